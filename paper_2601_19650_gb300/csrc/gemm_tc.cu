@@ -26,8 +26,9 @@
 // Kernel: persistent, one CTA per SM (cta_group::1) looping over 128 x BN output tiles of
 // all the problems of a call (a lockstep group of CBC instances is one call).  Warp 0
 // issues TMA loads of 64-wide K atoms (S slices of A and of B per atom, 128B swizzle,
-// two smem stages), warp 1 issues tcgen05.mma (one elected thread) into S TMEM
-// accumulators per K chunk, double buffered across chunks and tiles so the epilogue of
+// two smem stages), warp 1 issues tcgen05.mma (one elected thread; one MMA per slice of A,
+// against all the slices of B it meets side by side) into S TMEM accumulators per K chunk,
+// double buffered across chunks and tiles so the epilogue of
 // one chunk overlaps the MMAs of the next, and 4 (BN = 32) or 8 (BN = 64) epilogue warps
 // drain TMEM (tcgen05.ld) into int64 registers and write FP64, assembled with integer
 // operations.  Every wait is bounded (clock64); a timeout raises CBC_ERR_TIMEOUT in the
@@ -236,7 +237,8 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
   constexpr int B_BYTES = BN * KA * 2;
   constexpr int STAGE_BYTES = S * (A_BYTES + B_BYTES);
   constexpr uint32_t TMEM_COLS = 512;
-  static_assert(2 * S * BN <= 512, "TMEM budget");
+  static_assert(2 * S * BN <= 512, "TMEM budget");  // hence S BN <= 256, the widest MMA
+  static_assert(BN % 16 == 0, "MMA width");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
@@ -321,7 +323,6 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16(BM, BN);
       int jg = 0, cg = 0;  // atoms consumed, chunks issued (TMEM buffer cg & 1)
       bool run = true;
       for (int t = blockIdx.x; t < a.total_tiles && run; t += gridDim.x) {
@@ -345,18 +346,22 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
             tc_fence_after();
             const uint32_t sA = smem_u32(smem + stage * STAGE_BYTES);
             const uint32_t sB = sA + S * A_BYTES;
+            // One MMA per slice of A: the slices 0 .. S-1-s of B lie back to back in shared
+            // memory and the accumulators of the levels s .. S-1 they belong to (slice t of
+            // B: level s + t) back to back in TMEM, so they are one operand of (S-s) BN
+            // columns.  Issued one pair of slices at a time the MMAs were bound by reading
+            // A's 4 KB from shared memory again for every BN columns (8192 x 4096 x 1024
+            // complex, S = 5: 5.1 ms; stacked 3.3 ms, then bound by L2 reads of the slices).  s = 0 covers every
+            // level, so its first MMA of a chunk clears them all.
 #pragma unroll
-            for (int g = 0; g < S; ++g) {
-              const uint32_t d = tmem_base + (uint32_t)((buf * S + g) * BN);
+            for (int kk = 0; kk < KA / 16; ++kk) {
 #pragma unroll
-              for (int s = 0; s <= g; ++s) {
-                const int tt = g - s;
-#pragma unroll
-                for (int kk = 0; kk < KA / 16; ++kk) {
-                  uint64_t ad = sdesc_sw128(sA + s * A_BYTES + kk * 32);
-                  uint64_t bd = sdesc_sw128(sB + tt * B_BYTES + kk * 32);
-                  umma_bf16(d, ad, bd, idesc, (first && s == 0 && kk == 0) ? 0u : 1u);
-                }
+              for (int s = 0; s < S; ++s) {
+                const uint32_t d = tmem_base + (uint32_t)((buf * S + s) * BN);
+                const uint64_t ad = sdesc_sw128(sA + s * A_BYTES + kk * 32);
+                const uint64_t bd = sdesc_sw128(sB + kk * 32);
+                umma_bf16(d, ad, bd, idesc_bf16(BM, (S - s) * BN),
+                          (first && s == 0 && kk == 0) ? 0u : 1u);
               }
             }
             first = false;
