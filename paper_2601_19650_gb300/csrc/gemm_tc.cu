@@ -33,6 +33,7 @@
 // drain TMEM (tcgen05.ld) into int64 registers and write FP64, assembled with integer
 // operations.  Every wait is bounded (clock64); a timeout raises CBC_ERR_TIMEOUT in the
 // status word, all roles leave their loops, and TMEM is freed before the CTA exits.
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
@@ -458,15 +459,17 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
 }
 
 // ---------------- operand slicing ----------------
-// Logical rows are the rows of A, or the columns of B for the B^T side.  Two kernels:
-// the exponent of every logical row (max over K), then 32 x 32 tiles that are read
-// along whichever index is contiguous in memory, cut into slices in shared memory and
-// written to the [S][rows_pad][K2_pad] planes coalesced along K.
-template <typename T, bool SIDE_B>
-__device__ __forceinline__ T load_op(const T* src, const View& v, int r, int k, int conj) {
-  T x = SIDE_B ? src[v.roff(k) + v.coff(r)] : src[v.roff(r) + v.coff(k)];
-  return conj ? ops<T>::conj(x) : x;
-}
+// Logical rows are the rows of A, or the columns of B for the B^T side.  One launch cuts
+// both operands: a CTA takes 32 logical rows and a share of K, the CTAs of a cluster share
+// those rows' K range.  The elements are read once, along whichever index is contiguous in
+// memory, into shared memory (up to PACK_KEEP tiles; a longer share is read a second time,
+// from L2), the rows' exponents are combined through the cluster's shared memory, and the
+// slices leave coalesced along K to the [S][rows][K2_pad] planes.  Bound by HBM: 16 B read
+// and 4 S (A) or 8 S (B) B written per complex element.  Rows of padding are not written:
+// they reach only rows and columns of the accumulators that the epilogue skips.
+constexpr int PACK_ROWS = 32;
+constexpr int PACK_KEEP = 4;     // tiles held in shared memory
+constexpr int PACK_CLUSTER = 8;  // most CTAs that share the K range of one row block
 
 // exponent of |x| (biased-exponent field) without FP64 arithmetic: max|x| < 2^e with
 // e = field - 1022 for normal numbers; 0 maps to a floor value
@@ -479,61 +482,16 @@ __device__ __forceinline__ int expo_bits(double x) {
   return f - 1022;
 }
 
-// exponent of every logical row: 32 rows x 256 k per CTA, read along the contiguous
-// index, reduced in shared memory, combined across CTAs with an integer atomicMax
-template <typename T, bool SIDE_B>
-__global__ void __launch_bounds__(256) expo_kernel(const T* src, View v, int R, int K,
-                                                   int rowlanes, int* expo, int ebs, int* status) {
-  using O = ops<T>;
-  __shared__ int red[32][9];
-  src += (int64_t)blockIdx.z * v.bs;  // problem blockIdx.z of a batch
-  expo += (int64_t)blockIdx.z * ebs;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 256;
-  int best[4] = {-2000, -2000, -2000, -2000};
-  if (rowlanes) {  // lane -> row, warp -> k stripe
-    const int r = r0 + lane;
-    int b = -2000;
-    if (r < R)
-      for (int k = k0 + w; k < min(K, k0 + 256); k += 8) {
-        const T x = load_op<T, SIDE_B>(src, v, r, k, 0);
-        b = max(b, max(expo_bits(O::real(x)), expo_bits(O::imag(x))));
-      }
-    red[lane][w] = b;
-  } else {         // lane -> k, warp -> row group of 4
-    for (int q = 0; q < 4; ++q) {
-      const int r = r0 + w * 4 + q;
-      int b = -2000;
-      if (r < R)
-        for (int k = k0 + lane; k < min(K, k0 + 256); k += 32) {
-          const T x = load_op<T, SIDE_B>(src, v, r, k, 0);
-          b = max(b, max(expo_bits(O::real(x)), expo_bits(O::imag(x))));
-        }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
-      best[q] = b;
-    }
-    if (lane == 0)
-      for (int q = 0; q < 4; ++q) red[w * 4 + q][0] = best[q];
-  }
-  __syncthreads();
-  if (tid < 32) {
-    int b = red[tid][0];
-    if (rowlanes)
-      for (int q = 1; q < 8; ++q) b = max(b, red[tid][q]);
-    if (b >= 0x40000000) set_status(status, CBC_ERR_NUMERICAL);  // Inf or NaN in the row
-    if (r0 + tid < R && b > -2000) atomicMax(expo + r0 + tid, b);
-  }
-}
-
 // Balanced base-256 digits of t = x 2^(7-e) (|t| < 128): N = rint(t 256^(S-1)) (round to
-// nearest, ties to even), then the digits q_{S-1} .. q_1 are the balanced remainders of N
-// by 256 (in [-128, 127]) and q_0 the remaining quotient (|q_0| <= 128), so
-// t = sum_s q_s 256^-s up to 0.5 256^-(S-1).  N is taken straight from the bit pattern of
-// x (mantissa shifted with the rounding done on the bits that fall off): integer
-// operations only, since a scaling and an FP64-to-integer conversion per value would run
-// on the narrow FP64 pipe of this part.
-__device__ __forceinline__ void digits(double x, int e, int S, int (&q)[5]) {
+// nearest, ties to even), then t = sum_s q_s 256^-s up to 0.5 256^-(S-1) with q_1 .. q_{S-1}
+// the balanced remainders of N by 256 (in [-128, 127]) and q_0 the remaining quotient
+// (|q_0| <= 128).  N is taken straight from the bit pattern of x (mantissa shifted with the
+// rounding done on the bits that fall off): integer operations only, since a scaling and an
+// FP64-to-integer conversion per value would run on the narrow FP64 pipe of this part.
+// Returned is N + sum_{i<S-1} 128 256^i: its byte i is q_{S-1-i} + 128 for i < S-1, and its
+// bits from 8 (S-1) up are q_0.
+template <int S>
+__device__ __forceinline__ long long digit_word(double x, int e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7ffu);
   const unsigned long long mant = (b & 0xfffffffffffffull) | (ex ? (1ull << 52) : 0ull);
@@ -551,82 +509,167 @@ __device__ __forceinline__ void digits(double x, int e, int S, int (&q)[5]) {
     N = (long long)qq;
   }
   if (b >> 63) N = -N;
-  for (int sl = S - 1; sl >= 1; --sl) {
-    const long long hi = (N + 128) >> 8;  // floor((N + 128) / 256)
-    q[sl] = (int)(N - (hi << 8));
-    N = hi;
-  }
-  q[0] = (int)N;
+  constexpr long long bias = (long long)(0x8080808080808080ull & ((1ull << (8 * (S - 1))) - 1ull));
+  return N + bias;
 }
 
-__device__ __forceinline__ uint32_t bf16x2_bits(double lo, double hi) {
-  __nv_bfloat162 p = __floats2bfloat162_rn((float)lo, (float)hi);
-  return *reinterpret_cast<uint32_t*>(&p);
+// digit q_s as the bits of a float (exact; its upper half is the bf16): 2^23 + 128 + q is
+// formed by placing the byte in the mantissa of 2^23
+template <int S>
+__device__ __forceinline__ uint32_t digit_f32(long long w, int s) {
+  const uint32_t u = (s == 0) ? (uint32_t)((int)(w >> (8 * (S - 1))) + 128)
+                              : (uint32_t)(w >> (8 * (S - 1 - s))) & 0xffu;
+  return __float_as_uint(__uint_as_float(0x4b000000u | u) - 8388736.0f);
+}
+__device__ __forceinline__ uint32_t bf16_pair(uint32_t flo, uint32_t fhi) {
+  return __byte_perm(flo, fhi, 0x7632);
 }
 
-template <typename T, bool SIDE_B, bool ROWLANES>
-__global__ void __launch_bounds__(256) slice_kernel(const T* src, View v, int conj, int R, int K,
-                                                    int K2p, size_t plane, int S,
-                                                    __nv_bfloat16* out, const int* expo, int ebs,
-                                                    int rows_pad) {
+template <typename T>
+struct PackSide {
+  const T* src;
+  View v;              // of the operand as a matrix: rows x K for A, K x columns for B
+  int conj, rows, rowlanes;
+  __nv_bfloat16* out;  // planes; problem p at row block p
+  int* expo;           // exponents of the logical rows, ebs per problem
+  int ebs, rows_pad;   // packed rows of one problem in a plane
+};
+template <typename T>
+struct PackArgs {
+  PackSide<T> a, b;
+  int blocks_a;        // row blocks of A (then those of B)
+  int K, K2p, tiles_per_cta;
+  size_t plane_a, plane_b;
+  int* status;
+};
+
+template <typename T, bool SIDE_B, int S>
+__device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T>& o, size_t plane,
+                                          int block, T* tiles, int* s_max, int* s_exp) {
   using O = ops<T>;
   constexpr bool CPLX = O::cplx;
-  // problem blockIdx.z of a batch: its source, exponents and packed rows
-  src += (int64_t)blockIdx.z * v.bs;
-  expo += (int64_t)blockIdx.z * ebs;
-  out += (size_t)blockIdx.z * rows_pad * K2p;
-  __shared__ T tile[32][33];
-  __shared__ int se[32];
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 32;
-  for (int q = tid >> 5; q < 32; q += 8) {
-    const int r = ROWLANES ? r0 + lane : r0 + q;
-    const int k = ROWLANES ? k0 + q : k0 + lane;
-    T x = (r < R && k < K) ? load_op<T, SIDE_B>(src, v, r, k, conj) : O::zero();
-    if (ROWLANES)
-      tile[lane][q] = x;
-    else
-      tile[q][lane] = x;
+  constexpr int KT = CPLX ? 32 : 64;  // logical K of a tile: one 64-wide packed atom
+  constexpr int LD = KT + 1;
+  constexpr int NQ = PACK_ROWS * KT / 256;
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int nranks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int r0 = block * PACK_ROWS;
+  const T* src = o.src + (int64_t)blockIdx.z * o.v.bs;
+  const int ntiles = g.K2p / KA;
+  const int t_begin = rank * g.tiles_per_cta;
+  const int t_end = min(ntiles, t_begin + g.tiles_per_cta);
+  const bool keep = g.tiles_per_cta <= PACK_KEEP;
+  auto off_r = [&](int r) -> int64_t { return SIDE_B ? o.v.coff(r) : o.v.roff(r); };
+  auto off_k = [&](int k) -> int64_t { return SIDE_B ? o.v.roff(k) : o.v.coff(k); };
+  // element q of this thread in a tile.  Rows on the lanes: row = lane, k = warp + 8 q; K on
+  // the lanes: k = lane (+ 32), row = warp + 8 (q mod 4)
+  const bool rl = o.rowlanes != 0;
+  int64_t ro[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int r = r0 + (rl ? lane : warp + 8 * q);
+    ro[q] = r < o.rows ? off_r(r) : -1;
   }
-  if (tid < 32) {
-    const int e = expo[r0 + tid];
-    se[tid] = (e < -1100) ? 0 : e;  // all-zero (or padding) rows
-  }
+  int best[4] = {-2000, -2000, -2000, -2000};
+  auto load_tile = [&](int t, T* dst) {
+    T x[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int k = t * KT + (rl ? warp + 8 * q : lane + 32 * (q >> 2));
+      const int64_t rr = ro[q & 3];
+      x[q] = (rr >= 0 && k < g.K) ? src[rr + off_k(k)] : O::zero();
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      if (rl)
+        dst[lane * LD + warp + 8 * q] = x[q];
+      else
+        dst[(warp + 8 * (q & 3)) * LD + lane + 32 * (q >> 2)] = x[q];
+      const int b = max(expo_bits(O::real(x[q])), expo_bits(O::imag(x[q])));
+      best[q & 3] = max(best[q & 3], b);
+    }
+  };
+  if (tid < PACK_ROWS) s_max[tid] = -2000;
   __syncthreads();
-  // 32 logical rows x 32 logical k; real: one bf16 per (row, k); complex: one bf16 pair
-  constexpr int NPR = (CPLX && SIDE_B) ? 2 : 1;  // packed rows per logical row
-  for (int idx = tid; idx < 32 * 32 * NPR; idx += 256) {
-    const int kk = idx & 31;
-    const int prl = idx >> 5;            // packed row within the tile
-    const int lr = prl / NPR, half = prl % NPR;
-    const T x = tile[lr][kk];
-    const int e = se[lr];
-    const int prow = (r0 + lr) * NPR + half;
-    if constexpr (!CPLX) {
-      int q[5];
-      digits(O::real(x), e, S, q);
-      __nv_bfloat16* o = out + (size_t)prow * K2p + (k0 + kk);
-      for (int sl = 0; sl < S; ++sl) o[sl * plane] = __float2bfloat16_rn((float)q[sl]);
-    } else {
-      double a0, a1;  // the two K positions of this (packed row, k)
-      const double xr = O::real(x), xi = O::imag(x);
-      if (!SIDE_B) {
-        a0 = xr;
-        a1 = xi;
-      } else if (half == 0) {
-        a0 = xr;   // row 2n:   [ br, -bi ]
-        a1 = -xi;
-      } else {
-        a0 = xi;   // row 2n+1: [ bi,  br ]
-        a1 = xr;
-      }
-      int q0[5], q1[5];
-      digits(a0, e, S, q0);
-      digits(a1, e, S, q1);
-      uint32_t* o = reinterpret_cast<uint32_t*>(out) + ((size_t)prow * K2p + 2 * (k0 + kk)) / 2;
-      for (int sl = 0; sl < S; ++sl) o[sl * (plane / 2)] = bf16x2_bits(q0[sl], q1[sl]);
+  for (int t = t_begin; t < t_end; ++t) load_tile(t, tiles + (keep ? (t - t_begin) * PACK_ROWS * LD : 0));
+  if (rl) {
+    atomicMax(s_max + lane, max(max(best[0], best[1]), max(best[2], best[3])));
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      int b = best[q];
+#pragma unroll
+      for (int w = 16; w > 0; w >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, w));
+      if (lane == 0) s_max[warp + 8 * q] = b;
     }
   }
+  __syncthreads();
+  if (nranks > 1) cluster.sync();
+  if (tid < PACK_ROWS) {
+    int b = s_max[tid];
+    for (int q = 0; q < nranks; ++q)
+      if (q != rank) b = max(b, cluster.map_shared_rank(s_max, q)[tid]);
+    if (b >= 0x40000000) set_status(g.status, CBC_ERR_NUMERICAL);  // Inf or NaN in the row
+    b = (b < -1100) ? 0 : b;  // an all-zero (or padding) row
+    s_exp[tid] = b;
+    if (rank == 0 && r0 + tid < o.rows) o.expo[(int64_t)blockIdx.z * o.ebs + r0 + tid] = b;
+  }
+  __syncthreads();
+  uint32_t* out = reinterpret_cast<uint32_t*>(o.out + (size_t)blockIdx.z * o.rows_pad * g.K2p);
+  const size_t pl = plane / 2, ld = (size_t)g.K2p / 2;  // in words of two bf16
+  for (int t = t_begin; t < t_end; ++t) {
+    const T* tile = tiles;
+    if (keep) {
+      tile += (t - t_begin) * PACK_ROWS * LD;
+    } else {
+      __syncthreads();
+      load_tile(t, tiles);
+      __syncthreads();
+    }
+#pragma unroll 1
+    for (int q = 0; q < 4; ++q) {
+      const int lr = warp + 8 * q;
+      if (r0 + lr >= o.rows) continue;
+      const int e = s_exp[lr];
+      if constexpr (!CPLX) {
+        const long long w0 = digit_word<S>(tile[lr * LD + 2 * lane], e);
+        const long long w1 = digit_word<S>(tile[lr * LD + 2 * lane + 1], e);
+        uint32_t* d = out + (size_t)(r0 + lr) * ld + t * 32 + lane;
+#pragma unroll
+        for (int sl = 0; sl < S; ++sl)
+          d[sl * pl] = bf16_pair(digit_f32<S>(w0, sl), digit_f32<S>(w1, sl));
+      } else {
+        T x = tile[lr * LD + lane];
+        if (o.conj) x = O::conj(x);
+        const long long wr = digit_word<S>(O::real(x), e), wi = digit_word<S>(O::imag(x), e);
+        uint32_t* d = out + (size_t)(SIDE_B ? 2 : 1) * (r0 + lr) * ld + t * 32 + lane;
+#pragma unroll
+        for (int sl = 0; sl < S; ++sl) {
+          const uint32_t fr = digit_f32<S>(wr, sl), fi = digit_f32<S>(wi, sl);
+          if (!SIDE_B) {
+            d[sl * pl] = bf16_pair(fr, fi);
+          } else {  // rows 2n: [br, -bi] and 2n + 1: [bi, br]
+            d[sl * pl] = bf16_pair(fr, fi ^ 0x80000000u);
+            d[sl * pl + ld] = bf16_pair(fi, fr);
+          }
+        }
+      }
+    }
+  }
+  if (nranks > 1) cluster.sync();  // no CTA leaves while another still reads its row maxima
+}
+
+template <typename T, int S>
+__global__ void __launch_bounds__(256) pack_kernel(PackArgs<T> g) {
+  extern __shared__ __align__(16) unsigned char pack_smem[];
+  __shared__ int s_max[PACK_ROWS], s_exp[PACK_ROWS];
+  T* tiles = reinterpret_cast<T*>(pack_smem);
+  const int block = blockIdx.x / (int)cooperative_groups::this_cluster().num_blocks();
+  if (block < g.blocks_a)
+    pack_rows<T, false, S>(g, g.a, g.plane_a, block, tiles, s_max, s_exp);
+  else
+    pack_rows<T, true, S>(g, g.b, g.plane_b, block - g.blocks_a, tiles, s_max, s_exp);
 }
 
 // strides of the logical (row, k) indices at the origin, to pick the read pattern
@@ -637,26 +680,45 @@ bool rows_contiguous(const View& v) {
   return sr == 1 && sk != 1;
 }
 
-// nb problems (sources v.bs elements apart) go to consecutive row blocks of the planes
-template <typename T, bool SIDE_B>
-void pack_operand(const T* src, const View& v, bool conj, int R, int K, int rows_pad, int K2p,
-                  int S, __nv_bfloat16* out, int* expo, int* status, cudaStream_t s, int nb) {
-  constexpr bool CPLX = ops<T>::cplx;
-  const int nrows = (CPLX && SIDE_B) ? rows_pad / 2 : rows_pad;  // logical rows (padded)
-  const int klog = CPLX ? K2p / 2 : K2p;                           // logical K (padded)
-  const bool rl = rows_contiguous<SIDE_B>(v);
-  note_launches(CBC_K_AUX, 2);
-  cudaMemsetAsync(expo, 0xC0, sizeof(int) * nrows * nb, s);  // a large negative floor
-  expo_kernel<T, SIDE_B><<<dim3((K + 255) / 256, (nrows + 31) / 32, nb), 256, 0, s>>>(
-      src, v, R, K, rl ? 1 : 0, expo, nrows, status);
-  dim3 grid(klog / 32, nrows / 32, nb);
-  const size_t plane = (size_t)nb * rows_pad * K2p;
-  if (rl)
-    slice_kernel<T, SIDE_B, true><<<grid, 256, 0, s>>>(src, v, conj ? 1 : 0, R, K, K2p, plane, S,
-                                                       out, expo, nrows, rows_pad);
-  else
-    slice_kernel<T, SIDE_B, false><<<grid, 256, 0, s>>>(src, v, conj ? 1 : 0, R, K, K2p, plane, S,
-                                                        out, expo, nrows, rows_pad);
+template <typename T, int S>
+cudaError_t launch_pack(PackArgs<T> g, int nb, cudaStream_t s) {
+  constexpr int KT = ops<T>::cplx ? 32 : 64;
+  const void* k = (const void*)pack_kernel<T, S>;
+  cudaError_t e = allow_max_smem(k);
+  if (e != cudaSuccess) return e;
+  const int tiles = g.K2p / KA;
+  // as many CTAs along K as keep their share in shared memory, up to PACK_CLUSTER
+  int cs = 1;
+  while (cs < PACK_CLUSTER && cs * PACK_KEEP < tiles) cs *= 2;
+  g.tiles_per_cta = (tiles + cs - 1) / cs;
+  const int held = g.tiles_per_cta <= PACK_KEEP ? g.tiles_per_cta : 1;
+  const size_t smem = (size_t)held * PACK_ROWS * (KT + 1) * sizeof(T);
+  const int blocks = g.blocks_a + (g.b.rows + PACK_ROWS - 1) / PACK_ROWS;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)cs * blocks, 1, nb);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  note_launches(CBC_K_AUX, 1);
+  return cudaLaunchKernelEx(&cfg, pack_kernel<T, S>, g);
+}
+
+// both operands of nb problems (sources v.bs elements apart) into their planes
+template <typename T>
+cudaError_t pack_operands(const PackArgs<T>& g, int S, int nb, cudaStream_t s) {
+  switch (S) {
+    case 2: return launch_pack<T, 2>(g, nb, s);
+    case 3: return launch_pack<T, 3>(g, nb, s);
+    case 4: return launch_pack<T, 4>(g, nb, s);
+    default: return launch_pack<T, 5>(g, nb, s);
+  }
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -822,8 +884,18 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
   int* eb = reinterpret_cast<int*>(w);
   if (K <= 0) return cudaErrorInvalidValue;
   // slices of A (rows) and of B (columns, embedded); problem p owns row block p
-  pack_operand<T, false>(A, va, conjA, M, K, g.Mp, g.K2p, S, sa, ea, status, s, nb);
-  pack_operand<T, true>(B, vb, conjB, N, K, g.N2p, g.K2p, S, sb, eb, status, s, nb);
+  PackArgs<T> pk{};
+  pk.a = {A, va, conjA ? 1 : 0, M, rows_contiguous<false>(va) ? 1 : 0, sa, ea, g.Mp, g.Mp};
+  pk.b = {B, vb, conjB ? 1 : 0, N, rows_contiguous<true>(vb) ? 1 : 0, sb, eb,
+          CPLX ? g.N2p / 2 : g.N2p, g.N2p};
+  pk.blocks_a = (M + PACK_ROWS - 1) / PACK_ROWS;
+  pk.K = K;
+  pk.K2p = g.K2p;
+  pk.plane_a = b * g.Mp * g.K2p;
+  pk.plane_b = b * g.N2p * g.K2p;
+  pk.status = status;
+  cudaError_t pe = pack_operands<T>(pk, S, nb, s);
+  if (pe != cudaSuccess) return pe;
   CUtensorMap ma;
   if (!make_map(&ma, sa, g.K2p, nb * g.Mp, S, BM)) return cudaErrorInvalidValue;
   const int atoms = g.K2p / KA;
