@@ -70,7 +70,9 @@ enum cbc_dtype { CBC_F32 = 0, CBC_F64 = 1, CBC_C64 = 2, CBC_C128 = 3 };
 
 /* Arithmetic of cbc_apply.
  * CBC_PREC_FP64 : every contraction, Gram matrix, eigensolve, Cholesky and triangular
- *                 solve in FP64 (the plain baseline).
+ *                 solve in FP64.  Products whose operands' rows span less than 2^36 run on
+ *                 the tensor cores with 8 bf16 slices per operand, summed exactly and
+ *                 rounded to FP64 at the end; the others on the FP64 pipes.
  * CBC_PREC_MIXED: the dense contractions and Gram products run on the tensor cores
  *                 (tcgen05) with bf16 operand slices and FP32 partial sums that are
  *                 combined in FP64; the eigensolve, Cholesky and triangular solves stay
@@ -250,7 +252,7 @@ int ttno_destroy(ttno_t t); /* NULL is a no-op */
 /* Dense product used by every contraction of the sweeps, exposed as a building block
  * (and for kernel-level tests): C = op(A) op(B) with row-major DEVICE matrices of
  * dtype CBC_F64 or CBC_C128.  op(X) = X, X^T (trans), conj(X) (conj) or X^H (both).
- *   precision  CBC_PREC_FP64: FP64 SIMT; CBC_PREC_MIXED: tensor cores with `slices`
+ *   precision  CBC_PREC_FP64: FP64 accuracy (see cbc_apply); CBC_PREC_MIXED: tensor cores with `slices`
  *              bf16 slices per operand (2..5; 0 = 4), exact FP32 partial sums, FP64
  *              result (see cbc_apply)
  *   M, N, K    op(A) is M x K, op(B) is K x N, C is M x N (ldc >= N), K >= 1
@@ -309,7 +311,7 @@ int cbc_selftest_wait(long long limit_cycles, int* returned_out, void* stream);
  * Gram matrix counts only its Hermitian half).  Not thread safe across concurrent
  * cbc_apply calls.                                                                  */
 enum cbc_kclass {
-  CBC_K_GEMM_F64 = 0, /* FP64 SIMT contractions and Gram products                     */
+  CBC_K_GEMM_F64 = 0, /* FP64 contractions and Gram products                          */
   CBC_K_GEMM_TC = 1,  /* tcgen05 split-precision contractions and Gram products        */
   CBC_K_EIG = 2,      /* truncation eigensolver after the tridiagonal reduction        */
   CBC_K_CHOLQR = 3,   /* Cholesky and triangular solves of CholeskyQR2                */

@@ -79,8 +79,9 @@ int cholqr2_t(int m, int n, int nb, T* S, cudaStream_t s) {
   if (e == cudaSuccess) e = row_norms2<T>(S, m, n, n, sbs, rn, s, nb);
   if (e == cudaSuccess) e = scale_rows<T>(S, m, n, sbs, rn, s, nb);
   for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
-    e = gemm_f64<T>(m, m, n, nb, S, View::rowmajor(n, sbs), false, S, View::transposed(n, sbs),
-                    true, G, View::rowmajor(m, (int64_t)m * m), s);
+    e = gemm_f64_pooled<T>(m, m, n, nb, S, View::rowmajor(n, sbs), false, S,
+                           View::transposed(n, sbs), true, G, View::rowmajor(m, (int64_t)m * m),
+                           status, s);
     if (e == cudaSuccess) e = cholesky_lower<T>(G, m, status, bar, num_sms(), s, nb);
     if (e == cudaSuccess) e = trsm_lower_left<T>(G, S, m, n, status, bar, num_sms(), s, nb);
   }

@@ -682,10 +682,10 @@ int cbc_gemm(int precision, int slices, int dtype, int M, int N, int K, const vo
                                  conjB, (double*)C, vc, slices, ws, status, s);
     }
   } else if (e == cudaSuccess) {
-    e = cplx ? gemm_f64<zdbl>(M, N, K, 1, (const zdbl*)A, va, conjA, (const zdbl*)B, vb, conjB,
-                              (zdbl*)C, vc, s)
-             : gemm_f64<double>(M, N, K, 1, (const double*)A, va, conjA, (const double*)B, vb,
-                                conjB, (double*)C, vc, s);
+    e = cplx ? gemm_f64_pooled<zdbl>(M, N, K, 1, (const zdbl*)A, va, conjA, (const zdbl*)B, vb,
+                                   conjB, (zdbl*)C, vc, status, s)
+             : gemm_f64_pooled<double>(M, N, K, 1, (const double*)A, va, conjA, (const double*)B,
+                                     vb, conjB, (double*)C, vc, status, s);
   }
   int hs = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, s);

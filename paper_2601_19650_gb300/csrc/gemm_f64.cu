@@ -1,8 +1,8 @@
-// FP64 SIMT strided GEMM: the arithmetic of the plain-FP64 CBC path.
+// FP64 SIMT strided GEMM: the products of the plain-FP64 CBC path that the tensor cores do
+// not take (gemm_f64_split in gemm_tc.cu): short K, operands of a very wide range or with
+// Inf or NaN, and callers without room for slices.
 //
-// Every contraction of Sec. III (Eqs. (tt_cbc_first_contraction) ...
-// (cbc_final_contraction)) and every Gram product is one call of this kernel on leg
-// views of the node tensors (kernels.cuh: View).  On GB300 the FP64 pipe delivers
+// It works on leg views of the node tensors (kernels.cuh: View).  On GB300 the FP64 pipe delivers
 // about 2 DFMA per clock per SM, so this kernel is FP64-throughput bound by design: a
 // 64x64 output tile per CTA, 16-deep K slices staged in shared memory, 4x4 outputs
 // per thread, and a K split (FP64 atomics into a zeroed C) when the output tiles
@@ -26,6 +26,8 @@ struct GemmArgs {
   View vb;
   T* C;
   View vc;
+  const int* cond;  // not NULL: run only if *cond is set
+  int tiles_n, tiles_m, total;  // tiles of one (problem, split); of the launch
 };
 
 template <typename T, bool CA, bool CB, bool ATOMIC>
@@ -36,93 +38,97 @@ __global__ void __launch_bounds__(NT) gemm_f64_kernel(GemmArgs<T> g) {
   __shared__ int64_t a_row[BM];
   __shared__ int64_t b_col[BN];
 
+  if (g.cond && !*g.cond) return;
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
-  const int bm = blockIdx.y * BM, bn = blockIdx.x * BN;
-  const int batch = blockIdx.z / g.splits;
-  const int split = blockIdx.z % g.splits;
-  const int kbeg = split * g.kchunk;
-  const int kend = min(g.K, kbeg + g.kchunk);
+  for (int tile = blockIdx.x; tile < g.total; tile += gridDim.x) {
+    const int bn = tile % g.tiles_n * BN, bm = tile / g.tiles_n % g.tiles_m * BM;
+    const int z = tile / (g.tiles_n * g.tiles_m);
+    const int batch = z / g.splits;
+    const int split = z % g.splits;
+    const int kbeg = split * g.kchunk;
+    const int kend = min(g.K, kbeg + g.kchunk);
 
-  const T* A = g.A + (int64_t)batch * g.va.bs;
-  const T* B = g.B + (int64_t)batch * g.vb.bs;
-  T* C = g.C + (int64_t)batch * g.vc.bs;
+    const T* A = g.A + (int64_t)batch * g.va.bs;
+    const T* B = g.B + (int64_t)batch * g.vb.bs;
+    T* C = g.C + (int64_t)batch * g.vc.bs;
 
-  for (int i = tid; i < BM; i += NT) a_row[i] = (bm + i < g.M) ? g.va.roff(bm + i) : -1;
-  for (int i = tid; i < BN; i += NT) b_col[i] = (bn + i < g.N) ? g.vb.coff(bn + i) : -1;
-  __syncthreads();
-
-  T acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = O::zero();
-
-  for (int k0 = kbeg; k0 < kend; k0 += BK) {
-    // A tile: BM x BK, consecutive threads walk K (the contiguous leg of most views)
-#pragma unroll
-    for (int q = 0; q < (BM * BK) / NT; ++q) {
-      int idx = tid + q * NT;
-      int kk = idx % BK, mm = idx / BK;
-      int k = k0 + kk;
-      T v = O::zero();
-      int64_t ro = a_row[mm];
-      if (ro >= 0 && k < kend) {
-        v = A[ro + g.va.coff(k)];
-        if (CA) v = O::conj(v);
-      }
-      As[kk][mm] = v;
-    }
-    // B tile: BK x BN, consecutive threads walk N
-#pragma unroll
-    for (int q = 0; q < (BN * BK) / NT; ++q) {
-      int idx = tid + q * NT;
-      int nn = idx % BN, kk = idx / BN;
-      int k = k0 + kk;
-      T v = O::zero();
-      int64_t co = b_col[nn];
-      if (co >= 0 && k < kend) {
-        v = B[g.vb.roff(k) + co];
-        if (CB) v = O::conj(v);
-      }
-      Bs[kk][nn] = v;
-    }
+    for (int i = tid; i < BM; i += NT) a_row[i] = (bm + i < g.M) ? g.va.roff(bm + i) : -1;
+    for (int i = tid; i < BN; i += NT) b_col[i] = (bn + i < g.N) ? g.vb.coff(bn + i) : -1;
     __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      T a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = O::fma(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
 
+    T acc[4][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int r = bm + ty + 16 * i;
-    if (r >= g.M) continue;
-    int64_t ro = g.vc.roff(r);
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int c = bn + tx + 16 * j;
-      if (c >= g.N) continue;
-      T* dst = C + ro + g.vc.coff(c);
-      if (ATOMIC) {
-        if constexpr (O::cplx) {
-          double* d = reinterpret_cast<double*>(dst);
-          atomicAdd(d, O::real(acc[i][j]));
-          atomicAdd(d + 1, O::imag(acc[i][j]));
-        } else {
-          atomicAdd(reinterpret_cast<double*>(dst), O::real(acc[i][j]));
+      for (int j = 0; j < 4; ++j) acc[i][j] = O::zero();
+
+    for (int k0 = kbeg; k0 < kend; k0 += BK) {
+      // A tile: BM x BK, consecutive threads walk K (the contiguous leg of most views)
+#pragma unroll
+      for (int q = 0; q < (BM * BK) / NT; ++q) {
+        int idx = tid + q * NT;
+        int kk = idx % BK, mm = idx / BK;
+        int k = k0 + kk;
+        T v = O::zero();
+        int64_t ro = a_row[mm];
+        if (ro >= 0 && k < kend) {
+          v = A[ro + g.va.coff(k)];
+          if (CA) v = O::conj(v);
         }
-      } else {
-        *dst = acc[i][j];
+        As[kk][mm] = v;
+      }
+      // B tile: BK x BN, consecutive threads walk N
+#pragma unroll
+      for (int q = 0; q < (BN * BK) / NT; ++q) {
+        int idx = tid + q * NT;
+        int nn = idx % BN, kk = idx / BN;
+        int k = k0 + kk;
+        T v = O::zero();
+        int64_t co = b_col[nn];
+        if (co >= 0 && k < kend) {
+          v = B[g.vb.roff(k) + co];
+          if (CB) v = O::conj(v);
+        }
+        Bs[kk][nn] = v;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int kk = 0; kk < BK; ++kk) {
+        T a[4], b[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = O::fma(a[i], b[j], acc[i][j]);
+      }
+      __syncthreads();
+    }
+
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      int r = bm + ty + 16 * i;
+      if (r >= g.M) continue;
+      int64_t ro = g.vc.roff(r);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        int c = bn + tx + 16 * j;
+        if (c >= g.N) continue;
+        T* dst = C + ro + g.vc.coff(c);
+        if (ATOMIC) {
+          if constexpr (O::cplx) {
+            double* d = reinterpret_cast<double*>(dst);
+            atomicAdd(d, O::real(acc[i][j]));
+            atomicAdd(d + 1, O::imag(acc[i][j]));
+          } else {
+            atomicAdd(reinterpret_cast<double*>(dst), O::real(acc[i][j]));
+          }
+        } else {
+          *dst = acc[i][j];
+        }
       }
     }
   }
@@ -148,7 +154,7 @@ int g_num_sms = 0;
 template <typename T>
 cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va, bool conjA,
                      const T* B, const View& vb, bool conjB, T* C, const View& vc,
-                     cudaStream_t s) {
+                     cudaStream_t s, const int* cond) {
   if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
   if (g_num_sms == 0) {
     int dev = 0;
@@ -160,7 +166,7 @@ cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va,
   int ksteps = (K + BK - 1) / BK;
   int splits = 1;
   int target = 2 * g_num_sms;
-  if (tiles < target && ksteps >= 16) {
+  if (!cond && tiles < target && ksteps >= 16) {
     splits = (target + tiles - 1) / tiles;
     splits = min(splits, ksteps / 8);
     splits = max(splits, 1);
@@ -172,8 +178,10 @@ cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va,
     zero_view_kernel<T><<<256, 256, 0, s>>>(C, vc, M, N, batch);
     return cudaGetLastError();
   }
-  GemmArgs<T> g{M, N, K, splits, kchunk, A, va, B, vb, C, vc};
-  dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, batch * splits);
+  GemmArgs<T> g{M,  N, K,  splits, kchunk, A, va, B, vb, C, vc, cond,
+                (N + BN - 1) / BN, (M + BM - 1) / BM, tiles * splits};
+  // a product that usually does not run (cond) is launched as one resident wave
+  const int grid = cond ? std::min(g.total, target) : g.total;
   note_launches(CBC_K_GEMM_F64, splits > 1 ? 2 : 1);
   if (splits > 1) {
     int zb = (int)std::min<int64_t>(4096, ((int64_t)M * N * batch + 255) / 256);
@@ -199,9 +207,9 @@ cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va,
 
 template cudaError_t gemm_f64<double>(int, int, int, int, const double*, const View&, bool,
                                       const double*, const View&, bool, double*, const View&,
-                                      cudaStream_t);
+                                      cudaStream_t, const int*);
 template cudaError_t gemm_f64<zdbl>(int, int, int, int, const zdbl*, const View&, bool,
                                     const zdbl*, const View&, bool, zdbl*, const View&,
-                                    cudaStream_t);
+                                    cudaStream_t, const int*);
 
 }  // namespace cbc

@@ -16,7 +16,9 @@
 // hence exact.  The epilogue warps read the S level sums of a chunk from TMEM,
 // convert them to integers and fold them into one int64 per output element,
 // I += sum_g C_g << 8(S-1-g); the final value is 2^(ea+eb-14-8(S-1)) * I in FP64.
-// With S slices an operand keeps ~8S-1 bits relative to its row maximum.
+// With S slices an operand keeps ~8S-1 bits relative to its row maximum.  2 to 5 slices
+// serve the mixed path; 8 serve the FP64 path (gemm_f64_split at the end of this file), with
+// x = 2^(e-6) sum_s 2^(-8s) q_s and the level sums in two int64 per output element.
 //
 // Complex operands use the real 2x2 embedding: A' = [re, im] interleaved along K
 // (M x 2K) and B' = [[br, bi], [-bi, br]] blocks (2K x 2N), so C' = A' B' holds
@@ -25,8 +27,8 @@
 //
 // Kernel: persistent, one CTA per SM (cta_group::1) looping over 128 x BN output tiles of
 // all the problems of a call (a lockstep group of CBC instances is one call).  Warp 0
-// issues TMA loads of 64-wide K atoms (S slices of A and of B per atom, 128B swizzle,
-// two smem stages), warp 1 issues tcgen05.mma (one elected thread; one MMA per slice of A,
+// issues TMA loads of 64-wide K atoms (32-wide for 8 slices; S slices of A and of B per
+// atom, 128B or 64B swizzle, two smem stages), warp 1 issues tcgen05.mma (one elected thread; one MMA per slice of A,
 // against all the slices of B it meets side by side) into S TMEM accumulators per K chunk,
 // double buffered across chunks and tiles so the epilogue of
 // one chunk overlaps the MMAs of the next, and 4 (BN = 32) or 8 (BN = 64) epilogue warps
@@ -50,7 +52,13 @@ namespace cbc {
 namespace tc {
 
 constexpr int BM = 128;          // rows of the output tile (TMEM lanes)
-constexpr int KA = 64;           // bf16 elements per K atom (one 128-byte swizzle row)
+constexpr int KA = 64;           // K is padded to this many bf16 elements
+// bf16 elements per K atom of a smem stage: one 128-byte swizzle row, or one of 64 bytes
+// for 8 slices, of which two stages of 128-byte rows do not fit in shared memory
+__host__ __device__ constexpr int ka(int S) { return S > 5 ? 32 : 64; }
+// an operand element is x = 2^(e - head) (q_0 + q_1 2^-8 + ...): 8 slices keep one bit less
+// so that the digit word and its bias fit in 64 bits
+__host__ __device__ constexpr int head(int S) { return S > 5 ? 6 : 7; }
 constexpr int NSTAGE = 2;
 // warps: 0 TMA, 1 MMA, then 4 epilogue warps (one per TMEM lane quarter) per group of 32
 // accumulator columns, or of 16 when BN is not a multiple of 32 (BN = 48)
@@ -109,15 +117,17 @@ __device__ __forceinline__ void tma_load_3d(const CUtensorMap* map, uint64_t* ba
       : "memory");
 }
 
-// UMMA shared-memory descriptor: K-major tile, 128-byte swizzle, 8-row core groups
-// 1024 bytes apart.
-__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
+// UMMA shared-memory descriptor: K-major tile of ROWB-byte rows with the swizzle of that
+// width, 8-row core groups back to back.
+template <int ROWB>
+__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
+  static_assert(ROWB == 128 || ROWB == 64, "swizzle width");
   uint64_t d = 0;
   d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
   d |= (uint64_t)1 << 16;               // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(1024 >> 4) << 32;     // stride byte offset
+  d |= (uint64_t)(8 * ROWB >> 4) << 32; // stride byte offset
   d |= (uint64_t)1 << 46;               // descriptor version of the tcgen05 family
-  d |= (uint64_t)2 << 61;               // 128-byte swizzle
+  d |= (uint64_t)(ROWB == 128 ? 2 : 4) << 61;  // 128-byte or 64-byte swizzle
   return d;
 }
 
@@ -181,7 +191,7 @@ __device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[CW]) {
 
 struct TcArgs {
   int M, N2;             // real-embedded output rows / columns
-  int atoms_total;       // K2_pad / 64
+  int atoms_total;       // K2_pad / ka(S)
   int atoms_per_split;   // multiple of atoms_per_chunk
   int atoms_per_chunk;
   const int* expA;       // [M_pad]
@@ -191,6 +201,7 @@ struct TcArgs {
   char* C;               // FP64 output (double or zdbl) through the view
   View vc;               // vc.bs: elements between the outputs of consecutive problems
   int* status;
+  const int* skip;       // not NULL: nothing runs when *skip is set (see split_f64)
   int splits;            // K splits per problem
   int Mp, N2p;           // packed rows of one problem in the A and B planes
   int ebsB;              // entries of expB per problem
@@ -230,16 +241,35 @@ __device__ __noinline__ double i64_ldexp(long long a, int e) {
                                           (mant & ((1ull << 52) - 1ull))));
 }
 
+// ldexp(hi 2^32 + lo, e) with one rounding: the 128-bit sum is shifted down to 63 bits with
+// the bits that fall off kept as a sticky bit, which rounds the same way
+__device__ __noinline__ double i96_ldexp(long long hi, long long lo, int e) {
+  const __int128 t = ((__int128)hi << 32) + (__int128)lo;
+  const bool neg = t < 0;
+  const unsigned __int128 m = neg ? -(unsigned __int128)t : (unsigned __int128)t;
+  const unsigned long long top = (unsigned long long)(m >> 64);
+  unsigned long long w = (unsigned long long)m;
+  int sh = 0;
+  if (top != 0ull || (w >> 63)) {
+    sh = 65 - (top ? __clzll((long long)top) : 64);
+    const unsigned __int128 rest = m & (((unsigned __int128)1 << sh) - 1);
+    w = (unsigned long long)(m >> sh) | (rest != 0 ? 1ull : 0ull);
+  }
+  return i64_ldexp(neg ? -(long long)w : (long long)w, e + sh);
+}
+
 template <int S, int BN>
 __global__ void __launch_bounds__(nthreads(BN), 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    TcArgs a) {
-  constexpr int A_BYTES = BM * KA * 2;
-  constexpr int B_BYTES = BN * KA * 2;
+  constexpr int KAS = ka(S);
+  constexpr int A_BYTES = BM * KAS * 2;
+  constexpr int B_BYTES = BN * KAS * 2;
   constexpr int STAGE_BYTES = S * (A_BYTES + B_BYTES);
   constexpr uint32_t TMEM_COLS = 512;
   static_assert(2 * S * BN <= 512, "TMEM budget");  // hence S BN <= 256, the widest MMA
   static_assert(BN % 16 == 0, "MMA width");
+  if (a.skip && *a.skip) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
@@ -312,7 +342,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
           uint8_t* sA = smem + stage * STAGE_BYTES;
           uint8_t* sB = sA + S * A_BYTES;
           mbar_expect_tx(full + stage, STAGE_BYTES);
-          const int k = (q.a_begin + j) * KA;
+          const int k = (q.a_begin + j) * KAS;
 #pragma unroll
           for (int s = 0; s < S; ++s) {
             tma_load_3d(&tmA, full + stage, sA + s * A_BYTES, k, q.prob * a.Mp + q.m0, s);
@@ -355,12 +385,12 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
             // complex, S = 5: 5.1 ms; stacked 3.3 ms, then bound by L2 reads of the slices).  s = 0 covers every
             // level, so its first MMA of a chunk clears them all.
 #pragma unroll
-            for (int kk = 0; kk < KA / 16; ++kk) {
+            for (int kk = 0; kk < KAS / 16; ++kk) {
 #pragma unroll
               for (int s = 0; s < S; ++s) {
                 const uint32_t d = tmem_base + (uint32_t)((buf * S + s) * BN);
-                const uint64_t ad = sdesc_sw128(sA + s * A_BYTES + kk * 32);
-                const uint64_t bd = sdesc_sw128(sB + kk * 32);
+                const uint64_t ad = sdesc<2 * KAS>(sA + s * A_BYTES + kk * 32);
+                const uint64_t bd = sdesc<2 * KAS>(sB + kk * 32);
                 umma_bf16(d, ad, bd, idesc_bf16(BM, (S - s) * BN),
                           (first && s == 0 && kk == 0) ? 0u : 1u);
               }
@@ -386,9 +416,12 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
     for (int t = blockIdx.x; t < a.total_tiles && run; t += gridDim.x) {
       const Tile q = tile_of(t);
       const int row = q.m0 + quarter * 32 + lane;
-      long long acc[CW];
+      // 8 slices span 2 x 32 bits more than one int64 holds: levels 0-3 and 4-7 apart
+      constexpr int NACC = S > 5 ? 2 : 1;
+      constexpr int LV = S / NACC;  // levels per accumulator
+      long long acc[NACC][CW];
 #pragma unroll
-      for (int i = 0; i < CW; ++i) acc[i] = 0;
+      for (int i = 0; i < NACC * CW; ++i) acc[i / CW][i % CW] = 0;
       for (int c = 0; c < q.n_chunks; ++c, ++cg) {
         const int buf = cg & 1, use = cg >> 1;
         if (!mbar_wait(tfull + buf, use & 1, abort_flag, a.status)) {
@@ -398,7 +431,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
         tc_fence_after();
 #pragma unroll
         for (int g = 0; g < S; ++g) {
-          const int shift = 8 * (S - 1 - g);
+          const int shift = 8 * (LV - 1 - g % LV);
           uint32_t r[CW];
           tmem_ld<CW>(tmem_base + ((uint32_t)(quarter * 32) << 16) +
                           (uint32_t)((buf * S + g) * BN + colg * CW),
@@ -406,7 +439,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
 #pragma unroll
           for (int i = 0; i < CW; ++i) {
             long long qv = (long long)__float2int_rn(__uint_as_float(r[i]));
-            acc[i] += qv << shift;
+            acc[g / LV][i] += qv << shift;
           }
         }
         tc_fence_before();
@@ -426,7 +459,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
         const int myexp = myok ? expB[myn] : 0;
         const bool rowok = row < a.M;
         const int ea = rowok ? a.expA[q.prob * a.Mp + row] : 0;
-        const int bias = -14 - 8 * (S - 1);
+        const int bias = -2 * head(S) - 8 * (S - 1);
         const int64_t ro = rowok ? a.vc.roff(row) : 0;
 #pragma unroll
         for (int i = 0; i < CW; ++i) {
@@ -434,7 +467,11 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
           const int eb = __shfl_sync(0xffffffffu, myexp, i);
           const int col = q.n0 + colg * CW + i;
           if (rowok && col < a.N2) {
-            const double v = i64_ldexp(acc[i], ea + eb + bias);
+            double v;
+            if constexpr (NACC == 2)
+              v = i96_ldexp(acc[0][i], acc[1][i], ea + eb + bias);
+            else
+              v = i64_ldexp(acc[0][i], ea + eb + bias);
             double* dst;
             if (a.cplx)
               dst = reinterpret_cast<double*>(Cp + 16 * (ro + co)) + (col & 1);
@@ -468,6 +505,10 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
 // and 4 S (A) or 8 S (B) B written per complex element.  Rows of padding are not written:
 // they reach only rows and columns of the accumulators that the epilogue skips.
 constexpr int PACK_ROWS = 32;
+// FP64 products as 8 slices (gemm_f64_split): an operand whose rows span more than this many
+// powers of two, or that holds Inf or NaN, is left to the SIMT kernel.  Within it every entry
+// keeps at least 62 - 36 bits and the largest ones all 53; Gaussian rows span about 2^25.
+constexpr int SPLIT_RANGE = 36;
 constexpr int PACK_KEEP = 4;     // tiles held in shared memory
 constexpr int PACK_CLUSTER = 8;  // most CTAs that share the K range of one row block
 
@@ -482,7 +523,7 @@ __device__ __forceinline__ int expo_bits(double x) {
   return f - 1022;
 }
 
-// Balanced base-256 digits of t = x 2^(7-e) (|t| < 128): N = rint(t 256^(S-1)) (round to
+// Balanced base-256 digits of t = x 2^(head-e) (|t| < 2^head): N = rint(t 256^(S-1)) (round to
 // nearest, ties to even), then t = sum_s q_s 256^-s up to 0.5 256^-(S-1) with q_1 .. q_{S-1}
 // the balanced remainders of N by 256 (in [-128, 127]) and q_0 the remaining quotient
 // (|q_0| <= 128).  N is taken straight from the bit pattern of x (mantissa shifted with the
@@ -495,7 +536,7 @@ __device__ __forceinline__ long long digit_word(double x, int e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7ffu);
   const unsigned long long mant = (b & 0xfffffffffffffull) | (ex ? (1ull << 52) : 0ull);
-  const int k = (ex ? ex : 1) - 1075 + 7 + 8 * (S - 1) - e;  // N = rint(mant 2^k)
+  const int k = (ex ? ex : 1) - 1075 + head(S) + 8 * (S - 1) - e;  // N = rint(mant 2^k)
   long long N;
   if (k >= 0) {
     N = (long long)(mant << min(k, 63));
@@ -541,11 +582,13 @@ struct PackArgs {
   int K, K2p, tiles_per_cta;
   size_t plane_a, plane_b;
   int* status;
+  int* wide;           // not NULL: set when an operand does not suit the split (split_f64)
 };
 
 template <typename T, bool SIDE_B, int S>
 __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T>& o, size_t plane,
-                                          int block, T* tiles, int* s_max, int* s_exp) {
+                                          int block, T* tiles, int* s_max, int* s_min,
+                                          int* s_exp) {
   using O = ops<T>;
   constexpr bool CPLX = O::cplx;
   constexpr int KT = CPLX ? 32 : 64;  // logical K of a tile: one 64-wide packed atom
@@ -572,6 +615,7 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
     ro[q] = r < o.rows ? off_r(r) : -1;
   }
   int best[4] = {-2000, -2000, -2000, -2000};
+  int low[4] = {2000, 2000, 2000, 2000};
   auto load_tile = [&](int t, T* dst) {
     T x[NQ];
 #pragma unroll
@@ -586,15 +630,23 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
         dst[lane * LD + warp + 8 * q] = x[q];
       else
         dst[(warp + 8 * (q & 3)) * LD + lane + 32 * (q >> 2)] = x[q];
-      const int b = max(expo_bits(O::real(x[q])), expo_bits(O::imag(x[q])));
-      best[q & 3] = max(best[q & 3], b);
+      const int br = expo_bits(O::real(x[q])), bi = expo_bits(O::imag(x[q]));
+      best[q & 3] = max(best[q & 3], max(br, bi));
+      if constexpr (S > 5) {  // the smallest nonzero entry
+        if (br > -2000) low[q & 3] = min(low[q & 3], br);
+        if (bi > -2000) low[q & 3] = min(low[q & 3], bi);
+      }
     }
   };
-  if (tid < PACK_ROWS) s_max[tid] = -2000;
+  if (tid < PACK_ROWS) {
+    s_max[tid] = -2000;
+    s_min[tid] = 2000;
+  }
   __syncthreads();
   for (int t = t_begin; t < t_end; ++t) load_tile(t, tiles + (keep ? (t - t_begin) * PACK_ROWS * LD : 0));
   if (rl) {
     atomicMax(s_max + lane, max(max(best[0], best[1]), max(best[2], best[3])));
+    if constexpr (S > 5) atomicMin(s_min + lane, min(min(low[0], low[1]), min(low[2], low[3])));
   } else {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -602,15 +654,23 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
 #pragma unroll
       for (int w = 16; w > 0; w >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, w));
       if (lane == 0) s_max[warp + 8 * q] = b;
+      if constexpr (S > 5) atomicMin(s_min + warp + 8 * q, low[q]);
     }
   }
   __syncthreads();
   if (nranks > 1) cluster.sync();
   if (tid < PACK_ROWS) {
-    int b = s_max[tid];
+    int b = s_max[tid], lo = s_min[tid];
     for (int q = 0; q < nranks; ++q)
-      if (q != rank) b = max(b, cluster.map_shared_rank(s_max, q)[tid]);
-    if (b >= 0x40000000) set_status(g.status, CBC_ERR_NUMERICAL);  // Inf or NaN in the row
+      if (q != rank) {
+        b = max(b, cluster.map_shared_rank(s_max, q)[tid]);
+        if constexpr (S > 5) lo = min(lo, cluster.map_shared_rank(s_min, q)[tid]);
+      }
+    if constexpr (S > 5) {
+      if (b >= 0x40000000 || (lo < 2000 && b - lo > SPLIT_RANGE)) *g.wide = 1;
+    } else if (b >= 0x40000000) {
+      set_status(g.status, CBC_ERR_NUMERICAL);  // Inf or NaN in the row
+    }
     b = (b < -1100) ? 0 : b;  // an all-zero (or padding) row
     s_exp[tid] = b;
     if (rank == 0 && r0 + tid < o.rows) o.expo[(int64_t)blockIdx.z * o.ebs + r0 + tid] = b;
@@ -663,13 +723,13 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
 template <typename T, int S>
 __global__ void __launch_bounds__(256) pack_kernel(PackArgs<T> g) {
   extern __shared__ __align__(16) unsigned char pack_smem[];
-  __shared__ int s_max[PACK_ROWS], s_exp[PACK_ROWS];
+  __shared__ int s_max[PACK_ROWS], s_min[PACK_ROWS], s_exp[PACK_ROWS];
   T* tiles = reinterpret_cast<T*>(pack_smem);
   const int block = blockIdx.x / (int)cooperative_groups::this_cluster().num_blocks();
   if (block < g.blocks_a)
-    pack_rows<T, false, S>(g, g.a, g.plane_a, block, tiles, s_max, s_exp);
+    pack_rows<T, false, S>(g, g.a, g.plane_a, block, tiles, s_max, s_min, s_exp);
   else
-    pack_rows<T, true, S>(g, g.b, g.plane_b, block - g.blocks_a, tiles, s_max, s_exp);
+    pack_rows<T, true, S>(g, g.b, g.plane_b, block - g.blocks_a, tiles, s_max, s_min, s_exp);
 }
 
 // strides of the logical (row, k) indices at the origin, to pick the read pattern
@@ -717,6 +777,7 @@ cudaError_t pack_operands(const PackArgs<T>& g, int S, int nb, cudaStream_t s) {
     case 2: return launch_pack<T, 2>(g, nb, s);
     case 3: return launch_pack<T, 3>(g, nb, s);
     case 4: return launch_pack<T, 4>(g, nb, s);
+    case 8: return launch_pack<T, 8>(g, nb, s);
     default: return launch_pack<T, 5>(g, nb, s);
   }
 }
@@ -735,20 +796,21 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-bool make_map(CUtensorMap* m, void* base, int K2_pad, int rows_pad, int S, int box_rows) {
+bool make_map(CUtensorMap* m, void* base, int K2_pad, int64_t rows_pad, int S, int box_rows) {
   auto fn = encode_fn();
   if (!fn) return false;
   cuuint64_t dims[3] = {(cuuint64_t)K2_pad, (cuuint64_t)rows_pad, (cuuint64_t)S};
   cuuint64_t strides[2] = {(cuuint64_t)K2_pad * 2, (cuuint64_t)rows_pad * K2_pad * 2};
-  cuuint32_t box[3] = {(cuuint32_t)KA, (cuuint32_t)box_rows, 1};
+  cuuint32_t box[3] = {(cuuint32_t)ka(S), (cuuint32_t)box_rows, 1};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, es,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  ka(S) == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
 
-int atoms_per_chunk_for(int S) { return std::max(1, (1024 / S) / KA); }
+int atoms_per_chunk_for(int S) { return std::max(1, (1024 / S) / ka(S)); }
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct Geo {
@@ -767,8 +829,13 @@ Geo geometry(int M, int N, int K, bool cplx, int S) {
 
 // Tile widths a slice count can use: two sets of S accumulators of BN columns fit the
 // 512 TMEM columns of an SM (2 S BN <= 512) and two smem stages of S (128 + BN) x 64 bf16
-// fit the 227 KB opt-in shared memory.  S = 5: 32 or 48; S = 4: 32 or 64; S <= 3: 64.
+// fit the 227 KB opt-in shared memory.  S = 5: 32 or 48; S = 4: 32 or 64; S <= 3: 64;
+// S = 8: 32.
 int bn_candidates(int S, int (&out)[2]) {
+  if (S == 8) {
+    out[0] = 32;
+    return 1;
+  }
   if (S == 5) {
     out[0] = 32;
     out[1] = 48;
@@ -785,7 +852,7 @@ int bn_candidates(int S, int (&out)[2]) {
 
 template <int S, int BN>
 constexpr size_t smem_bytes() {
-  return (size_t)NSTAGE * S * (BM * KA * 2 + BN * KA * 2) + 1024 + 256;
+  return (size_t)NSTAGE * S * (BM + BN) * ka(S) * 2 + 1024 + 256;
 }
 
 template <int S, int BN>
@@ -812,6 +879,7 @@ cudaError_t launch(int S, int BN, const CUtensorMap& ma, const CUtensorMap& mb, 
     case 4064: return launch_bn<4, 64>(ma, mb, args, grid, s);
     case 5032: return launch_bn<5, 32>(ma, mb, args, grid, s);
     case 5048: return launch_bn<5, 48>(ma, mb, args, grid, s);
+    case 8032: return launch_bn<8, 32>(ma, mb, args, grid, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -831,6 +899,17 @@ std::map<TuneKey, int> g_tuned;
 int g_sms = 0;
 
 }  // namespace tc
+
+namespace {
+// The SIMT kernel walks K at ~1 us (real) or ~4 us (complex) per 16 terms whatever M and N
+// are, the split costs ~10 us of launches more.  cbc_gemm in all, SIMT / split:
+//   real     256 x 256: K = 16 46 / 57 us, 64 100 / 58; 128 x 128 x 32 63 / 56;
+//            1000 x 1000 x 16 61 / 79, x 1000 2107 / 142
+//   complex  16 x 16 x 16 96 / 55, 1000 x 1000 x 8 158 / 106, 128 x 2048 x 128 556 / 69,
+//            1000^3 8097 / 389 us
+constexpr int SPLIT_MIN_K_REAL = 28, SPLIT_MIN_K_CPLX = 8;
+constexpr size_t SPLIT_MAX_BYTES = size_t(16) << 30;
+}  // namespace
 
 size_t gemm_tc_workspace_bytes(int M, int N, int K, bool cplx, int S, int nb) {
   using namespace tc;
@@ -856,14 +935,14 @@ static View transpose_view(const View& v) {
 template <typename T>
 cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA, const T* B,
                     const View& vb, bool conjB, T* C, const View& vc, int S, void* ws,
-                    int* status, cudaStream_t s, int nb) {
+                    int* status, cudaStream_t s, int nb, int* wide) {
   using namespace tc;
   if (M <= 0 || N <= 0 || nb <= 0) return cudaSuccess;
-  if (S < 2 || S > 5) return cudaErrorInvalidValue;
+  if ((S < 2 || S > 5) && !(S == 8 && wide)) return cudaErrorInvalidValue;
   // keep the long dimension on the 128-row side: C^T = B^T A^T
   if (M < BM && N > M) {
     return gemm_tc<T>(N, M, K, B, transpose_view(vb), conjB, A, transpose_view(va), conjA, C,
-                      transpose_view(vc), S, ws, status, s, nb);
+                      transpose_view(vc), S, ws, status, s, nb, wide);
   }
   constexpr bool CPLX = ops<T>::cplx;
   if (g_sms == 0) {
@@ -894,11 +973,12 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
   pk.plane_a = b * g.Mp * g.K2p;
   pk.plane_b = b * g.N2p * g.K2p;
   pk.status = status;
+  pk.wide = wide;
   cudaError_t pe = pack_operands<T>(pk, S, nb, s);
   if (pe != cudaSuccess) return pe;
   CUtensorMap ma;
   if (!make_map(&ma, sa, g.K2p, nb * g.Mp, S, BM)) return cudaErrorInvalidValue;
-  const int atoms = g.K2p / KA;
+  const int atoms = g.K2p / ka(S);
   const int apc = atoms_per_chunk_for(S);
   const int chunks = (atoms + apc - 1) / apc;
   // one launch with tile width BN; a partial last column tile reads the next problem's
@@ -925,6 +1005,7 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
     args.C = reinterpret_cast<char*>(C);
     args.vc = vc;
     args.status = status;
+    args.skip = wide;
     args.splits = splits;
     args.Mp = g.Mp;
     args.N2p = g.N2p;
@@ -938,8 +1019,9 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
     args.tiles_n = tiles_n;
     args.total_tiles = args.tiles_m * args.tiles_n * splits * nb;
     dim3 grid(std::min(args.total_tiles, g_sms));
-    note_launches(CBC_K_GEMM_TC, 1);
-    note_flops(CBC_K_TC_ISSUED,
+    note_launches(S == 8 ? CBC_K_GEMM_F64 : CBC_K_GEMM_TC, 1);
+    if (S != 8)
+      note_flops(CBC_K_TC_ISSUED,
                2.0 * g.Mp * ((double)tiles_n * BN) * g.K2p * (S * (S + 1) / 2) * nb);
     return launch(S, BN, ma, mb, args, grid, s);
   };
@@ -981,11 +1063,44 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
   return e;
 }
 
+// ---- FP64 products on the tensor cores -------------------------------------------------
+// 8 slices hold 62 bits of an entry relative to its row's (column's) maximum and their
+// products are summed exactly, so the only rounding is the one to 53 bits at the end (one
+// more per K split): on rows that span fewer powers of two than SPLIT_RANGE the error is
+// below that of an FP64 sum.  Operands outside that are found while they are cut; then the
+// tensor-core kernel returns at once and the SIMT kernel behind it does the product.
+// Relative error against 80-bit sums, Gaussian entries: 4e-17 to 2e-16 where the SIMT kernel
+// has 1e-16 (K = 16) to 1e-15 (K = 1000).
+size_t gemm_f64_split_bytes(int M, int N, int K, bool cplx, int nb) {
+  if (K < (cplx ? SPLIT_MIN_K_CPLX : SPLIT_MIN_K_REAL)) return 0;
+  const size_t b = gemm_tc_workspace_bytes(M, N, K, cplx, 8, nb) + 256;
+  return b <= SPLIT_MAX_BYTES ? b : 0;
+}
+
+template <typename T>
+cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& va, bool conjA,
+                           const T* B, const View& vb, bool conjB, T* C, const View& vc, void* ws,
+                           int* status, cudaStream_t s) {
+  int* wide = static_cast<int*>(ws);
+  cudaError_t e = cudaMemsetAsync(wide, 0, sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  e = gemm_tc<T>(M, N, K, A, va, conjA, B, vb, conjB, C, vc, 8, static_cast<char*>(ws) + 256,
+                 status, s, nb, wide);
+  if (e != cudaSuccess) return e;
+  return gemm_f64<T>(M, N, K, nb, A, va, conjA, B, vb, conjB, C, vc, s, wide);
+}
+
+template cudaError_t gemm_f64_split<double>(int, int, int, int, const double*, const View&, bool,
+                                            const double*, const View&, bool, double*,
+                                            const View&, void*, int*, cudaStream_t);
+template cudaError_t gemm_f64_split<zdbl>(int, int, int, int, const zdbl*, const View&, bool,
+                                          const zdbl*, const View&, bool, zdbl*, const View&,
+                                          void*, int*, cudaStream_t);
 template cudaError_t gemm_tc<double>(int, int, int, const double*, const View&, bool,
                                      const double*, const View&, bool, double*, const View&, int,
-                                     void*, int*, cudaStream_t, int);
+                                     void*, int*, cudaStream_t, int, int*);
 template cudaError_t gemm_tc<zdbl>(int, int, int, const zdbl*, const View&, bool, const zdbl*,
                                    const View&, bool, zdbl*, const View&, int, void*, int*,
-                                   cudaStream_t, int);
+                                   cudaStream_t, int, int*);
 
 }  // namespace cbc

@@ -60,7 +60,17 @@ struct View {
 template <typename T>
 cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va, bool conjA,
                      const T* B, const View& vb, bool conjB, T* C, const View& vc,
-                     cudaStream_t s);
+                     cudaStream_t s, const int* cond = nullptr);
+// (cond: a device word; not NULL: the product runs only if it is set.)
+
+// The FP64 product as 8 bf16 slices per operand on the tensor cores, with an error no larger
+// than gemm_f64's (gemm_tc.cu).  gemm_f64_split_bytes gives the bytes it needs at `ws`, or 0
+// where gemm_f64 is to be used: small products, and slices beyond 16 GB.
+size_t gemm_f64_split_bytes(int M, int N, int K, bool cplx, int nb);
+template <typename T>
+cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& va, bool conjA,
+                           const T* B, const View& vb, bool conjB, T* C, const View& vc, void* ws,
+                           int* status, cudaStream_t s);
 
 // The same product on the tensor cores with S bf16 slices per operand (gemm_tc.cu);
 // `ws` must hold gemm_tc_workspace_bytes(M, N, K, cplx, S, nb) bytes.  nb problems of
@@ -69,7 +79,7 @@ size_t gemm_tc_workspace_bytes(int M, int N, int K, bool cplx, int S, int nb = 1
 template <typename T>
 cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA, const T* B,
                     const View& vb, bool conjB, T* C, const View& vc, int S, void* ws,
-                    int* status, cudaStream_t s, int nb = 1);
+                    int* status, cudaStream_t s, int nb = 1, int* wide = nullptr);
 
 // ---- Hermitian eigensolver (FP64): A (m x m, row-major, overwritten) -----------------
 // Finds the eigenvalues in descending order and the eigenvectors of the `k` largest,

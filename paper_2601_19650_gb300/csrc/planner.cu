@@ -36,6 +36,16 @@ struct Arena {
     ptrs.push_back(p);
     return static_cast<T*>(p);
   }
+  // room that the caller can do without: NULL, and no error kept, when there is none
+  void* try_get(size_t bytes) {
+    void* p = nullptr;
+    if (pool_malloc(&p, bytes, s) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    ptrs.push_back(p);
+    return p;
+  }
   // scopes: release() frees (stream-ordered) everything allocated after mark()
   size_t mark() const { return ptrs.size(); }
   void release(size_t mk) {
@@ -135,6 +145,19 @@ cudaError_t tgemm(const Prec& pr, bool fwd, bool gram, int M, int N, int K, cons
     }
     pr.ar->release(mk);  // the slices are dead once the launch is queued
     return e;
+  }
+  const size_t wb = gemm_f64_split_bytes(M, N, K, ops<T>::cplx, pr.nb);
+  if (wb > 0) {
+    const size_t mk = pr.ar->mark();
+    if (void* ws = pr.ar->try_get(wb)) {
+      cudaError_t e;
+      {
+        KTimer t(CBC_K_GEMM_F64, s, 0, fl);
+        e = gemm_f64_split<T>(M, N, K, pr.nb, A, va, ca, B, vb, cb, C, vc, ws, pr.status, s);
+      }
+      pr.ar->release(mk);
+      return e;
+    }
   }
   KTimer t(CBC_K_GEMM_F64, s, 0, fl);
   return gemm_f64<T>(M, N, K, pr.nb, A, va, ca, B, vb, cb, C, vc, s);

@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "../../include/cbc.h"
+#include "kernels.cuh"
 
 namespace cbc {
 
@@ -115,6 +116,23 @@ void note_flops(int cls, double flops);
 // stream-ordered device allocation from the library's own pool on the current device
 // (freed with cudaFreeAsync); the caller's default pool is never touched
 cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t s);
+
+// gemm_f64_split with slices from the library's pool where that is the faster way and the
+// pool has room for them, else gemm_f64
+template <typename T>
+cudaError_t gemm_f64_pooled(int M, int N, int K, int nb, const T* A, const View& va, bool conjA,
+                            const T* B, const View& vb, bool conjB, T* C, const View& vc,
+                            int* status, cudaStream_t s) {
+  void* ws = nullptr;
+  const size_t wb = gemm_f64_split_bytes(M, N, K, ops<T>::cplx, nb);
+  if (wb > 0 && pool_malloc(&ws, wb, s) == cudaSuccess) {
+    cudaError_t e = gemm_f64_split<T>(M, N, K, nb, A, va, conjA, B, vb, conjB, C, vc, ws, status, s);
+    const cudaError_t f = cudaFreeAsync(ws, s);
+    return e != cudaSuccess ? e : f;
+  }
+  if (wb > 0) cudaGetLastError();  // no room: not an error
+  return gemm_f64<T>(M, N, K, nb, A, va, conjA, B, vb, conjB, C, vc, s);
+}
 
 int fail(int code, const char* fmt, ...);
 int cuda_fail(cudaError_t e, const char* what);

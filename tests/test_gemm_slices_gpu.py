@@ -24,3 +24,42 @@ def test_slicing_edges(K, trans, cplx):
     eb = 2.0 ** (np.floor(np.log2(np.abs(np.stack([b.real, b.imag])).max(axis=(0, 1)))) + 1)
     bound = (2 if cplx else 1) * K * np.outer(ea, eb) * 2.0 ** (-8 * S) * (3 + S * S / 2)
     assert np.all(np.abs(C - ref) <= bound)
+
+
+def _fp64_case(rng, M, N, K, cplx, grade=None):
+    A, B = _rand(rng, (M, K), cplx), _rand(rng, (K, N), cplx)
+    if grade is not None:  # entries of a row fall by 2^-grade along K
+        A = A * 2.0 ** (-np.linspace(0, grade, K))[None, :]
+    return A, B
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("shape", [(128, 64, 28), (1, 1, 8), (33, 31, 127), (129, 33, 129),
+                                   (256, 40, 1025), (65, 300, 4097)])
+@pytest.mark.parametrize("grade", [None, 20, 80])
+def test_fp64_split(shape, grade, cplx):
+    """FP64 products on the tensor cores and, for rows that span too much, behind them: the
+    componentwise bound K eps |A||B| of an FP64 sum (sqrt 2 more per complex product), in
+    80-bit arithmetic; split operands add at most 2^(e_a+e_b) K 2^-58."""
+    rng = np.random.default_rng(5)
+    M, N, K = shape
+    A, B = _fp64_case(rng, M, N, K, cplx, grade)
+    C, _ = _run(0, 0, A, B)
+    wide = np.clongdouble if cplx else np.longdouble
+    ref = A.astype(wide) @ B.astype(wide)
+    eps = 2.0 ** -53
+    bound = 4 * (K + 2) * eps * (np.abs(A) @ np.abs(B))
+    if grade != 80:
+        bound = bound + K * 2.0 ** -55 * np.outer(np.abs(A).max(1), np.abs(B).max(0))
+    assert np.all(np.abs(C - ref) <= bound)
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+def test_fp64_nonfinite_passes_through(bad):
+    """Inf and NaN go through an FP64 product as through any sum."""
+    rng = np.random.default_rng(9)
+    A, B = _fp64_case(rng, 70, 40, 64, False)
+    A[3, 5] = bad
+    C, ref = _run(0, 0, A, B)
+    assert np.array_equal(np.isnan(C), np.isnan(ref)) and np.array_equal(np.isinf(C), np.isinf(ref))
+    assert np.abs(np.delete(C, 3, 0) - np.delete(ref, 3, 0)).max() <= 1e-12
