@@ -128,17 +128,26 @@ __device__ __forceinline__ bool grid_sync(GridBarrier* bar, int* status,
   return s_ok != 0;
 }
 
-// 1/x for finite nonzero x by Newton-Raphson on f(r) = 1/r - x, r <- r (2 - x r),
-// started from the single-precision reciprocal of the mantissa (the exponent is split
-// off with frexp so any double works): ~23 -> 46 -> 92 correct bits.  Used where a
-// long dependent chain of FP64 divisions would otherwise dominate the latency.
+// 1/x for finite nonzero x: the hardware's ~20-bit FP64 approximation r, then one cubic
+// step r (1 + e + e^2) with e = 1 - x r (the Newton series of 1/x cut after the square, an
+// error of e^3).  A dependent FP64 operation takes ~64 clocks on this part and the
+// approximation ~19, so this chain is ~210 clocks; an FP32 seed behind frexp / ldexp and two
+// Newton steps took ~2.5 times that, in the chains that bound the eigensolver and Cholesky.
+// Arguments near the ends of the exponent range take that longer way.
 __device__ __forceinline__ double rcp64(double x) {
-  int ex;
-  double f = frexp(x, &ex);
+  const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+  if (ex - 3u < 2040u) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+  }
+  int sh;
+  double f = frexp(x, &sh);
   double r = (double)__frcp_rn((float)f);
   r = fma(r, fma(-f, r, 1.0), r);
   r = fma(r, fma(-f, r, 1.0), r);
-  return ldexp(r, -ex);
+  return ldexp(r, -sh);
 }
 
 // 1/sqrt(x) for finite x > 0 by Newton-Raphson on f(r) = 1/r^2 - x,
