@@ -168,6 +168,18 @@ __device__ __forceinline__ double rsqrt64(double x) {
   return ldexp(r, -ex / 2);
 }
 
+// The same in the way of rcp64: r (1 + e/2 + 3 e^2/8) with e = 1 - x r^2, five dependent
+// operations.  (The pivots of Cholesky keep rsqrt64: whether a rank-deficient block breaks
+// down hangs on its last bit.)
+__device__ __forceinline__ double rsqrt64_short(double x) {
+  const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+  if (ex - 1u >= 2046u) return rsqrt64(x);
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x * r, r, 1.0);
+  return fma(r, e * fma(0.375, e, 0.5), r);
+}
+
 // Row i of entry t of a packed lower triangle (t = i (i + 1) / 2 + c, 0 <= c <= i).  The
 // estimate comes from a single-precision square root (FP64 throughput per SM is two
 // orders of magnitude below FP32 on this part) and is corrected in integer arithmetic.

@@ -23,7 +23,6 @@
 
 #include <algorithm>
 #include <type_traits>
-#include <cstdlib>
 
 #include "df.cuh"
 #include "kernels.cuh"
@@ -208,16 +207,26 @@ __global__ void __launch_bounds__(TPB) tridiag_kernel(TriArgs<T> a) {
   }
 }
 
-// ---- tridiagonalisation with the rows in shared memory -----------------------------
-// Same reduction as tridiag_kernel, for m small enough that every CTA keeps its rows in
-// shared memory.  Column j needs two exchanges through global memory: the Householder
-// vector v_j (with tau_j) from the CTA that owns row j, and p = tau_j A v_j, one entry
-// from the owner of each row.  Both travel as plain data: the receiving buffers are
-// filled with the all-ones bit pattern before the launch, each entry is written once
-// with a relaxed store, and readers poll every entry until it differs from that
-// pattern, so no fence, counter or atomic sits on the dependency chain.  Each CTA also
-// publishes its share of v^H p (its own rows); every CTA adds the P shares in one fixed
-// order, so all CTAs apply the same rank-2 update.  Every wait is bounded.
+// ---- tridiagonalisation of a lone matrix with the rows in shared memory ----------------
+// For m <= 1024 with every CTA's rows r = cta + P t in its shared memory.  The reduction is
+// a chain of m columns, and what bounds it is that chain: one exchange between the CTAs
+// through L2 (~1600 clocks) and, on this part, ~64 clocks for every dependent FP64 operation
+// and for every FP64 instruction of a warp.  So per column:
+//   * one exchange.  Every CTA publishes A u for its own rows together with their entries of
+//     the next column; every CTA then forms w and the next column x by itself, with the same
+//     operations in the same order, so no Householder vector travels.  Both go out as plain
+//     data into buffers filled with the all-ones bit pattern before the launch, each entry
+//     written once with a relaxed store and polled until it differs from that pattern: no
+//     fence, counter or atomic on the chain.  Every wait is bounded.
+//   * the reflector unscaled, u = x - beta e_1 and H = I - gamma u u^H: only beta stands
+//     between the norm and A u; gamma and the scaled vector for the back transformation are
+//     formed while the exchange is under way.  u^H A u is real, so w = gamma A u + c u with a
+//     real c = -|gamma|^2 (u^H A u) / 2.
+//   * both sums over the block in integers: the terms are aligned to the largest one and
+//     added exactly (no FP64 instruction, and the same value in every CTA);
+//   * the rank-2 update of the rows while one warp computes beta.
+// Two exchanges per column and FP64 sums / this: m = 256 complex 2.93 / 1.40 ms, 64 0.55 /
+// 0.26 ms, 512 real 5.29 / 3.00 ms, 1000 real 13.7 / 9.0 ms.
 template <typename T>
 struct Tri2Args {
   const T* A;
@@ -225,17 +234,15 @@ struct Tri2Args {
   double* d;
   double* e;
   T* tau;
-  T* V;    // m x m; row j: [j] = tau_j, [j+1, m) = v_j; sentinel-filled before the launch
-  T* Pg;   // m x m; row j: [j+1, m) = tau_j A v_j;     sentinel-filled before the launch
-  T* Dg;   // (m-1) x P; [j][q] = CTA q's share of v_j^H p_j; sentinel-filled too
+  T* V;    // m x m; row j: [j+1, m) = v_j
+  T* X;    // m x m pairs; row j: [j+1, m) = (A u_j, column j+1 before its update by u_j);
+           // sentinel-filled before the launch
   int* status;
-  int P;            // CTAs per matrix; CTA b handles matrix b / P of a batch
-  int64_t a_bs;     // elements between consecutive matrices A
-  size_t wb;        // bytes between the workspaces (d .. Pg) of consecutive matrices
 };
 
 constexpr long long kSentinel = -1LL;  // all bits set: a NaN that arithmetic never yields
 constexpr long long kWaitCycles = 4000000000LL;
+constexpr int kLoneMaxM = 1024;
 
 __device__ __forceinline__ double pub_value(double x) {
   return (__double_as_longlong(x) == kSentinel) ? __longlong_as_double(0x7ff8000000000000LL) : x;
@@ -261,403 +268,291 @@ __device__ __forceinline__ bool ld_pub(const zdbl* p, zdbl* v) {
   return __double_as_longlong(x) != kSentinel && __double_as_longlong(y) != kSentinel;
 }
 
-
-// dst[lo, hi) <- src[lo, hi) as the entries get published (and their double-float forms
-// into ddst when given).  False (for the whole CTA) when a wait ran out or another CTA
-// has reported an error.
-template <typename T>
-__device__ bool gather_pub(const T* src, T* dst, int lo, int hi, int* status,
-                           typename dfof<T>::type* ddst = nullptr) {
-  bool ok = true;
-  for (int c = lo + threadIdx.x; c < hi && ok; c += blockDim.x) {
-    T v;
-    if (!ld_pub(src + c, &v)) {
-      const long long t0 = clock64();
-      while (!ld_pub(src + c, &v)) {
-        if (*((volatile int*)status) != 0) {
-          ok = false;
-          break;
-        }
-        if (clock64() - t0 > kWaitCycles) {
-          set_status(status, CBC_ERR_TIMEOUT);
-          ok = false;
-          break;
-        }
+// N pairs of published values at p[i] (skipped where p[i] is NULL), all loads in flight
+// together; false when the wait ran out or another CTA has reported an error
+template <typename T, int N>
+__device__ __forceinline__ bool wait_pairs(const T* const (&p)[N], T (&y)[N], T (&z)[N],
+                                           int* status) {
+  bool all = true;
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (p[i]) {
+      const bool a = ld_pub(p[i], &y[i]), b = ld_pub(p[i] + 1, &z[i]);
+      all = all && a && b;
+    }
+  if (all) return true;
+  const long long t0 = clock64();
+  while (true) {
+    all = true;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (p[i]) {
+        const bool a = ld_pub(p[i], &y[i]), b = ld_pub(p[i] + 1, &z[i]);
+        all = all && a && b;
       }
-    }
-    dst[c] = v;
-    if (ddst) ddst[c] = to_df(v);
-  }
-  return __syncthreads_and(ok) != 0;
-}
-
-// Two ranges in one polling pass (one barrier).
-template <typename T>
-__device__ bool gather_pub2(const T* s1, T* d1, int lo1, int hi1, const T* s2, T* d2, int lo2,
-                            int hi2, int* status) {
-  bool ok = true;
-  const int n1 = hi1 - lo1, n = n1 + (hi2 - lo2);
-  for (int q = threadIdx.x; q < n && ok; q += blockDim.x) {
-    const T* src = (q < n1) ? s1 + lo1 + q : s2 + lo2 + (q - n1);
-    T* dst = (q < n1) ? d1 + lo1 + q : d2 + lo2 + (q - n1);
-    T v;
-    if (!ld_pub(src, &v)) {
-      const long long t0 = clock64();
-      while (!ld_pub(src, &v)) {
-        if (*((volatile int*)status) != 0) {
-          ok = false;
-          break;
-        }
-        if (clock64() - t0 > kWaitCycles) {
-          set_status(status, CBC_ERR_TIMEOUT);
-          ok = false;
-          break;
-        }
-      }
-    }
-    *dst = v;
-  }
-  return __syncthreads_and(ok) != 0;
-}
-
-// (sum x, sum y) over the CTA; sh holds at least 66 doubles
-__device__ __forceinline__ double2 block_sum2(double x, double y, double* sh) {
-  x = warp_sum(x);
-  y = warp_sum(y);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (lane == 0) {
-    sh[w] = x;
-    sh[32 + w] = y;
-  }
-  __syncthreads();
-  if (w == 0) {
-    double a = (lane < nw) ? sh[lane] : 0.0, b = (lane < nw) ? sh[32 + lane] : 0.0;
-    a = warp_sum(a);
-    b = warp_sum(b);
-    if (lane == 0) {
-      sh[64] = a;
-      sh[65] = b;
+    if (all) return true;
+    if (*((volatile int*)status) != 0) return false;
+    if (clock64() - t0 > kWaitCycles) {
+      set_status(status, CBC_ERR_TIMEOUT);
+      return false;
     }
   }
-  __syncthreads();
-  return make_double2(sh[64], sh[65]);
 }
 
-// Householder vector of column j from the owner's updated row j (zlarfg convention:
-// H = I - tau v v^H, H^H x = beta e_1 with beta real); written to vs (shared) and
-// published to V.
-template <typename T>
-__device__ void householder_pub(const Tri2Args<T>& a, const T* row, int j, T* vs, double* sh) {
-  using O = ops<T>;
-  const int m = a.m;
-  double xn2 = 0.0;
-  for (int c = j + 2 + threadIdx.x; c < m; c += blockDim.x) xn2 += O::abs2(row[c]);
-  xn2 = block_sum2(xn2, 0.0, sh).x;
-  const T alpha = O::conj(row[j + 1]);
-  const double ar = O::real(alpha), ai = O::imag(alpha);
-  T tau, scale;
-  double beta;
-  const bool trivial = (xn2 == 0.0 && ai == 0.0);
-  if (trivial) {
-    tau = O::zero();
-    beta = ar;
-    scale = O::zero();
+// Exact sums of up to 256 doubles in 64-bit integers.  A term m 2^(e-1075) (m of 53 bits)
+// enters as m 2^2 shifted right by its distance to the largest exponent, rounded, so what is
+// lost is below 2^-55 of the largest term.
+struct WarpSum {
+  long long sum;
+  int e;  // exponent field of the largest term
+};
+__device__ __forceinline__ WarpSum warp_isum(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ffu);
+  const int emax = __reduce_max_sync(0xffffffffu, e);
+  const unsigned long long m = e ? ((b & 0xfffffffffffffull) | (1ull << 52)) << 2 : 0ull;
+  const int sh = emax - e;
+  unsigned long long q = 0ull;
+  if (sh == 0)
+    q = m;
+  else if (sh < 60)
+    q = (m + (1ull << (sh - 1))) >> sh;
+  // three limbs (26, 26 and the rest) through the 32-bit warp reduction
+  const long long s = (b >> 63) ? -(long long)q : (long long)q;
+  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)s & 0x3ffffffu);
+  const unsigned mid = __reduce_add_sync(0xffffffffu, (unsigned)(s >> 26) & 0x3ffffffu);
+  const int hi = __reduce_add_sync(0xffffffffu, (int)(s >> 52));
+  return {((long long)hi << 52) + ((long long)mid << 26) + (long long)lo, emax};
+}
+// total of the warps' sums, rounded to a double
+template <int NW>
+__device__ __forceinline__ double block_isum(const WarpSum* s) {
+  int E = 0;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) E = max(E, s[w].e);
+  long long t = 0;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) t += s[w].sum >> min(E - s[w].e, 63);
+  if (E == 0x7ff) return __longlong_as_double(0x7ff8000000000000LL);  // a NaN or Inf among them
+  if (t == 0) return 0.0;
+  const unsigned long long neg = t < 0 ? 1ull : 0ull;
+  unsigned long long m = neg ? 0ull - (unsigned long long)t : (unsigned long long)t;
+  const int top = 63 - __clzll((long long)m);
+  int ex = E + top - 54;  // the term 2^54 of a sum has the exponent field E
+  if (top > 52) {
+    const int sh = top - 52;
+    m = (m + (1ull << (sh - 1))) >> sh;
+    if (m >> 53) {
+      m >>= 1;
+      ++ex;
+    }
   } else {
-    const double n2 = ar * ar + ai * ai + xn2;
-    const double rn = rsqrt64(n2);  // 1 / ||x||
-    const double nrm = n2 * rn;
-    beta = (ar >= 0.0) ? -nrm : nrm;
-    const double ib = (ar >= 0.0) ? -rn : rn;  // 1 / beta
-    tau = O::make((beta - ar) * ib, -ai * ib);
-    const double zr = ar - beta, zi = ai;
-    const double iden = rcp64(zr * zr + zi * zi);
-    scale = O::make(zr * iden, -zi * iden);
+    m <<= 52 - top;
   }
-  T* vg = a.V + (int64_t)j * m;
-  for (int c = j + 1 + threadIdx.x; c < m; c += blockDim.x) {
-    const T v = (c == j + 1) ? O::one() : (trivial ? O::zero() : O::conj(row[c]) * scale);
-    vs[c] = v;
-    st_pub(vg + c, v);
-  }
-  if (threadIdx.x == 0) {
-    vs[j] = tau;
-    st_pub(vg + j, tau);
-    a.tau[j] = tau;
-    a.e[j] = beta;
-    a.d[j] = O::real(row[j]);
-  }
-  __syncthreads();
+  if (ex <= 0) return 0.0;
+  if (ex >= 0x7ff) return __longlong_as_double(0x7ff0000000000000LL);
+  return __longlong_as_double(
+      (long long)((neg << 63) | ((unsigned long long)ex << 52) | (m & 0xfffffffffffffull)));
 }
 
-// householder_pub by one warp (lane = this thread's lane): no CTA barrier, so the other
-// warps of the owner CTA keep updating their rows meanwhile.
-template <typename T>
-__device__ void householder_pub_warp(const Tri2Args<T>& a, const T* row, int j, T* vs,
-                                     int lane) {
-  using O = ops<T>;
-  const int m = a.m;
-  double xn2 = 0.0;
-  for (int c = j + 2 + lane; c < m; c += 32) xn2 += O::abs2(row[c]);
-  xn2 = warp_sum(xn2);
-  const T alpha = O::conj(row[j + 1]);
-  const double ar = O::real(alpha), ai = O::imag(alpha);
-  T tau, scale;
-  double beta;
-  const bool trivial = (xn2 == 0.0 && ai == 0.0);
-  if (trivial) {
-    tau = O::zero();
-    beta = ar;
-    scale = O::zero();
-  } else {
-    const double n2 = ar * ar + ai * ai + xn2;
-    const double rn = rsqrt64(n2);  // 1 / ||x||
-    const double nrm = n2 * rn;
-    beta = (ar >= 0.0) ? -nrm : nrm;
-    const double ib = (ar >= 0.0) ? -rn : rn;  // 1 / beta
-    tau = O::make((beta - ar) * ib, -ai * ib);
-    const double zr = ar - beta, zi = ai;
-    const double iden = rcp64(zr * zr + zi * zi);
-    scale = O::make(zr * iden, -zi * iden);
-  }
-  T* vg = a.V + (int64_t)j * m;
-  for (int c = j + 1 + lane; c < m; c += 32) {
-    const T v = (c == j + 1) ? O::one() : (trivial ? O::zero() : O::conj(row[c]) * scale);
-    st_pub(vg + c, v);
-    vs[c] = v;
-  }
-
-  if (lane == 0) {
-    vs[j] = tau;
-    st_pub(vg + j, tau);
-    a.tau[j] = tau;
-    a.e[j] = beta;
-    a.d[j] = O::real(row[j]);
-  }
-  __syncwarp();
+// the sum of x over the warp's lanes: every lane for a real x; for a complex one lane 0 holds
+// the real part and lane 16 the imaginary part (one FP64 addition per level either way)
+__device__ __forceinline__ double warp_sum_parts(double x) { return warp_sum(x); }
+__device__ __forceinline__ double warp_sum_parts(zdbl x) {
+  const bool up = threadIdx.x & 16;
+  double v = (up ? x.im : x.re) + __shfl_xor_sync(0xffffffffu, up ? x.re : x.im, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
-// DF: rows as double-float pairs (mixed path); else FP64 throughout.
-template <typename T, bool DF>
-__global__ void __launch_bounds__(TPB) tridiag_smem_kernel(Tri2Args<T> a0) {
+// NE: columns per thread (m <= 256 NE)
+template <typename T, int NE>
+__global__ void __launch_bounds__(TPB) tridiag_lone_kernel(Tri2Args<T> a) {
   using O = ops<T>;
-  extern __shared__ unsigned char sm_raw[];
-  __shared__ double sh[72];
-  __shared__ T part[TPB / 32];
-  const int P = a0.P, inst = blockIdx.x / P, cta = blockIdx.x % P;
-  Tri2Args<T> a = a0;
-  {
-    const size_t off = (size_t)inst * a0.wb;
-    a.A = a0.A + (int64_t)inst * a0.a_bs;
-    a.d = byte_shift(a0.d, off);
-    a.e = byte_shift(a0.e, off);
-    a.tau = byte_shift(a0.tau, off);
-    a.V = byte_shift(a0.V, off);
-    a.Pg = byte_shift(a0.Pg, off);
-    a.Dg = byte_shift(a0.Dg, off);
-  }
-  const int m = a.m;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  constexpr int NW = TPB / 32, NC = O::cplx ? 2 : 1;
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  __shared__ WarpSum s_norm[NW], s_dot[NW];
+  __shared__ double s_acc[NW][NW][NC];
+  __shared__ double s_beta, s_ib;
+  __shared__ T s_typ;
+  const int P = gridDim.x, cta = blockIdx.x, m = a.m;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nr = (m - cta + P - 1) / P;  // own rows r = cta + P t
   T* rows = reinterpret_cast<T*>(sm_raw);
-  T* vbuf = rows + (size_t)nr * m;  // v of two consecutive columns
-  T* psm = vbuf + 2 * (size_t)m;    // p, then w
-  T* pown = psm + m;                // p of the own rows (by local row index)
-  T* dsm = pown + m;                // the P shares of v^H p
-  // DF only: v and w as double-float, and the owner's row j+1 back in FP64
-  using D = typename dfof<T>::type;
-  D* rdf = reinterpret_cast<D*>(rows);
-  D* vdfb = reinterpret_cast<D*>(dsm + P);  // two buffers, like vbuf
-  D* wdf = vdfb + 2 * (size_t)m;
-  T* hrow = reinterpret_cast<T*>(wdf + m);
+  T* ubuf = rows + (size_t)((m + P - 1) / P) * m;  // u of this column and of the one before
+  T* wsm = ubuf + 2 * (size_t)m;                   // w of the one before
   for (int t = 0; t < nr; ++t)
-    for (int c = threadIdx.x; c < m; c += blockDim.x) {
-      const T x = a.A[(int64_t)(cta + P * t) * m + c];
-      if constexpr (DF)
-        rdf[(size_t)t * m + c] = to_df(x);
-      else
-        rows[(size_t)t * m + c] = x;
-    }
-  __syncthreads();
-  // own row t as FP64 (DF: converted into hrow from column `from` on)
-  auto row64 = [&](int t, int from) -> const T* {
-    if constexpr (DF) {
-      for (int c = from + threadIdx.x; c < m; c += blockDim.x) hrow[c] = from_df(rdf[(size_t)t * m + c]);
-      __syncthreads();
-      return hrow;
-    } else {
-      return rows + (size_t)t * m;
-    }
-  };
-  if (m == 1) {
-    if (cta == 0) {
-      const T* r0 = row64(0, 0);
-      if (threadIdx.x == 0) a.d[0] = O::real(r0[0]);
-    }
-    return;
-  }
-  if (cta == 0) {
-    householder_pub(a, row64(0, 0), 0, vbuf, sh);
-    if constexpr (DF) {
-      for (int c = 1 + threadIdx.x; c < m; c += blockDim.x) vdfb[c] = to_df(vbuf[c]);
-      __syncthreads();
-    }
-  }
-  for (int j = 0; j < m - 1; ++j) {
-    T* vsm = vbuf + (size_t)(j & 1) * m;
-    D* vdf = vdfb + (size_t)(j & 1) * m;
-    // v_j and tau_j (the owner of row j computed them into vsm itself)
-    // (the double-float copy of v goes with the gather; the owner converts its own v)
-    if (j % P != cta) {
-      if (!gather_pub(a.V + (int64_t)j * m, vsm, j, m, a.status, DF ? vdf : nullptr)) return;
-    } else if (DF && j > 0) {
-      for (int c = j + 1 + threadIdx.x; c < m; c += blockDim.x) vdf[c] = to_df(vsm[c]);
-      __syncthreads();
-    }
-    const T tau = vsm[j];
-    // phase B: p_r = tau sum_{c>j} A[r][c] v_c for own rows r > j
-    const int t0 = (j + 1 - cta + P - 1) / P;  // first own row beyond j
-    const int live = nr - t0;
-    T* pg = a.Pg + (int64_t)j * m;
-    if (live > 0) {
-      int S = 1;
-      while (S * 2 * live <= nw) S *= 2;
-      if (S == 1) {
-        // rows ta and ta + nw per warp pass; a reduce-scatter butterfly leaves row ta's
-        // sum in lanes 0-15 and row tb's in lanes 16-31 (5 add levels for both rows)
-        for (int item = warp; item < live; item += 2 * nw) {
-          const int ta = t0 + item;
-          const bool two = item + nw < live;
-          const int tb = two ? ta + nw : ta;
-          T xa = O::zero(), xb = O::zero();
-          if constexpr (DF) {
-            const D* ra = rdf + (size_t)ta * m;
-            const D* rb = rdf + (size_t)tb * m;
-            D ya = to_df(O::zero()), yb = ya;
-            for (int c = j + 1 + lane; c < m; c += 32) {
-              const D vc = vdf[c];
-              ya = dff(ra[c], vc, ya);
-              if (two) yb = dff(rb[c], vc, yb);
-            }
-            xa = from_df(ya);
-            xb = from_df(yb);
-          } else {
-            const T* ra = rows + (size_t)ta * m;
-            const T* rb = rows + (size_t)tb * m;
-            for (int c = j + 1 + lane; c < m; c += 32) {
-              const T vc = vsm[c];
-              xa = O::fma(ra[c], vc, xa);
-              if (two) xb = O::fma(rb[c], vc, xb);
-            }
-          }
-          if (two) {
-            T keep = (lane < 16) ? xa : xb;
-            keep = keep + shfl_xor((lane < 16) ? xb : xa, 16);
+    for (int c = tid; c < m; c += TPB) rows[(size_t)t * m + c] = a.A[(int64_t)(cta + P * t) * m + c];
+  T x[NE];  // column k of the current matrix at rows c = tid + 256 i
 #pragma unroll
-            for (int o = 8; o > 0; o >>= 1) keep = keep + shfl_xor(keep, o);
-            if ((lane & 15) == 0) {
-              const int t = (lane == 0) ? ta : tb;
-              const T pr = tau * keep;
-              pown[t] = pr;
-              st_pub(pg + cta + P * t, pr);
-            }
-          } else {
-            xa = warp_sum(xa);
-            if (lane == 0) {
-              const T pr = tau * xa;
-              pown[ta] = pr;
-              st_pub(pg + cta + P * ta, pr);
-            }
-          }
-        }
-      } else {
-        for (int item = warp; item < live * S; item += nw) {
-          const int t = t0 + item / S, sg = item % S;
-          T acc = O::zero();
-          if constexpr (DF) {
-            const D* row = rdf + (size_t)t * m;
-            D y = to_df(O::zero());
-            for (int c = j + 1 + sg * 32 + lane; c < m; c += S * 32) y = dff(row[c], vdf[c], y);
-            acc = from_df(y);
-          } else {
-            const T* row = rows + (size_t)t * m;
-            for (int c = j + 1 + sg * 32 + lane; c < m; c += S * 32) acc = O::fma(row[c], vsm[c], acc);
-          }
-          acc = warp_sum(acc);
-          if (lane == 0) part[item] = acc;
-        }
-        __syncthreads();
-        if (threadIdx.x < live) {
-          T sp = part[threadIdx.x * S];
-          for (int q = 1; q < S; ++q) sp = sp + part[threadIdx.x * S + q];
-          const T pr = tau * sp;
-          pown[t0 + threadIdx.x] = pr;
-          st_pub(pg + cta + P * (t0 + threadIdx.x), pr);
+  for (int i = 0; i < NE; ++i) {
+    const int c = tid + TPB * i;
+    x[i] = c < m ? a.A[(int64_t)c * m] : O::zero();
+  }
+  for (int k = 0;; ++k) {
+    T* u = ubuf + (size_t)(k & 1) * m;
+    const T* up = ubuf + (size_t)((k & 1) ^ 1) * m;
+    double part = 0.0;
+#pragma unroll
+    for (int i = 0; i < NE; ++i) {
+      const int c = tid + TPB * i;
+      if (c >= k && c < m) {
+        u[c] = x[i];
+        if (c == k && cta == 0) a.d[k] = O::real(x[i]);
+        if (c >= k + 2) {
+          if constexpr (O::cplx)
+            part = fma(x[i].re, x[i].re, fma(x[i].im, x[i].im, part));
+          else
+            part = fma(x[i], x[i], part);
         }
       }
     }
-    __syncthreads();
-    // this CTA's share of v^H p, published next to p
-    if (warp == 0) {
-      T dv = O::zero();
-      for (int t = t0 + lane; t < nr; t += 32) dv = O::fma(O::conj(vsm[cta + P * t]), pown[t], dv);
-      dv = warp_sum(dv);
-      if (lane == 0) st_pub(a.Dg + (int64_t)j * P + cta, dv);
-    }
-    // all of p and all shares; v^H p summed in one fixed order (the same in every CTA);
-    // then w = p - (conj(tau)/2)(v^H p) v in place
-    if (!gather_pub2(pg, psm, j + 1, m, a.Dg + (int64_t)j * P, dsm, 0, P, a.status)) return;
-    T dot = O::zero();
-    for (int q = lane; q < P; q += 32) dot = dot + dsm[q];
-    dot = warp_sum(dot);
-    const T coef = O::scale(-0.5, O::conj(tau) * dot);
-    for (int c = j + 1 + threadIdx.x; c < m; c += blockDim.x) {
-      psm[c] = O::fma(coef, vsm[c], psm[c]);
-      if constexpr (DF) wdf[c] = to_df(psm[c]);
+    if (k == m - 1) break;
+    {
+      const WarpSum s = warp_isum(part);
+      if (lane == 0) s_norm[warp] = s;
     }
     __syncthreads();
-    // phase C: own rows r > j: A[r][c] -= v_r conj(w_c) + w_r conj(v_c), c > j
-    auto update_row = [&](int t, int c0, int cstep) {
-      const int r = cta + P * t;
-      const T nvr = O::scale(-1.0, vsm[r]), nwr = O::scale(-1.0, psm[r]);
-      if constexpr (DF) {
-        D* row = rdf + (size_t)t * m;
-        const D dvr = to_df(nvr), dwr = to_df(nwr);
-        for (int c = j + 1 + c0; c < m; c += cstep)
-          row[c] = dff(dwr, dfconj(vdf[c]), dff(dvr, dfconj(wdf[c]), row[c]));
-      } else {
+    const int t0 = (k + 1 > cta) ? (k + 1 - cta + P - 1) / P : 0;  // first own row beyond k
+    if (warp == 0) {  // beta, and u's first entry alpha - beta
+      const double xn2 = block_isum<NW>(s_norm);
+      const T alpha = u[k + 1];
+      const double ar = O::real(alpha), ai = O::imag(alpha);
+      // xn2 = 0 and alpha real: H is the identity (tests on the bits: an FP64 comparison costs
+      // as much as an addition)
+      double beta = ar, ib = 0.0, z = 0.0;
+      const double n2 = O::cplx ? fma(ar, ar, fma(ai, ai, xn2)) : fma(ar, ar, xn2);
+      const bool rest = __double_as_longlong(xn2) != 0ll ||
+                        (__double_as_longlong(ai) & 0x7fffffffffffffffll) != 0ll;
+      if (rest && __double_as_longlong(n2) != 0ll) {
+        const double rn = rsqrt64_short(n2);  // 1 / ||x||
+        const bool pos = __double2hiint(ar) >= 0;
+        const double nrm = n2 * rn;
+        beta = pos ? -nrm : nrm;
+        ib = pos ? -rn : rn;
+        z = ar - beta;
+      }
+      __syncwarp();
+      if (lane == 0) {
+        u[k + 1] = O::make(z, rest ? ai : 0.0);
+        s_beta = beta;
+        s_ib = ib;
+      }
+    } else if (k > 0 && (warp & 3)) {
+      // meanwhile the update of column k-1, A -= u w^H + w u^H, by the warps that don't share
+      // warp 0's FP64 unit
+      for (int t = t0; t < nr; ++t) {
         T* row = rows + (size_t)t * m;
-        for (int c = j + 1 + c0; c < m; c += cstep)
-          row[c] = O::fma(nwr, O::conj(vsm[c]), O::fma(nvr, O::conj(psm[c]), row[c]));
+        const int r = cta + P * t;
+        const T nu = O::scale(-1.0, up[r]), nw = O::scale(-1.0, wsm[r]);
+        for (int c = k + 1 + (warp - 1 - (warp >> 2)) * 32 + lane; c < m; c += 6 * 32)
+          row[c] = O::fma(nw, O::conj(up[c]), O::fma(nu, O::conj(wsm[c]), row[c]));
       }
-    };
-    if (j + 1 < m - 1 && (j + 1) % P == cta) {
-      // the next column's owner: warp 0 updates that row and publishes v_{j+1} while
-      // the other warps update the remaining rows
-      if (warp == 0) {
-        update_row(t0, lane, 32);
-        __syncwarp();
-        const T* hr;
-        if constexpr (DF) {
-          for (int c = j + 1 + lane; c < m; c += 32) hrow[c] = from_df(rdf[(size_t)t0 * m + c]);
-          __syncwarp();
-          hr = hrow;
-        } else {
-          hr = rows + (size_t)t0 * m;
-        }
-        householder_pub_warp(a, hr, j + 1, vbuf + (size_t)((j + 1) & 1) * m, lane);
-      } else {
-        for (int t = t0 + 1 + (warp - 1); t < nr; t += nw - 1) update_row(t, lane, 32);
-      }
-    } else {
-      for (int t = t0 + warp; t < nr; t += nw) update_row(t, lane, 32);
-    }
-    if (j + 1 == m - 1 && (m - 1) % P == cta) {
-      __syncthreads();
-      const T* rl = row64((m - 1 - cta) / P, m - 1);
-      if (threadIdx.x == 0) a.d[m - 1] = O::real(rl[m - 1]);
     }
     __syncthreads();
+    // A u for the own rows: S warps per row
+    const int live = nr - t0;
+    T* xg = a.X + (int64_t)k * m * 2;
+    int S = NW;
+    while (S > 1 && (S * live > NW || 32 * S >= 2 * (m - k - 1))) S >>= 1;
+    for (int l0 = 0; l0 < live; l0 += NW / S) {
+      const int li = l0 + warp / S, seg = warp % S;
+      if (li < live) {
+        const T* row = rows + (size_t)(t0 + li) * m;
+        T acc = O::zero();
+        for (int c = k + 1 + seg * 32 + lane; c < m; c += S * 32) acc = O::fma(row[c], u[c], acc);
+        const double v = warp_sum_parts(acc);
+        const int r = cta + P * (t0 + li);
+        if (seg == 0 && lane == 1) st_pub(xg + 2 * r + 1, row[k + 1]);
+        if ((lane & 15) == 0 && lane < 16 * NC) {
+          if (S == 1)
+            st_pub(reinterpret_cast<double*>(xg + 2 * r) + (lane >> 4), v);
+          else
+            s_acc[li][seg][lane >> 4] = v;
+        }
+      }
+    }
+    if (S > 1) {  // (then S live <= NW: all rows were done in one round)
+      __syncthreads();
+      if (tid < live * NC) {
+        const int li = tid / NC, q = tid % NC;
+        double v = s_acc[li][0][q];
+        for (int s = 1; s < S; ++s) v += s_acc[li][s][q];
+        st_pub(reinterpret_cast<double*>(xg + 2 * (cta + P * (t0 + li))) + q, v);
+      }
+    }
+    // while the others' rows arrive: gamma = -1 / (beta conj(alpha - beta)), tau and the
+    // scaled reflector of the own rows for the back transformation
+    const T up0 = u[k + 1];
+    const double zr = O::real(up0), zi = O::imag(up0), ib = s_ib;
+    T gamma = O::zero(), scale = O::zero();
+    if (ib != 0.0) {
+      const double iden = rcp64(O::cplx ? fma(zr, zr, zi * zi) : zr * zr);
+      const double f = -ib * iden;
+      gamma = O::make(zr * f, zi * f);
+      scale = O::make(zr * iden, -zi * iden);  // 1 / (alpha - beta)
+    }
+    if (tid >= TPB - 32) {
+      for (int t = t0 + lane; t < nr; t += 32) {
+        const int r = cta + P * t;
+        a.V[(int64_t)k * m + r] = (r == k + 1) ? O::one() : u[r] * scale;
+      }
+      if (cta == 0 && lane == 31) {
+        a.tau[k] = O::make(-zr * ib, -zi * ib);
+        a.e[k] = s_beta;
+      }
+    }
+    T ty[NE], col[NE];
+    double dp = 0.0;
+    bool ok;
+    {
+      const T* src[NE];
+#pragma unroll
+      for (int i = 0; i < NE; ++i) {
+        const int c = tid + TPB * i;
+        src[i] = (c > k && c < m) ? xg + 2 * c : nullptr;
+        ty[i] = col[i] = O::zero();
+      }
+      ok = wait_pairs<T, NE>(src, ty, col, a.status);
+#pragma unroll
+      for (int i = 0; i < NE; ++i) {
+        const int c = tid + TPB * i;
+        if (src[i]) {
+          const T uc = u[c], y = ty[i];
+          if constexpr (O::cplx)
+            dp = fma(uc.re, y.re, fma(uc.im, y.im, dp));
+          else
+            dp = fma(uc, y, dp);
+          ty[i] = gamma * y;
+          if (c == k + 1) s_typ = ty[i];
+        }
+      }
+    }
+    {
+      const WarpSum s = warp_isum(dp);
+      if (lane == 0) s_dot[warp] = s;
+    }
+    if (!__syncthreads_and(ok)) return;
+    const double dot = block_isum<NW>(s_dot);
+    const double gr = O::real(gamma), gi = O::imag(gamma);
+    const double cf = O::cplx ? -0.5 * fma(gr, gr * dot, gi * (gi * dot)) : -0.5 * (gr * (gr * dot));
+    // w = gamma A u + c u, and column k+1 after the update: x - u conj(w_{k+1}) - w conj(u_{k+1})
+    const T nwc = O::conj(s_typ + O::scale(cf, up0)), nuc = O::conj(up0);
+#pragma unroll
+    for (int i = 0; i < NE; ++i) {
+      const int c = tid + TPB * i;
+      if (c > k && c < m) {
+        const T uc = u[c];
+        T w;
+        if constexpr (O::cplx)
+          w = zdbl{fma(cf, uc.re, ty[i].re), fma(cf, uc.im, ty[i].im)};
+        else
+          w = fma(cf, uc, ty[i]);
+        wsm[c] = w;
+        x[i] = O::fma(-w, nuc, O::fma(-uc, nwc, col[i]));
+      }
+    }
   }
 }
 
@@ -1246,8 +1141,7 @@ size_t eig_workspace_bytes(int m, int kmax, bool cplx) {
   b += align256(sizeof(double) * 4);                 // dot
   b += align256(sizeof(GridBarrier));                // barrier
   b += align256(sizeof(double) * (size_t)m * kmax);  // X
-  b += align256(ts * (size_t)m * m);                 // p of every column (exchange)
-  b += align256(ts * (size_t)m * m);                 // shares of v^H p (exchange)
+  b += align256(2 * ts * (size_t)m * m);             // exchange of the lone reduction
   return b;
 }
 
@@ -1274,8 +1168,7 @@ cudaError_t heev_top(T* A, int m, int kmax, int64_t max_bond, double tol, double
   double* dot = (double*)take(sizeof(double) * 4);
   GridBarrier* bar = (GridBarrier*)take(sizeof(GridBarrier));
   double* X = (double*)take(sizeof(double) * (size_t)m * kmax);
-  T* Pg = (T*)take(ts * (size_t)m * m);
-  T* Dg = (T*)take(ts * (size_t)m * m);
+  T* Xg = (T*)take(2 * ts * (size_t)m * m);
 
   cudaError_t err = cudaSuccess;
   // algorithmic FP64 flops: Householder tridiagonalisation (16/3) m^3 complex,
@@ -1283,41 +1176,27 @@ cudaError_t heev_top(T* A, int m, int kmax, int64_t max_bond, double tol, double
   const double cm = ops<T>::cplx ? 4.0 : 1.0;
   const double fl_tri = cm * (4.0 / 3.0) * m * (double)m * m * nb;
   const double fl_rest = cm * 2.0 * m * (double)m * kmax * nb;
-  // 1. tridiagonalisation.  Rows in shared memory when they fit: one thread-block
-  // cluster of up to 16 CTAs per matrix for a batch or when `prefer_cluster`
-  // (co-scheduled and, unlike cooperative launches, concurrent with other streams'
-  // work), else a cooperative launch over ~m/4 CTAs per matrix (the fastest single
-  // reduction); rows in global memory beyond that.  CBC_TRIDIAG_CTAS overrides the CTA
-  // count (1..16 selects a cluster).
-  int Pw = 0;
-  if (const char* env = getenv("CBC_TRIDIAG_CTAS")) Pw = std::max(0, std::min(num_sms, atoi(env)));
-  auto shm_for = [&](int P) {
-    return (((size_t)((m + P - 1) / P) + (df ? 8 : 4)) * m + P) * ts;
-  };
-  // double-float rows pay off when the batch makes the reduction throughput bound; a
-  // lone reduction is latency bound and runs faster in FP64
-  df = df && nb > 1;
-  const void* ksm = df ? (const void*)tridiag_smem_kernel<T, true>
-                       : (const void*)tridiag_smem_kernel<T, false>;
-  const size_t shm_cap = 160 * 1024;
-  int P = Pw > 0 ? Pw : std::max(1, std::min(16, m / 2));
-  bool cluster = false;
-  if ((Pw > 0 || prefer_cluster || nb > 1) && P <= 16 && shm_for(P) <= shm_cap) {
-    err = allow_max_smem(ksm);
-    if (err != cudaSuccess) return err;
-    cluster = cluster_ctas(ksm, P, TPB, shm_for(P)) == P;
-  }
-  if (!cluster && Pw <= 0) P = std::max(1, std::min(num_sms, m / 4));
-  // batches (and concurrent instances) use the cluster reduction with the rows' lower
-  // triangles in shared memory and the exchanges through distributed shared memory
-  // (tridiag_cluster.cu); CBC_TRIDIAG_CTAS selects the polling kernels above instead
+  // 1. tridiagonalisation.  A batch or an instance that runs next to others (prefer_cluster):
+  // one thread-block cluster per matrix (tridiag_cluster.cu), co-scheduled and, unlike a
+  // cooperative launch, concurrent with other streams' work.  Else, and where no cluster
+  // holds the matrix, a cooperative launch per matrix, with the rows in shared memory up to
+  // kLoneMaxM and in global memory beyond.
+  df = df && nb > 1;  // a lone reduction runs in FP64
   int Pc = 0;
-  if ((nb > 1 || prefer_cluster) && Pw <= 0 && m >= 2) Pc = tridiag_cluster_size<T>(m, df);
-  if (Pc > 0) cluster = false;
-  const bool in_smem = Pc == 0 && (cluster || shm_for(P) <= shm_cap);
+  if ((nb > 1 || prefer_cluster) && m >= 2) Pc = tridiag_cluster_size<T>(m, df);
+  // rows per CTA: more CTAs shorten the work on the rows but lengthen the exchange, which
+  // every CTA polls (m = 256 real: 2 rows 1.31 ms, 4 rows 1.00, 6 1.09; complex, with four
+  // times the work, 1.40, 1.45 and 1.64 ms)
+  const int R = std::max(ops<T>::cplx ? 2 : 4, (m + num_sms - 1) / num_sms);
+  const int Pl = (m + R - 1) / R;
+  const size_t shl = ((size_t)R + 3) * m * ts;
+  const bool lone = Pc == 0 && m <= kLoneMaxM && shl <= 200 * 1024;
+  const void* kl = m <= TPB ? (const void*)tridiag_lone_kernel<T, 1>
+                   : m <= 2 * TPB ? (const void*)tridiag_lone_kernel<T, 2>
+                                  : (const void*)tridiag_lone_kernel<T, 4>;
   {
-    // barrier, tau and e[0] start at zero; with the rows in shared memory the exchange
-    // buffers start as all-ones bit patterns (the "not yet written" mark)
+    // barrier, tau and e[0] start at zero; the exchange buffers of the lone reduction as
+    // all-ones bit patterns (the "not yet written" mark)
     WsInit wi{};
     auto add = [&](void* p, size_t bytes, unsigned long long v) {
       wi.seg[wi.nseg] = static_cast<unsigned long long*>(p);
@@ -1328,43 +1207,37 @@ cudaError_t heev_top(T* A, int m, int kmax, int64_t max_bond, double tol, double
     add(bar, sizeof(GridBarrier), 0ull);
     add(tau, ts * m, 0ull);
     add(e, sizeof(double), 0ull);
-    if (in_smem) {
-      add(V, ts * (size_t)m * m, ~0ull);
-      add(Pg, ts * (size_t)m * m, ~0ull);
-      add(Dg, ts * (size_t)m * m, ~0ull);
+    if (lone) {
+      add(Xg, ts * (size_t)m * m * 2, ~0ull);
     }
     wi.wb = wb;
     note_launches(CBC_K_AUX, 1);
     ws_init_kernel<<<dim3((unsigned)std::min<int64_t>(64, ((int64_t)m * m * (ts / 8) + 255) / 256), nb), 256, 0, s>>>(wi);
     err = cudaGetLastError();
-    if (err == cudaSuccess && in_smem) err = allow_max_smem(ksm);
+    if (err == cudaSuccess && lone) err = allow_max_smem(kl);
     if (err != cudaSuccess) return err;
   }
   {
-  KTimer tt(CBC_K_TRIDIAG, s, (cluster || Pc > 0) ? 1 : nb, fl_tri);
+  KTimer tt(CBC_K_TRIDIAG, s, Pc > 0 ? 1 : nb, fl_tri);
   if (Pc > 0) {
     err = tridiag_cluster<T>(A, m, d, e, tau, V, (int64_t)m * m, wb, nb, Pc, df, s);
-  } else if (cluster) {
-    Tri2Args<T> ta{A, m, d, e, tau, V, Pg, Dg, status, P, (int64_t)m * m, wb};
-    void* args[] = {&ta};
-    err = launch_cluster(ksm, P, nb * P, TPB, shm_for(P), args, s);
   } else {
     for (int b = 0; b < nb && err == cudaSuccess; ++b) {
       const size_t off = (size_t)b * wb;
       T* Ab = A + (int64_t)b * m * m;
-      if (in_smem) {
+      if (lone) {
         Tri2Args<T> ta{Ab, m, byte_shift(d, off), byte_shift(e, off), byte_shift(tau, off),
-                       byte_shift(V, off), byte_shift(Pg, off), byte_shift(Dg, off), status, P, 0, 0};
+                       byte_shift(V, off), byte_shift(Xg, off), status};
         void* args[] = {&ta};
-        err = cudaLaunchCooperativeKernel(ksm, dim3(P), dim3(TPB),
-                                          args, shm_for(P), s);
+        err = cudaLaunchCooperativeKernel(kl, dim3(Pl), dim3(TPB), args, shl, s);
       } else {
         TriArgs<T> ta{Ab, m, byte_shift(d, off), byte_shift(e, off), byte_shift(tau, off),
                       byte_shift(V, off), byte_shift(vbuf, off), byte_shift(p, off),
                       byte_shift(dot, off), byte_shift(bar, off), status};
         void* args[] = {&ta};
-        err = cudaLaunchCooperativeKernel((const void*)tridiag_kernel<T>, dim3(P), dim3(TPB), args,
-                                          0, s);
+        err = cudaLaunchCooperativeKernel((const void*)tridiag_kernel<T>,
+                                          dim3(std::max(1, std::min(num_sms, m / 4))), dim3(TPB),
+                                          args, 0, s);
       }
     }
   }
