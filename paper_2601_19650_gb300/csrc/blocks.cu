@@ -38,24 +38,23 @@ __global__ void wait_selftest_kernel(const unsigned int* word, int* status, long
 
 template <typename T>
 int heev_t(int m, int kmax, int nb, T* A, double* lam, T* U, bool mixed, cudaStream_t s) {
-  int* ints = nullptr;
+  int* status = nullptr;
   void* work = nullptr;
   const size_t wb = eig_workspace_bytes(m, kmax, ops<T>::cplx);
-  cudaError_t e = pool_malloc(reinterpret_cast<void**>(&ints), sizeof(int) * (1 + nb), s);
+  cudaError_t e = pool_malloc(reinterpret_cast<void**>(&status), sizeof(int), s);
   if (e != cudaSuccess) return cuda_fail(e, "cbc_heev: alloc");
   e = pool_malloc(&work, wb * nb, s);
   if (e != cudaSuccess) {
-    cudaFreeAsync(ints, s);
+    cudaFreeAsync(status, s);
     return cuda_fail(e, "cbc_heev: alloc");
   }
-  e = cudaMemsetAsync(ints, 0, sizeof(int) * (1 + nb), s);
+  e = cudaMemsetAsync(status, 0, sizeof(int), s);
   if (e == cudaSuccess)
-    e = heev_top<T>(A, m, kmax, kmax, 0.0, -1.0, lam, U, ints + 1, work, ints, num_sms(), s, nb,
-                    false, mixed);
+    e = heev_top<T>(A, m, kmax, lam, U, work, status, num_sms(), s, nb, false, mixed);
   int hs = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, ints, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, s);
   cudaFreeAsync(work, s);
-  cudaFreeAsync(ints, s);
+  cudaFreeAsync(status, s);
   cudaError_t e2 = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "cbc_heev");
   if (e2 != cudaSuccess) return cuda_fail(e2, "cbc_heev: synchronize");

@@ -6,19 +6,18 @@
 // values, so keeping the k largest eigenpairs keeps the same subspace as the truncated
 // SVD.  Stages:
 //   1. Householder reduction to a real symmetric tridiagonal T = Q^H K Q by one group
-//      of CTAs that wait on each other (a thread-block cluster when the rows fit in its
-//      shared memory, else a cooperative launch); rows of K are dealt round-robin to the
-//      CTAs so the shrinking trailing block stays balanced.  FP64 work is spread over
-//      several SMs because one GB300 SM retires only ~2 DFMA per clock.
+//      of CTAs that wait on each other (a thread-block cluster per matrix of a batch, else a
+//      cooperative launch); rows of K are dealt round-robin to the CTAs so the shrinking
+//      trailing block stays balanced.  FP64 work is spread over several SMs because one
+//      GB300 SM retires only ~2 DFMA per clock.
 //   2. Estimates of all eigenvalues of T by single-precision Sturm-count multisection,
 //      one warp per eigenvalue (a dependent chain of FP64 divisions per Sturm step is
 //      slow on this part; the estimates only need to separate the eigenvalues).
 //   3. Eigenvectors of T for the candidates (the kmax largest) by FP64 inverse
 //      iteration seeded with those estimates (one LU, four solves); eigenvalues =
-//      Rayleigh quotients.
-//   4. The rank rule (max_bond, relative floor, tolerance) on the refined eigenvalues,
-//      with the discarded weight taken as trace(T) minus the kept eigenvalues.
-//   5. Back transformation u = H_0 H_1 ... H_{m-2} x, one warp per kept eigenvector.
+//      Rayleigh quotients.  (The rank rule runs on the host, on weights measured on the
+//      factor.)
+//   4. Back transformation u = H_0 H_1 ... H_{m-2} x.
 #include <float.h>
 
 #include <algorithm>
@@ -558,7 +557,8 @@ __global__ void __launch_bounds__(TPB) tridiag_lone_kernel(Tri2Args<T> a) {
 
 // ---- eigenvalues of T: single-precision multisection, one warp per eigenvalue --------
 // The values only seed the shifts of the FP64 inverse iteration below, whose Rayleigh
-// quotients are the eigenvalues used for the rank rule.
+// quotients are the eigenvalues used for the rank rule.  T is scaled by a power of two to
+// entries below 1, so any norm fits FP32.
 __device__ __forceinline__ int sturm32(const float* dd, const float* e2, int m, float x,
                                        float pivmin) {
   int cnt = 0;
@@ -572,62 +572,102 @@ __device__ __forceinline__ int sturm32(const float* dd, const float* e2, int m, 
   return cnt;
 }
 
-__global__ void bisect32_kernel(const double* d, const double* e, int m, float* lam32,
-                                size_t wb) {
+// lam32: eigenvalues / *scale, descending; lam[j] for j >= kmax (the estimates that the
+// caller gets; the first kmax come from the inverse iteration)
+__global__ void bisect32_kernel(const double* d, const double* e, int m, int kmax, float* lam32,
+                                double* scale, double* lam, size_t wb) {
   extern __shared__ float shf[];
   d = byte_shift(d, blockIdx.y * wb);  // matrix blockIdx.y of a batch
   e = byte_shift(e, blockIdx.y * wb);
   lam32 = byte_shift(lam32, blockIdx.y * wb);
+  scale = byte_shift(scale, blockIdx.y * wb);
+  lam += (size_t)blockIdx.y * m;
   float* dd = shf;
   float* e2 = shf + m;
-  __shared__ float s_lo, s_hi, s_piv;
+  __shared__ int s_exp;
+  __shared__ float s_lo[32], s_hi[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if (threadIdx.x == 0) s_exp = 0;
+  __syncthreads();
+  auto field = [](double x) { return ((unsigned)__double2hiint(x) >> 20) & 0x7ffu; };
+  unsigned ex = 0;
+  for (int i = threadIdx.x; i < m; i += blockDim.x)
+    ex = max(ex, max(field(d[i]), i < m - 1 ? field(e[i]) : 0u));
+  ex = __reduce_max_sync(0xffffffffu, ex);
+  if (lane == 0) atomicMax(&s_exp, (int)ex);
+  __syncthreads();
+  const int E = min(s_exp, 2044);
+  const double inv = __hiloint2double((2045 - E) << 20, 0), sc = __hiloint2double((E + 1) << 20, 0);
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    dd[i] = (float)d[i];
-    e2[i] = (i < m - 1) ? (float)(e[i] * e[i]) : 0.f;
-  }
-  if (threadIdx.x == 0) {
-    double lo = DBL_MAX, hi = -DBL_MAX, emax = 0.0;
-    for (int i = 0; i < m; ++i) {
-      double r = 0.0;
-      if (i > 0) r += fabs(e[i - 1]);
-      if (i < m - 1) r += fabs(e[i]);
-      lo = fmin(lo, d[i] - r);
-      hi = fmax(hi, d[i] + r);
-      if (i < m - 1) emax = fmax(emax, e[i] * e[i]);
-    }
-    double span = fmax(fabs(lo), fabs(hi));
-    s_lo = (float)(lo - 1e-6 * span) - FLT_MIN;
-    s_hi = (float)(hi + 1e-6 * span) + FLT_MIN;
-    s_piv = FLT_MIN * (float)fmax(1.0, emax);
+    dd[i] = (float)(d[i] * inv);
+    e2[i] = (i < m - 1) ? (float)(e[i] * inv) : 0.f;
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int jj = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);  // descending index
+  float lo = FLT_MAX, hi = -FLT_MAX;  // Gershgorin
+  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    const float r = (i > 0 ? fabsf(e2[i - 1]) : 0.f) + fabsf(e2[i]);
+    lo = fminf(lo, dd[i] - r);
+    hi = fmaxf(hi, dd[i] + r);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (lane == 0) {
+    s_lo[warp] = lo;
+    s_hi[warp] = hi;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < m; i += blockDim.x) e2[i] *= e2[i];
+  for (int w = 0; w < nw; ++w) {
+    lo = fminf(lo, s_lo[w]);
+    hi = fmaxf(hi, s_hi[w]);
+  }
+  const float span = fmaxf(fabsf(lo), fabsf(hi));
+  lo -= 1e-6f * span + FLT_MIN;
+  hi += 1e-6f * span + FLT_MIN;
+  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *scale = sc;
+  const int jj = blockIdx.x * nw + warp;  // descending index
   if (jj >= m) return;
   const int target = m - 1 - jj;
-  float lo = s_lo, hi = s_hi;
   for (int round = 0; round < 12; ++round) {
     const float x = lo + (hi - lo) * (float)(lane + 1) * (1.f / 33.f);
-    const int cnt = sturm32(dd, e2, m, x, s_piv);
+    const int cnt = sturm32(dd, e2, m, x, FLT_MIN);
     const unsigned bits = __ballot_sync(0xffffffffu, cnt <= target);
     const int nle = __popc(bits);
     const float xl = __shfl_sync(0xffffffffu, x, max(nle - 1, 0));
     const float xh = __shfl_sync(0xffffffffu, x, min(nle, 31));
     if (nle > 0) lo = xl;
     if (nle < 32) hi = xh;
-    if (hi - lo <= 2e-7f * fmaxf(fabsf(lo), fabsf(hi)) + s_piv) break;
+    if (hi - lo <= 2e-7f * fmaxf(fabsf(lo), fabsf(hi)) + FLT_MIN) break;
   }
-  if (lane == 0) lam32[jj] = 0.5f * (lo + hi);
+  if (lane == 0) {
+    const float v = 0.5f * (lo + hi);
+    lam32[jj] = v;
+    if (jj >= kmax) lam[jj] = (double)v * sc;
+  }
 }
 
 // ---- eigenvectors of T by FP64 inverse iteration ----------------------------------
-// The LU of T - sigma I with partial pivoting (the layout of LAPACK's tridiagonal
-// factorisation) lives in shared memory, [i][member], with the pivots stored as
-// reciprocals so the solves are division free.  A candidate whose single-precision
-// eigenvalue is separated from its neighbours by more than 1e-4 of the spectral radius
-// gets a thread of its own (invit_kernel); a run of closer candidates is a cluster that
-// one warp iterates as a block, orthonormalising after every solve
-// (invit_cluster_kernel).  The eigenvalue is the FP64 Rayleigh quotient of the vector.
+// One LU of T - sigma I and four solves per candidate, in T's scaled units.  The chain of
+// dependent FP64 operations (~64 clocks each, and as many for every FP64 instruction a warp
+// issues) is the cost, so
+//   * the elimination runs from both ends of T to the middle, one lane per half, which
+//     halves the chain: the two halves meet in a 2 x 2 system;
+//   * partial pivoting without a branch: 7 FP64 operations per row and factorisation, 4 per
+//     row and solve (pivots kept as reciprocals, U scaled by them);
+//   * no normalisation between the solves: T has entries below 1 and a pivot is at least
+//     2^-52 of its span, so four solves grow a vector by
+//     less than 2^250;
+//   * norms, Rayleigh quotients and orthogonalisation by all lanes of the warp.
+// A candidate whose single-precision eigenvalue is separated from its neighbours by more
+// than 1e-4 of the spectral radius stands alone; a run of closer candidates is a cluster
+// that one warp iterates as a block, orthonormalising after every solve.
+// One thread per candidate from the top, and the clusters in a kernel behind / this: 128
+// candidates of m = 256 0.52 / 0.19 ms, 64 such matrices 2.7 / 1.0 ms; 1024 of m = 2048 31 /
+// 5.9 ms.
 __device__ __forceinline__ uint32_t hash32(uint32_t x) {
   x ^= x >> 16;
   x *= 0x7feb352dU;
@@ -640,299 +680,317 @@ __device__ __forceinline__ uint32_t hash32(uint32_t x) {
 struct InvArgs {
   const double* d;
   const double* e;
-  const float* lam32;  // descending
+  const float* lam32;   // descending, in scaled units
+  const double* scale;
   int m;
-  int kmax;            // candidates j < kmax
-  double* X;           // m x kmax (row i, column j)
-  double* rq;          // [kmax] Rayleigh quotients
-  size_t wb;           // workspace bytes between the matrices of a batch (blockIdx.y)
+  int kmax;             // candidates j < kmax
+  double* X;            // m x kmax (row i, column j)
+  double* lam;          // [m] per matrix: lam[j], j < kmax, Rayleigh quotients
+  size_t wb;            // workspace bytes between the matrices of a batch (blockIdx.y)
+  int per;              // lone candidates per warp
+  int cper;             // members of a cluster iterated together
+  int nclu;             // the first nclu CTAs of a matrix take its clusters, round robin
+  int staged;           // scaled d and e in shared memory
 };
 
-// Shared-memory arrays of the members handled by one CTA: element i of member t at
-// [i * tpb + t] (consecutive members' rows side by side).
-struct InvSmem {
-  double *dl, *di, *du, *du2, *b;  // multipliers, reciprocal pivots, U's two superdiagonals, vector
-  unsigned char* piv;
-  int tpb;
-  __device__ InvSmem(double* base, int m, int tpb_) : tpb(tpb_) {
-    dl = base;
-    di = dl + (size_t)m * tpb;
-    du = di + (size_t)m * tpb;
-    du2 = du + (size_t)m * tpb;
-    b = du2 + (size_t)m * tpb;
-    piv = reinterpret_cast<unsigned char*>(b + (size_t)m * tpb);
+constexpr int kInvMax = 16;  // members per warp: two lanes each
+
+// The state of one warp: member t on lanes 2t (rows 0, 1, ... of T) and 2t + 1 (rows m-1,
+// m-2, ...).  Row p of a half is element [p * ld + lane] of the arrays.
+struct Inv {
+  double *f, *r, *u1, *u2, *b;  // multipliers (last bit: rows swapped), 1/pivot, U's
+                                // superdiagonals / pivot, the vector
+  const double *d, *e;
+  double inv;                   // factor from d, e to scaled units (1 if they are scaled)
+  int m, h, n, ld, lane;        // h rows in the upper half, n in this lane's
+  bool top, swap;
+  double r1, f1, a2, r2;        // the factored 2 x 2 system in the middle
+
+  __device__ double D(int p) const { return d[top ? p : m - 1 - p] * inv; }
+  // the coupling of row p of the half to its next one (of the last row: to the other half)
+  __device__ double E(int p) const { return e[top ? p : m - 2 - p] * inv; }
+  __device__ double* at(int i, int t) const {  // element i of member t's vector
+    return b + (i < h ? (size_t)i * ld + 2 * t : (size_t)(m - 1 - i) * ld + 2 * t + 1);
+  }
+  static __device__ bool less_abs(double x, double y) {  // |x| < |y| on the bits
+    return (__double_as_longlong(x) & 0x7fffffffffffffffll) <
+           (__double_as_longlong(y) & 0x7fffffffffffffffll);
+  }
+  static __device__ double guard(double x, double tiny) {
+    return less_abs(x, tiny) ? __hiloint2double(__double2hiint(tiny) | (__double2hiint(x) & 0x80000000),
+                                                __double2loint(tiny))
+                             : x;
+  }
+
+  __device__ void factor(double sigma, double tiny) {
+    double dc = D(0) - sigma, uc = m > 1 ? E(0) : 0.0;
+    for (int p = 0; p < n - 1; ++p) {
+      const double li = E(p), dn = D(p + 1) - sigma, un = E(p + 1);
+      const bool sw = less_abs(dc, li);
+      const double rp = rcp64(guard(sw ? li : dc, tiny));
+      const double num = sw ? dc : li, A = sw ? dn : uc, B = sw ? un : 0.0, C = sw ? uc : dn;
+      double mult = num * rp;
+      mult = __longlong_as_double((__double_as_longlong(mult) & ~1ll) | (sw ? 1ll : 0ll));
+      const size_t o = (size_t)p * ld + lane;
+      f[o] = mult;
+      r[o] = rp;
+      u1[o] = A * rp;
+      u2[o] = B * rp;
+      dc = fma(-mult, A, C);
+      const double g = -mult * un;
+      uc = sw ? g : un;
+    }
+    // the last rows of both halves: dT x_T + uT x_B = b_T, uB x_T + dB x_B = b_B
+    const double dp = __shfl_xor_sync(0xffffffffu, dc, 1), upn = __shfl_xor_sync(0xffffffffu, uc, 1);
+    const double dT = top ? dc : dp, uT = top ? uc : upn, dB = top ? dp : dc, uB = top ? upn : uc;
+    swap = less_abs(dT, uB);
+    a2 = swap ? dB : uT;
+    r1 = rcp64(guard(swap ? uB : dT, tiny));
+    f1 = (swap ? dT : uB) * r1;
+    r2 = rcp64(guard(fma(-f1, a2, swap ? uT : dB), tiny));
+  }
+
+  __device__ void solve() {
+    double carry = b[lane];
+    int p = 0;
+    for (; p + 4 <= n - 1; p += 4) {  // four rows' operands in flight
+      double fl[4], nx[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        fl[q] = f[(size_t)(p + q) * ld + lane];
+        nx[q] = b[(size_t)(p + q + 1) * ld + lane];
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const bool sw = __double_as_longlong(fl[q]) & 1;
+        const double y = sw ? nx[q] : carry;
+        carry = fma(-fl[q], y, sw ? carry : nx[q]);
+        b[(size_t)(p + q) * ld + lane] = y;
+      }
+    }
+    for (; p < n - 1; ++p) {
+      const double fl = f[(size_t)p * ld + lane], nx = b[(size_t)(p + 1) * ld + lane];
+      const bool sw = __double_as_longlong(fl) & 1;
+      const double y = sw ? nx : carry;
+      carry = fma(-fl, y, sw ? carry : nx);
+      b[(size_t)p * ld + lane] = y;
+    }
+    const double cp = __shfl_xor_sync(0xffffffffu, carry, 1);
+    const double bT = top ? carry : cp, bB = top ? cp : carry;
+    const double c1 = swap ? bB : bT, c2 = swap ? bT : bB;
+    const double xB = fma(-f1, c1, c2) * r2;
+    const double xT = fma(-a2, xB, c1) * r1;
+    double x1 = top ? xT : xB, x2 = top ? xB : xT;
+    b[(size_t)(n - 1) * ld + lane] = x1;
+    p = n - 2;
+    for (; p >= 3; p -= 4) {
+      double y[4], v1[4], v2[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const size_t o = (size_t)(p - q) * ld + lane;
+        y[q] = b[o] * r[o];
+        v1[q] = u1[o];
+        v2[q] = u2[o];
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double x = fma(-v1[q], x1, fma(-v2[q], x2, y[q]));
+        b[(size_t)(p - q) * ld + lane] = x;
+        x2 = x1;
+        x1 = x;
+      }
+    }
+    for (; p >= 0; --p) {
+      const size_t o = (size_t)p * ld + lane;
+      const double x = fma(-u1[o], x1, fma(-u2[o], x2, b[o] * r[o]));
+      b[o] = x;
+      x2 = x1;
+      x1 = x;
+    }
+  }
+
+  // ---- by the whole warp, over the elements of one member's vector ----
+  __device__ void start(int t, int j) {
+    const int ln = threadIdx.x & 31;
+    for (int i = ln; i < m; i += 32) {
+      const uint32_t hsh = hash32((uint32_t)(i * 7919 + j * 104729 + 17));
+      *at(i, t) = ((double)(hsh & 0xffffff) / 16777216.0) - 0.5;
+    }
+  }
+  __device__ double norm2(int t) const {
+    double s = 0.0;
+    for (int i = threadIdx.x & 31; i < m; i += 32) {
+      const double x = *at(i, t);
+      s = fma(x, x, s);
+    }
+    return warp_sum(s);
+  }
+  __device__ void scale_by(int t, double f) {
+    for (int i = threadIdx.x & 31; i < m; i += 32) *at(i, t) *= f;
+  }
+  // Rayleigh quotient of member t's vector (in T's own units) and the unit vector as column j
+  __device__ void finish(const InvArgs& a, int t, int j, double sc) {
+    const int ln = threadIdx.x & 31;
+    double s = 0.0, q = 0.0;
+    for (int i = ln; i < m; i += 32) {
+      const double x = *at(i, t);
+      double tx = (d[i] * inv) * x;
+      if (i + 1 < m) tx = fma(2.0 * inv * e[i], *at(i + 1, t), tx);
+      q = fma(x, tx, q);
+      s = fma(x, x, s);
+    }
+    s = warp_sum(s);
+    q = warp_sum(q);
+    const double rn = (s > 0.0) ? rsqrt64_short(s) : 0.0;
+    for (int i = ln; i < m; i += 32) a.X[(size_t)i * a.kmax + j] = *at(i, t) * rn;
+    if (ln == 0) a.lam[j] = (q * rn * rn) * sc;
   }
 };
-#define SH(arr, i) w.arr[(size_t)(i) * w.tpb + t]
-
-// LU with partial pivoting of T - sigma I for member t (pivots kept as reciprocals, so the
-// solves are division free)
-__device__ void invit_factor(const double* d, const double* e, int m, double sigma, double tiny,
-                             const InvSmem& w, int t) {
-  double dcur = d[0] - sigma;
-  double ucur = (m > 1) ? e[0] : 0.0;  // superdiagonal entry of the current row
-  for (int i = 0; i < m - 1; ++i) {
-    const double li = e[i];
-    const double dn = d[i + 1] - sigma;
-    const double un = (i + 1 < m - 1) ? e[i + 1] : 0.0;
-    if (fabs(dcur) >= fabs(li)) {
-      double dv = (fabs(dcur) < tiny) ? ((dcur < 0.0) ? -tiny : tiny) : dcur;
-      double r = rcp64(dv);
-      double f = li * r;
-      SH(piv, i) = 0;
-      SH(dl, i) = f;
-      SH(di, i) = r;
-      SH(du, i) = ucur;
-      SH(du2, i) = 0.0;
-      dcur = dn - f * ucur;
-      ucur = un;
-    } else {
-      double r = rcp64(li);
-      double f = dcur * r;
-      SH(piv, i) = 1;
-      SH(dl, i) = f;
-      SH(di, i) = r;
-      SH(du, i) = dn;
-      SH(du2, i) = un;
-      dcur = ucur - f * dn;
-      ucur = -f * un;
-    }
-  }
-  double dv = (fabs(dcur) < tiny) ? ((dcur < 0.0) ? -tiny : tiny) : dcur;
-  SH(di, m - 1) = rcp64(dv);
-}
-
-// b <- (T - sigma I)^{-1} b for member t with its factors: L y = P b, then U x = y
-__device__ void invit_solve(int m, const InvSmem& w, int t) {
-  double carry = SH(b, 0);
-  for (int i = 0; i < m - 1; ++i) {
-    double nxt = SH(b, i + 1);
-    if (SH(piv, i) == 0) {
-      SH(b, i) = carry;
-      carry = nxt - SH(dl, i) * carry;
-    } else {
-      SH(b, i) = nxt;
-      carry = carry - SH(dl, i) * nxt;
-    }
-  }
-  SH(b, m - 1) = carry;
-  double x1 = 0.0, x2 = 0.0;
-  for (int i = m - 1; i >= 0; --i) {
-    double sv = SH(b, i) - SH(du, i) * x1 - SH(du2, i) * x2;
-    if (i == m - 1) sv = SH(b, i);
-    double xi = sv * SH(di, i);
-    SH(b, i) = xi;
-    x2 = x1;
-    x1 = xi;
-  }
-}
-
-// random start vector of candidate j (fixed hash, so every run is reproducible)
-__device__ void invit_start(int m, int j, const InvSmem& w, int t) {
-  for (int i = 0; i < m; ++i) {
-    uint32_t h = hash32((uint32_t)(i * 7919 + j * 104729 + 17));
-    SH(b, i) = ((double)(h & 0xffffff) / 16777216.0) - 0.5;
-  }
-}
-
-// sum_i x_i y_i over strided arrays with four independent partial sums (the FP64
-// latency chain is the cost of a lone thread's dot product)
-__device__ __forceinline__ double dot4(const double* x, size_t sx, const double* y, size_t sy,
-                                       int m) {
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-  int i = 0;
-  for (; i + 3 < m; i += 4) {
-    a0 = fma(x[(size_t)i * sx], y[(size_t)i * sy], a0);
-    a1 = fma(x[(size_t)(i + 1) * sx], y[(size_t)(i + 1) * sy], a1);
-    a2 = fma(x[(size_t)(i + 2) * sx], y[(size_t)(i + 2) * sy], a2);
-    a3 = fma(x[(size_t)(i + 3) * sx], y[(size_t)(i + 3) * sy], a3);
-  }
-  for (; i < m; ++i) a0 = fma(x[(size_t)i * sx], y[(size_t)i * sy], a0);
-  return (a0 + a1) + (a2 + a3);
-}
-
-// Rayleigh quotient of member t's (unit) vector, written with the vector to column j of X
-__device__ void invit_finish(const InvArgs& a, int j, const InvSmem& w, int t) {
-  const int m = a.m, K = a.kmax;
-  double rqv = 0.0;
-  for (int i = 0; i < m; ++i) {
-    const double xi = SH(b, i);
-    double tx = a.d[i] * xi;
-    if (i > 0) tx += a.e[i - 1] * SH(b, i - 1);
-    if (i < m - 1) tx += a.e[i] * SH(b, i + 1);
-    rqv += xi * tx;
-    a.X[(size_t)i * K + j] = xi;
-  }
-  a.rq[j] = rqv;
-}
-
-__device__ __forceinline__ void invit_shift(InvArgs& a) {
-  const size_t off = blockIdx.y * a.wb;
-  a.d = byte_shift(a.d, off);
-  a.e = byte_shift(a.e, off);
-  a.lam32 = byte_shift(a.lam32, off);
-  a.X = byte_shift(a.X, off);
-  a.rq = byte_shift(a.rq, off);
-}
 
 // Each solve shrinks the components along eigenvectors at distance delta by about
 // |lambda - sigma| / delta with |lambda - sigma| ~ 1e-7 span (single-precision shifts);
 // four solves reach FP64 accuracy for delta >= 1e-4 span.  Candidates closer than that
-// to a neighbour form a cluster (invit_cluster_kernel).
-__device__ __forceinline__ double invit_span(const InvArgs& a) {
-  return fmax(fabs((double)a.lam32[0]), fabs((double)a.lam32[a.m - 1])) + DBL_MIN;
-}
-__device__ __forceinline__ bool close_pair(const InvArgs& a, int j, double ortol) {
-  return (double)a.lam32[j] - (double)a.lam32[j + 1] <= ortol;  // descending
+// to a neighbour form a cluster.
+__device__ __forceinline__ bool close_pair(const float* lam32, int j, double ortol) {
+  return (double)lam32[j] - (double)lam32[j + 1] <= ortol;  // descending
 }
 
-// candidates that are not part of a cluster: one thread each
-__global__ void invit_kernel(InvArgs a) {
-  extern __shared__ double shd[];
-  invit_shift(a);
-  const int m = a.m, K = a.kmax, t = threadIdx.x;
-  const InvSmem w(shd, m, blockDim.x);
-  const int jj = blockIdx.x * blockDim.x + t;
-  if (jj >= K) return;
-  const double span = invit_span(a);
-  const double ortol = 1e-4 * span;
-  if ((jj > 0 && close_pair(a, jj - 1, ortol)) || (jj + 1 < K && close_pair(a, jj, ortol))) return;
-  const double tiny = 2.220446049250313e-16 * span;
-  invit_factor(a.d, a.e, m, (double)a.lam32[jj], tiny, w, t);
-  invit_start(m, jj, w, t);
-  for (int it = 0; it < 4; ++it) {
-    invit_solve(m, w, t);
-    const double nrm = dot4(&SH(b, 0), w.tpb, &SH(b, 0), w.tpb, m);
-    const double inv = (nrm > 0.0) ? rcp64(sqrt(nrm)) : 0.0;
-    for (int i = 0; i < m; ++i) SH(b, i) *= inv;
-  }
-  invit_finish(a, jj, w, t);
-}
-
-// The clusters of candidates (runs of neighbours closer than 1e-4 of the spectral radius),
-// each by one warp: `per` members at a time, one per lane, iterated as a block (block inverse
-// iteration): every lane solves with its own shift (shifts at least 1e-10 span apart),
-// then the block is orthonormalised (modified Gram-Schmidt, lanes in parallel) against
-// the cluster's finished columns and within itself, four times.  The vectors then span
-// the invariant subspace of the cluster's eigenvalues (any basis of it is a valid set of
-// eigenvectors when they are not resolved individually).
-// one cluster [jj, cend) by the warp, `per` members per pass
-__device__ void invit_cluster(const InvArgs& a, const InvSmem& w, int jj, int cend, int per,
-                              double span, double tiny) {
-  const int m = a.m, K = a.kmax, lane = threadIdx.x;
-  for (int j0 = jj; j0 < cend; j0 += per) {
-    const int nact = min(per, cend - j0);
-    const bool act = lane < nact;
-    const int t = act ? lane : 0;
-    const int j = j0 + lane;
-    if (act) {
-      double sigma = (double)a.lam32[jj];
-      for (int q = jj + 1; q <= j; ++q) sigma = fmin((double)a.lam32[q], sigma - 1e-10 * span);
-      invit_factor(a.d, a.e, m, sigma, tiny, w, t);
-      invit_start(m, j, w, t);
-    }
+// One cluster [jj, cend) by the warp, cper members at a time, iterated as a block (block
+// inverse iteration): every member solves with its own shift (shifts at least 1e-10 span
+// apart), then the block is orthonormalised (modified Gram-Schmidt) against the cluster's
+// finished columns and within itself, four times.  The vectors then span the invariant
+// subspace of the cluster's eigenvalues (any basis of it is a valid set of eigenvectors
+// when they are not resolved individually).
+__device__ void invit_cluster(const InvArgs& a, Inv& w, int jj, int cend, double span, double tiny,
+                              double sc) {
+  const int m = a.m, K = a.kmax, ln = threadIdx.x & 31;
+  for (int j0 = jj; j0 < cend; j0 += a.cper) {
+    const int nact = min(a.cper, cend - j0);
+    const int j = j0 + min(w.lane >> 1, nact - 1);
+    double sigma = (double)a.lam32[jj];
+    for (int q = jj + 1; q <= j; ++q) sigma = fmin((double)a.lam32[q], sigma - 1e-10 * span);
+    w.factor(sigma, tiny);
+    for (int t = 0; t < nact; ++t) w.start(t, j0 + t);
     __syncwarp();
     for (int it = 0; it < 4; ++it) {
-      if (act) {
-        invit_solve(m, w, t);
-        // against the finished columns of the cluster
-        for (int q = jj; q < j0; ++q) {
-          const double dv = dot4(a.X + q, (size_t)K, &SH(b, 0), w.tpb, m);
-          for (int i = 0; i < m; ++i) SH(b, i) -= dv * a.X[(size_t)i * K + q];
-        }
+      w.solve();
+      __syncwarp();
+      for (int t = 0; t < nact; ++t) {
+        const double s = w.norm2(t);
+        w.scale_by(t, s > 0.0 ? rsqrt64_short(s) : 0.0);
       }
       __syncwarp();
-      // within the block, in member order
-      for (int q = 0; q < nact; ++q) {
-        if (lane == q) {
-          const double nrm = dot4(&SH(b, 0), w.tpb, &SH(b, 0), w.tpb, m);
-          const double inv = (nrm > 0.0) ? rcp64(sqrt(nrm)) : 0.0;
-          for (int i = 0; i < m; ++i) SH(b, i) *= inv;
+      for (int t = 0; t < nact; ++t) {
+        for (int q = jj; q < j0 + t; ++q) {  // the finished columns, then the block's earlier ones
+          const bool fin = q < j0;
+          double dv = 0.0;
+          for (int i = ln; i < m; i += 32)
+            dv = fma(fin ? a.X[(size_t)i * K + q] : *w.at(i, q - j0), *w.at(i, t), dv);
+          dv = warp_sum(dv);
+          for (int i = ln; i < m; i += 32) {
+            double* x = w.at(i, t);
+            *x = fma(-dv, fin ? a.X[(size_t)i * K + q] : *w.at(i, q - j0), *x);
+          }
         }
-        __syncwarp();
-        if (act && lane > q) {
-          const double* bq = w.b + q;
-          const double dv = dot4(bq, w.tpb, &SH(b, 0), w.tpb, m);
-          for (int i = 0; i < m; ++i) SH(b, i) -= dv * bq[(size_t)i * w.tpb];
-        }
+        const double s = w.norm2(t);
+        w.scale_by(t, s > 0.0 ? rsqrt64_short(s) : 0.0);
         __syncwarp();
       }
     }
-    if (act) invit_finish(a, j, w, t);
+    for (int t = 0; t < nact; ++t) w.finish(a, t, j0 + t, sc);
     __syncwarp();
   }
 }
 
-__global__ void invit_cluster_kernel(InvArgs a, int per) {
+__global__ void __launch_bounds__(32) invit_kernel(InvArgs a) {
   extern __shared__ double shd[];
-  invit_shift(a);
-  const int K = a.kmax;
-  const InvSmem w(shd, a.m, per);
-  const double span = invit_span(a);
+  {
+    const size_t off = blockIdx.y * a.wb;
+    a.d = byte_shift(a.d, off);
+    a.e = byte_shift(a.e, off);
+    a.lam32 = byte_shift(a.lam32, off);
+    a.scale = byte_shift(a.scale, off);
+    a.X = byte_shift(a.X, off);
+    a.lam += (size_t)blockIdx.y * a.m;
+  }
+  const int m = a.m, K = a.kmax, ln = threadIdx.x;
+  const double sc = *a.scale;  // a power of two
+  const double inv = __hiloint2double((2046 << 20) - __double2hiint(sc), 0);
+  const bool clusters = (int)blockIdx.x < a.nclu;
+  const int per = clusters ? a.cper : a.per;
+  Inv w;
+  w.m = m;
+  w.h = (m + 1) / 2;
+  w.ld = 2 * per + (per >= 8 ? 1 : 0);  // odd rows where the whole warp walks a column
+  w.lane = ln < 2 * per ? ln : 2 * per - 2 + (ln & 1);  // idle lanes shadow the last member's
+  w.top = !(w.lane & 1);
+  w.n = w.top ? w.h : m - w.h;
+  const size_t sz = (size_t)w.h * w.ld;
+  w.f = shd;
+  w.r = w.f + sz;
+  w.u1 = w.r + sz;
+  w.u2 = w.u1 + sz;
+  w.b = w.u2 + sz;
+  w.d = a.d;
+  w.e = a.e;
+  w.inv = inv;
+  if (a.staged) {
+    double* sd = w.b + sz;
+    double* se = sd + m;
+    for (int i = ln; i < m; i += 32) {
+      sd[i] = a.d[i] * inv;
+      se[i] = (i < m - 1) ? a.e[i] * inv : 0.0;
+    }
+    w.d = sd;
+    w.e = se;
+    w.inv = 1.0;
+    __syncwarp();
+  }
+  if (m == 1) {
+    if (ln == 0 && blockIdx.x == gridDim.x - 1) {
+      a.X[0] = 1.0;
+      a.lam[0] = a.d[0];
+    }
+    return;
+  }
+  const double span = fmax(fabs((double)a.lam32[0]), fabs((double)a.lam32[m - 1])) + DBL_MIN;
   const double ortol = 1e-4 * span;
   const double tiny = 2.220446049250313e-16 * span;
-  // CTA c takes clusters c, c + gridDim.x, ... in order (a cluster: a run of two or more
-  // candidates whose neighbours are close); every lane scans the same candidates
-  int cidx = -1;
-  for (int jj = 0; jj + 1 < K;) {
-    if (!close_pair(a, jj, ortol)) {
-      ++jj;
-      continue;
-    }
-    int cend = jj + 2;
-    while (cend < K && close_pair(a, cend - 1, ortol)) ++cend;
-    ++cidx;
-    if (cidx % (int)gridDim.x == (int)blockIdx.x) invit_cluster(a, w, jj, cend, per, span, tiny);
-    jj = cend;
-  }
-}
-#undef SH
-
-// rank rule on the Rayleigh quotients of the candidates; the discarded weight is the
-// exact trace of T minus the kept eigenvalues.  Writes k and the full eigenvalue list.
-// floor_rel < 0 keeps all kmax candidates (the caller decides the rank from weights it
-// measures on the factor itself).
-__global__ void rank_kernel(const double* d, const double* rq, const float* lam32, int m,
-                            int kmax, long long max_bond, double tol, double floor_rel,
-                            int* k_dev, double* lam, size_t wb) {
-  __shared__ double s_tr;
-  // matrix blockIdx.x of a batch
-  d = byte_shift(d, blockIdx.x * wb);
-  rq = byte_shift(rq, blockIdx.x * wb);
-  lam32 = byte_shift(lam32, blockIdx.x * wb);
-  k_dev += blockIdx.x;
-  lam += (size_t)blockIdx.x * m;
-  if (threadIdx.x == 0) {
-    double tr = 0.0;
-    for (int i = 0; i < m; ++i) tr += d[i];
-    s_tr = tr;
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < m; j += blockDim.x) lam[j] = (j < kmax) ? rq[j] : (double)lam32[j];
-  if (threadIdx.x != 0) return;
-  const double l0 = rq[0];
-  int k = 1;
-  if (floor_rel < 0.0) {
-    k = kmax;  // every candidate: the caller applies the rank rule itself
-  } else if (l0 > 0.0) {
-    k = 0;
-    while (k < kmax && rq[k] > floor_rel * l0) ++k;
-    if (tol > 0.0) {
-      const double total = fmax(s_tr, 0.0);
-      double tail = total;
-      int kt = 0;
-      while (kt < kmax && tail > tol * tol * total) {
-        tail -= fmax(rq[kt], 0.0);
-        ++kt;
+  if (clusters) {
+    // clusters blockIdx.x, blockIdx.x + nclu, ... in order (a run of two or more candidates
+    // whose neighbours are close)
+    int cidx = -1;
+    for (int jj = 0; jj + 1 < K;) {
+      if (!close_pair(a.lam32, jj, ortol)) {
+        ++jj;
+        continue;
       }
-      if (kt < 1) kt = 1;
-      if (kt < k) k = kt;
+      int cend = jj + 2;
+      while (cend < K && close_pair(a.lam32, cend - 1, ortol)) ++cend;
+      ++cidx;
+      if (cidx % a.nclu == (int)blockIdx.x) invit_cluster(a, w, jj, cend, span, tiny, sc);
+      jj = cend;
     }
-    if (max_bond > 0 && k > max_bond) k = (int)max_bond;
-    if (k < 1) k = 1;
+    return;
   }
-  if (k > kmax) k = kmax;
-  *k_dev = k;
+  // candidates j0 .. j0 + per - 1, the lone ones among them
+  const int j0 = ((int)blockIdx.x - a.nclu) * per;
+  const int nact = min(per, K - j0);
+  auto lone = [&](int j) {
+    return !((j > 0 && close_pair(a.lam32, j - 1, ortol)) ||
+             (j + 1 < K && close_pair(a.lam32, j, ortol)));
+  };
+  bool any = false;
+  for (int t = 0; t < nact; ++t) any = any || lone(j0 + t);
+  if (!any) return;
+  const int j = j0 + min(w.lane >> 1, nact - 1);
+  w.factor((double)a.lam32[j], tiny);
+  for (int t = 0; t < nact; ++t) w.start(t, j0 + t);
+  __syncwarp();
+  for (int it = 0; it < 4; ++it) w.solve();
+  __syncwarp();
+  for (int t = 0; t < nact; ++t)
+    if (lone(j0 + t)) w.finish(a, t, j0 + t, sc);
 }
 
 // ---- back transformation: U[:, jj] = H_0 ... H_{m-2} X[:, jj] ------------------------
@@ -943,7 +1001,7 @@ __global__ void rank_kernel(const double* d, const double* rq, const float* lam3
 template <typename T>
 __global__ void __launch_bounds__(128) backtransform_kernel(const T* V, const T* tau,
                                                             const double* X, int m, int kmax,
-                                                            const int* k_dev, T* U, size_t wb) {
+                                                            T* U, size_t wb) {
   using O = ops<T>;
   extern __shared__ unsigned char smem_raw[];
   T* u = reinterpret_cast<T*>(smem_raw);
@@ -952,12 +1010,9 @@ __global__ void __launch_bounds__(128) backtransform_kernel(const T* V, const T*
   V = byte_shift(V, blockIdx.y * wb);
   tau = byte_shift(tau, blockIdx.y * wb);
   X = byte_shift(X, blockIdx.y * wb);
-  k_dev += blockIdx.y;
   U += (size_t)blockIdx.y * m * kmax;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int jj = blockIdx.x;
-  const int k = *k_dev;
-  if (jj >= k) return;
   for (int i = tid; i < m; i += 128) u[i] = O::make(X[(int64_t)i * kmax + jj], 0.0);
   __syncthreads();
   int par = 0;
@@ -997,8 +1052,7 @@ constexpr int BT_WARPS = 8;
 // per reflector in FP32 (the partial sums and tau * sum stay FP64).
 template <typename T, bool DF>
 __global__ void __launch_bounds__(32 * BT_WARPS) backtransform32_kernel(
-    const T* V, const T* tau, const double* X, int m, int kmax, const int* k_dev, T* U,
-    size_t wb) {
+    const T* V, const T* tau, const double* X, int m, int kmax, T* U, size_t wb) {
   using O = ops<T>;
   using D = typename dfof<T>::type;
   using E = typename std::conditional<DF, D, T>::type;  // element type of u and v in smem
@@ -1013,13 +1067,10 @@ __global__ void __launch_bounds__(32 * BT_WARPS) backtransform32_kernel(
   V = byte_shift(V, blockIdx.y * wb);
   tau = byte_shift(tau, blockIdx.y * wb);
   X = byte_shift(X, blockIdx.y * wb);
-  k_dev += blockIdx.y;
   U += (size_t)blockIdx.y * m * kmax;
-  const int k = *k_dev;
   const int c0 = blockIdx.x * 32;
-  if (c0 >= k) return;
   const int col = c0 + lane;
-  const bool live = col < k;
+  const bool live = col < kmax;
   const int rb = (m + BT_WARPS - 1) / BT_WARPS;
   const int r0 = warp * rb, r1 = min(m, r0 + rb);
   auto to_e = [](const T& x) -> E {
@@ -1133,12 +1184,12 @@ size_t eig_workspace_bytes(int m, int kmax, bool cplx) {
   b += align256(sizeof(double) * m);                 // d
   b += align256(sizeof(double) * m);                 // e
   b += align256(sizeof(float) * m);                  // lam32
-  b += align256(sizeof(double) * m);                 // rq
   b += align256(ts * m);                             // tau
   b += align256(ts * (size_t)m * m);                 // V
   b += align256(ts * 2 * m);                         // vbuf
   b += align256(ts * 2 * m);                         // p (two buffers)
   b += align256(sizeof(double) * 4);                 // dot
+  b += align256(sizeof(double));                     // scale of T
   b += align256(sizeof(GridBarrier));                // barrier
   b += align256(sizeof(double) * (size_t)m * kmax);  // X
   b += align256(2 * ts * (size_t)m * m);             // exchange of the lone reduction
@@ -1146,9 +1197,8 @@ size_t eig_workspace_bytes(int m, int kmax, bool cplx) {
 }
 
 template <typename T>
-cudaError_t heev_top(T* A, int m, int kmax, int64_t max_bond, double tol, double floor_rel,
-                     double* lam, T* U, int* k_dev, void* work, int* status, int num_sms,
-                     cudaStream_t s, int nb, bool prefer_cluster, bool df) {
+cudaError_t heev_top(T* A, int m, int kmax, double* lam, T* U, void* work, int* status,
+                     int num_sms, cudaStream_t s, int nb, bool prefer_cluster, bool df) {
   char* w = static_cast<char*>(work);
   auto take = [&](size_t bytes) {
     char* p = w;
@@ -1160,12 +1210,12 @@ cudaError_t heev_top(T* A, int m, int kmax, int64_t max_bond, double tol, double
   double* d = (double*)take(sizeof(double) * m);
   double* e = (double*)take(sizeof(double) * m);
   float* lam32 = (float*)take(sizeof(float) * m);
-  double* rq = (double*)take(sizeof(double) * m);
   T* tau = (T*)take(ts * m);
   T* V = (T*)take(ts * (size_t)m * m);
   T* vbuf = (T*)take(ts * 2 * m);
   T* p = (T*)take(ts * 2 * m);
   double* dot = (double*)take(sizeof(double) * 4);
+  double* scale = (double*)take(sizeof(double));
   GridBarrier* bar = (GridBarrier*)take(sizeof(GridBarrier));
   double* X = (double*)take(sizeof(double) * (size_t)m * kmax);
   T* Xg = (T*)take(2 * ts * (size_t)m * m);
@@ -1243,36 +1293,35 @@ cudaError_t heev_top(T* A, int m, int kmax, int64_t max_bond, double tol, double
   }
   }
   if (err != cudaSuccess) return err;
-  KTimer te(CBC_K_EIG, s, 4, fl_rest);
+  KTimer te(CBC_K_EIG, s, 3, fl_rest);
   // 2. eigenvalue estimates
   const int wpb = 8;
   bisect32_kernel<<<dim3((m + wpb - 1) / wpb, nb), 32 * wpb, 2 * sizeof(float) * m, s>>>(
-      d, e, m, lam32, wb);
-  // 3. eigenvectors of T for the candidates, FP64.  The LU and the solves are long
-  // dependent FP64 chains: alone, one candidate per CTA runs fastest (a whole SM and its
-  // FP64 unit per chain); in a batch with many candidates per SM, up to 16 candidates
-  // share a warp (one per lane), which issues 16x fewer FP64 warp instructions.
-  int tpb = 1;
-  if ((size_t)nb * kmax >= 4 * (size_t)num_sms)
-    tpb = (int)std::max<size_t>(1, std::min<size_t>(16, (200 * 1024 - 64) / ((size_t)m * 41)));
-  size_t shi = (size_t)tpb * m * 41 + 64;
-  err = allow_max_smem((const void*)invit_kernel);
-  if (err != cudaSuccess) return err;
-  InvArgs ia{d, e, lam32, m, kmax, X, rq, wb};
-  invit_kernel<<<dim3((kmax + tpb - 1) / tpb, nb), tpb, shi, s>>>(ia);
-  // clusters: one warp each, four CTAs per matrix that share its clusters round robin, as
-  // many members per pass as shared memory holds
-  if (kmax >= 2) {
-    const int per = (int)std::max<size_t>(1, std::min<size_t>(32, (200 * 1024 - 64) / ((size_t)m * 41)));
-    const size_t shc = (size_t)per * m * 41 + 64;
-    err = allow_max_smem((const void*)invit_cluster_kernel);
+      d, e, m, kmax, lam32, scale, lam, wb);
+  // 3. eigenvectors of T for the candidates, FP64: as few per warp as gives every SM one warp
+  // (a warp costs the same for one member as for 16), and at most what shared memory holds
+  {
+    const size_t room = 216 * 1024, half = (size_t)(m + 1) / 2;
+    auto bytes = [&](int per) {
+      return 5 * half * (size_t)(2 * per + (per >= 8 ? 1 : 0)) * sizeof(double);
+    };
+    int cper = kInvMax;
+    while (cper > 1 && bytes(cper) > room) --cper;
+    const int nclu = kmax >= 2 ? std::min(4, kmax / 2) : 0;
+    const int sms = std::max(1, num_sms - nclu * nb);
+    const int per = (int)std::min<int64_t>(
+        cper, std::max<int64_t>(1, ((int64_t)nb * kmax + sms - 1) / sms));
+    size_t sh = std::max(bytes(per), nclu > 0 ? bytes(cper) : 0);
+    const bool staged = sh + 2 * (size_t)m * sizeof(double) <= 226 * 1024;
+    if (staged) sh += 2 * (size_t)m * sizeof(double);
+    err = allow_max_smem((const void*)invit_kernel);
     if (err != cudaSuccess) return err;
-    invit_cluster_kernel<<<dim3(std::min(4, kmax / 2), nb), 32, shc, s>>>(ia, per);
+    InvArgs ia{d, e, lam32, scale, m, kmax, X, lam, wb, per, cper, nclu, staged ? 1 : 0};
+    invit_kernel<<<dim3(nclu + (kmax + per - 1) / per, nb), 32, sh, s>>>(ia);
+    err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
   }
-  // 4. rank rule on the refined eigenvalues
-  rank_kernel<<<nb, 256, 0, s>>>(d, rq, lam32, m, kmax, (long long)max_bond, tol, floor_rel,
-                                 k_dev, lam, wb);
-  // 5. back transformation: 32 vectors per CTA (fewer FP64 instructions) when u fits in
+  // 4. back transformation: 32 vectors per CTA (fewer FP64 instructions) when u fits in
   // shared memory and the batch gives enough CTAs to spread the FP64 work over the SMs;
   // else one vector per CTA
   const size_t shm32 = ((size_t)m * 32 + 3 * (size_t)m) * ts;
@@ -1283,10 +1332,10 @@ cudaError_t heev_top(T* A, int m, int kmax, int64_t max_bond, double tol, double
     if (err != cudaSuccess) return err;
     if (df)
       backtransform32_kernel<T, true><<<dim3((kmax + 31) / 32, nb), 32 * BT_WARPS, shm32, s>>>(
-          V, tau, X, m, kmax, k_dev, U, wb);
+          V, tau, X, m, kmax, U, wb);
     else
       backtransform32_kernel<T, false><<<dim3((kmax + 31) / 32, nb), 32 * BT_WARPS, shm32, s>>>(
-          V, tau, X, m, kmax, k_dev, U, wb);
+          V, tau, X, m, kmax, U, wb);
     return cudaGetLastError();
   }
   size_t shm = (size_t)m * ts;
@@ -1294,14 +1343,13 @@ cudaError_t heev_top(T* A, int m, int kmax, int64_t max_bond, double tol, double
     err = allow_max_smem((const void*)backtransform_kernel<T>);
     if (err != cudaSuccess) return err;
   }
-  backtransform_kernel<T><<<dim3(kmax, nb), 128, shm, s>>>(V, tau, X, m, kmax, k_dev, U, wb);
+  backtransform_kernel<T><<<dim3(kmax, nb), 128, shm, s>>>(V, tau, X, m, kmax, U, wb);
   return cudaGetLastError();
 }
 
-template cudaError_t heev_top<double>(double*, int, int, int64_t, double, double, double*,
-                                      double*, int*, void*, int*, int, cudaStream_t, int, bool,
-                                      bool);
-template cudaError_t heev_top<zdbl>(zdbl*, int, int, int64_t, double, double, double*, zdbl*,
-                                    int*, void*, int*, int, cudaStream_t, int, bool, bool);
+template cudaError_t heev_top<double>(double*, int, int, double*, double*, void*, int*, int,
+                                      cudaStream_t, int, bool, bool);
+template cudaError_t heev_top<zdbl>(zdbl*, int, int, double*, zdbl*, void*, int*, int,
+                                    cudaStream_t, int, bool, bool);
 
 }  // namespace cbc

@@ -82,17 +82,14 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
                     int* status, cudaStream_t s, int nb = 1, int* wide = nullptr);
 
 // ---- Hermitian eigensolver (FP64): A (m x m, row-major, overwritten) -----------------
-// Finds the eigenvalues in descending order and the eigenvectors of the `k` largest,
-// where k = min(max_bond (if > 0), #{lambda_j > floor * lambda_0}, smallest k with
-// sum_{j>=k} lambda_j <= tol^2 sum_j lambda_j (if tol > 0)), at least 1; floor < 0 gives
-// k = kmax (every candidate).  Outputs: lam[m], U (m x kmax, row-major, column j =
-// eigenvector j), *k_dev.  Workspace: eig_workspace_bytes(m, kmax).
-struct EigWork;
+// Finds the eigenvalues in descending order (the first kmax as FP64 Rayleigh quotients of the
+// vectors, the rest as single-precision estimates) and the eigenvectors of the kmax largest.
+// Outputs: lam[m], U (m x kmax, row-major, column j = eigenvector j); nb matrices m*m (lam m,
+// U m*kmax) elements apart.  Workspace: nb * eig_workspace_bytes(m, kmax).
 size_t eig_workspace_bytes(int m, int kmax, bool cplx);
 template <typename T>
-cudaError_t heev_top(T* A, int m, int kmax, int64_t max_bond, double tol, double floor_rel,
-                     double* lam, T* U, int* k_dev, void* work, int* status, int num_sms,
-                     cudaStream_t s, int nb = 1, bool prefer_cluster = false,
+cudaError_t heev_top(T* A, int m, int kmax, double* lam, T* U, void* work, int* status,
+                     int num_sms, cudaStream_t s, int nb = 1, bool prefer_cluster = false,
                      bool df = false);
 
 // Householder tridiagonalisation by one thread-block cluster per matrix (rows in shared
@@ -141,11 +138,6 @@ cudaError_t launch_cluster(const void* func, int cluster, int grid, int threads,
 template <typename T>
 cudaError_t normalize_inplace(T* x, int64_t n, double* log_acc, int* status, double* scratch,
                               cudaStream_t s, int nb = 1, bool shared_log = false);
-// L[r, c] = sqrt(lam[r]) * conj(V[c, r]) for r < k (V: n x ldv row-major), L: k x n;
-// nb problems: V n*ldv, lam n, k_dev 1 and L l_bs elements apart
-template <typename T>
-cudaError_t scaled_adjoint(const T* V, int ldv, const double* lam, const int* k_dev, int n,
-                           T* L, cudaStream_t s, int nb = 1, int64_t l_bs = 0);
 // out = in with its axes permuted: out dims are in dims[perm[0]], in dims[perm[1]], ...
 // (row-major, rank <= 8); nb tensors of the same shape, back to back in in and out
 template <typename T>

@@ -56,23 +56,6 @@ __global__ void scale_kernel(T* x, int64_t n, const double* sumsq, double* log_a
     x[i] = ops<T>::scale(inv, x[i]);
 }
 
-template <typename T>
-__global__ void scaled_adjoint_kernel(const T* V, int ldv, const double* lam, const int* k_dev,
-                                      int n, T* L, int64_t l_bs) {
-  V += (int64_t)blockIdx.y * n * ldv;
-  lam += (int64_t)blockIdx.y * n;
-  k_dev += blockIdx.y;
-  L += (int64_t)blockIdx.y * l_bs;
-  int k = *k_dev;
-  int64_t total = (int64_t)k * n;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    int r = (int)(t / n), c = (int)(t % n);
-    double sl = sqrt(fmax(lam[r], 0.0));
-    L[t] = ops<T>::scale(sl, ops<T>::conj(V[(int64_t)c * ldv + r]));
-  }
-}
-
 // between nb separate tensors (ptrs[b], n elements each) and one buffer holding them
 // `stride` elements apart; instance blockIdx.y
 template <typename T>
@@ -388,15 +371,6 @@ cudaError_t normalize_inplace(T* x, int64_t n, double* log_acc, int* status, dou
 }
 
 template <typename T>
-cudaError_t scaled_adjoint(const T* V, int ldv, const double* lam, const int* k_dev, int n, T* L,
-                           cudaStream_t s, int nb, int64_t l_bs) {
-  note_launches(CBC_K_AUX, 1);
-  scaled_adjoint_kernel<T><<<dim3(grid_for((int64_t)ldv * n), nb), 256, 0, s>>>(V, ldv, lam, k_dev,
-                                                                              n, L, l_bs);
-  return cudaGetLastError();
-}
-
-template <typename T>
 cudaError_t group_copy(T* const* ptrs, T* buf, int64_t stride, int64_t n, int nb, bool to_group,
                        cudaStream_t s) {
   note_launches(CBC_K_AUX, 1);
@@ -600,10 +574,6 @@ template cudaError_t normalize_inplace<double>(double*, int64_t, double*, int*, 
                                                cudaStream_t, int, bool);
 template cudaError_t normalize_inplace<zdbl>(zdbl*, int64_t, double*, int*, double*, cudaStream_t,
                                              int, bool);
-template cudaError_t scaled_adjoint<double>(const double*, int, const double*, const int*, int,
-                                            double*, cudaStream_t, int, int64_t);
-template cudaError_t scaled_adjoint<zdbl>(const zdbl*, int, const double*, const int*, int, zdbl*,
-                                          cudaStream_t, int, int64_t);
 template cudaError_t permute<double>(const double*, double*, int, const int64_t*, const int*,
                                      cudaStream_t, int);
 template cudaError_t permute<zdbl>(const zdbl*, zdbl*, int, const int64_t*, const int*,

@@ -110,7 +110,6 @@ int sweeps(const Args& a, Bump& b, bool dry) {
   NA_GET(d_int, int, 4);
   NA_GET(d_dbl, double, 4);
   int* status = d_int;
-  int* k_dev = d_int + 1;
   double* log_fwd = d_dbl;
   double* log_out = d_dbl + 1;
   double* dscr = d_dbl + 2;
@@ -171,7 +170,7 @@ int sweeps(const Args& a, Bump& b, bool dry) {
       else
         NA_CK(gemm_f64<T>(n, n, m, 1, Lp, View::transposed(n), true, Lp, View::rowmajor(n), false,
                           K, View::rowmajor(n), s));
-      NA_CK(heev_top<T>(K, g, kmax, kmax, 0.0, -1.0, lam, U, k_dev, work, status, num_sms(), s));
+      NA_CK(heev_top<T>(K, g, kmax, lam, U, work, status, num_sms(), s));
       if (rows) {  // U^H M, kmax x n, in the environment buffer
         NA_CK(gemm_f64<T>(kmax, n, m, 1, U, View::transposed(kmax), true, Lp, View::rowmajor(n),
                           false, envn, View::rowmajor(n), s));

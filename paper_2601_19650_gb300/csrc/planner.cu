@@ -93,11 +93,10 @@ int status_to_rc(int st) {
   }
 }
 
-// device scalars of one call: one status word; k, the two log scales and the
-// reduction scratch per instance of a group
+// device scalars of one call: one status word; the two log scales and the reduction scratch
+// per instance of a group
 struct Scalars {
   int* status;
-  int* k;
   double* log_fwd;
   double* log_out;
   double* scratch;
@@ -241,8 +240,7 @@ int refine_level2(Arena& ar, const Prec& pr, const T* M, int m, int n, int kmax,
   else        // R^H R
     CK(tgemm<T>(pr, true, true, n, n, m, R, View::transposed(n), true, R, View::rowmajor(n),
                 false, K2, View::rowmajor(n), s));
-  CK(heev_top<T>(K2, g, k2, k2, 0.0, -1.0, lam2, U2, sc.k, work, sc.status, num_sms(), s, 1,
-                 o.concurrent, false));
+  CK(heev_top<T>(K2, g, k2, lam2, U2, work, sc.status, num_sms(), s, 1, o.concurrent, false));
   // U2 <- U2 - U1r (U1r^H U2)
   CK(tgemm<T>(pr, true, false, jlo, k2, g, U1, View::transposed(kmax), true, U2,
               View::rowmajor(k2), false, C, View::rowmajor(k2), s));
@@ -328,8 +326,7 @@ int compress_rows(Arena& ar, const Prec& pr, const T* M, int m, int n, int64_t m
   // ||M||_F^2, the weight of the cut: the trace of the Gram (g reads instead of m n)
   CK(trace_real<T>(K, g, (int64_t)g * g, total_dev, s, nb));
   // every candidate; the mixed path reduces batches to tridiagonal form in double-float
-  CK(heev_top<T>(K, g, kmax, kmax, 0.0, -1.0, lam, U, sc.k, work, sc.status, num_sms(), s, nb,
-                 o.concurrent, pr.mixed));
+  CK(heev_top<T>(K, g, kmax, lam, U, work, sc.status, num_sms(), s, nb, o.concurrent, pr.mixed));
   const int64_t ubs = (int64_t)g * kmax;
   T* W = nullptr;
   int64_t wbs;
@@ -524,12 +521,12 @@ int run_tt_group(const std::vector<const Net*>& sts, const std::vector<const Net
       }
   Arena ar(s);   // scalars, environments: the whole call
   Arena tmp(s);  // per-site temporaries, released after each site
-  int* d_int = ar.get<int>(std::max(4, 1 + nb));
+  int* d_int = ar.get<int>(4);
   double* d_dbl = ar.get<double>(std::max(4, 3 * nb));
   CKA(d_int); CKA(d_dbl);
-  CK(cudaMemsetAsync(d_int, 0, std::max(4, 1 + nb) * sizeof(int), s));
+  CK(cudaMemsetAsync(d_int, 0, 4 * sizeof(int), s));
   CK(cudaMemsetAsync(d_dbl, 0, std::max(4, 3 * nb) * sizeof(double), s));
-  Scalars sc{d_int, d_int + 1, d_dbl, d_dbl + nb, d_dbl + 2 * nb};
+  Scalars sc{d_int, d_dbl, d_dbl + nb, d_dbl + 2 * nb};
   Prec pr;
   pr.mixed = (o.precision == CBC_PREC_MIXED);
   pr.cholqr_f64 = o.cholqr_f64;
@@ -812,7 +809,7 @@ int run_tt_direct(const Net& st, const Net& op, int64_t max_bond, double tol, co
   CKA(d_int); CKA(d_dbl);
   CK(cudaMemsetAsync(d_int, 0, 4 * sizeof(int), s));
   CK(cudaMemsetAsync(d_dbl, 0, 4 * sizeof(double), s));
-  Scalars sc{d_int, d_int + 1, d_dbl, d_dbl + 1, d_dbl + 2};
+  Scalars sc{d_int, d_dbl, d_dbl + 1, d_dbl + 2};
   Prec pr;
   pr.mixed = (o.precision == CBC_PREC_MIXED);
   pr.cholqr_f64 = o.cholqr_f64;
@@ -1098,15 +1095,15 @@ int run_tree(const Net& st, const Net& op, int64_t max_bond, double tol, const O
   const auto& ch = st.children;
   Arena ar(s);   // environments and scalars: the whole call
   Arena tmp(s);  // per group: gathers, contractions, workspaces
-  // scalars: status, k per group member, the output's log scale, and per member the
-  // forward log scales (unused) and the normalisation scratch
-  int* d_int = ar.get<int>(1 + n);
+  // scalars: status, the output's log scale, and per member the forward log scales (unused)
+  // and the normalisation scratch
+  int* d_int = ar.get<int>(4);
   double* d_dbl = ar.get<double>(1 + 2 * (size_t)n);
   CKA(d_int);
   CKA(d_dbl);
-  CK(cudaMemsetAsync(d_int, 0, (1 + n) * sizeof(int), s));
+  CK(cudaMemsetAsync(d_int, 0, 4 * sizeof(int), s));
   CK(cudaMemsetAsync(d_dbl, 0, (1 + 2 * (size_t)n) * sizeof(double), s));
-  Scalars sc{d_int, d_int + 1, d_dbl + 1, d_dbl, d_dbl + 1 + n};
+  Scalars sc{d_int, d_dbl + 1, d_dbl, d_dbl + 1 + n};
   Prec pr;
   pr.mixed = (o.precision == CBC_PREC_MIXED);
   pr.cholqr_f64 = o.cholqr_f64;
@@ -1485,9 +1482,9 @@ int run_tree(const Net& st, const Net& op, int64_t max_bond, double tol, const O
     int rc = run_groups(groups, step3);
     if (rc != CBC_OK) return rc;
   }
-  int h[2];
+  int h[1];
   double hl = 0.0;
-  CK(cudaMemcpyAsync(h, sc.status, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(h, sc.status, sizeof(int), cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(&hl, sc.log_out, sizeof(double), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   if (h[0] != 0) return status_to_rc(h[0]);

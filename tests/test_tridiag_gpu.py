@@ -1,6 +1,6 @@
 """The reductions to tridiagonal form at the edges of their ranges, through cbc_heev: sizes
 around the columns per thread (256) and the rows per CTA, reflectors that are the identity
-(diagonal, block-diagonal and low-rank matrices)."""
+(diagonal, block-diagonal and low-rank matrices), and matrices of very small or large norm."""
 import numpy as np
 import pytest
 
@@ -45,7 +45,7 @@ def test_lone_sizes(m, cplx):
 
 @pytest.mark.parametrize("cplx", [False, True])
 @pytest.mark.parametrize("nb,mixed", [(1, False), (3, False), (3, True)])
-@pytest.mark.parametrize("kind", ["diagonal", "blocks", "rank"])
+@pytest.mark.parametrize("kind", ["diagonal", "blocks", "rank", "tiny", "huge"])
 def test_special_matrices(kind, nb, mixed, cplx):
     m = 48
     a = _random(m, cplx)
@@ -60,4 +60,8 @@ def test_special_matrices(kind, nb, mixed, cplx):
         x = _random(28, cplx, 2)[:, :5]
         a[20:, 20:] = x @ x.conj().T
         a += 0.5 * np.diag(np.linspace(0.0, 1.0, m))
+    elif kind == "tiny":
+        a = a * (1e-60 if not mixed else 1e-12)
+    elif kind == "huge":
+        a = a * (1e60 if not mixed else 1e12)
     _check(a, kmax=m // 2, nb=nb, mixed=mixed)
