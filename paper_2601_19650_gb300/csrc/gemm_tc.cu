@@ -31,8 +31,8 @@
 // atom, 128B or 64B swizzle, two smem stages), warp 1 issues tcgen05.mma (one elected thread; one MMA per slice of A,
 // against all the slices of B it meets side by side) into S TMEM accumulators per K chunk,
 // double buffered across chunks and tiles so the epilogue of
-// one chunk overlaps the MMAs of the next, and 4 (BN = 32) or 8 (BN = 64) epilogue warps
-// drain TMEM (tcgen05.ld) into int64 registers and write FP64, assembled with integer
+// one chunk overlaps the MMAs of the next, and 4 epilogue warps per 16
+// columns drain TMEM (tcgen05.ld) into int64 registers and write FP64, assembled with integer
 // operations.  Every wait is bounded (clock64); a timeout raises CBC_ERR_TIMEOUT in the
 // status word, all roles leave their loops, and TMEM is freed before the CTA exits.
 #include <cooperative_groups.h>
@@ -60,11 +60,14 @@ __host__ __device__ constexpr int ka(int S) { return S > 5 ? 32 : 64; }
 // so that the digit word and its bias fit in 64 bits
 __host__ __device__ constexpr int head(int S) { return S > 5 ? 6 : 7; }
 constexpr int NSTAGE = 2;
-// warps: 0 TMA, 1 MMA, then 4 epilogue warps (one per TMEM lane quarter) per group of 32
-// accumulator columns, or of 16 when BN is not a multiple of 32 (BN = 48)
-__host__ __device__ constexpr int epi_cols(int BN) { return (BN % 32 == 0) ? 32 : 16; }
+// warps: 0 TMA, 1 MMA, then 4 epilogue warps (one per TMEM lane quarter) per group of 16
+// accumulator columns: a tile's last sums leave through integer chains that one warp per
+// scheduler cannot hide (64-wide tiles, chosen for long K, keep 32 per warp and their
+// registers)
+__host__ __device__ constexpr int epi_cols(int BN) { return BN == 64 ? 32 : 16; }
 __host__ __device__ constexpr int epi_warps(int BN) { return (BN / epi_cols(BN)) * 4; }
 __host__ __device__ constexpr int nthreads(int BN) { return 64 + 32 * epi_warps(BN); }
+int g_sms = 0;
 constexpr long long WAIT_CYCLES = 4000000000LL;  // ~2 s at 2 GHz
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -157,6 +160,16 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+      "%11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
@@ -171,16 +184,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-      "%11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
 template <int CW>
 __device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[CW]) {
   if constexpr (CW == 32)
@@ -209,53 +212,46 @@ struct TcArgs {
   int total_tiles;       // tiles_m * tiles_n * splits * problems
 };
 
-// ldexp((double)a, e) formed with integer operations: the int64 is rounded to 53 bits
-// (round to nearest, ties to even, as the conversion instruction does) and the exponent
-// field written directly, so the epilogue keeps off the narrow FP64 pipe of this part.
-// Results outside the normal range take the FP64 route.  Not inlined: the epilogue calls
-// it once per accumulator, and 32 inlined copies per instantiation overflow the
-// instruction cache.
-__device__ __noinline__ double i64_ldexp(long long a, int e) {
-  if (a == 0) return 0.0;
-  const unsigned long long neg = a < 0 ? 1ull : 0ull;
-  const unsigned long long m = neg ? 0ull - (unsigned long long)a : (unsigned long long)a;
-  int top = 63 - __clzll((long long)m);
-  unsigned long long mant;
-  if (top > 52) {
-    const int sh = top - 52;
-    const unsigned long long rem = m & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
-    mant = m >> sh;
-    if (rem > half || (rem == half && (mant & 1ull))) {
-      ++mant;
-      if (mant == (1ull << 53)) {
-        mant >>= 1;
-        ++top;
-      }
-    }
-  } else {
-    mant = m << (52 - top);
+// (n + sticky) 2^e with n normalised (bit 63 set) and sticky != 0 for bits that fell off below
+// it, rounded to a double (to nearest, ties to even) in integer operations: the epilogue keeps
+// off the narrow FP64 pipe of this part.  Adding the 53-bit significand to the exponent field
+// less one carries into the exponent both for its leading bit and when rounding overflows.
+__device__ __forceinline__ double round_ldexp(unsigned long long n, bool sticky, int e, bool neg) {
+  const unsigned long long r = n + 0x3ffull + (((n >> 11) & 1ull) | (sticky ? 1ull : 0ull));
+  const unsigned long long mant = (r >> 11) | (r < n ? 1ull << 53 : 0ull);
+  const int E = 63 + e + 1023;  // exponent field of n 2^e
+  if (E <= 0 || E >= 2046) {
+    const double v = ldexp((double)mant, e + 11);
+    return neg ? -v : v;
   }
-  const int E = top + e + 1023;
-  if (E <= 0 || E >= 2047) return ldexp((double)a, e);
-  return __longlong_as_double((long long)((neg << 63) | ((unsigned long long)E << 52) |
-                                          (mant & ((1ull << 52) - 1ull))));
+  return __longlong_as_double((long long)(((unsigned long long)(E - 1) << 52) + mant +
+                                          (neg ? 1ull << 63 : 0ull)));
 }
-
-// ldexp(hi 2^32 + lo, e) with one rounding: the 128-bit sum is shifted down to 63 bits with
-// the bits that fall off kept as a sticky bit, which rounds the same way
-__device__ __noinline__ double i96_ldexp(long long hi, long long lo, int e) {
-  const __int128 t = ((__int128)hi << 32) + (__int128)lo;
-  const bool neg = t < 0;
-  const unsigned __int128 m = neg ? -(unsigned __int128)t : (unsigned __int128)t;
-  const unsigned long long top = (unsigned long long)(m >> 64);
-  unsigned long long w = (unsigned long long)m;
-  int sh = 0;
-  if (top != 0ull || (w >> 63)) {
-    sh = 65 - (top ? __clzll((long long)top) : 64);
-    const unsigned __int128 rest = m & (((unsigned __int128)1 << sh) - 1);
-    w = (unsigned long long)(m >> sh) | (rest != 0 ? 1ull : 0ull);
+// ldexp((double)a, e)
+__device__ __forceinline__ double i64_ldexp(long long a, int e) {
+  if (a == 0) return 0.0;
+  const unsigned long long m = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
+  const int lz = __clzll((long long)m);
+  return round_ldexp(m << lz, false, e - lz, a < 0);
+}
+// ldexp(hi 2^32 + lo, e) with one rounding
+__device__ __forceinline__ double i96_ldexp(long long hi, long long lo, int e) {
+  hi += lo >> 32;
+  unsigned long long h = (unsigned long long)hi;
+  unsigned long long l = (unsigned long long)lo << 32;  // its low half, left aligned
+  const bool neg = hi < 0;
+  if (neg) {  // -(h 2^64 + l)
+    l = 0ull - l;
+    h = ~h + (l == 0ull ? 1ull : 0ull);
   }
-  return i64_ldexp(neg ? -(long long)w : (long long)w, e + sh);
+  if (h == 0ull) {
+    if (l == 0ull) return 0.0;
+    const int lz = __clzll((long long)l);
+    return round_ldexp(l << lz, false, e - 32 - lz, neg);
+  }
+  const int lz = __clzll((long long)h);
+  const unsigned long long n = (h << lz) | (lz ? l >> (64 - lz) : 0ull);
+  return round_ldexp(n, (l << lz) != 0ull, e + 32 - lz, neg);
 }
 
 template <int S, int BN>
@@ -434,8 +430,8 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
           const int shift = 8 * (LV - 1 - g % LV);
           uint32_t r[CW];
           tmem_ld<CW>(tmem_base + ((uint32_t)(quarter * 32) << 16) +
-                          (uint32_t)((buf * S + g) * BN + colg * CW),
-                      r);
+                        (uint32_t)((buf * S + g) * BN + colg * CW),
+                    r);
 #pragma unroll
           for (int i = 0; i < CW; ++i) {
             long long qv = (long long)__float2int_rn(__uint_as_float(r[i]));
@@ -461,26 +457,41 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
         const int ea = rowok ? a.expA[q.prob * a.Mp + row] : 0;
         const int bias = -2 * head(S) - 8 * (S - 1);
         const int64_t ro = rowok ? a.vc.roff(row) : 0;
+        const bool pair = a.cplx && !a.atomic && (reinterpret_cast<uintptr_t>(a.C) & 15) == 0;
+        auto value = [&](int i, int e) {
+          if constexpr (NACC == 2)
+            return i96_ldexp(acc[0][i], acc[1][i], e);
+          else
+            return i64_ldexp(acc[0][i], e);
+        };
+        auto put = [&](double* dst, double v) {
+          if (a.atomic)
+            atomicAdd(dst, v);
+          else
+            *dst = v;
+        };
 #pragma unroll
-        for (int i = 0; i < CW; ++i) {
+        for (int i = 0; i < CW; i += 2) {
+          // a complex element, in one store where C is 16-byte aligned, or two real ones
           const long long co = __shfl_sync(0xffffffffu, mycoff, i);
-          const int eb = __shfl_sync(0xffffffffu, myexp, i);
+          const long long co1 = __shfl_sync(0xffffffffu, mycoff, i + 1);
+          const int e0 = ea + bias + __shfl_sync(0xffffffffu, myexp, i);
+          const int e1 = ea + bias + __shfl_sync(0xffffffffu, myexp, i + 1);
           const int col = q.n0 + colg * CW + i;
           if (rowok && col < a.N2) {
-            double v;
-            if constexpr (NACC == 2)
-              v = i96_ldexp(acc[0][i], acc[1][i], ea + eb + bias);
-            else
-              v = i64_ldexp(acc[0][i], ea + eb + bias);
-            double* dst;
-            if (a.cplx)
-              dst = reinterpret_cast<double*>(Cp + 16 * (ro + co)) + (col & 1);
-            else
-              dst = reinterpret_cast<double*>(Cp + 8 * (ro + co));
-            if (a.atomic)
-              atomicAdd(dst, v);
-            else
-              *dst = v;
+            const double v0 = value(i, e0), v1 = value(i + 1, e1);
+            if (a.cplx) {
+              double* dst = reinterpret_cast<double*>(Cp + 16 * (ro + co));
+              if (pair) {
+                *reinterpret_cast<double2*>(dst) = make_double2(v0, v1);
+              } else {
+                put(dst, v0);
+                put(dst + 1, v1);
+              }
+            } else {
+              put(reinterpret_cast<double*>(Cp + 8 * (ro + co)), v0);
+              if (col + 1 < a.N2) put(reinterpret_cast<double*>(Cp + 8 * (ro + co1)), v1);
+            }
           }
         }
       }
@@ -498,10 +509,10 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
 // ---------------- operand slicing ----------------
 // Logical rows are the rows of A, or the columns of B for the B^T side.  One launch cuts
 // both operands: a CTA takes 32 logical rows and a share of K, the CTAs of a cluster share
-// those rows' K range.  The elements are read once, along whichever index is contiguous in
-// memory, into shared memory (up to PACK_KEEP tiles; a longer share is read a second time,
-// from L2), the rows' exponents are combined through the cluster's shared memory, and the
-// slices leave coalesced along K to the [S][rows][K2_pad] planes.  Bound by HBM: 16 B read
+// those rows' K range.  The elements are copied to shared memory once, along whichever index
+// is contiguous in memory and all at once (up to `keep` tiles; a longer share is copied a
+// second time, from L2), the rows' exponents are combined through the cluster's shared
+// memory, and the slices leave coalesced along K to the [S][rows][K2_pad] planes.  Bound by HBM: 16 B read
 // and 4 S (A) or 8 S (B) B written per complex element.  Rows of padding are not written:
 // they reach only rows and columns of the accumulators that the epilogue skips.
 constexpr int PACK_ROWS = 32;
@@ -509,7 +520,10 @@ constexpr int PACK_ROWS = 32;
 // powers of two, or that holds Inf or NaN, is left to the SIMT kernel.  Within it every entry
 // keeps at least 62 - 36 bits and the largest ones all 53; Gaussian rows span about 2^25.
 constexpr int SPLIT_RANGE = 36;
-constexpr int PACK_KEEP = 4;     // tiles held in shared memory
+// tiles held in shared memory: more cover a longer share in one copy, fewer leave room for
+// other CTAs on the SM
+constexpr int PACK_KEEP = 4, PACK_KEEP_FEW = 8;
+constexpr int PACK_FEW_CTAS = 304;
 constexpr int PACK_CLUSTER = 8;  // most CTAs that share the K range of one row block
 
 // exponent of |x| (biased-exponent field) without FP64 arithmetic: max|x| < 2^e with
@@ -523,12 +537,12 @@ __device__ __forceinline__ int expo_bits(double x) {
   return f - 1022;
 }
 
-// Balanced base-256 digits of t = x 2^(head-e) (|t| < 2^head): N = rint(t 256^(S-1)) (round to
-// nearest, ties to even), then t = sum_s q_s 256^-s up to 0.5 256^-(S-1) with q_1 .. q_{S-1}
+// Balanced base-256 digits of t = x 2^(head-e) (|t| < 2^head): N = t 256^(S-1) rounded to the
+// nearest integer, then t = sum_s q_s 256^-s up to 0.5 256^-(S-1) with q_1 .. q_{S-1}
 // the balanced remainders of N by 256 (in [-128, 127]) and q_0 the remaining quotient
-// (|q_0| <= 128).  N is taken straight from the bit pattern of x (mantissa shifted with the
-// rounding done on the bits that fall off): integer operations only, since a scaling and an
-// FP64-to-integer conversion per value would run on the narrow FP64 pipe of this part.
+// (|q_0| <= 128).  N is taken straight from the bit pattern of x (the mantissa plus half a
+// unit, shifted): integer operations only, since a scaling and an FP64-to-integer conversion
+// per value would run on the narrow FP64 pipe of this part.
 // Returned is N + sum_{i<S-1} 128 256^i: its byte i is q_{S-1-i} + 128 for i < S-1, and its
 // bits from 8 (S-1) up are q_0.
 template <int S>
@@ -536,20 +550,15 @@ __device__ __forceinline__ long long digit_word(double x, int e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7ffu);
   const unsigned long long mant = (b & 0xfffffffffffffull) | (ex ? (1ull << 52) : 0ull);
-  const int k = (ex ? ex : 1) - 1075 + head(S) + 8 * (S - 1) - e;  // N = rint(mant 2^k)
-  long long N;
-  if (k >= 0) {
-    N = (long long)(mant << min(k, 63));
-  } else if (k <= -64) {
-    N = 0;
-  } else {
-    const int sh = -k;
-    unsigned long long qq = mant >> sh;
-    const unsigned long long rem = mant & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
-    if (rem > half || (rem == half && (qq & 1ull))) ++qq;
-    N = (long long)qq;
-  }
-  if (b >> 63) N = -N;
+  // N = mant 2^-sh; the largest exponent of a row, ex = e + 1022, has the smallest sh
+  constexpr int MIN_SH = 53 - head(S) - 8 * (S - 1);
+  const int sh = MIN_SH + e + 1022 - (ex ? ex : 1);
+  unsigned long long n;
+  if (MIN_SH < 1 && sh <= 0)
+    n = mant << -sh;
+  else
+    n = sh < 64 ? (mant + (1ull << (sh - 1))) >> sh : 0ull;
+  const long long N = (b >> 63) ? -(long long)n : (long long)n;
   constexpr long long bias = (long long)(0x8080808080808080ull & ((1ull << (8 * (S - 1))) - 1ull));
   return N + bias;
 }
@@ -558,9 +567,14 @@ __device__ __forceinline__ long long digit_word(double x, int e) {
 // formed by placing the byte in the mantissa of 2^23
 template <int S>
 __device__ __forceinline__ uint32_t digit_f32(long long w, int s) {
-  const uint32_t u = (s == 0) ? (uint32_t)((int)(w >> (8 * (S - 1))) + 128)
-                              : (uint32_t)(w >> (8 * (S - 1 - s))) & 0xffu;
-  return __float_as_uint(__uint_as_float(0x4b000000u | u) - 8388736.0f);
+  uint32_t u;
+  if (s == 0) {
+    u = 0x4b000000u + (uint32_t)((int)(w >> (8 * (S - 1))) + 128);
+  } else {
+    const int byte = S - 1 - s;
+    u = __byte_perm(byte < 4 ? (uint32_t)w : (uint32_t)(w >> 32), 0x4b000000u, 0x7540 + (byte & 3));
+  }
+  return __float_as_uint(__uint_as_float(u) - 8388736.0f);
 }
 __device__ __forceinline__ uint32_t bf16_pair(uint32_t flo, uint32_t fhi) {
   return __byte_perm(flo, fhi, 0x7632);
@@ -579,13 +593,31 @@ template <typename T>
 struct PackArgs {
   PackSide<T> a, b;
   int blocks_a;        // row blocks of A (then those of B)
-  int K, K2p, tiles_per_cta;
+  int K, K2p, tiles_per_cta, keep;
   size_t plane_a, plane_b;
   int* status;
   int* wide;           // not NULL: set when an operand does not suit the split (split_f64)
 };
 
-template <typename T, bool SIDE_B, int S>
+// one element to shared memory, zero if !in; complex ones in one copy where the operand is
+// 16-byte aligned (a caller's need not be), else in two
+__device__ __forceinline__ void copy_async(double* dst, const double* src, bool in, bool) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src),
+               "r"(in ? 8 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async(zdbl* dst, const zdbl* src, bool in, bool al16) {
+  if (al16) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src),
+                 "r"(in ? 16 : 0)
+                 : "memory");
+  } else {
+    copy_async(&dst->re, &src->re, in, false);
+    copy_async(&dst->im, &src->im, in, false);
+  }
+}
+
+template <typename T, bool SIDE_B, int S, int ROWS>
 __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T>& o, size_t plane,
                                           int block, T* tiles, int* s_max, int* s_min,
                                           int* s_exp) {
@@ -593,74 +625,85 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
   constexpr bool CPLX = O::cplx;
   constexpr int KT = CPLX ? 32 : 64;  // logical K of a tile: one 64-wide packed atom
   constexpr int LD = KT + 1;
-  constexpr int NQ = PACK_ROWS * KT / 256;
+  constexpr int NQ = ROWS * KT / 256, RQ = ROWS / 8;
   cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
   const int nranks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int r0 = block * PACK_ROWS;
+  const int r0 = block * ROWS;
   const T* src = o.src + (int64_t)blockIdx.z * o.v.bs;
   const int ntiles = g.K2p / KA;
   const int t_begin = rank * g.tiles_per_cta;
   const int t_end = min(ntiles, t_begin + g.tiles_per_cta);
-  const bool keep = g.tiles_per_cta <= PACK_KEEP;
   auto off_r = [&](int r) -> int64_t { return SIDE_B ? o.v.coff(r) : o.v.roff(r); };
-  auto off_k = [&](int k) -> int64_t { return SIDE_B ? o.v.roff(k) : o.v.coff(k); };
-  // element q of this thread in a tile.  Rows on the lanes: row = lane, k = warp + 8 q; K on
-  // the lanes: k = lane (+ 32), row = warp + 8 (q mod 4)
-  const bool rl = o.rowlanes != 0;
-  int64_t ro[4];
+  // (the two divisions of a two-level index only where it has two levels)
+  const bool flat = (SIDE_B ? o.v.r_in : o.v.c_in) == 0x7fffffff;
+  const int64_t ks = SIDE_B ? o.v.rs_in : o.v.cs_in;
+  auto off_k = [&](int k) -> int64_t {
+    return flat ? k * ks : (SIDE_B ? o.v.roff(k) : o.v.coff(k));
+  };
+  // element q of this thread in a tile.  Rows on the lanes: row = lane mod ROWS, the lanes
+  // beyond on the next k; K on the lanes: k = lane + 32 (q / RQ), row = warp + 8 (q mod RQ)
+  const bool rl = o.rowlanes != 0, al16 = (reinterpret_cast<uintptr_t>(o.src) & 15) == 0;
+  int64_t ro[RQ];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int r = r0 + (rl ? lane : warp + 8 * q);
+  for (int q = 0; q < RQ; ++q) {
+    const int r = r0 + (rl ? lane % ROWS : warp + 8 * q);
     ro[q] = r < o.rows ? off_r(r) : -1;
   }
-  int best[4] = {-2000, -2000, -2000, -2000};
-  int low[4] = {2000, 2000, 2000, 2000};
-  auto load_tile = [&](int t, T* dst) {
-    T x[NQ];
+  // tiles [t, min(t + keep, t_end)) into shared memory
+  auto load_tiles = [&](int t) {
+    const int te = min(t + g.keep, t_end);
+    for (int i = t; i < te; ++i) {
+      T* dst = tiles + (i - t) * ROWS * LD;
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      const int k = t * KT + (rl ? warp + 8 * q : lane + 32 * (q >> 2));
-      const int64_t rr = ro[q & 3];
-      x[q] = (rr >= 0 && k < g.K) ? src[rr + off_k(k)] : O::zero();
-    }
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      if (rl)
-        dst[lane * LD + warp + 8 * q] = x[q];
-      else
-        dst[(warp + 8 * (q & 3)) * LD + lane + 32 * (q >> 2)] = x[q];
-      const int br = expo_bits(O::real(x[q])), bi = expo_bits(O::imag(x[q]));
-      best[q & 3] = max(best[q & 3], max(br, bi));
-      if constexpr (S > 5) {  // the smallest nonzero entry
-        if (br > -2000) low[q & 3] = min(low[q & 3], br);
-        if (bi > -2000) low[q & 3] = min(low[q & 3], bi);
+      for (int q = 0; q < NQ; ++q) {
+        const int kk = rl ? lane / ROWS + (32 / ROWS) * (warp + 8 * q) : lane + 32 * (q / RQ);
+        const int k = i * KT + kk;
+        const int64_t rr = ro[q % RQ];
+        const bool in = rr >= 0 && k < g.K;
+        copy_async(dst + (rl ? lane % ROWS : warp + 8 * (q % RQ)) * LD + kk, in ? src + rr + off_k(k) : src,
+                   in, al16);
       }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
   };
-  if (tid < PACK_ROWS) {
-    s_max[tid] = -2000;
-    s_min[tid] = 2000;
+  // largest (and smallest nonzero) exponents of rows warp + 8 q
+  int best[RQ], low[RQ];
+#pragma unroll
+  for (int q = 0; q < RQ; ++q) {
+    best[q] = -2000;
+    low[q] = 2000;
   }
-  __syncthreads();
-  for (int t = t_begin; t < t_end; ++t) load_tile(t, tiles + (keep ? (t - t_begin) * PACK_ROWS * LD : 0));
-  if (rl) {
-    atomicMax(s_max + lane, max(max(best[0], best[1]), max(best[2], best[3])));
-    if constexpr (S > 5) atomicMin(s_min + lane, min(min(low[0], low[1]), min(low[2], low[3])));
-  } else {
+  for (int t = t_begin; t < t_end; t += g.keep) {
+    if (t > t_begin) __syncthreads();
+    load_tiles(t);
+    __syncthreads();
+    const int n = min(g.keep, t_end - t);
+    for (int i = 0; i < n; ++i)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      int b = best[q];
+      for (int q = 0; q < NQ; ++q) {
+        const T x = tiles[(i * ROWS + warp + 8 * (q % RQ)) * LD + lane + 32 * (q / RQ)];
+        const int br = expo_bits(O::real(x)), bi = expo_bits(O::imag(x));
+        best[q % RQ] = max(best[q % RQ], max(br, bi));
+        if constexpr (S > 5) {
+          if (br > -2000) low[q % RQ] = min(low[q % RQ], br);
+          if (bi > -2000) low[q % RQ] = min(low[q % RQ], bi);
+        }
+      }
+  }
 #pragma unroll
-      for (int w = 16; w > 0; w >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, w));
-      if (lane == 0) s_max[warp + 8 * q] = b;
-      if constexpr (S > 5) atomicMin(s_min + warp + 8 * q, low[q]);
+  for (int q = 0; q < RQ; ++q) {
+    const int b = __reduce_max_sync(0xffffffffu, best[q]);
+    if (lane == 0) s_max[warp + 8 * q] = b;
+    if constexpr (S > 5) {
+      const int l = __reduce_min_sync(0xffffffffu, low[q]);
+      if (lane == 0) s_min[warp + 8 * q] = l;
     }
   }
   __syncthreads();
   if (nranks > 1) cluster.sync();
-  if (tid < PACK_ROWS) {
-    int b = s_max[tid], lo = s_min[tid];
+  if (tid < ROWS) {
+    int b = s_max[tid], lo = S > 5 ? s_min[tid] : 2000;
     for (int q = 0; q < nranks; ++q)
       if (q != rank) {
         b = max(b, cluster.map_shared_rank(s_max, q)[tid]);
@@ -678,17 +721,17 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
   __syncthreads();
   uint32_t* out = reinterpret_cast<uint32_t*>(o.out + (size_t)blockIdx.z * o.rows_pad * g.K2p);
   const size_t pl = plane / 2, ld = (size_t)g.K2p / 2;  // in words of two bf16
+  const bool held = t_end - t_begin <= g.keep;  // the whole share is still there
   for (int t = t_begin; t < t_end; ++t) {
-    const T* tile = tiles;
-    if (keep) {
-      tile += (t - t_begin) * PACK_ROWS * LD;
-    } else {
+    const int i = (t - t_begin) % g.keep;
+    const T* tile = tiles + i * ROWS * LD;
+    if (!held && i == 0) {
       __syncthreads();
-      load_tile(t, tiles);
+      load_tiles(t);
       __syncthreads();
     }
 #pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < RQ; ++q) {
       const int lr = warp + 8 * q;
       if (r0 + lr >= o.rows) continue;
       const int e = s_exp[lr];
@@ -720,16 +763,16 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
   if (nranks > 1) cluster.sync();  // no CTA leaves while another still reads its row maxima
 }
 
-template <typename T, int S>
+template <typename T, int S, int ROWS>
 __global__ void __launch_bounds__(256) pack_kernel(PackArgs<T> g) {
   extern __shared__ __align__(16) unsigned char pack_smem[];
-  __shared__ int s_max[PACK_ROWS], s_min[PACK_ROWS], s_exp[PACK_ROWS];
+  __shared__ int s_max[ROWS], s_min[ROWS], s_exp[ROWS];
   T* tiles = reinterpret_cast<T*>(pack_smem);
   const int block = blockIdx.x / (int)cooperative_groups::this_cluster().num_blocks();
   if (block < g.blocks_a)
-    pack_rows<T, false, S>(g, g.a, g.plane_a, block, tiles, s_max, s_min, s_exp);
+    pack_rows<T, false, S, ROWS>(g, g.a, g.plane_a, block, tiles, s_max, s_min, s_exp);
   else
-    pack_rows<T, true, S>(g, g.b, g.plane_b, block - g.blocks_a, tiles, s_max, s_min, s_exp);
+    pack_rows<T, true, S, ROWS>(g, g.b, g.plane_b, block - g.blocks_a, tiles, s_max, s_min, s_exp);
 }
 
 // strides of the logical (row, k) indices at the origin, to pick the read pattern
@@ -740,24 +783,18 @@ bool rows_contiguous(const View& v) {
   return sr == 1 && sk != 1;
 }
 
-template <typename T, int S>
-cudaError_t launch_pack(PackArgs<T> g, int nb, cudaStream_t s) {
+template <typename T, int S, int ROWS>
+cudaError_t launch_pack(PackArgs<T> g, int cs, int nb, cudaStream_t s) {
   constexpr int KT = ops<T>::cplx ? 32 : 64;
-  const void* k = (const void*)pack_kernel<T, S>;
-  cudaError_t e = allow_max_smem(k);
+  cudaError_t e = allow_max_smem((const void*)pack_kernel<T, S, ROWS>);
   if (e != cudaSuccess) return e;
-  const int tiles = g.K2p / KA;
-  // as many CTAs along K as keep their share in shared memory, up to PACK_CLUSTER
-  int cs = 1;
-  while (cs < PACK_CLUSTER && cs * PACK_KEEP < tiles) cs *= 2;
-  g.tiles_per_cta = (tiles + cs - 1) / cs;
-  const int held = g.tiles_per_cta <= PACK_KEEP ? g.tiles_per_cta : 1;
-  const size_t smem = (size_t)held * PACK_ROWS * (KT + 1) * sizeof(T);
-  const int blocks = g.blocks_a + (g.b.rows + PACK_ROWS - 1) / PACK_ROWS;
+  g.blocks_a = (g.a.rows + ROWS - 1) / ROWS;
+  const int blocks = g.blocks_a + (g.b.rows + ROWS - 1) / ROWS;
+  g.keep = std::min(PACK_KEEP * PACK_ROWS / ROWS, g.tiles_per_cta);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)cs * blocks, 1, nb);
   cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = (size_t)g.keep * ROWS * (KT + 1) * sizeof(T);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -767,18 +804,32 @@ cudaError_t launch_pack(PackArgs<T> g, int nb, cudaStream_t s) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   note_launches(CBC_K_AUX, 1);
-  return cudaLaunchKernelEx(&cfg, pack_kernel<T, S>, g);
+  return cudaLaunchKernelEx(&cfg, pack_kernel<T, S, ROWS>, g);
+}
+
+template <typename T, int S>
+cudaError_t pack_slices(PackArgs<T> g, int nb, cudaStream_t s) {
+  const int tiles = g.K2p / KA;
+  // as many CTAs along K as keep their share in shared memory, up to PACK_CLUSTER
+  int cs = 1;
+  while (cs < PACK_CLUSTER && cs * PACK_KEEP < tiles) cs *= 2;
+  g.tiles_per_cta = (tiles + cs - 1) / cs;
+  const int64_t ctas =
+      (int64_t)cs * nb *
+      ((g.a.rows + PACK_ROWS - 1) / PACK_ROWS + (g.b.rows + PACK_ROWS - 1) / PACK_ROWS);
+  if (ctas < 2 * g_sms) return launch_pack<T, S, PACK_ROWS / 2>(g, cs, nb, s);
+  return launch_pack<T, S, PACK_ROWS>(g, cs, nb, s);
 }
 
 // both operands of nb problems (sources v.bs elements apart) into their planes
 template <typename T>
 cudaError_t pack_operands(const PackArgs<T>& g, int S, int nb, cudaStream_t s) {
   switch (S) {
-    case 2: return launch_pack<T, 2>(g, nb, s);
-    case 3: return launch_pack<T, 3>(g, nb, s);
-    case 4: return launch_pack<T, 4>(g, nb, s);
-    case 8: return launch_pack<T, 8>(g, nb, s);
-    default: return launch_pack<T, 5>(g, nb, s);
+    case 2: return pack_slices<T, 2>(g, nb, s);
+    case 3: return pack_slices<T, 3>(g, nb, s);
+    case 4: return pack_slices<T, 4>(g, nb, s);
+    case 8: return pack_slices<T, 8>(g, nb, s);
+    default: return pack_slices<T, 5>(g, nb, s);
   }
 }
 
@@ -896,8 +947,6 @@ struct TuneKey {
 std::mutex g_tune_mu;
 std::map<TuneKey, int> g_tuned;
 
-int g_sms = 0;
-
 }  // namespace tc
 
 namespace {
@@ -967,7 +1016,6 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
   pk.a = {A, va, conjA ? 1 : 0, M, rows_contiguous<false>(va) ? 1 : 0, sa, ea, g.Mp, g.Mp};
   pk.b = {B, vb, conjB ? 1 : 0, N, rows_contiguous<true>(vb) ? 1 : 0, sb, eb,
           CPLX ? g.N2p / 2 : g.N2p, g.N2p};
-  pk.blocks_a = (M + PACK_ROWS - 1) / PACK_ROWS;
   pk.K = K;
   pk.K2p = g.K2p;
   pk.plane_a = b * g.Mp * g.K2p;

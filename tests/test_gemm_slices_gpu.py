@@ -63,3 +63,26 @@ def test_fp64_nonfinite_passes_through(bad):
     C, ref = _run(0, 0, A, B)
     assert np.array_equal(np.isnan(C), np.isnan(ref)) and np.array_equal(np.isinf(C), np.isinf(ref))
     assert np.abs(np.delete(C, 3, 0) - np.delete(ref, 3, 0)).max() <= 1e-12
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_operands_on_odd_doubles(prec):
+    """Complex operands whose storage starts on an odd double (8-byte aligned only)."""
+    import torch
+
+    from paper_2601_19650_gb300 import _cbc
+    rng = np.random.default_rng(4)
+    M, N, K = 70, 45, 130
+    A, B = _rand(rng, (M, K), True), _rand(rng, (K, N), True)
+
+    def shifted(x):
+        buf = torch.zeros(2 * x.size + 1, dtype=torch.float64, device="cuda")
+        buf[1:] = torch.from_numpy(np.ascontiguousarray(x).view(np.float64).reshape(-1)).to("cuda")
+        return buf, buf.data_ptr() + 8
+
+    (ka, pa), (kb, pb) = shifted(A), shifted(B)
+    kc, pc = shifted(np.zeros((M, N), dtype=np.complex128))
+    _cbc.cbc_gemm(prec, 5, _cbc.CBC_C128, M, N, K, pa, K, False, False, pb, N, False, False, pc, N)
+    C = kc[1:].cpu().numpy().view(np.complex128).reshape(M, N)
+    # 5 slices: K terms, each off by at most 16 2^(e_a+e_b-40) with entries below 2^3
+    assert np.abs(C - A @ B).max() <= (1e-12 if prec == 0 else 2 * K * 16 * 2.0 ** (6 - 40))
