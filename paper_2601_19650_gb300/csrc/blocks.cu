@@ -48,11 +48,19 @@ int heev_t(int m, int kmax, int nb, T* A, double* lam, T* U, bool mixed, cudaStr
     cudaFreeAsync(status, s);
     return cuda_fail(e, "cbc_heev: alloc");
   }
+  // without room for the back transformation by products the call takes the other way
+  void* bt = nullptr;
+  const size_t btb = eig_bt_bytes(m, kmax, ops<T>::cplx, nb);
+  if (btb > 0 && pool_malloc(&bt, btb, s) != cudaSuccess) {
+    cudaGetLastError();
+    bt = nullptr;
+  }
   e = cudaMemsetAsync(status, 0, sizeof(int), s);
   if (e == cudaSuccess)
-    e = heev_top<T>(A, m, kmax, lam, U, work, status, num_sms(), s, nb, false, mixed);
+    e = heev_top<T>(A, m, kmax, lam, U, work, status, num_sms(), s, nb, false, mixed, bt);
   int hs = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (bt) cudaFreeAsync(bt, s);
   cudaFreeAsync(work, s);
   cudaFreeAsync(status, s);
   cudaError_t e2 = cudaStreamSynchronize(s);

@@ -1153,6 +1153,80 @@ __global__ void __launch_bounds__(32 * BT_WARPS) backtransform32_kernel(
     }
 }
 
+// ---- back transformation by matrix products -----------------------------------------
+// Blocks of BT_NB reflectors in the compact WY form H_j0 .. H_{j0+b-1} = I - V T V^H (V: one
+// column per reflector, T upper triangular), applied from the last block to the first,
+// U <- U - (V T)(V^H U), with the products on the tensor cores (8 slices: an error below that
+// of FP64 sums; U's columns may span any range here, since what counts is their norm).  One
+// reflector at a time the transformation is a chain of m dot products, each ~3000 clocks of
+// FP64 reductions, and FP64 work of 8 m^2 kmax flops on its pipes.
+// One at a time / products, with the rest of the eigensolver behind the reduction: m = 2048
+// complex, 1024 vectors 73.9 / 10.6 ms; 64 matrices of m = 256, 128 vectors 4.0 / 2.6 ms.
+constexpr int BT_NB = 64, BT_HALF = 32;
+
+// U = X (real) as nb matrices of n elements, X wb bytes apart
+template <typename T>
+__global__ void widen_x_kernel(const double* X, int64_t n, T* U, size_t wb) {
+  X = byte_shift(X, blockIdx.y * wb);
+  U += (int64_t)blockIdx.y * n;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    U[i] = ops<T>::make(X[i], 0.0);
+}
+
+// NaN into U when *flag is set (an Inf or NaN among V, T or X, which the slices don't carry)
+template <typename T>
+__global__ void poison_kernel(const int* flag, T* U, int64_t n) {
+  if (!*flag) return;
+  const double nan = __longlong_as_double(0x7ff8000000000000LL);
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    U[i] = ops<T>::make(nan, ops<T>::cplx ? nan : 0.0);
+}
+
+// T of BT_HALF reflectors from G = V^H V (BT_HALF x BT_HALF, leading dimension BT_NB):
+// T^-1 = diag(1 / tau) + the strict upper triangle of G, so column i of T is x_i = tau_i,
+// x_r = -tau_r sum_{r < l <= i} G[r][l] x_l.  One CTA per half block (blockIdx.x: block and
+// half, blockIdx.y: matrix), four lanes per column that share each sum.
+template <typename T>
+__global__ void __launch_bounds__(128) wy_t_kernel(const T* G, const T* tau, int m, T* Tm,
+                                                   size_t wb, int64_t bs) {
+  using O = ops<T>;
+  __shared__ T g[BT_HALF][BT_HALF + 1];
+  __shared__ T tt[BT_HALF];
+  const int blk = blockIdx.x >> 1, half = blockIdx.x & 1;
+  const int64_t at = blockIdx.y * bs + (int64_t)blk * BT_NB * BT_NB + half * BT_HALF * (BT_NB + 1);
+  tau = byte_shift(tau, blockIdx.y * wb);
+  G += at;
+  Tm += at;
+  for (int i = threadIdx.x; i < BT_HALF * BT_HALF; i += blockDim.x)
+    g[i / BT_HALF][i % BT_HALF] = G[(int64_t)(i / BT_HALF) * BT_NB + i % BT_HALF];
+  if (threadIdx.x < BT_HALF) {
+    const int j = blk * BT_NB + half * BT_HALF + threadIdx.x;
+    tt[threadIdx.x] = j < m - 1 ? tau[j] : O::zero();
+  }
+  __syncthreads();
+  const int i = threadIdx.x >> 2, sub = threadIdx.x & 3;  // column i, terms l = sub (mod 4)
+  T x[BT_HALF / 4];                                       // x_l, l = sub + 4 q
+#pragma unroll
+  for (int q = 0; q < BT_HALF / 4; ++q) x[q] = (sub + 4 * q == i) ? tt[i] : O::zero();
+#pragma unroll
+  for (int r = BT_HALF - 1; r >= 0; --r) {
+    T acc = O::zero();
+#pragma unroll
+    for (int q = 0; q < BT_HALF / 4; ++q)
+      if (4 * q + 3 > r) {
+        const int l = sub + 4 * q;
+        if (l > r) acc = O::fma(g[r][l], x[q], acc);
+      }
+    acc = acc + shfl_xor(acc, 1);
+    acc = acc + shfl_xor(acc, 2);
+    if (r < i && (r & 3) == sub) x[r >> 2] = O::scale(-1.0, tt[r] * acc);
+  }
+#pragma unroll
+  for (int q = 0; q < BT_HALF / 4; ++q) Tm[(int64_t)(sub + 4 * q) * BT_NB + i] = x[q];
+}
+
 // Initial contents of a batch of eigensolver workspaces in one launch: up to 6 segments
 // of 64-bit words per instance (instance blockIdx.y, workspaces wb bytes apart).
 struct WsInit {
@@ -1196,9 +1270,126 @@ size_t eig_workspace_bytes(int m, int kmax, bool cplx) {
   return b;
 }
 
+// Where the products pay: they cost ~12 launches and ~70 us per block of 64 reflectors before
+// the work counts, one reflector at a time costs ~1.9 us each.  One at a time / products, the
+// eigensolver behind the reduction in us: lone m = 128 complex, 64 vectors 340 / 362; 256, 128
+// vectors 722 / 588; 512 real, 256 vectors 1250 / 997; 64 matrices of m = 32 195 / 238, of 64
+// 769 / 334; 5 of m = 97 real 214 / 344.
+static bool bt_products(int m, int kmax, int nb) {
+  return m >= 48 && (double)m * m * kmax * nb >= 4e6;
+}
+
+static size_t bt_gemm_bytes(int m, int kmax, bool cplx, int nb) {
+  const int nblk = (m + BT_NB - 1) / BT_NB;
+  const int rep = nb > 1 ? nb : nblk;  // the products on V alone: a block of all matrices, or
+                                       // all blocks of a lone one
+  size_t b = 0;
+  auto need = [&](int M, int N, int K, int n) {
+    b = std::max(b, gemm_tc_workspace_bytes(M, N, K, cplx, 8, n));
+  };
+  need(BT_NB, BT_NB, m, rep);                      // V^H V
+  need(BT_HALF, BT_HALF, BT_HALF, nb * nblk);      // T
+  need(m, BT_NB, BT_NB, rep);                      // V T
+  need(BT_NB, kmax, m, nb);                        // V^H U
+  need(m, kmax, BT_NB, nb);                        // (V T)(V^H U)
+  return b;
+}
+
+size_t eig_bt_bytes(int m, int kmax, bool cplx, int nb) {
+  if (!bt_products(m, kmax, nb)) return 0;
+  const size_t ts = cplx ? sizeof(zdbl) : sizeof(double);
+  const size_t nblk = (m + BT_NB - 1) / BT_NB;
+  return 256 + align256(2 * nb * nblk * BT_NB * BT_NB * ts) +
+         align256(nb * nblk * BT_HALF * BT_HALF * ts) + align256((size_t)nb * BT_NB * kmax * ts) +
+         bt_gemm_bytes(m, kmax, cplx, nb);
+}
+
+// U = H_0 .. H_{m-2} X.  V (rows v_j, zero up to the diagonal), tau, X and Y (room for m rows
+// more than m columns each) lie in the matrices' workspaces, wb bytes apart.
+template <typename T>
+static cudaError_t backtransform_products(const T* V, const T* tau, const double* X, T* Y, int m,
+                                          int kmax, T* U, size_t wb, void* bt, int* status,
+                                          cudaStream_t s, int nb) {
+  const int nblk = (m + BT_NB - 1) / BT_NB;
+  const int64_t we = (int64_t)(wb / sizeof(T)), sq = BT_NB * BT_NB, tbs = nblk * sq;
+  char* w = static_cast<char*>(bt);
+  auto take = [&](size_t bytes) {
+    char* p = w;
+    w += align256(bytes);
+    return p;
+  };
+  int* flag = reinterpret_cast<int*>(take(4));
+  T* G = reinterpret_cast<T*>(take(2 * nb * tbs * sizeof(T)));
+  T* Tm = G + nb * tbs;
+  T* tmp = reinterpret_cast<T*>(take(sizeof(T) * nb * nblk * BT_HALF * BT_HALF));
+  T* W = reinterpret_cast<T*>(take(sizeof(T) * (size_t)nb * BT_NB * kmax));
+  void* ws = w;
+  TcWide opt;
+  opt.wide = flag;
+  TcWide sub = opt;
+  sub.subtract = true;
+  cudaError_t e = cudaMemsetAsync(bt, 0, (char*)(G + 2 * nb * tbs) - (char*)bt, s);  // flag, G, T
+  auto mul = [&](int M, int N, int K, const T* A, View va, int64_t abs, bool ca, const T* B,
+                 View vb, int64_t bbs, T* C, int64_t ldc, int64_t cbs, int n, const TcWide& o) {
+    if (e != cudaSuccess) return;
+    va.bs = abs;
+    vb.bs = bbs;
+    e = gemm_tc<T>(M, N, K, A, va, ca, B, vb, false, C, View::rowmajor(ldc, cbs), 8, ws, status, s,
+                   n, o);
+  };
+  const int64_t n = (int64_t)m * kmax;
+  note_launches(CBC_K_EIG, 3);
+  widen_x_kernel<T><<<dim3((unsigned)std::min<int64_t>(256, (n + 255) / 256), nb), 256, 0, s>>>(
+      X, n, U, wb);
+  // G = V^H V per block.  V's rows beyond m are not there: the last block has m - j0 of them
+  const int full = m / BT_NB;  // blocks of BT_NB rows
+  for (int q = 0; q < nblk; ++q) {
+    const int j0 = q * BT_NB, b = std::min(BT_NB, m - j0);
+    const bool all = nb == 1 && q == 0 && full > 1;  // a lone matrix: every full block at once
+    const int64_t vbs = nb > 1 ? we : (int64_t)BT_NB * m, gbs = nb > 1 ? tbs : sq;
+    const int c0 = all ? 0 : j0;  // v_j starts at column j + 1
+    const T* Vb = V + (int64_t)j0 * m + c0;
+    mul(b, b, m - c0, Vb, View::rowmajor(m), vbs, true, Vb, View::transposed(m), vbs,
+        G + q * sq, BT_NB, gbs, nb > 1 ? nb : (all ? full : 1), opt);
+    if (all) q = full - 1;
+  }
+  if (e != cudaSuccess) return e;
+  wy_t_kernel<T><<<dim3(2 * nblk, nb), 128, 0, s>>>(G, tau, m, Tm, wb, tbs);
+  // the halves of a block: T12 = -T1 (V1^H V2) T2
+  const int64_t hf = BT_HALF * BT_HALF;
+  mul(BT_HALF, BT_HALF, BT_HALF, G + BT_HALF, View::rowmajor(BT_NB), sq, false,
+      Tm + BT_HALF * (BT_NB + 1), View::rowmajor(BT_NB), sq, tmp, BT_HALF, hf, nb * nblk, opt);
+  mul(BT_HALF, BT_HALF, BT_HALF, Tm, View::rowmajor(BT_NB), sq, false, tmp,
+      View::rowmajor(BT_HALF), hf, Tm + BT_HALF, BT_NB, sq, nb * nblk, sub);
+  // Y = V T per block, m x BT_NB each
+  const int64_t ybs = (int64_t)BT_NB * m;
+  for (int q = 0; q < nblk; ++q) {
+    const int j0 = q * BT_NB, b = std::min(BT_NB, m - j0);
+    const bool all = nb == 1 && q == 0 && full > 1;
+    const int c0 = all ? 0 : j0;
+    mul(m - c0, BT_NB, b, V + (int64_t)j0 * m + c0, View::transposed(m), nb > 1 ? we : ybs, false,
+        Tm + q * sq, View::rowmajor(BT_NB), nb > 1 ? tbs : sq, Y + q * ybs + (int64_t)c0 * BT_NB,
+        BT_NB, nb > 1 ? we : ybs, nb > 1 ? nb : (all ? full : 1), opt);
+    if (all) q = full - 1;
+  }
+  for (int q = nblk - 1; q >= 0; --q) {
+    const int j0 = q * BT_NB, b = std::min(BT_NB, m - j0), r = m - j0;
+    const T* Vb = V + (int64_t)j0 * m + j0;
+    T* Ub = U + (int64_t)j0 * kmax;
+    mul(b, kmax, r, Vb, View::rowmajor(m), we, true, Ub, View::rowmajor(kmax), n, W, kmax,
+        (int64_t)BT_NB * kmax, nb, opt);
+    mul(r, kmax, b, Y + q * ybs + (int64_t)j0 * BT_NB, View::rowmajor(BT_NB), we, false, W,
+        View::rowmajor(kmax), (int64_t)BT_NB * kmax, Ub, kmax, n, nb, sub);
+  }
+  if (e != cudaSuccess) return e;
+  poison_kernel<T><<<(unsigned)std::min<int64_t>(256, (n * nb + 255) / 256), 256, 0, s>>>(
+      flag, U, n * nb);
+  return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t heev_top(T* A, int m, int kmax, double* lam, T* U, void* work, int* status,
-                     int num_sms, cudaStream_t s, int nb, bool prefer_cluster, bool df) {
+                     int num_sms, cudaStream_t s, int nb, bool prefer_cluster, bool df, void* bt) {
   char* w = static_cast<char*>(work);
   auto take = [&](size_t bytes) {
     char* p = w;
@@ -1244,6 +1435,7 @@ cudaError_t heev_top(T* A, int m, int kmax, double* lam, T* U, void* work, int* 
   const void* kl = m <= TPB ? (const void*)tridiag_lone_kernel<T, 1>
                    : m <= 2 * TPB ? (const void*)tridiag_lone_kernel<T, 2>
                                   : (const void*)tridiag_lone_kernel<T, 4>;
+  const bool products = bt && bt_products(m, kmax, nb);
   {
     // barrier, tau and e[0] start at zero; the exchange buffers of the lone reduction as
     // all-ones bit patterns (the "not yet written" mark)
@@ -1257,6 +1449,7 @@ cudaError_t heev_top(T* A, int m, int kmax, double* lam, T* U, void* work, int* 
     add(bar, sizeof(GridBarrier), 0ull);
     add(tau, ts * m, 0ull);
     add(e, sizeof(double), 0ull);
+    if (products) add(V, ts * (size_t)m * m, 0ull);  // v_j is zero up to column j
     if (lone) {
       add(Xg, ts * (size_t)m * m * 2, ~0ull);
     }
@@ -1321,7 +1514,11 @@ cudaError_t heev_top(T* A, int m, int kmax, double* lam, T* U, void* work, int* 
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
   }
-  // 4. back transformation: 32 vectors per CTA (fewer FP64 instructions) when u fits in
+  // 4. back transformation: by matrix products where there is room for them (the exchange
+  // buffer of the reduction holds V T)
+  if (products)
+    return backtransform_products<T>(V, tau, X, Xg, m, kmax, U, wb, bt, status, s, nb);
+  // else 32 vectors per CTA (fewer FP64 instructions) when u fits in
   // shared memory and the batch gives enough CTAs to spread the FP64 work over the SMs;
   // else one vector per CTA
   const size_t shm32 = ((size_t)m * 32 + 3 * (size_t)m) * ts;
@@ -1348,8 +1545,8 @@ cudaError_t heev_top(T* A, int m, int kmax, double* lam, T* U, void* work, int* 
 }
 
 template cudaError_t heev_top<double>(double*, int, int, double*, double*, void*, int*, int,
-                                      cudaStream_t, int, bool, bool);
+                                      cudaStream_t, int, bool, bool, void*);
 template cudaError_t heev_top<zdbl>(zdbl*, int, int, double*, zdbl*, void*, int*, int,
-                                    cudaStream_t, int, bool, bool);
+                                    cudaStream_t, int, bool, bool, void*);
 
 }  // namespace cbc

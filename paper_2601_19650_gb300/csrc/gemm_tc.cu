@@ -204,7 +204,8 @@ struct TcArgs {
   char* C;               // FP64 output (double or zdbl) through the view
   View vc;               // vc.bs: elements between the outputs of consecutive problems
   int* status;
-  const int* skip;       // not NULL: nothing runs when *skip is set (see split_f64)
+  const int* skip;       // not NULL: nothing runs when *skip is set (gemm_f64_split)
+  int subtract;          // C - A B instead of A B
   int splits;            // K splits per problem
   int Mp, N2p;           // packed rows of one problem in the A and B planes
   int ebsB;              // entries of expB per problem
@@ -457,7 +458,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
         const int ea = rowok ? a.expA[q.prob * a.Mp + row] : 0;
         const int bias = -2 * head(S) - 8 * (S - 1);
         const int64_t ro = rowok ? a.vc.roff(row) : 0;
-        const bool pair = a.cplx && !a.atomic && (reinterpret_cast<uintptr_t>(a.C) & 15) == 0;
+        const bool pair = a.cplx && !a.atomic && !a.subtract && (reinterpret_cast<uintptr_t>(a.C) & 15) == 0;
         auto value = [&](int i, int e) {
           if constexpr (NACC == 2)
             return i96_ldexp(acc[0][i], acc[1][i], e);
@@ -466,9 +467,9 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
         };
         auto put = [&](double* dst, double v) {
           if (a.atomic)
-            atomicAdd(dst, v);
+            atomicAdd(dst, a.subtract ? -v : v);
           else
-            *dst = v;
+            *dst = a.subtract ? *dst - v : v;
         };
 #pragma unroll
         for (int i = 0; i < CW; i += 2) {
@@ -516,10 +517,6 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
 // and 4 S (A) or 8 S (B) B written per complex element.  Rows of padding are not written:
 // they reach only rows and columns of the accumulators that the epilogue skips.
 constexpr int PACK_ROWS = 32;
-// FP64 products as 8 slices (gemm_f64_split): an operand whose rows span more than this many
-// powers of two, or that holds Inf or NaN, is left to the SIMT kernel.  Within it every entry
-// keeps at least 62 - 36 bits and the largest ones all 53; Gaussian rows span about 2^25.
-constexpr int SPLIT_RANGE = 36;
 // tiles held in shared memory: more cover a longer share in one copy, fewer leave room for
 // other CTAs on the SM
 constexpr int PACK_KEEP = 4, PACK_KEEP_FEW = 8;
@@ -596,7 +593,8 @@ struct PackArgs {
   int K, K2p, tiles_per_cta, keep;
   size_t plane_a, plane_b;
   int* status;
-  int* wide;           // not NULL: set when an operand does not suit the split (split_f64)
+  int* wide;           // 8 slices: set when an operand holds Inf or NaN or a row spans more
+  int range;           // than 2^range
 };
 
 // one element to shared memory, zero if !in; complex ones in one copy where the operand is
@@ -710,7 +708,7 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
         if constexpr (S > 5) lo = min(lo, cluster.map_shared_rank(s_min, q)[tid]);
       }
     if constexpr (S > 5) {
-      if (b >= 0x40000000 || (lo < 2000 && b - lo > SPLIT_RANGE)) *g.wide = 1;
+      if (b >= 0x40000000 || (lo < 2000 && b - lo > g.range)) *g.wide = 1;
     } else if (b >= 0x40000000) {
       set_status(g.status, CBC_ERR_NUMERICAL);  // Inf or NaN in the row
     }
@@ -956,6 +954,10 @@ namespace {
 //            1000 x 1000 x 16 61 / 79, x 1000 2107 / 142
 //   complex  16 x 16 x 16 96 / 55, 1000 x 1000 x 8 158 / 106, 128 x 2048 x 128 556 / 69,
 //            1000^3 8097 / 389 us
+// An operand whose rows span more than this many powers of two, or that holds Inf or NaN, is
+// left to the SIMT kernel.  Within it every entry keeps at least 62 - 36 bits and the largest
+// ones all 53; Gaussian rows span about 2^25.
+constexpr int SPLIT_RANGE = 36;
 constexpr int SPLIT_MIN_K_REAL = 28, SPLIT_MIN_K_CPLX = 8;
 constexpr size_t SPLIT_MAX_BYTES = size_t(16) << 30;
 }  // namespace
@@ -984,14 +986,14 @@ static View transpose_view(const View& v) {
 template <typename T>
 cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA, const T* B,
                     const View& vb, bool conjB, T* C, const View& vc, int S, void* ws,
-                    int* status, cudaStream_t s, int nb, int* wide) {
+                    int* status, cudaStream_t s, int nb, const TcWide& opt) {
   using namespace tc;
   if (M <= 0 || N <= 0 || nb <= 0) return cudaSuccess;
-  if ((S < 2 || S > 5) && !(S == 8 && wide)) return cudaErrorInvalidValue;
+  if ((S < 2 || S > 5) && !(S == 8 && opt.wide)) return cudaErrorInvalidValue;
   // keep the long dimension on the 128-row side: C^T = B^T A^T
   if (M < BM && N > M) {
     return gemm_tc<T>(N, M, K, B, transpose_view(vb), conjB, A, transpose_view(va), conjA, C,
-                      transpose_view(vc), S, ws, status, s, nb, wide);
+                      transpose_view(vc), S, ws, status, s, nb, opt);
   }
   constexpr bool CPLX = ops<T>::cplx;
   if (g_sms == 0) {
@@ -1021,7 +1023,8 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
   pk.plane_a = b * g.Mp * g.K2p;
   pk.plane_b = b * g.N2p * g.K2p;
   pk.status = status;
-  pk.wide = wide;
+  pk.wide = opt.wide;
+  pk.range = opt.range;
   cudaError_t pe = pack_operands<T>(pk, S, nb, s);
   if (pe != cudaSuccess) return pe;
   CUtensorMap ma;
@@ -1053,12 +1056,13 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
     args.C = reinterpret_cast<char*>(C);
     args.vc = vc;
     args.status = status;
-    args.skip = wide;
+    args.skip = opt.skip ? opt.wide : nullptr;
+    args.subtract = opt.subtract ? 1 : 0;
     args.splits = splits;
     args.Mp = g.Mp;
     args.N2p = g.N2p;
     args.ebsB = CPLX ? g.N2p / 2 : g.N2p;
-    if (splits > 1) {
+    if (splits > 1 && !opt.subtract) {
       // the split partial sums are added into a zeroed C
       cudaError_t e = gemm_f64<T>(M, N, 0, nb, A, va, false, B, vb, false, C, vc, s);
       if (e != cudaSuccess) return e;
@@ -1133,7 +1137,7 @@ cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& 
   cudaError_t e = cudaMemsetAsync(wide, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   e = gemm_tc<T>(M, N, K, A, va, conjA, B, vb, conjB, C, vc, 8, static_cast<char*>(ws) + 256,
-                 status, s, nb, wide);
+                 status, s, nb, TcWide{wide, SPLIT_RANGE, true, false});
   if (e != cudaSuccess) return e;
   return gemm_f64<T>(M, N, K, nb, A, va, conjA, B, vb, conjB, C, vc, s, wide);
 }
@@ -1146,9 +1150,9 @@ template cudaError_t gemm_f64_split<zdbl>(int, int, int, int, const zdbl*, const
                                           void*, int*, cudaStream_t);
 template cudaError_t gemm_tc<double>(int, int, int, const double*, const View&, bool,
                                      const double*, const View&, bool, double*, const View&, int,
-                                     void*, int*, cudaStream_t, int, int*);
+                                     void*, int*, cudaStream_t, int, const TcWide&);
 template cudaError_t gemm_tc<zdbl>(int, int, int, const zdbl*, const View&, bool, const zdbl*,
                                    const View&, bool, zdbl*, const View&, int, void*, int*,
-                                   cudaStream_t, int, int*);
+                                   cudaStream_t, int, const TcWide&);
 
 }  // namespace cbc

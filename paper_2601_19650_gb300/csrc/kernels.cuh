@@ -75,26 +75,37 @@ cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& 
 // The same product on the tensor cores with S bf16 slices per operand (gemm_tc.cu);
 // `ws` must hold gemm_tc_workspace_bytes(M, N, K, cplx, S, nb) bytes.  nb problems of
 // one shape, their operands va.bs / vb.bs / vc.bs elements apart, in one launch.
+// S = 8 (62 bits of every entry, relative to its row's maximum) needs TcWide::wide, a device
+// word that is set when an operand holds Inf or NaN or one of its rows spans more than
+// 2^range; `skip`: then C is left alone.  `subtract`: C - A B into C.
+struct TcWide {
+  int* wide = nullptr;
+  int range = 1 << 20;
+  bool skip = false;
+  bool subtract = false;
+};
 size_t gemm_tc_workspace_bytes(int M, int N, int K, bool cplx, int S, int nb = 1);
 template <typename T>
 cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA, const T* B,
                     const View& vb, bool conjB, T* C, const View& vc, int S, void* ws,
-                    int* status, cudaStream_t s, int nb = 1, int* wide = nullptr);
+                    int* status, cudaStream_t s, int nb = 1, const TcWide& opt = TcWide());
 
 // ---- Hermitian eigensolver (FP64): A (m x m, row-major, overwritten) -----------------
 // Finds the eigenvalues in descending order (the first kmax as FP64 Rayleigh quotients of the
 // vectors, the rest as single-precision estimates) and the eigenvectors of the kmax largest.
 // Outputs: lam[m], U (m x kmax, row-major, column j = eigenvector j); nb matrices m*m (lam m,
-// U m*kmax) elements apart.  Workspace: nb * eig_workspace_bytes(m, kmax).
+// U m*kmax) elements apart.  Workspace: nb * eig_workspace_bytes(m, kmax), and in `bt`, which
+// may be NULL, eig_bt_bytes(m, kmax, nb) for the back transformation by matrix products.
 size_t eig_workspace_bytes(int m, int kmax, bool cplx);
 template <typename T>
 cudaError_t heev_top(T* A, int m, int kmax, double* lam, T* U, void* work, int* status,
                      int num_sms, cudaStream_t s, int nb = 1, bool prefer_cluster = false,
-                     bool df = false);
+                     bool df = false, void* bt = nullptr);
+size_t eig_bt_bytes(int m, int kmax, bool cplx, int nb);  // 0: the products are not used
 
 // Householder tridiagonalisation by one thread-block cluster per matrix (rows in shared
 // memory, exchanges through distributed shared memory; tridiag_cluster.cu).  Outputs as
-// the eigensolver's first stage: d, e, tau, V (row j = [tau_j, 1, v_j...] from column j),
+// the eigensolver's first stage: d, e, tau, V (row j = [1, v_j...] from column j + 1),
 // per matrix wb bytes apart; A: nb matrices a_bs elements apart.  df: double-float rows.
 // tridiag_cluster_size returns the cluster size that fits (4, 8 or 16), 0 if none.
 template <typename T>

@@ -222,6 +222,8 @@ int refine_level2(Arena& ar, const Prec& pr, const T* M, int m, int n, int kmax,
   T* P2 = ar.get<T>((size_t)g * k2);
   T* W2c = rows ? nullptr : ar.get<T>((size_t)m * k2);
   char* work = ar.get<char>(eig_workspace_bytes(g, k2, ops<T>::cplx));
+  const size_t btb = eig_bt_bytes(g, k2, ops<T>::cplx, 1);
+  void* bt = btb > 0 ? ar.try_get(btb) : nullptr;
   double* dv = ar.get<double>(k2 + 4);
   CKA(P); CKA(R); CKA(K2); CKA(lam2); CKA(U2); CKA(C); CKA(P2); CKA(work); CKA(dv);
   if (!rows) CKA(W2c);
@@ -240,7 +242,8 @@ int refine_level2(Arena& ar, const Prec& pr, const T* M, int m, int n, int kmax,
   else        // R^H R
     CK(tgemm<T>(pr, true, true, n, n, m, R, View::transposed(n), true, R, View::rowmajor(n),
                 false, K2, View::rowmajor(n), s));
-  CK(heev_top<T>(K2, g, k2, lam2, U2, work, sc.status, num_sms(), s, 1, o.concurrent, false));
+  CK(heev_top<T>(K2, g, k2, lam2, U2, work, sc.status, num_sms(), s, 1, o.concurrent, false,
+                 bt));
   // U2 <- U2 - U1r (U1r^H U2)
   CK(tgemm<T>(pr, true, false, jlo, k2, g, U1, View::transposed(kmax), true, U2,
               View::rowmajor(k2), false, C, View::rowmajor(k2), s));
@@ -310,6 +313,8 @@ int compress_rows(Arena& ar, const Prec& pr, const T* M, int m, int n, int64_t m
   double* lam = ar.get<double>((size_t)nb * g);
   T* U = ar.get<T>((size_t)nb * g * kmax);
   char* work = ar.get<char>(nb * eig_workspace_bytes(g, kmax, ops<T>::cplx));
+  const size_t btb = eig_bt_bytes(g, kmax, ops<T>::cplx, nb);
+  void* bt = btb > 0 ? ar.try_get(btb) : nullptr;
   double* dv = ar.get<double>((size_t)nb * (kmax + 2));  // w [nb][kmax], beyond [nb], total [nb]
   CKA(K); CKA(lam); CKA(U); CKA(work); CKA(dv);
   double* w_dev = dv;
@@ -326,7 +331,8 @@ int compress_rows(Arena& ar, const Prec& pr, const T* M, int m, int n, int64_t m
   // ||M||_F^2, the weight of the cut: the trace of the Gram (g reads instead of m n)
   CK(trace_real<T>(K, g, (int64_t)g * g, total_dev, s, nb));
   // every candidate; the mixed path reduces batches to tridiagonal form in double-float
-  CK(heev_top<T>(K, g, kmax, lam, U, work, sc.status, num_sms(), s, nb, o.concurrent, pr.mixed));
+  CK(heev_top<T>(K, g, kmax, lam, U, work, sc.status, num_sms(), s, nb, o.concurrent, pr.mixed,
+                 bt));
   const int64_t ubs = (int64_t)g * kmax;
   T* W = nullptr;
   int64_t wbs;

@@ -47,7 +47,7 @@ struct TriClArgs {
   int m;
   double* d;       // per-matrix outputs, workspaces wb bytes apart:
   double* e;       //   diagonal, off-diagonal (beta_j), tau_j, and the reflectors
-  T* tau;          //   V (row j: [j] = tau_j, [j+1] = 1, [c] = v_c)
+  T* tau;          //   V (row j: [j+1] = 1, [c] = v_c)
   T* V;
   int64_t a_bs;    // elements between consecutive matrices A
   size_t wb;       // bytes between consecutive workspaces
@@ -227,7 +227,6 @@ __global__ void __launch_bounds__(TCL_THREADS) tridiag_cluster_kernel(TriClArgs<
       s_scaleE = AR::cvt(scale);
       s_trivial = trivial ? 1 : 0;
       if (cta == 0) {
-        V[(int64_t)j * m + j] = tau;
         tau_out[j] = tau;
         e[j] = beta;
       }

@@ -65,3 +65,13 @@ def test_special_matrices(kind, nb, mixed, cplx):
     elif kind == "huge":
         a = a * (1e60 if not mixed else 1e12)
     _check(a, kmax=m // 2, nb=nb, mixed=mixed)
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("m", [48, 63, 64, 65, 127, 128, 129, 193])
+def test_back_transformation_blocks(m, cplx):
+    """Batches large enough for the back transformation by products, around its blocks of 64
+    reflectors (two halves of 32) and a last block that is short."""
+    k = m // 2 + 1
+    nb = int(4e6 / (m * m * k)) + 1
+    _check(_random(m, cplx), kmax=k, nb=nb)
