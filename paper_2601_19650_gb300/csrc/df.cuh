@@ -30,9 +30,32 @@ template <>
 struct dfof<zdbl> {
   using type = dfz;
 };
+// Conversions between FP64 and double-float in integer operations (an FP64 instruction, a
+// conversion included, costs a warp ~64 clocks on this part); values far outside the FP32
+// range go through the conversion instructions.
 __device__ __forceinline__ df1 df_make(double x) {
-  const float h = __double2float_rn(x);
-  return {h, __double2float_rn(x - (double)h)};
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ffu);
+  if (ex - 960 > 180 || ex < 960) {
+    if ((b << 1) == 0ull) return {0.f, 0.f};
+    const float h = __double2float_rn(x);
+    return {h, __double2float_rn(x - (double)h)};
+  }
+  // mantissa = q 2^29 + rem, q of 24 bits rounded to nearest, |rem| <= 2^28
+  const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
+  const int q = (int)((m + (1ull << 28)) >> 29);
+  const int rem = (int)(m - ((unsigned long long)q << 29));
+  const unsigned sg = (unsigned)(b >> 32) & 0x80000000u;
+  const float h = __int2float_rn(q) * __uint_as_float(sg | ((unsigned)(ex - 1046 + 127) << 23));
+  const float l = __int2float_rn(rem) * __uint_as_float(sg | ((unsigned)(ex - 1075 + 127) << 23));
+  return {h, l};
+}
+__device__ __forceinline__ double df_widen(float f) {
+  const unsigned u = __float_as_uint(f), ex = (u >> 23) & 0xffu;
+  if (ex - 1u >= 254u) return (u << 1) ? (double)f : 0.0;
+  const unsigned long long b = ((unsigned long long)(u & 0x80000000u) << 32) |
+                               (((unsigned long long)(u & 0x7fffffffu) << 29) + (896ull << 52));
+  return __longlong_as_double((long long)b);
 }
 __device__ __forceinline__ df1 df_neg(df1 a) { return {-a.h, -a.l}; }
 // c + a b
@@ -50,7 +73,7 @@ __device__ __forceinline__ df1 df_fma(df1 a, df1 b, df1 c) {
 }
 __device__ __forceinline__ df1 to_df(double x) { return df_make(x); }
 __device__ __forceinline__ dfz to_df(zdbl x) { return {df_make(x.re), df_make(x.im)}; }
-__device__ __forceinline__ double from_df(df1 a) { return (double)a.h + (double)a.l; }
+__device__ __forceinline__ double from_df(df1 a) { return df_widen(a.h) + df_widen(a.l); }
 __device__ __forceinline__ zdbl from_df(dfz a) { return {from_df(a.re), from_df(a.im)}; }
 __device__ __forceinline__ df1 dff(df1 a, df1 b, df1 c) { return df_fma(a, b, c); }
 __device__ __forceinline__ dfz dff(dfz a, dfz b, dfz c) {  // c + a b, complex

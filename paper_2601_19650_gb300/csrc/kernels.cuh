@@ -107,12 +107,16 @@ size_t eig_bt_bytes(int m, int kmax, bool cplx, int nb);  // 0: the products are
 // memory, exchanges through distributed shared memory; tridiag_cluster.cu).  Outputs as
 // the eigensolver's first stage: d, e, tau, V (row j = [1, v_j...] from column j + 1),
 // per matrix wb bytes apart; A: nb matrices a_bs elements apart.  df: double-float rows.
-// tridiag_cluster_size returns the cluster size that fits (4, 8 or 16), 0 if none.
+// tridiag_cluster_shape returns the cluster that fits (ctas = 0 if none).
+struct TriClusterShape {
+  int ctas = 0, threads = 0;
+};
 template <typename T>
-int tridiag_cluster_size(int m, bool df);
+TriClusterShape tridiag_cluster_shape(int m, int nb, bool df);
 template <typename T>
 cudaError_t tridiag_cluster(const T* A, int m, double* d, double* e, T* tau, T* V, int64_t a_bs,
-                            size_t wb, int nb, int P, bool df, cudaStream_t s);
+                            size_t wb, int nb, const TriClusterShape& sh, bool df,
+                            cudaStream_t s);
 
 // ---- Cholesky QR (FP64) ------------------------------------------------------------
 // Q = C^{-1} S with G = S S^H = C C^H, S: m x n (m <= n), row-major, in place on S.
