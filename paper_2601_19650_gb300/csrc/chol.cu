@@ -5,15 +5,19 @@
 // the GPU path forms G = S S^H, factors G = C C^H, and solves Q = C^{-1} S; doing it
 // twice (CholeskyQR2) restores orthonormality to FP64 round-off.
 //
-// Cholesky: one group of CTAs that wait on each other (a thread-block cluster of up to
-// 16 CTAs, else a cooperative launch), 32-wide column blocks.  Per block, CTA 0 factors
-// the diagonal block in shared memory, every other row of the panel is solved by one
-// warp (shuffles carry the solved entries), and the trailing lower triangle is updated
-// from a shared-memory copy of the panel; bounded grid barriers separate the phases.
+// Cholesky: one thread-block cluster per matrix with the rows in shared memory
+// (chol_cluster_kernel), a CTA per matrix for larger batches (chol1_kernel); for matrices
+// that no cluster holds, a group of CTAs that wait on each other works in 32-wide column
+// blocks on global memory (chol_kernel): per block, CTA 0 factors the diagonal block in shared
+// memory, every other row of the panel is solved by one warp (shuffles carry the solved
+// entries), and the trailing lower triangle is updated from a shared-memory copy of the panel;
+// bounded grid barriers separate the phases.
 // Triangular solve: columns of S are independent, so each warp owns one column and runs
 // the forward substitution in 32-row groups without any inter-CTA synchronisation.
 // Divisions use Newton reciprocals (rcp64): long dependent chains of FP64 divisions are
 // slow on this part.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "df.cuh"
@@ -169,6 +173,11 @@ __global__ void __launch_bounds__(TPB) chol_kernel(CholArgs<T> a) {
   }
 }
 
+// offset of own row t (r = q + P t) in rank q's packed triangle: sum_{u<t} (q + P u + 1)
+__device__ __forceinline__ int tri_off(int q, int P, int t) {
+  return t * (q + 1) + P * (t * (t - 1) / 2);
+}
+
 // One CTA per matrix of a batch (blockIdx.x), the lower triangle packed in shared memory
 // ((i, l) at i (i + 1) / 2 + l): right-looking, one column per step, no grid barriers.
 // For batches, where the matrices themselves fill the SMs.
@@ -225,6 +234,120 @@ __global__ void __launch_bounds__(TPB) chol1_kernel(T* G, int m, int* status) {
   for (int64_t t = threadIdx.x; t < tri; t += blockDim.x) {
     const int i = tri_row(t);
     G[(int64_t)i * m + (t - (int64_t)i * (i + 1) / 2)] = L[t];
+  }
+}
+
+// One thread-block cluster of P CTAs (a power of two) per matrix, the lower triangle of each
+// CTA's rows r = rank + P t packed in shared memory; right-looking, two columns per step.  A
+// CTA sets its rows' entries of the next two columns aside while it updates them; after the
+// step's one cluster barrier every CTA reads both columns from their owners (distributed
+// shared memory) and updates the second by the first itself.  The updates need 1 / pivot only,
+// A[r][c] -= (A[r][j] / pivot) conj(A[c][j]); the roots and the scaled columns come from one
+// warp beside them.  Bound by that chain (~64 clocks per dependent FP64 operation).  Column
+// blocks of 32 with three barriers through global memory each / one column per step / this:
+// m = 128 complex 466 / 260 / 206 us (64 218 / 101 / 72).
+constexpr int CHT = 128;
+template <typename T>
+__global__ void __launch_bounds__(CHT) chol_cluster_kernel(T* G, int m, int rows_cap, int nr_cap,
+                                                           int* status) {
+  using O = ops<T>;
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int P = (int)cluster.num_blocks(), lp = 31 - __clz(P), pm = P - 1;
+  const int cta = (int)cluster.block_rank();
+  G += (int64_t)(blockIdx.x >> lp) * m * m;
+  extern __shared__ unsigned char sm_raw[];
+  T* rows = reinterpret_cast<T*>(sm_raw);
+  T* set = rows + rows_cap;      // [2][nr_cap][2] own rows' entries of these two columns and the next
+  T* col0 = set + 4 * nr_cap;    // [m] the columns
+  T* col1 = col0 + m;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = CHT / 32;
+  const int nr = (m - cta + pm) >> lp;
+  for (int t = warp; t < nr; t += nw) {
+    const int r = cta + (t << lp);
+    T* dst = rows + tri_off(cta, P, t);
+    for (int c = lane; c <= r; c += 32) {
+      const T x = G[(int64_t)r * m + c];
+      dst[c] = x;
+      if (c < 2) set[2 * t + c] = x;
+    }
+  }
+  // not positive or not finite, on the bits
+  auto no_pivot = [](double p) {
+    return (unsigned)__double2hiint(p) >= 0x7ff00000u || __double_as_longlong(p) == 0ll;
+  };
+  // 1 / pivot rounded up by one unit, so that a row that repeats an earlier one ends in a pivot
+  // that is not positive
+  // (below 2^-1019, where it would overflow, of 2^100 pivot)
+  auto tiny = [](double p) { return __double2hiint(p) < 0x00400000; };
+  auto inv_pivot = [&](double p) {
+    return __longlong_as_double(__double_as_longlong(rcp64(tiny(p) ? 0x1p100 * p : p)) + 1ll);
+  };
+  // -x / pivot
+  auto over = [&](double p, double rp, T x) {
+    return O::scale(-rp, tiny(p) ? O::scale(0x1p100, x) : x);
+  };
+  bool bad = false;
+  for (int j = 0; j < m && !bad; j += 2) {
+    const T* now = set + ((j >> 1) & 1) * 2 * nr_cap;
+    T* next = set + (((j >> 1) & 1) ^ 1) * 2 * nr_cap;
+    const bool two = j + 1 < m;
+    cluster.sync();
+    for (int c = j + tid; c < m; c += CHT) {
+      const T* src = cluster.map_shared_rank(now, c & pm) + 2 * (c >> lp);
+      col0[c] = src[0];
+      if (c > j) col1[c] = src[1];
+    }
+    __syncthreads();
+    const double p0 = O::real(col0[j]);
+    if (no_pivot(p0)) {
+      bad = true;  // in every CTA
+      break;
+    }
+    const double rp0 = inv_pivot(p0);
+    if (two) {
+      const T a1 = over(p0, rp0, O::conj(col0[j + 1]));
+      for (int c = j + 1 + tid; c < m; c += CHT) col1[c] = O::fma(a1, col0[c], col1[c]);
+    }
+    __syncthreads();
+    const double p1 = two ? O::real(col1[j + 1]) : 1.0;
+    if (no_pivot(p1)) {
+      bad = true;
+      break;
+    }
+    if (warp == nw - 1) {  // the scaled columns
+      const double rc0 = rsqrt64_short(p0), rc1 = rsqrt64_short(p1);
+      for (int t = ((j > cta) ? (j - cta + pm) >> lp : 0) + lane; t < nr; t += 32) {
+        const int r = cta + (t << lp);
+        T* row = rows + tri_off(cta, P, t) + j;
+        row[0] = (r == j) ? O::make(p0 * rc0, 0.0) : O::scale(rc0, col0[r]);
+        if (r > j) row[1] = (r == j + 1) ? O::make(p1 * rc1, 0.0) : O::scale(rc1, col1[r]);
+      }
+    }
+    const double rp1 = inv_pivot(p1);
+    const int t0 = (j + 2 > cta) ? (j + 2 - cta + pm) >> lp : 0;  // first own row beyond j + 1
+    // (by the other warps alone where there are few rows)
+    const int uw = nr <= 16 ? nw - 1 : nw;
+    for (int t = warp < uw ? t0 + warp : nr; t < nr; t += uw) {
+      const int r = cta + (t << lp);
+      T* row = rows + tri_off(cta, P, t);
+      const T f0 = over(p0, rp0, col0[r]), f1 = over(p1, rp1, col1[r]);
+      for (int c = j + 2 + lane; c <= r; c += 32) {
+        const T x = O::fma(f1, O::conj(col1[c]), O::fma(f0, O::conj(col0[c]), row[c]));
+        row[c] = x;
+        if (c < j + 4) next[2 * t + c - j - 2] = x;
+      }
+    }
+  }
+  cluster.sync();  // no CTA leaves while another still reads its columns
+  if (bad) {
+    if (tid == 0) set_status(status, CBC_ERR_NOT_POSITIVE_DEFINITE);
+    return;
+  }
+  for (int t = warp; t < nr; t += nw) {
+    const int r = cta + (t << lp);
+    const T* src = rows + tri_off(cta, P, t);
+    for (int c = lane; c <= r; c += 32) G[(int64_t)r * m + c] = src[c];
   }
 }
 
@@ -349,9 +472,38 @@ __global__ void to_df_kernel(const T* C, typename dfof<T>::type* D, df1* R, int 
 template <typename T>
 cudaError_t cholesky_lower(T* G, int m, int* status, void* bar, int num_sms, cudaStream_t s,
                            int nb) {
-  // FP64 is scarce per SM on this part: spread the trailing updates over several SMs,
-  // one cluster of up to 16 CTAs per matrix when it fits (concurrent with other
-  // streams' work), else a cooperative launch over more SMs per matrix
+  // the rows in the shared memory of one cluster per matrix: as many CTAs (and FP64 units) as
+  // the batch leaves idle, 4 rows each at least; where that is one, a kernel without a cluster
+  {
+    const void* kc = (const void*)chol_cluster_kernel<T>;
+    cudaError_t err = allow_max_smem(kc);
+    if (err != cudaSuccess) return err;
+    int want = 1;
+    while (want < 16 && want * 4 < m && 2 * want * nb <= num_sms) want *= 2;
+    const size_t tri_bytes = (size_t)m * (m + 1) / 2 * sizeof(T);
+    if (want == 1 && nb > 1 && tri_bytes <= 200 * 1024) {
+      err = allow_max_smem((const void*)chol1_kernel<T>);
+      if (err != cudaSuccess) return err;
+      note_launches(CBC_K_CHOLQR, 1);
+      chol1_kernel<T><<<nb, TPB, tri_bytes, s>>>(G, m, status);
+      return cudaGetLastError();
+    }
+    for (int P = want; P <= 16; P *= 2) {
+      int rows_cap = 0, nr_cap = (m + P - 1) / P;
+      for (int q = 0; q < P && q < m; ++q) {
+        const int nr = (m - q + P - 1) / P;
+        rows_cap = std::max(rows_cap, nr * (q + 1) + P * (nr * (nr - 1) / 2));
+      }
+      const size_t smem = ((size_t)rows_cap + 4 * nr_cap + 2 * m) * sizeof(T);
+      if (smem > 220 * 1024 || cluster_ctas(kc, P, CHT, smem) != P) continue;
+      note_launches(CBC_K_CHOLQR, 1);
+      void* args[] = {&G, &m, &rows_cap, &nr_cap, &status};
+      return launch_cluster(kc, P, nb * P, CHT, smem, args, s);
+    }
+  }
+  // larger matrices: column blocks with the matrix in global memory, one cluster of up to 16
+  // CTAs per matrix when it fits (concurrent with other streams' work), else a cooperative
+  // launch over more SMs per matrix
   cudaError_t err = cudaMemsetAsync(bar, 0, sizeof(GridBarrier) * nb, s);
   if (err != cudaSuccess) return err;
   // the panel in shared memory when it fits, else read from global memory
@@ -363,15 +515,6 @@ cudaError_t cholesky_lower(T* G, int m, int* status, void* bar, int num_sms, cud
     if (err != cudaSuccess) return err;
   }
   note_launches(CBC_K_CHOLQR, 1);
-  // a batch of 8 or more: one CTA per matrix (its FP64 work spread over the batch
-  // instead of over a cluster per matrix)
-  const size_t tri_bytes = (size_t)m * (m + 1) / 2 * sizeof(T);
-  if (nb >= 8 && tri_bytes <= 200 * 1024) {
-    err = allow_max_smem((const void*)chol1_kernel<T>);
-    if (err != cudaSuccess) return err;
-    chol1_kernel<T><<<nb, TPB, tri_bytes, s>>>(G, m, status);
-    return cudaGetLastError();
-  }
   int P = std::max(1, std::min(16, (m * m) / 256));
   if (cluster_ctas(kch, P, TPB, shm) == P) {
     CholArgs<T> a{G, m, status, (GridBarrier*)bar, P};

@@ -1,0 +1,65 @@
+"""The Cholesky factor of CholeskyQR2 at the edges of its kernels, through cbc_cholqr2: sizes
+around a pair of columns and the rows per CTA, batches that take clusters of 16, 4 and 2 CTAs
+and one CTA each, a row whose pivot is denormal, and rows that repeat an earlier one."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(S):
+    import torch
+
+    from paper_2601_19650_gb300 import _cbc as c
+    nb, m, n = S.shape
+    d = torch.from_numpy(np.ascontiguousarray(S)).to("cuda")
+    c.cbc_cholqr2(c.CBC_C128 if np.iscomplexobj(S) else c.CBC_F64, m, n, nb, d.data_ptr())
+    return d.cpu().numpy()
+
+
+def _random(nb, m, cplx):
+    r = np.random.default_rng([nb, m, cplx])
+    shape = (nb, m, 2 * m + 3)
+    return r.standard_normal(shape) + (1j * r.standard_normal(shape) if cplx else 0)
+
+
+def _check(S, Q):
+    # two passes leave a few roundings of sums of up to 800 terms: well below 1e-13
+    for s, q in zip(S, Q):
+        m = len(s)
+        assert np.abs(q @ q.conj().T - np.eye(m)).max() < 1e-13
+        # S = R Q row by row (the rows' norms may differ), R lower triangular, diagonal > 0
+        norm = np.linalg.norm(s, axis=1, keepdims=True)
+        R = (s / norm) @ q.conj().T
+        assert np.linalg.norm(s / norm - R @ q, axis=1).max() < 1e-12
+        assert np.abs(np.triu(R, 1)).max() < 1e-12
+        dg = np.diag(R)
+        assert np.all(dg.real > 0) and np.abs(dg.imag).max() < 1e-12
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("m,nb", [(1, 1), (2, 1), (3, 1), (4, 1), (5, 1), (17, 1), (31, 3),
+                                  (33, 1), (63, 1), (65, 3), (129, 1), (200, 1), (257, 1),
+                                  (400, 1), (33, 20), (64, 20), (65, 70), (7, 100), (130, 100)])
+def test_sizes_and_batches(m, nb, cplx):
+    S = _random(nb, m, cplx)
+    _check(S, _run(S))
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("row", [0, 3, 4, 11])
+def test_denormal_pivot(row, cplx):
+    S = _random(1, 12, cplx)
+    S[0, row] *= 2.0 ** -516  # its squared norm is below 2^-1024: 1 / pivot overflows
+    _check(S, _run(S))
+
+
+@pytest.mark.parametrize("nb", [1, 20])
+@pytest.mark.parametrize("pair", [(3, 7), (0, 1), (6, 7), (7, 8), (5, 39)])
+def test_repeated_row_is_reported(pair, nb):
+    from paper_2601_19650_gb300 import _cbc as c
+    S = np.random.default_rng(3).standard_normal((nb, 40, 200))
+    S[nb - 1, pair[1]] = S[nb - 1, pair[0]]
+    with pytest.raises(c.CBCError) as ei:
+        _run(S)
+    assert ei.value.code == 4
