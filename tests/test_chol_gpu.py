@@ -1,6 +1,6 @@
 """The Cholesky factor of CholeskyQR2 at the edges of its kernels, through cbc_cholqr2: sizes
 around a pair of columns and the rows per CTA, batches that take clusters of 16, 4 and 2 CTAs
-and one CTA each, a row whose pivot is denormal, and rows that repeat an earlier one."""
+and one CTA each, a row far smaller than the others (the rows are scaled to unit norm before), and rows that repeat an earlier one."""
 import numpy as np
 import pytest
 
@@ -48,9 +48,9 @@ def test_sizes_and_batches(m, nb, cplx):
 
 @pytest.mark.parametrize("cplx", [False, True])
 @pytest.mark.parametrize("row", [0, 3, 4, 11])
-def test_denormal_pivot(row, cplx):
+def test_tiny_row(row, cplx):
     S = _random(1, 12, cplx)
-    S[0, row] *= 2.0 ** -516  # its squared norm is below 2^-1024: 1 / pivot overflows
+    S[0, row] *= 2.0 ** -516  # its squared norm is denormal
     _check(S, _run(S))
 
 
