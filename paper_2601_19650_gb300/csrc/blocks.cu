@@ -81,6 +81,12 @@ int cholqr2_t(int m, int n, int nb, T* S, cudaStream_t s) {
   if (e == cudaSuccess) e = pool_malloc(&bar, sizeof(GridBarrier) * nb, s);
   if (e == cudaSuccess) e = pool_malloc(reinterpret_cast<void**>(&rn), sizeof(double) * m * nb, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), s);
+  void* tw = nullptr;
+  const size_t tb = trsm_products_bytes(m, n, ops<T>::cplx, nb, false);
+  if (e == cudaSuccess && tb > 0 && pool_malloc(&tw, tb, s) != cudaSuccess) {
+    cudaGetLastError();  // without room the solve takes the other way
+    tw = nullptr;
+  }
   const int64_t sbs = (int64_t)m * n;
   // unit rows first (the sweeps do the same): same row space, better conditioned Gram
   if (e == cudaSuccess) e = row_norms2<T>(S, m, n, n, sbs, rn, s, nb);
@@ -90,10 +96,13 @@ int cholqr2_t(int m, int n, int nb, T* S, cudaStream_t s) {
                            View::transposed(n, sbs), true, G, View::rowmajor(m, (int64_t)m * m),
                            status, s);
     if (e == cudaSuccess) e = cholesky_lower<T>(G, m, status, bar, num_sms(), s, nb);
-    if (e == cudaSuccess) e = trsm_lower_left<T>(G, S, m, n, status, bar, num_sms(), s, nb);
+    if (e == cudaSuccess)
+      e = tw ? trsm_products<T>(G, S, m, n, status, tw, s, nb)
+             : trsm_lower_left<T>(G, S, m, n, status, bar, num_sms(), s, nb);
   }
   int hs = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (tw) cudaFreeAsync(tw, s);
   if (G) cudaFreeAsync(G, s);
   if (status) cudaFreeAsync(status, s);
   if (bar) cudaFreeAsync(bar, s);

@@ -12,8 +12,9 @@
 // memory, every other row of the panel is solved by one warp (shuffles carry the solved
 // entries), and the trailing lower triangle is updated from a shared-memory copy of the panel;
 // bounded grid barriers separate the phases.
-// Triangular solve: columns of S are independent, so each warp owns one column and runs
-// the forward substitution in 32-row groups without any inter-CTA synchronisation.
+// Triangular solve: where there is enough of it, by matrix products with inverted diagonal
+// blocks (trsm_products); else columns of S are independent, so each warp owns one column and
+// runs the forward substitution in 32-row groups without any inter-CTA synchronisation.
 // Divisions use Newton reciprocals (rcp64): long dependent chains of FP64 divisions are
 // slow on this part.
 #include <cooperative_groups.h>
@@ -467,6 +468,67 @@ __global__ void to_df_kernel(const T* C, typename dfof<T>::type* D, df1* R, int 
     R[i] = df_make(rcp64(O::real(C[(int64_t)i * m + i])));
 }
 
+// ---- triangular solve by matrix products -----------------------------------------------
+// Blocks of TRB rows, X_b = C_bb^-1 (S_b - C_b,<b X_<b), with the inverses of the diagonal
+// blocks and every product on the tensor cores (8 slices, an error below that of FP64 sums).
+// A product with an inverse leaves a residual of the block's condition number times rounding,
+// substitution one of rounding, so each block is corrected once: X_b += C_bb^-1 (S_b - C_bb
+// X_b).  Bound by the chain of products; warp-per-column substitution / this, 64 of 128 x 256
+// complex: 2360 / 700 us.
+// (S comes with rows of unit norm: a slice has one exponent per column, and rows far smaller
+// than others would be lost in the products with the inverses.)
+constexpr int TRB = 64, TRH = 32;
+
+// The diagonal blocks of C (lower triangular, m x m, nb of them) as TRB x TRB matrices with
+// zeros above the diagonal (D; rows beyond m: unit rows), and the inverses of their two TRH x
+// TRH diagonal halves (Inv); both zeroed before.  One CTA per half (blockIdx.x: block and half,
+// blockIdx.y: matrix), four lanes per column of the inverse: x_r = -(1 / L_rr) sum_{i <= l < r}
+// L[r][l] x_l.
+template <typename T>
+__global__ void __launch_bounds__(128) trsm_inv_kernel(const T* C, int m, T* D, T* Inv,
+                                                       int64_t bs) {
+  using O = ops<T>;
+  __shared__ T g[TRH][TRH + 1];
+  __shared__ double rl[TRH];
+  const int blk = blockIdx.x >> 1, half = blockIdx.x & 1;
+  const int r0 = blk * TRB + half * TRH;
+  C += (int64_t)blockIdx.y * m * m;
+  D += blockIdx.y * bs + (int64_t)blk * TRB * TRB + half * TRH * TRB;  // its rows
+  Inv += blockIdx.y * bs + (int64_t)blk * TRB * TRB + half * TRH * (TRB + 1);
+  for (int e = threadIdx.x; e < TRH * TRH; e += blockDim.x) {
+    const int i = e / TRH, l = e % TRH, r = r0 + i;
+    T x = (i == l) ? O::one() : O::zero();
+    if (r < m) x = l <= i ? C[(int64_t)r * m + r0 + l] : O::zero();
+    g[i][l] = x;
+    D[(int64_t)i * TRB + half * TRH + l] = x;
+    if (half == 1 && r < m) D[(int64_t)i * TRB + l] = C[(int64_t)r * m + r0 - TRH + l];
+  }
+  __syncthreads();
+  if (threadIdx.x < TRH) rl[threadIdx.x] = rcp64(O::real(g[threadIdx.x][threadIdx.x]));
+  __syncthreads();
+  const int i = threadIdx.x >> 2, sub = threadIdx.x & 3;  // column i, terms l = sub (mod 4)
+  T x[TRH / 4];                                           // x_l, l = sub + 4 q
+#pragma unroll
+  for (int q = 0; q < TRH / 4; ++q) x[q] = (sub + 4 * q == i) ? O::make(rl[i], 0.0) : O::zero();
+#pragma unroll
+  for (int r = 1; r < TRH; ++r) {
+    T acc = O::zero();
+#pragma unroll
+    for (int q = 0; q < TRH / 4; ++q)
+      if (4 * q < r) {
+        const int l = sub + 4 * q;
+        if (l < r) acc = O::fma(g[r][l], x[q], acc);
+      }
+    acc = acc + shfl_xor(acc, 1);
+    acc = acc + shfl_xor(acc, 2);
+    if (r > i && (r & 3) == sub) x[r >> 2] = O::scale(-rl[r], acc);
+  }
+#pragma unroll
+  for (int q = 0; q < TRH / 4; ++q) Inv[(int64_t)(sub + 4 * q) * TRB + i] = x[q];
+}
+
+size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
+
 }  // namespace
 
 template <typename T>
@@ -531,6 +593,73 @@ cudaError_t cholesky_lower(T* G, int m, int* status, void* bar, int num_sms, cud
   return cudaSuccess;
 }
 
+size_t trsm_products_bytes(int m, int n, bool cplx, int nb, bool df) {
+  // Each block is a chain of four products (~75 us where they are small), so the line is work
+  // per block.  Both solves of a CholeskyQR2, substitution / products in us: 128 x 256 complex,
+  // 16 of them 1350 / 550, one 231 / 465; 64 of 64 x 128 complex 718 / 410; complex 400 x 800
+  // 2586 / 1370, 256 x 512 694 / 806; real 600 x 1200 1265 / 1720.  Double-float substitution
+  // takes about half as long.
+  const double line = df ? 1.2e8 : 6e7;
+  if ((double)m * m * n * nb * (cplx ? 4 : 1) < line * ((m + TRB - 1) / TRB)) return 0;
+  const size_t ts = cplx ? sizeof(zdbl) : sizeof(double);
+  const size_t nblk = (m + TRB - 1) / TRB;
+  size_t g = gemm_tc_workspace_bytes(TRH, TRH, TRH, cplx, 8, (int)(nb * nblk));
+  g = std::max(g, gemm_tc_workspace_bytes(std::min(TRB, m), n, m, cplx, 8, nb));
+  return 256 + al256(2 * nb * nblk * TRB * TRB * ts) + al256(nb * nblk * TRH * TRH * ts) +
+         al256((size_t)nb * TRB * n * ts) + g;
+}
+
+template <typename T>
+cudaError_t trsm_products(const T* C, T* S, int m, int n, int* status, void* ws, cudaStream_t s,
+                          int nb) {
+  const int nblk = (m + TRB - 1) / TRB;
+  const int64_t sq = TRB * TRB, bs = nblk * sq, hf = TRH * TRH, mn = (int64_t)m * n;
+  char* w = static_cast<char*>(ws);
+  auto take = [&](size_t bytes) {
+    char* p = w;
+    w += al256(bytes);
+    return p;
+  };
+  TcWide set;
+  set.wide = reinterpret_cast<int*>(take(4));  // (Inf and NaN are met by the next Gram)
+  T* D = reinterpret_cast<T*>(take(2 * nb * bs * sizeof(T)));
+  T* Inv = D + nb * bs;
+  T* tmp = reinterpret_cast<T*>(take(sizeof(T) * nb * nblk * hf));
+  T* X = reinterpret_cast<T*>(take(sizeof(T) * (size_t)nb * TRB * n));
+  void* gw = w;
+  cudaError_t e = cudaMemsetAsync(D, 0, 2 * nb * bs * sizeof(T), s);
+  if (e != cudaSuccess) return e;
+  note_launches(CBC_K_CHOLQR, 1);
+  trsm_inv_kernel<T><<<dim3(2 * nblk, nb), 128, 0, s>>>(C, m, D, Inv, bs);
+  // dst = A B (acc 0), dst - A B (-1) or base + A B (1)
+  auto mul = [&](int M, int N, int K, const T* A, int64_t lda, int64_t abs, const T* B,
+                 int64_t ldb, int64_t bbs, T* dst, int64_t ldc, int64_t cbs, int cnt, int acc,
+                 const T* base) {
+    if (e != cudaSuccess) return;
+    TcWide o = set;
+    o.acc = acc;
+    o.base = base;
+    o.base_bs = (int64_t)TRB * n;  // (X)
+    e = gemm_tc<T>(M, N, K, A, View::rowmajor(lda, abs), false, B, View::rowmajor(ldb, bbs), false,
+                   dst, View::rowmajor(ldc, cbs), 8, gw, status, s, cnt, o);
+  };
+  // the inverse of a block from its halves': Inv21 = -Inv22 (C21 Inv11)
+  mul(TRH, TRH, TRH, D + TRH * TRB, TRB, sq, Inv, TRB, sq, tmp, TRH, hf, nb * nblk, 0, nullptr);
+  mul(TRH, TRH, TRH, Inv + TRH * (TRB + 1), TRB, sq, tmp, TRH, hf, Inv + TRH * TRB, TRB, sq,
+      nb * nblk, -1, nullptr);
+  for (int q = 0; q < nblk; ++q) {
+    const int r0 = q * TRB, h = std::min(TRB, m - r0);
+    T* Sb = S + (int64_t)r0 * n;
+    const T *Db = D + q * sq, *Ib = Inv + q * sq;
+    if (q > 0)
+      mul(h, n, r0, C + (int64_t)r0 * m, m, (int64_t)m * m, S, n, mn, Sb, n, mn, nb, -1, nullptr);
+    mul(h, n, h, Ib, TRB, bs, Sb, n, mn, X, n, (int64_t)TRB * n, nb, 0, nullptr);
+    mul(h, n, h, Db, TRB, bs, X, n, (int64_t)TRB * n, Sb, n, mn, nb, -1, nullptr);
+    mul(h, n, h, Ib, TRB, bs, Sb, n, mn, Sb, n, mn, nb, 1, X);
+  }
+  return e;
+}
+
 template <typename T>
 cudaError_t trsm_lower_left(const T* C, T* S, int m, int n, int* status, void* bar, int num_sms,
                             cudaStream_t s, int nb, void* dfbuf) {
@@ -585,6 +714,10 @@ cudaError_t trsm_lower_left(const T* C, T* S, int m, int n, int* status, void* b
 
 template cudaError_t cholesky_lower<double>(double*, int, int*, void*, int, cudaStream_t, int);
 template cudaError_t cholesky_lower<zdbl>(zdbl*, int, int*, void*, int, cudaStream_t, int);
+template cudaError_t trsm_products<double>(const double*, double*, int, int, int*, void*,
+                                           cudaStream_t, int);
+template cudaError_t trsm_products<zdbl>(const zdbl*, zdbl*, int, int, int*, void*, cudaStream_t,
+                                         int);
 template cudaError_t trsm_lower_left<double>(const double*, double*, int, int, int*, void*, int,
                                              cudaStream_t, int, void*);
 template cudaError_t trsm_lower_left<zdbl>(const zdbl*, zdbl*, int, int, int*, void*, int,

@@ -1272,7 +1272,7 @@ static cudaError_t backtransform_products(const T* V, const T* tau, const double
   TcWide opt;
   opt.wide = flag;
   TcWide sub = opt;
-  sub.subtract = true;
+  sub.acc = -1;
   cudaError_t e = cudaMemsetAsync(bt, 0, (char*)(G + 2 * nb * tbs) - (char*)bt, s);  // flag, G, T
   auto mul = [&](int M, int N, int K, const T* A, View va, int64_t abs, bool ca, const T* B,
                  View vb, int64_t bbs, T* C, int64_t ldc, int64_t cbs, int n, const TcWide& o) {

@@ -205,7 +205,9 @@ struct TcArgs {
   View vc;               // vc.bs: elements between the outputs of consecutive problems
   int* status;
   const int* skip;       // not NULL: nothing runs when *skip is set (gemm_f64_split)
-  int subtract;          // C - A B instead of A B
+  int acc;               // 1 or -1: base + A B or base - A B instead of A B
+  const char* base;      // rows and columns as C's (C itself when it is split along K)
+  int64_t base_shift;    // base's bytes from problem to problem less C's
   int splits;            // K splits per problem
   int Mp, N2p;           // packed rows of one problem in the A and B planes
   int ebsB;              // entries of expB per problem
@@ -458,7 +460,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
         const int ea = rowok ? a.expA[q.prob * a.Mp + row] : 0;
         const int bias = -2 * head(S) - 8 * (S - 1);
         const int64_t ro = rowok ? a.vc.roff(row) : 0;
-        const bool pair = a.cplx && !a.atomic && !a.subtract && (reinterpret_cast<uintptr_t>(a.C) & 15) == 0;
+        const bool pair = a.cplx && !a.atomic && !a.acc && (reinterpret_cast<uintptr_t>(a.C) & 15) == 0;
         auto value = [&](int i, int e) {
           if constexpr (NACC == 2)
             return i96_ldexp(acc[0][i], acc[1][i], e);
@@ -467,9 +469,13 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
         };
         auto put = [&](double* dst, double v) {
           if (a.atomic)
-            atomicAdd(dst, a.subtract ? -v : v);
+            atomicAdd(dst, a.acc < 0 ? -v : v);
+          else if (a.acc)
+            *dst = *reinterpret_cast<const double*>(a.base + (reinterpret_cast<char*>(dst) - a.C) +
+                                                    q.prob * a.base_shift) +
+                   (a.acc < 0 ? -v : v);
           else
-            *dst = a.subtract ? *dst - v : v;
+            *dst = v;
         };
 #pragma unroll
         for (int i = 0; i < CW; i += 2) {
@@ -1040,7 +1046,7 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
     const int tiles_n = (g.N2p + BN - 1) / BN;
     const int tiles = (g.Mp / BM) * tiles_n * nb;
     int splits = 1;
-    if (tiles < g_sms && chunks > 1) splits = std::min(chunks, std::max(1, g_sms / tiles));
+    if (tiles < g_sms && chunks > 1 && !opt.base) splits = std::min(chunks, std::max(1, g_sms / tiles));
     const int chunks_per_split = (chunks + splits - 1) / splits;
     splits = (chunks + chunks_per_split - 1) / chunks_per_split;
     TcArgs args;
@@ -1057,12 +1063,14 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
     args.vc = vc;
     args.status = status;
     args.skip = opt.skip ? opt.wide : nullptr;
-    args.subtract = opt.subtract ? 1 : 0;
+    args.acc = opt.acc;
+    args.base = opt.base ? static_cast<const char*>(opt.base) : args.C;
+    args.base_shift = opt.base ? (opt.base_bs - vc.bs) * (int64_t)sizeof(T) : 0;
     args.splits = splits;
     args.Mp = g.Mp;
     args.N2p = g.N2p;
     args.ebsB = CPLX ? g.N2p / 2 : g.N2p;
-    if (splits > 1 && !opt.subtract) {
+    if (splits > 1 && !opt.acc) {
       // the split partial sums are added into a zeroed C
       cudaError_t e = gemm_f64<T>(M, N, 0, nb, A, va, false, B, vb, false, C, vc, s);
       if (e != cudaSuccess) return e;
@@ -1137,7 +1145,7 @@ cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& 
   cudaError_t e = cudaMemsetAsync(wide, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   e = gemm_tc<T>(M, N, K, A, va, conjA, B, vb, conjB, C, vc, 8, static_cast<char*>(ws) + 256,
-                 status, s, nb, TcWide{wide, SPLIT_RANGE, true, false});
+                 status, s, nb, TcWide{wide, SPLIT_RANGE, true});
   if (e != cudaSuccess) return e;
   return gemm_f64<T>(M, N, K, nb, A, va, conjA, B, vb, conjB, C, vc, s, wide);
 }

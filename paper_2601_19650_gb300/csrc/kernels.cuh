@@ -77,12 +77,15 @@ cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& 
 // one shape, their operands va.bs / vb.bs / vc.bs elements apart, in one launch.
 // S = 8 (62 bits of every entry, relative to its row's maximum) needs TcWide::wide, a device
 // word that is set when an operand holds Inf or NaN or one of its rows spans more than
-// 2^range; `skip`: then C is left alone.  `subtract`: C - A B into C.
+// 2^range; `skip`: then C is left alone.  acc = 1 or -1: base + A B or base - A B into C, with
+// base (NULL: C itself) laid out as C but for its problems, base_bs elements apart.
 struct TcWide {
   int* wide = nullptr;
   int range = 1 << 20;
   bool skip = false;
-  bool subtract = false;
+  int acc = 0;
+  const void* base = nullptr;
+  int64_t base_bs = 0;
 };
 size_t gemm_tc_workspace_bytes(int M, int N, int K, bool cplx, int S, int nb = 1);
 template <typename T>
@@ -129,6 +132,14 @@ cudaError_t cholesky_lower(T* G, int m, int* status, void* bar, int num_sms, cud
 template <typename T>
 cudaError_t trsm_lower_left(const T* C, T* S, int m, int n, int* status, void* bar,
                             int num_sms, cudaStream_t s, int nb = 1, void* dfbuf = nullptr);
+// The same solve by products on the tensor cores, to FP64 accuracy (`df`: the other way would
+// be double-float): `ws` holds
+// trsm_products_bytes (0 where trsm_lower_left is the better way) bytes; S has
+// rows of unit norm.
+size_t trsm_products_bytes(int m, int n, bool cplx, int nb, bool df);
+template <typename T>
+cudaError_t trsm_products(const T* C, T* S, int m, int n, int* status, void* ws, cudaStream_t s,
+                          int nb);
 inline size_t trsm_df_bytes(int m, int nb, bool cplx) {
   return (size_t)nb * ((size_t)m * m * (cplx ? 16 : 8) + (size_t)m * 8);
 }

@@ -1,6 +1,8 @@
 """The Cholesky factor of CholeskyQR2 at the edges of its kernels, through cbc_cholqr2: sizes
 around a pair of columns and the rows per CTA, batches that take clusters of 16, 4 and 2 CTAs
-and one CTA each, a row far smaller than the others (the rows are scaled to unit norm before), and rows that repeat an earlier one."""
+and one CTA each, a row far smaller than the others (the rows are scaled to unit norm before), and rows that repeat an
+earlier one; and the triangular solve by products (batches with enough work) at the edges of
+its blocks of 64 rows and their halves, nearly dependent rows among them."""
 import numpy as np
 import pytest
 
@@ -63,3 +65,19 @@ def test_repeated_row_is_reported(pair, nb):
     with pytest.raises(c.CBCError) as ei:
         _run(S)
     assert ei.value.code == 4
+
+
+@pytest.mark.parametrize("m,n,nb,cplx", [(33, 70, 200, True), (40, 41, 240, True),
+                                         (64, 64, 60, True), (65, 131, 56, True),
+                                         (97, 195, 24, True), (130, 261, 12, True),
+                                         (128, 130, 32, False), (128, 130, 64, False),
+                                         (129, 300, 40, False)])
+def test_solve_by_products(m, n, nb, cplx):
+    # by products where m^2 n nb (times 4 if complex) is 6e7 or more per block of 64 rows: all
+    # of these but the 32 of 128 x 130, which lie below the line
+    r = np.random.default_rng([m, n, nb])
+    S = r.standard_normal((nb, m, n)) + (1j * r.standard_normal((nb, m, n)) if cplx else 0)
+    S[:, 5] = S[:, 4] + 1e-5 * S[:, 5]
+    S[:, m - 1] = S[:, 0] + 1e-5 * S[:, m - 1]
+    S[:, 7] *= 2.0 ** -300
+    _check(S, _run(S))
