@@ -549,6 +549,9 @@ __device__ __forceinline__ int expo_bits(double x) {
 // Returned is N + sum_{i<S-1} 128 256^i: its byte i is q_{S-1-i} + 128 for i < S-1, and its
 // bits from 8 (S-1) up are q_0.
 template <int S>
+constexpr long long DIGIT_BIAS =
+    (long long)(0x8080808080808080ull & ((1ull << (8 * (S - 1))) - 1ull));
+template <int S>
 __device__ __forceinline__ long long digit_word(double x, int e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7ffu);
@@ -562,8 +565,12 @@ __device__ __forceinline__ long long digit_word(double x, int e) {
   else
     n = sh < 64 ? (mant + (1ull << (sh - 1))) >> sh : 0ull;
   const long long N = (b >> 63) ? -(long long)n : (long long)n;
-  constexpr long long bias = (long long)(0x8080808080808080ull & ((1ull << (8 * (S - 1))) - 1ull));
-  return N + bias;
+  return N + DIGIT_BIAS<S>;
+}
+// the word of -x from x's
+template <int S>
+__device__ __forceinline__ long long negated_word(long long w) {
+  return 2 * DIGIT_BIAS<S> - w;
 }
 
 // digit q_s as the bits of a float (exact; its upper half is the bf16): 2^23 + 128 + q is
@@ -750,6 +757,9 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
         T x = tile[lr * LD + lane];
         if (o.conj) x = O::conj(x);
         const long long wr = digit_word<S>(O::real(x), e), wi = digit_word<S>(O::imag(x), e);
+        // -x has digits of its own (a digit of -128 carries), and products that leave out the
+        // last levels depend on them
+        const long long wn = negated_word<S>(wi);
         uint32_t* d = out + (size_t)(SIDE_B ? 2 : 1) * (r0 + lr) * ld + t * 32 + lane;
 #pragma unroll
         for (int sl = 0; sl < S; ++sl) {
@@ -757,7 +767,7 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
           if (!SIDE_B) {
             d[sl * pl] = bf16_pair(fr, fi);
           } else {  // rows 2n: [br, -bi] and 2n + 1: [bi, br]
-            d[sl * pl] = bf16_pair(fr, fi ^ 0x80000000u);
+            d[sl * pl] = bf16_pair(fr, digit_f32<S>(wn, sl));
             d[sl * pl + ld] = bf16_pair(fi, fr);
           }
         }

@@ -86,3 +86,59 @@ def test_operands_on_odd_doubles(prec):
     C = kc[1:].cpu().numpy().view(np.complex128).reshape(M, N)
     # 5 slices: K terms, each off by at most 16 2^(e_a+e_b-40) with entries below 2^3
     assert np.abs(C - A @ B).max() <= (1e-12 if prec == 0 else 2 * K * 16 * 2.0 ** (6 - 40))
+
+
+def _digits(x, e, S):
+    """The balanced base-256 digits q_0 .. q_{S-1} of x 2^(7-e), rounded to nearest, ties to
+    even, in Python integers."""
+    from fractions import Fraction
+    n = round(Fraction(float(x)) * Fraction(2) ** (7 - e + 8 * (S - 1)))
+    q = [0] * S
+    for s in range(S - 1, 0, -1):
+        hi = (n + 128) >> 8
+        q[s], n = n - (hi << 8), hi
+    q[0] = n
+    return q
+
+
+def _planes(rows, S):
+    e = np.frexp(np.abs(rows).max(axis=1))[1]
+    q = np.array([[_digits(x, int(ei), S) for x in r] for r, ei in zip(rows, e)], dtype=object)
+    return q, e
+
+
+@pytest.mark.parametrize("ties", [False])
+@pytest.mark.parametrize("S", [4, 5])
+@pytest.mark.parametrize("cplx,conj", [(False, False), (True, False), (True, True)])
+def test_split_product_bits(cplx, conj, S, ties):
+    """The split product bit for bit: exact integer sums of the digits' products of the first
+    S levels, rounded once.  Digits of -x are not the negated digits of x where one is -128;
+    `ties`: half of the entries lie halfway between two last digits."""
+    rng = np.random.default_rng([S, cplx, ties])
+    M, N, K = 40, 20, 48
+    def draw(shape):
+        top = 2 ** (7 + 8 * (S - 1))
+        n = rng.integers(-top + 1, top - 1, shape).astype(float)
+        n[0, :], n[:, 0] = 0.75 * top, 0.75 * top  # every row and column: exponent 0
+        f = 0.5 * rng.integers(0, 2, shape) if ties else rng.integers(0, 8, shape) / 8 + 1 / 16
+        return (n + f) * 2.0 ** (-7 - 8 * (S - 1))
+    A, B = draw((M, K)), draw((K, N))
+    if cplx:
+        A, B = A + 1j * draw((M, K)), B + 1j * draw((K, N))
+    C, _ = _run(1, S, A, B, False, False, False, conj)
+    b = B.conj() if conj else B
+    if cplx:
+        ra = np.stack([A.real, A.imag], axis=2).reshape(M, 2 * K)
+        rb = np.stack([np.stack([b.real, -b.imag], 1).reshape(2 * K, N),
+                       np.stack([b.imag, b.real], 1).reshape(2 * K, N)], 2).reshape(2 * K, 2 * N).T
+    else:
+        ra, rb = A, b.T
+    (qa, ea), (qb, eb) = _planes(ra, S), _planes(rb, S)
+    want = np.zeros((len(ra), len(rb)))
+    for i in range(len(ra)):
+        for j in range(len(rb)):
+            t = sum(int((qa[i, :, s] * qb[j, :, g - s]).sum()) << (8 * (S - 1 - g))
+                    for g in range(S) for s in range(g + 1))
+            want[i, j] = np.ldexp(float(t), int(ea[i] + eb[j]) - 14 - 8 * (S - 1))
+    got = np.stack([C.real, C.imag], axis=2).reshape(M, 2 * N) if cplx else C
+    assert np.array_equal(got, want)
