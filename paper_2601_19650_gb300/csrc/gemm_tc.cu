@@ -541,10 +541,11 @@ __device__ __forceinline__ int expo_bits(double x) {
 }
 
 // Balanced base-256 digits of t = x 2^(head-e) (|t| < 2^head): N = t 256^(S-1) rounded to the
-// nearest integer, then t = sum_s q_s 256^-s up to 0.5 256^-(S-1) with q_1 .. q_{S-1}
+// nearest integer (ties to even: of the 14 bits that 5 slices drop, all but the first are zero
+// in one entry of 2^14), then t = sum_s q_s 256^-s up to 0.5 256^-(S-1) with q_1 .. q_{S-1}
 // the balanced remainders of N by 256 (in [-128, 127]) and q_0 the remaining quotient
-// (|q_0| <= 128).  N is taken straight from the bit pattern of x (the mantissa plus half a
-// unit, shifted): integer operations only, since a scaling and an FP64-to-integer conversion
+// (|q_0| <= 128).  N is taken straight from the bit pattern of x (the mantissa plus what
+// rounds it, shifted): integer operations only, since a scaling and an FP64-to-integer conversion
 // per value would run on the narrow FP64 pipe of this part.
 // Returned is N + sum_{i<S-1} 128 256^i: its byte i is q_{S-1-i} + 128 for i < S-1, and its
 // bits from 8 (S-1) up are q_0.
@@ -563,7 +564,7 @@ __device__ __forceinline__ long long digit_word(double x, int e) {
   if (MIN_SH < 1 && sh <= 0)
     n = mant << -sh;
   else
-    n = sh < 64 ? (mant + (1ull << (sh - 1))) >> sh : 0ull;
+    n = sh < 64 ? (mant + ((1ull << (sh - 1)) - 1ull) + ((mant >> sh) & 1ull)) >> sh : 0ull;
   const long long N = (b >> 63) ? -(long long)n : (long long)n;
   return N + DIGIT_BIAS<S>;
 }

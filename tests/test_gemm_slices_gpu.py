@@ -107,7 +107,7 @@ def _planes(rows, S):
     return q, e
 
 
-@pytest.mark.parametrize("ties", [False])
+@pytest.mark.parametrize("ties", [False, True])
 @pytest.mark.parametrize("S", [4, 5])
 @pytest.mark.parametrize("cplx,conj", [(False, False), (True, False), (True, True)])
 def test_split_product_bits(cplx, conj, S, ties):
