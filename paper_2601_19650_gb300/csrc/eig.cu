@@ -530,7 +530,7 @@ __global__ void bisect32_kernel(const double* d, const double* e, int m, int kma
   float* dd = shf;
   float* e2 = shf + m;
   __shared__ int s_exp;
-  __shared__ float s_lo[32], s_hi[32];
+  __shared__ double s_lo[32], s_hi[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   if (threadIdx.x == 0) s_exp = 0;
   __syncthreads();
@@ -545,33 +545,35 @@ __global__ void bisect32_kernel(const double* d, const double* e, int m, int kma
   const double inv = __hiloint2double((2045 - E) << 20, 0), sc = __hiloint2double((E + 1) << 20, 0);
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
     dd[i] = (float)(d[i] * inv);
-    e2[i] = (i < m - 1) ? (float)(e[i] * inv) : 0.f;
+    const double ei = (i < m - 1) ? e[i] * inv : 0.0;
+    e2[i] = (float)(ei * ei);
   }
-  __syncthreads();
-  float lo = FLT_MAX, hi = -FLT_MAX;  // Gershgorin
+  // Gershgorin's bounds and the squares are formed in FP64 and rounded once: the estimates are
+  // points of the grid that the bounds span, to FP32 accuracy, and move with them
+  double glo = DBL_MAX, ghi = -DBL_MAX;
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    const float r = (i > 0 ? fabsf(e2[i - 1]) : 0.f) + fabsf(e2[i]);
-    lo = fminf(lo, dd[i] - r);
-    hi = fmaxf(hi, dd[i] + r);
+    double r = 0.0;
+    if (i > 0) r += fabs(e[i - 1] * inv);
+    if (i < m - 1) r += fabs(e[i] * inv);
+    glo = fmin(glo, d[i] * inv - r);
+    ghi = fmax(ghi, d[i] * inv + r);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, o));
+    ghi = fmax(ghi, __shfl_xor_sync(0xffffffffu, ghi, o));
   }
   if (lane == 0) {
-    s_lo[warp] = lo;
-    s_hi[warp] = hi;
+    s_lo[warp] = glo;
+    s_hi[warp] = ghi;
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < m; i += blockDim.x) e2[i] *= e2[i];
   for (int w = 0; w < nw; ++w) {
-    lo = fminf(lo, s_lo[w]);
-    hi = fmaxf(hi, s_hi[w]);
+    glo = fmin(glo, s_lo[w]);
+    ghi = fmax(ghi, s_hi[w]);
   }
-  const float span = fmaxf(fabsf(lo), fabsf(hi));
-  lo -= 1e-6f * span + FLT_MIN;
-  hi += 1e-6f * span + FLT_MIN;
+  const double span = fmax(fabs(glo), fabs(ghi));
+  float lo = (float)(glo - 1e-6 * span) - FLT_MIN, hi = (float)(ghi + 1e-6 * span) + FLT_MIN;
   __syncthreads();
   if (blockIdx.x == 0 && threadIdx.x == 0) *scale = sc;
   const int jj = blockIdx.x * nw + warp;  // descending index

@@ -75,3 +75,34 @@ def test_back_transformation_blocks(m, cplx):
     k = m // 2 + 1
     nb = int(4e6 / (m * m * k)) + 1
     _check(_random(m, cplx), kmax=k, nb=nb)
+
+
+@pytest.mark.parametrize("nb", [1, 3])
+@pytest.mark.parametrize("m", [2, 33, 64, 257])
+def test_estimates_bits(m, nb):
+    """The eigenvalue estimates beyond kmax are points of the FP32 bisection's grid between
+    Gershgorin's bounds in FP64: bit for bit on diagonal matrices, whose counts are exact."""
+    import torch
+
+    from paper_2601_19650_gb300 import _cbc as c
+    f = np.float32
+    dg = np.random.default_rng(m).standard_normal(m)
+    A = torch.from_numpy(np.stack([np.diag(dg)] * nb)).cuda()
+    lam = torch.zeros(nb, m, dtype=torch.float64, device="cuda")
+    U = torch.zeros(nb, m, 1, dtype=torch.float64, device="cuda")
+    c.cbc_heev(c.CBC_F64, m, 1, nb, A.data_ptr(), lam.data_ptr(), U.data_ptr(), False)
+    span = np.abs(dg).max()
+    d32, want = dg.astype(f), np.zeros(m)
+    for j in range(1, m):
+        lo, hi = f(dg.min() - 1e-6 * span), f(dg.max() + 1e-6 * span)
+        for _ in range(12):
+            step = (hi - lo) * np.arange(1, 33, dtype=f)
+            # fma(step, 1 / 33, lo): one rounding
+            x = (lo.astype(np.float64) + step.astype(np.float64) * np.float64(f(1) / f(33))).astype(f)
+            n = int(sum((d32 < v).sum() <= m - 1 - j for v in x))
+            lo, hi = (x[n - 1] if n else lo), (x[n] if n < 32 else hi)
+            if hi - lo <= f(2e-7) * max(abs(lo), abs(hi)):
+                break
+        want[j] = f(0.5) * (lo + hi)
+    for b in range(nb):
+        assert np.array_equal(lam[b, 1:].cpu().numpy(), want[1:])
