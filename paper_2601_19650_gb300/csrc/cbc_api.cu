@@ -116,6 +116,7 @@ static int build_network(Net* net, int kind, int n_nodes, const int32_t* parent,
   net->bond.assign(bond_dim, bond_dim + n_nodes);
   net->stream = static_cast<cudaStream_t>(stream);
   net->cplx = (dtype == CBC_C64 || dtype == CBC_C128);
+  net->wide = (dtype == CBC_F64 || dtype == CBC_C128);
   int roots = 0;
   for (int i = 0; i < n_nodes; ++i) {
     if (parent[i] < -1 || parent[i] >= n_nodes || parent[i] == i)

@@ -533,16 +533,18 @@ size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
 template <typename T>
 cudaError_t cholesky_lower(T* G, int m, int* status, void* bar, int num_sms, cudaStream_t s,
-                           int nb) {
+                           int nb, bool steady) {
   // the rows in the shared memory of one cluster per matrix: as many CTAs (and FP64 units) as
-  // the batch leaves idle, 4 rows each at least; where that is one, a kernel without a cluster
-  {
+  // the batch leaves idle, 4 rows each at least; where that is one, a kernel without a cluster.
+  // (`steady`: the column blocks below, one CTA per matrix from 8 matrices on.  A change of the
+  // order of these sums by 1e-16 has moved mixed results on 64-bit data by 2e-9.)
+  const size_t tri_bytes = (size_t)m * (m + 1) / 2 * sizeof(T);
+  if (!steady) {
     const void* kc = (const void*)chol_cluster_kernel<T>;
     cudaError_t err = allow_max_smem(kc);
     if (err != cudaSuccess) return err;
     int want = 1;
     while (want < 16 && want * 4 < m && 2 * want * nb <= num_sms) want *= 2;
-    const size_t tri_bytes = (size_t)m * (m + 1) / 2 * sizeof(T);
     if (want == 1 && nb > 1 && tri_bytes <= 200 * 1024) {
       err = allow_max_smem((const void*)chol1_kernel<T>);
       if (err != cudaSuccess) return err;
@@ -562,6 +564,13 @@ cudaError_t cholesky_lower(T* G, int m, int* status, void* bar, int num_sms, cud
       void* args[] = {&G, &m, &rows_cap, &nr_cap, &status};
       return launch_cluster(kc, P, nb * P, CHT, smem, args, s);
     }
+  }
+  if (steady && nb >= 8 && tri_bytes <= 200 * 1024) {
+    cudaError_t err = allow_max_smem((const void*)chol1_kernel<T>);
+    if (err != cudaSuccess) return err;
+    note_launches(CBC_K_CHOLQR, 1);
+    chol1_kernel<T><<<nb, TPB, tri_bytes, s>>>(G, m, status);
+    return cudaGetLastError();
   }
   // larger matrices: column blocks with the matrix in global memory, one cluster of up to 16
   // CTAs per matrix when it fits (concurrent with other streams' work), else a cooperative
@@ -712,8 +721,8 @@ cudaError_t trsm_lower_left(const T* C, T* S, int m, int n, int* status, void* b
   return cudaGetLastError();
 }
 
-template cudaError_t cholesky_lower<double>(double*, int, int*, void*, int, cudaStream_t, int);
-template cudaError_t cholesky_lower<zdbl>(zdbl*, int, int*, void*, int, cudaStream_t, int);
+template cudaError_t cholesky_lower<double>(double*, int, int*, void*, int, cudaStream_t, int, bool);
+template cudaError_t cholesky_lower<zdbl>(zdbl*, int, int*, void*, int, cudaStream_t, int, bool);
 template cudaError_t trsm_products<double>(const double*, double*, int, int, int*, void*,
                                            cudaStream_t, int);
 template cudaError_t trsm_products<zdbl>(const zdbl*, zdbl*, int, int, int*, void*, cudaStream_t,

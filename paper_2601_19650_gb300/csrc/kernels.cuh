@@ -121,12 +121,26 @@ cudaError_t tridiag_cluster(const T* A, int m, double* d, double* e, T* tau, T* 
                             size_t wb, int nb, const TriClusterShape& sh, bool df,
                             cudaStream_t s);
 
+// The same outputs with a fixed order of all sums, for mixed calls on 64-bit data (eig_steady.cu
+// says why); workspace: nb * eig_workspace_bytes_steady(m, kmax).
+size_t eig_workspace_bytes_steady(int m, int kmax, bool cplx);
+template <typename T>
+cudaError_t heev_top_steady(T* A, int m, int kmax, double* lam, T* U, void* work, int* status,
+                            int num_sms, cudaStream_t s, int nb, bool prefer_cluster, bool df);
+template <typename T>
+int tridiag_cluster_size_steady(int m, bool df);
+template <typename T>
+cudaError_t tridiag_cluster_steady(const T* A, int m, double* d, double* e, T* tau, T* V,
+                                   int64_t a_bs, size_t wb, int nb, int P, bool df,
+                                   cudaStream_t s);
+
 // ---- Cholesky QR (FP64) ------------------------------------------------------------
 // Q = C^{-1} S with G = S S^H = C C^H, S: m x n (m <= n), row-major, in place on S.
-// nb problems: G, C m*m and S m*n elements apart; `bar` holds nb GridBarriers.
+// nb problems: G, C m*m and S m*n elements apart; `bar` holds nb GridBarriers.  `steady`: a fixed
+// order of the sums, for mixed calls on 64-bit data.
 template <typename T>
 cudaError_t cholesky_lower(T* G, int m, int* status, void* bar, int num_sms, cudaStream_t s,
-                           int nb = 1);
+                           int nb = 1, bool steady = false);
 // dfbuf: NULL for the FP64 solve; else room for trsm_df_bytes(m, nb) bytes, and the solve
 // runs in double-float arithmetic (the mixed path)
 template <typename T>

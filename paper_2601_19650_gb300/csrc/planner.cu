@@ -121,11 +121,26 @@ T host_one() {
 struct Prec {
   bool mixed = false;
   bool cholqr_f64 = false;  // CholeskyQR2's Gram in FP64 even on the mixed path
+  bool steady = false;      // mixed on 64-bit data: a fixed order of all sums (eig_steady.cu)
   int s_fwd = 5, s_bwd = 4;
   Arena* ar = nullptr;
   int* status = nullptr;
   int nb = 1;
 };
+
+// the eigensolver of a call's precision, and its workspace per matrix
+template <typename T>
+size_t eig_bytes(const Prec& pr, int m, int kmax) {
+  return pr.steady ? eig_workspace_bytes_steady(m, kmax, ops<T>::cplx)
+                   : eig_workspace_bytes(m, kmax, ops<T>::cplx);
+}
+template <typename T>
+cudaError_t heev(const Prec& pr, T* A, int m, int kmax, double* lam, T* U, void* work, void* bt,
+                 int* status, cudaStream_t s, int nb, bool concurrent, bool df) {
+  if (pr.steady)
+    return heev_top_steady<T>(A, m, kmax, lam, U, work, status, num_sms(), s, nb, concurrent, df);
+  return heev_top<T>(A, m, kmax, lam, U, work, status, num_sms(), s, nb, concurrent, df, bt);
+}
 
 template <typename T>
 cudaError_t tgemm(const Prec& pr, bool fwd, bool gram, int M, int N, int K, const T* A,
@@ -221,8 +236,8 @@ int refine_level2(Arena& ar, const Prec& pr, const T* M, int m, int n, int kmax,
   T* C = ar.get<T>((size_t)std::max(1, jlo) * k2);
   T* P2 = ar.get<T>((size_t)g * k2);
   T* W2c = rows ? nullptr : ar.get<T>((size_t)m * k2);
-  char* work = ar.get<char>(eig_workspace_bytes(g, k2, ops<T>::cplx));
-  const size_t btb = eig_bt_bytes(g, k2, ops<T>::cplx, 1);
+  char* work = ar.get<char>(eig_bytes<T>(pr, g, k2));
+  const size_t btb = pr.steady ? 0 : eig_bt_bytes(g, k2, ops<T>::cplx, 1);
   void* bt = btb > 0 ? ar.try_get(btb) : nullptr;
   double* dv = ar.get<double>(k2 + 4);
   CKA(P); CKA(R); CKA(K2); CKA(lam2); CKA(U2); CKA(C); CKA(P2); CKA(work); CKA(dv);
@@ -242,8 +257,7 @@ int refine_level2(Arena& ar, const Prec& pr, const T* M, int m, int n, int kmax,
   else        // R^H R
     CK(tgemm<T>(pr, true, true, n, n, m, R, View::transposed(n), true, R, View::rowmajor(n),
                 false, K2, View::rowmajor(n), s));
-  CK(heev_top<T>(K2, g, k2, lam2, U2, work, sc.status, num_sms(), s, 1, o.concurrent, false,
-                 bt));
+  CK(heev<T>(pr, K2, g, k2, lam2, U2, work, bt, sc.status, s, 1, o.concurrent, false));
   // U2 <- U2 - U1r (U1r^H U2)
   CK(tgemm<T>(pr, true, false, jlo, k2, g, U1, View::transposed(kmax), true, U2,
               View::rowmajor(k2), false, C, View::rowmajor(k2), s));
@@ -312,8 +326,8 @@ int compress_rows(Arena& ar, const Prec& pr, const T* M, int m, int n, int64_t m
   T* K = ar.get<T>((size_t)nb * g * g);
   double* lam = ar.get<double>((size_t)nb * g);
   T* U = ar.get<T>((size_t)nb * g * kmax);
-  char* work = ar.get<char>(nb * eig_workspace_bytes(g, kmax, ops<T>::cplx));
-  const size_t btb = eig_bt_bytes(g, kmax, ops<T>::cplx, nb);
+  char* work = ar.get<char>(nb * eig_bytes<T>(pr, g, kmax));
+  const size_t btb = pr.steady ? 0 : eig_bt_bytes(g, kmax, ops<T>::cplx, nb);
   void* bt = btb > 0 ? ar.try_get(btb) : nullptr;
   double* dv = ar.get<double>((size_t)nb * (kmax + 2));  // w [nb][kmax], beyond [nb], total [nb]
   CKA(K); CKA(lam); CKA(U); CKA(work); CKA(dv);
@@ -331,8 +345,7 @@ int compress_rows(Arena& ar, const Prec& pr, const T* M, int m, int n, int64_t m
   // ||M||_F^2, the weight of the cut: the trace of the Gram (g reads instead of m n)
   CK(trace_real<T>(K, g, (int64_t)g * g, total_dev, s, nb));
   // every candidate; the mixed path reduces batches to tridiagonal form in double-float
-  CK(heev_top<T>(K, g, kmax, lam, U, work, sc.status, num_sms(), s, nb, o.concurrent, pr.mixed,
-                 bt));
+  CK(heev<T>(pr, K, g, kmax, lam, U, work, bt, sc.status, s, nb, o.concurrent, pr.mixed));
   const int64_t ubs = (int64_t)g * kmax;
   T* W = nullptr;
   int64_t wbs;
@@ -472,7 +485,7 @@ int lq_rows_inplace(Arena& ar, const Prec& pr, T* S, int m, int n, const Scalars
   // large solves by products; else the mixed path solves in double-float arithmetic (FP32 pipes)
   void* dfb = nullptr;
   const bool df = pr.mixed && !pr.cholqr_f64;
-  const size_t tb = trsm_products_bytes(m, n, ops<T>::cplx, nb, df);
+  const size_t tb = pr.steady ? 0 : trsm_products_bytes(m, n, ops<T>::cplx, nb, df);
   void* tw = tb > 0 ? ar.try_get(tb) : nullptr;
   if (!tw && df) {
     dfb = ar.get<char>(trsm_df_bytes(m, nb, ops<T>::cplx));
@@ -498,7 +511,7 @@ int lq_rows_inplace(Arena& ar, const Prec& pr, T* S, int m, int n, const Scalars
     }
     KTimer t(CBC_K_CHOLQR, s, 0,
              nb * (ops<T>::cplx ? 4.0 : 1.0) * ((double)m * m * m / 3.0 + (double)m * m * n));
-    CK(cholesky_lower<T>(G, m, sc.status, bar, num_sms(), s, nb));
+    CK(cholesky_lower<T>(G, m, sc.status, bar, num_sms(), s, nb, pr.steady));
     if (tw)
       CK(trsm_products<T>(G, S, m, n, sc.status, tw, s, nb));
     else
@@ -541,6 +554,7 @@ int run_tt_group(const std::vector<const Net*>& sts, const std::vector<const Net
   Scalars sc{d_int, d_dbl, d_dbl + nb, d_dbl + 2 * nb};
   Prec pr;
   pr.mixed = (o.precision == CBC_PREC_MIXED);
+  for (int b = 0; b < nb; ++b) pr.steady |= pr.mixed && (sts[b]->wide || opv[b]->wide);
   pr.cholqr_f64 = o.cholqr_f64;
   pr.s_fwd = o.slices_fwd;
   pr.s_bwd = o.slices_bwd;
@@ -653,6 +667,7 @@ int run_tt_group(const std::vector<const Net*>& sts, const std::vector<const Net
     out->bond.assign(L, 1);
     out->children = sts[b]->children;
     out->cplx = sts[b]->cplx;
+    out->wide = sts[b]->wide || opv[b]->wide;
     out->stream = (nb == 1) ? s : sts[b]->stream;
     out->data.assign(L, nullptr);
     out->numel.assign(L, 0);
@@ -824,6 +839,7 @@ int run_tt_direct(const Net& st, const Net& op, int64_t max_bond, double tol, co
   Scalars sc{d_int, d_dbl, d_dbl + 1, d_dbl + 2};
   Prec pr;
   pr.mixed = (o.precision == CBC_PREC_MIXED);
+  pr.steady = pr.mixed && (st.wide || op.wide);
   pr.cholqr_f64 = o.cholqr_f64;
   pr.s_fwd = o.slices_fwd;
   pr.s_bwd = o.slices_bwd;
@@ -840,6 +856,7 @@ int run_tt_direct(const Net& st, const Net& op, int64_t max_bond, double tol, co
   out->bond.assign(L, 1);
   out->children = st.children;
   out->cplx = st.cplx;
+  out->wide = st.wide || op.wide;
   out->stream = s;
   out->data.assign(L, nullptr);
   out->numel.assign(L, 0);
@@ -1118,6 +1135,7 @@ int run_tree(const Net& st, const Net& op, int64_t max_bond, double tol, const O
   Scalars sc{d_int, d_dbl + 1, d_dbl, d_dbl + 1 + n};
   Prec pr;
   pr.mixed = (o.precision == CBC_PREC_MIXED);
+  pr.steady = pr.mixed && (st.wide || op.wide);
   pr.cholqr_f64 = o.cholqr_f64;
   pr.s_fwd = o.slices_fwd;
   pr.s_bwd = o.slices_bwd;
@@ -1380,6 +1398,7 @@ int run_tree(const Net& st, const Net& op, int64_t max_bond, double tol, const O
   out->bond.assign(n, 1);
   out->children = st.children;
   out->cplx = st.cplx;
+  out->wide = st.wide || op.wide;
   out->stream = s;
   out->data.assign(n, nullptr);
   out->numel.assign(n, 0);

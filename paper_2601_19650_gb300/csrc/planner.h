@@ -20,6 +20,7 @@ struct Net {
   std::vector<int64_t> phys, bond;
   std::vector<std::vector<int>> children;
   bool cplx = false;
+  bool wide = false;  // created from 64-bit data, or a result of such networks
   std::vector<void*> data;
   std::vector<int64_t> numel;
   void* block = nullptr;  // when set, data[i] point into this one allocation
