@@ -62,9 +62,9 @@ FP64_NOMINAL_TFLOPS = 1.25   # GB300 FP64, nominal: the fallback when the DGEMM 
 # workload; each entry names the summary under profiles/ it comes from.  A class whose
 # kernel changed after its capture has no entry (traffic null).
 PROFILED_TRAFFIC = {}
-KERNEL_OF_CLASS = {"tridiag": "tridiag_cluster_kernel", "eig": "bisect32/invit/rank/backtransform",
-                   "gemm_tc": "gemm_tc_kernel (+ operand slicing)", "cholqr": "chol_kernel + trsm",
-                   "gemm_f64": "gemm_f64_kernel"}
+KERNEL_OF_CLASS = {"tridiag": "tridiag_cluster_kernel", "eig": "bisect32/invit/backtransform",
+                   "gemm_tc": "gemm_tc_kernel (+ operand slicing)", "cholqr": "chol_cluster_kernel + trsm",
+                   "gemm_f64": "gemm_tc_kernel<8> / gemm_f64_kernel"}
 
 
 def instance_seeds(rank: int, B: int):
