@@ -643,14 +643,16 @@ struct InvArgs {
 constexpr int kInvMax = 16;  // members per warp: two lanes each
 
 // The state of one warp: member t on lanes 2t (rows 0, 1, ... of T) and 2t + 1 (rows m-1,
-// m-2, ...).  Row p of a half is element [p * ld + lane] of the arrays.
+// m-2, ...).  Row p of a half is element [p * ld + lane] of the arrays.  Lanes without a member
+// (act false, n = 1: no rows to walk) take part in the shuffles and touch no shared column:
+// the solves work in place, so only the lane that owns a column may read or write it.
 struct Inv {
   double *f, *r, *u1, *u2, *b;  // multipliers (last bit: rows swapped), 1/pivot, U's
                                 // superdiagonals / pivot, the vector
   const double *d, *e;
   double inv;                   // factor from d, e to scaled units (1 if they are scaled)
   int m, h, n, ld, lane;        // h rows in the upper half, n in this lane's
-  bool top, swap;
+  bool act, top, swap;
   double r1, f1, a2, r2;        // the factored 2 x 2 system in the middle
 
   __device__ double D(int p) const { return d[top ? p : m - 1 - p] * inv; }
@@ -698,7 +700,7 @@ struct Inv {
   }
 
   __device__ void solve() {
-    double carry = b[lane];
+    double carry = act ? b[lane] : 0.0;
     int p = 0;
     for (; p + 4 <= n - 1; p += 4) {  // four rows' operands in flight
       double fl[4], nx[4];
@@ -728,7 +730,7 @@ struct Inv {
     const double xB = fma(-f1, c1, c2) * r2;
     const double xT = fma(-a2, xB, c1) * r1;
     double x1 = top ? xT : xB, x2 = top ? xB : xT;
-    b[(size_t)(n - 1) * ld + lane] = x1;
+    if (act) b[(size_t)(n - 1) * ld + lane] = x1;
     p = n - 2;
     for (; p >= 3; p -= 4) {
       double y[4], v1[4], v2[4];
@@ -869,9 +871,10 @@ __global__ void __launch_bounds__(32) invit_kernel(InvArgs a) {
   w.m = m;
   w.h = (m + 1) / 2;
   w.ld = 2 * per + (per >= 8 ? 1 : 0);  // odd rows where the whole warp walks a column
-  w.lane = ln < 2 * per ? ln : 2 * per - 2 + (ln & 1);  // idle lanes shadow the last member's
+  w.act = ln < 2 * per;
+  w.lane = w.act ? ln : (ln & 1);
   w.top = !(w.lane & 1);
-  w.n = w.top ? w.h : m - w.h;
+  w.n = !w.act ? 1 : (w.top ? w.h : m - w.h);
   const size_t sz = (size_t)w.h * w.ld;
   w.f = shd;
   w.r = w.f + sz;
