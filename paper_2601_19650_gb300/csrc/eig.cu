@@ -1124,10 +1124,12 @@ __global__ void widen_x_kernel(const double* X, int64_t n, T* U, size_t wb) {
     U[i] = ops<T>::make(X[i], 0.0);
 }
 
-// NaN into U when *flag is set (an Inf or NaN among V, T or X, which the slices don't carry)
+// NaN into U (n elements) of every matrix blockIdx.y whose flag is set (an Inf or NaN among its
+// V, T or X, which the slices don't carry)
 template <typename T>
 __global__ void poison_kernel(const int* flag, T* U, int64_t n) {
-  if (!*flag) return;
+  if (!flag[blockIdx.y]) return;
+  U += blockIdx.y * n;
   const double nan = __longlong_as_double(0x7ff8000000000000LL);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
@@ -1249,7 +1251,7 @@ size_t eig_bt_bytes(int m, int kmax, bool cplx, int nb) {
   if (!bt_products(m, kmax, nb)) return 0;
   const size_t ts = cplx ? sizeof(zdbl) : sizeof(double);
   const size_t nblk = (m + BT_NB - 1) / BT_NB;
-  return 256 + align256(2 * nb * nblk * BT_NB * BT_NB * ts) +
+  return align256(sizeof(int) * nb) + align256(2 * nb * nblk * BT_NB * BT_NB * ts) +
          align256(nb * nblk * BT_HALF * BT_HALF * ts) + align256((size_t)nb * BT_NB * kmax * ts) +
          bt_gemm_bytes(m, kmax, cplx, nb);
 }
@@ -1268,7 +1270,7 @@ static cudaError_t backtransform_products(const T* V, const T* tau, const double
     w += align256(bytes);
     return p;
   };
-  int* flag = reinterpret_cast<int*>(take(4));
+  int* flag = reinterpret_cast<int*>(take(sizeof(int) * nb));  // one per matrix
   T* G = reinterpret_cast<T*>(take(2 * nb * tbs * sizeof(T)));
   T* Tm = G + nb * tbs;
   T* tmp = reinterpret_cast<T*>(take(sizeof(T) * nb * nblk * BT_HALF * BT_HALF));
@@ -1279,9 +1281,11 @@ static cudaError_t backtransform_products(const T* V, const T* tau, const double
   TcWide sub = opt;
   sub.acc = -1;
   cudaError_t e = cudaMemsetAsync(bt, 0, (char*)(G + 2 * nb * tbs) - (char*)bt, s);  // flag, G, T
+  // (n problems: one per matrix, all blocks of all matrices, or blocks of a lone one)
   auto mul = [&](int M, int N, int K, const T* A, View va, int64_t abs, bool ca, const T* B,
-                 View vb, int64_t bbs, T* C, int64_t ldc, int64_t cbs, int n, const TcWide& o) {
+                 View vb, int64_t bbs, T* C, int64_t ldc, int64_t cbs, int n, TcWide o) {
     if (e != cudaSuccess) return;
+    o.per = n / nb;
     va.bs = abs;
     vb.bs = bbs;
     e = gemm_tc<T>(M, N, K, A, va, ca, B, vb, false, C, View::rowmajor(ldc, cbs), 8, ws, status, s,
@@ -1332,8 +1336,8 @@ static cudaError_t backtransform_products(const T* V, const T* tau, const double
         View::rowmajor(kmax), (int64_t)BT_NB * kmax, Ub, kmax, n, nb, sub);
   }
   if (e != cudaSuccess) return e;
-  poison_kernel<T><<<(unsigned)std::min<int64_t>(256, (n * nb + 255) / 256), 256, 0, s>>>(
-      flag, U, n * nb);
+  poison_kernel<T><<<dim3((unsigned)std::min<int64_t>(256, (n + 255) / 256), nb), 256, 0, s>>>(
+      flag, U, n);
   return cudaGetLastError();
 }
 

@@ -607,8 +607,8 @@ struct PackArgs {
   int K, K2p, tiles_per_cta, keep;
   size_t plane_a, plane_b;
   int* status;
-  int* wide;           // 8 slices: set when an operand holds Inf or NaN or a row spans more
-  int range;           // than 2^range
+  int* wide;           // 8 slices: word (problem / per) is set when an operand holds Inf or NaN
+  int per, range;      // or a row spans more than 2^range
 };
 
 // one element to shared memory, zero if !in; complex ones in one copy where the operand is
@@ -722,7 +722,7 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
         if constexpr (S > 5) lo = min(lo, cluster.map_shared_rank(s_min, q)[tid]);
       }
     if constexpr (S > 5) {
-      if (b >= 0x40000000 || (lo < 2000 && b - lo > g.range)) *g.wide = 1;
+      if (b >= 0x40000000 || (lo < 2000 && b - lo > g.range)) g.wide[blockIdx.z / g.per] = 1;
     } else if (b >= 0x40000000) {
       set_status(g.status, CBC_ERR_NUMERICAL);  // Inf or NaN in the row
     }
@@ -1041,6 +1041,7 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
   pk.plane_b = b * g.N2p * g.K2p;
   pk.status = status;
   pk.wide = opt.wide;
+  pk.per = opt.per;
   pk.range = opt.range;
   cudaError_t pe = pack_operands<T>(pk, S, nb, s);
   if (pe != cudaSuccess) return pe;
@@ -1156,7 +1157,7 @@ cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& 
   cudaError_t e = cudaMemsetAsync(wide, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   e = gemm_tc<T>(M, N, K, A, va, conjA, B, vb, conjB, C, vc, 8, static_cast<char*>(ws) + 256,
-                 status, s, nb, TcWide{wide, SPLIT_RANGE, true});
+                 status, s, nb, TcWide{wide, 0x7fffffff, SPLIT_RANGE, true});
   if (e != cudaSuccess) return e;
   return gemm_f64<T>(M, N, K, nb, A, va, conjA, B, vb, conjB, C, vc, s, wide);
 }

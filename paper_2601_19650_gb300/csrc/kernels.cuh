@@ -75,12 +75,13 @@ cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& 
 // The same product on the tensor cores with S bf16 slices per operand (gemm_tc.cu);
 // `ws` must hold gemm_tc_workspace_bytes(M, N, K, cplx, S, nb) bytes.  nb problems of
 // one shape, their operands va.bs / vb.bs / vc.bs elements apart, in one launch.
-// S = 8 (62 bits of every entry, relative to its row's maximum) needs TcWide::wide, a device
-// word that is set when an operand holds Inf or NaN or one of its rows spans more than
-// 2^range; `skip`: then C is left alone.  acc = 1 or -1: base + A B or base - A B into C, with
+// S = 8 (62 bits of every entry, relative to its row's maximum) needs TcWide::wide, device
+// words of which number p / per is set when an operand of problem p holds Inf or NaN or one of
+// its rows spans more than 2^range; `skip` (one word): then C is left alone.  acc = 1 or -1: base + A B or base - A B into C, with
 // base (NULL: C itself) laid out as C but for its problems, base_bs elements apart.
 struct TcWide {
   int* wide = nullptr;
+  int per = 0x7fffffff;
   int range = 1 << 20;
   bool skip = false;
   int acc = 0;
