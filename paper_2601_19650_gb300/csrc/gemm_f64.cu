@@ -26,7 +26,7 @@ struct GemmArgs {
   View vb;
   T* C;
   View vc;
-  const int* cond;  // not NULL: run only if *cond is set
+  const int* cond;  // not NULL: only the problems whose word is set
   int tiles_n, tiles_m, total;  // tiles of one (problem, split); of the launch
 };
 
@@ -38,13 +38,13 @@ __global__ void __launch_bounds__(NT) gemm_f64_kernel(GemmArgs<T> g) {
   __shared__ int64_t a_row[BM];
   __shared__ int64_t b_col[BN];
 
-  if (g.cond && !*g.cond) return;
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
   for (int tile = blockIdx.x; tile < g.total; tile += gridDim.x) {
     const int bn = tile % g.tiles_n * BN, bm = tile / g.tiles_n % g.tiles_m * BM;
     const int z = tile / (g.tiles_n * g.tiles_m);
     const int batch = z / g.splits;
+    if (g.cond && !g.cond[batch]) continue;
     const int split = z % g.splits;
     const int kbeg = split * g.kchunk;
     const int kend = min(g.K, kbeg + g.kchunk);

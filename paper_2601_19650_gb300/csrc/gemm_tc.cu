@@ -204,7 +204,7 @@ struct TcArgs {
   char* C;               // FP64 output (double or zdbl) through the view
   View vc;               // vc.bs: elements between the outputs of consecutive problems
   int* status;
-  const int* skip;       // not NULL: nothing runs when *skip is set (gemm_f64_split)
+  const int* skip;       // not NULL: nothing runs for problem p when skip[p] is set (gemm_f64_split)
   int acc;               // 1 or -1: base + A B or base - A B instead of A B
   const char* base;      // rows and columns as C's (C itself when it is split along K)
   int64_t base_shift;    // base's bytes from problem to problem less C's
@@ -268,7 +268,6 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
   constexpr uint32_t TMEM_COLS = 512;
   static_assert(2 * S * BN <= 512, "TMEM budget");  // hence S BN <= 256, the widest MMA
   static_assert(BN % 16 == 0, "MMA width");
-  if (a.skip && *a.skip) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
@@ -296,6 +295,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
     q.prob = z / a.splits;
     q.a_begin = (z % a.splits) * a.atoms_per_split;
     q.n_atoms = max(0, min(a.atoms_total, q.a_begin + a.atoms_per_split) - q.a_begin);
+    if (a.skip && a.skip[q.prob]) q.n_atoms = 0;  // (no role has anything to do in the tile)
     q.n_chunks = (q.n_atoms + a.atoms_per_chunk - 1) / a.atoms_per_chunk;
     return q;
   };
@@ -1140,12 +1140,12 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
 // products are summed exactly, so the only rounding is the one to 53 bits at the end (one
 // more per K split): on rows that span fewer powers of two than SPLIT_RANGE the error is
 // below that of an FP64 sum.  Operands outside that are found while they are cut; then the
-// tensor-core kernel returns at once and the SIMT kernel behind it does the product.
+// tensor-core kernel leaves their problem out and the SIMT kernel behind it does it.
 // Relative error against 80-bit sums, Gaussian entries: 4e-17 to 2e-16 where the SIMT kernel
 // has 1e-16 (K = 16) to 1e-15 (K = 1000).
 size_t gemm_f64_split_bytes(int M, int N, int K, bool cplx, int nb) {
   if (K < (cplx ? SPLIT_MIN_K_CPLX : SPLIT_MIN_K_REAL)) return 0;
-  const size_t b = gemm_tc_workspace_bytes(M, N, K, cplx, 8, nb) + 256;
+  const size_t b = gemm_tc_workspace_bytes(M, N, K, cplx, 8, nb) + tc::a256(sizeof(int) * nb);
   return b <= SPLIT_MAX_BYTES ? b : 0;
 }
 
@@ -1153,11 +1153,12 @@ template <typename T>
 cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& va, bool conjA,
                            const T* B, const View& vb, bool conjB, T* C, const View& vc, void* ws,
                            int* status, cudaStream_t s) {
-  int* wide = static_cast<int*>(ws);
-  cudaError_t e = cudaMemsetAsync(wide, 0, sizeof(int), s);
+  int* wide = static_cast<int*>(ws);  // one word per problem
+  const size_t wb = tc::a256(sizeof(int) * nb);
+  cudaError_t e = cudaMemsetAsync(wide, 0, wb, s);
   if (e != cudaSuccess) return e;
-  e = gemm_tc<T>(M, N, K, A, va, conjA, B, vb, conjB, C, vc, 8, static_cast<char*>(ws) + 256,
-                 status, s, nb, TcWide{wide, 0x7fffffff, SPLIT_RANGE, true});
+  e = gemm_tc<T>(M, N, K, A, va, conjA, B, vb, conjB, C, vc, 8, static_cast<char*>(ws) + wb,
+                 status, s, nb, TcWide{wide, 1, SPLIT_RANGE, true});
   if (e != cudaSuccess) return e;
   return gemm_f64<T>(M, N, K, nb, A, va, conjA, B, vb, conjB, C, vc, s, wide);
 }

@@ -61,7 +61,7 @@ template <typename T>
 cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va, bool conjA,
                      const T* B, const View& vb, bool conjB, T* C, const View& vc,
                      cudaStream_t s, const int* cond = nullptr);
-// (cond: a device word; not NULL: the product runs only if it is set.)
+// (cond: a device word per problem; not NULL: only the problems whose word is set.)
 
 // The FP64 product as 8 bf16 slices per operand on the tensor cores, with an error no larger
 // than gemm_f64's (gemm_tc.cu).  gemm_f64_split_bytes gives the bytes it needs at `ws`, or 0
@@ -77,7 +77,7 @@ cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& 
 // one shape, their operands va.bs / vb.bs / vc.bs elements apart, in one launch.
 // S = 8 (62 bits of every entry, relative to its row's maximum) needs TcWide::wide, device
 // words of which number p / per is set when an operand of problem p holds Inf or NaN or one of
-// its rows spans more than 2^range; `skip` (one word): then C is left alone.  acc = 1 or -1: base + A B or base - A B into C, with
+// its rows spans more than 2^range; `skip` (per = 1): then the problem's C is left alone.  acc = 1 or -1: base + A B or base - A B into C, with
 // base (NULL: C itself) laid out as C but for its problems, base_bs elements apart.
 struct TcWide {
   int* wide = nullptr;
