@@ -1,6 +1,6 @@
 // FP64 SIMT strided GEMM: the products of the plain-FP64 CBC path that the tensor cores do
-// not take (gemm_f64_split in gemm_tc.cu): short K, operands of a very wide range or with
-// Inf or NaN, and callers without room for slices.
+// not take (gemm_f64_split in gemm_tc.cu): short K, operands that split_guard.cuh turns down,
+// and callers without room for slices.
 //
 // It works on leg views of the node tensors (kernels.cuh: View).  On GB300 the FP64 pipe delivers
 // about 2 DFMA per clock per SM, so this kernel is FP64-throughput bound by design: a
@@ -11,6 +11,7 @@
 
 #include "kernels.cuh"
 #include "planner.h"
+#include "split_guard.cuh"
 
 namespace cbc {
 namespace {
@@ -26,7 +27,7 @@ struct GemmArgs {
   View vb;
   T* C;
   View vc;
-  const int* cond;  // not NULL: only the problems whose word is set
+  const int* guard;  // not NULL: only the problems that the split turns down
   int tiles_n, tiles_m, total;  // tiles of one (problem, split); of the launch
 };
 
@@ -44,7 +45,7 @@ __global__ void __launch_bounds__(NT) gemm_f64_kernel(GemmArgs<T> g) {
     const int bn = tile % g.tiles_n * BN, bm = tile / g.tiles_n % g.tiles_m * BM;
     const int z = tile / (g.tiles_n * g.tiles_m);
     const int batch = z / g.splits;
-    if (g.cond && !g.cond[batch]) continue;
+    if (g.guard && split_holds(g.guard + batch * GUARD_WORDS, O::cplx ? 2 * g.K : g.K)) continue;
     const int split = z % g.splits;
     const int kbeg = split * g.kchunk;
     const int kend = min(g.K, kbeg + g.kchunk);
@@ -154,7 +155,7 @@ int g_num_sms = 0;
 template <typename T>
 cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va, bool conjA,
                      const T* B, const View& vb, bool conjB, T* C, const View& vc,
-                     cudaStream_t s, const int* cond) {
+                     cudaStream_t s, const int* guard) {
   if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
   if (g_num_sms == 0) {
     int dev = 0;
@@ -166,7 +167,7 @@ cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va,
   int ksteps = (K + BK - 1) / BK;
   int splits = 1;
   int target = 2 * g_num_sms;
-  if (!cond && tiles < target && ksteps >= 16) {
+  if (!guard && tiles < target && ksteps >= 16) {
     splits = (target + tiles - 1) / tiles;
     splits = min(splits, ksteps / 8);
     splits = max(splits, 1);
@@ -178,10 +179,10 @@ cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va,
     zero_view_kernel<T><<<256, 256, 0, s>>>(C, vc, M, N, batch);
     return cudaGetLastError();
   }
-  GemmArgs<T> g{M,  N, K,  splits, kchunk, A, va, B, vb, C, vc, cond,
+  GemmArgs<T> g{M,  N, K,  splits, kchunk, A, va, B, vb, C, vc, guard,
                 (N + BN - 1) / BN, (M + BM - 1) / BM, tiles * splits};
-  // a product that usually does not run (cond) is launched as one resident wave
-  const int grid = cond ? std::min(g.total, target) : g.total;
+  // a product that usually does not run (guard) is launched as one resident wave
+  const int grid = guard ? std::min(g.total, target) : g.total;
   note_launches(CBC_K_GEMM_F64, splits > 1 ? 2 : 1);
   if (splits > 1) {
     int zb = (int)std::min<int64_t>(4096, ((int64_t)M * N * batch + 255) / 256);

@@ -47,6 +47,7 @@
 
 #include "kernels.cuh"
 #include "planner.h"
+#include "split_guard.cuh"
 
 namespace cbc {
 namespace tc {
@@ -204,7 +205,8 @@ struct TcArgs {
   char* C;               // FP64 output (double or zdbl) through the view
   View vc;               // vc.bs: elements between the outputs of consecutive problems
   int* status;
-  const int* skip;       // not NULL: nothing runs for problem p when skip[p] is set (gemm_f64_split)
+  const int* guard;      // not NULL: nothing runs for problems that it turns down (gemm_f64_split)
+  int guard_k;           // terms of the real sums
   int acc;               // 1 or -1: base + A B or base - A B instead of A B
   const char* base;      // rows and columns as C's (C itself when it is split along K)
   int64_t base_shift;    // base's bytes from problem to problem less C's
@@ -286,6 +288,8 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
   struct Tile {
     int m0, n0, prob, a_begin, n_atoms, n_chunks;
   };
+  int seen = -1;  // the last problem whose guard was looked at
+  bool holds = true;
   auto tile_of = [&](int t) {
     Tile q;
     const int mt = t % a.tiles_m, r = t / a.tiles_m;
@@ -295,7 +299,11 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
     q.prob = z / a.splits;
     q.a_begin = (z % a.splits) * a.atoms_per_split;
     q.n_atoms = max(0, min(a.atoms_total, q.a_begin + a.atoms_per_split) - q.a_begin);
-    if (a.skip && a.skip[q.prob]) q.n_atoms = 0;  // (no role has anything to do in the tile)
+    if (a.guard && q.prob != seen) {
+      seen = q.prob;
+      holds = split_holds(a.guard + (int64_t)q.prob * GUARD_WORDS, a.guard_k);
+    }
+    if (!holds) q.n_atoms = 0;  // (no role has anything to do in the tile)
     q.n_chunks = (q.n_atoms + a.atoms_per_chunk - 1) / a.atoms_per_chunk;
     return q;
   };
@@ -591,6 +599,21 @@ __device__ __forceinline__ uint32_t bf16_pair(uint32_t flo, uint32_t fhi) {
   return __byte_perm(flo, fhi, 0x7632);
 }
 
+// Adds to cnt[t - 2] how many of the warp's entries x0, x1 are below 2^(e-t), t = 2 .. 8 (at most
+// 64: eight bits each; a subnormal entry counts as below all).
+__device__ __forceinline__ void count_levels(double x0, double x1, int e, int* cnt) {
+  auto below = [&](double x) {
+    const int f = ((unsigned)__double2hiint(x) >> 20) & 0x7ff;
+    const int n = f ? min(max(e + 1021 - f, 0), GUARD_LEVELS) : GUARD_LEVELS;  // levels above |x|
+    return 0x0101010101010101ull & ((1ull << (8 * n)) - 1ull);
+  };
+  const unsigned long long w = below(x0) + below(x1);
+  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)w);
+  const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(w >> 32));
+  const int lane = threadIdx.x & 31;
+  if (lane < GUARD_LEVELS) cnt[lane] += ((lane < 4 ? lo : hi) >> (8 * (lane & 3))) & 255u;
+}
+
 template <typename T>
 struct PackSide {
   const T* src;
@@ -607,8 +630,9 @@ struct PackArgs {
   int K, K2p, tiles_per_cta, keep;
   size_t plane_a, plane_b;
   int* status;
-  int* wide;           // 8 slices: word (problem / per) is set when an operand holds Inf or NaN
-  int per, range;      // or a row spans more than 2^range
+  int* wide;           // 8 slices: word (problem / per) is set when an operand holds Inf or NaN,
+  int per;
+  int* guard;          // or the words of split_guard.cuh are filled in
 };
 
 // one element to shared memory, zero if !in; complex ones in one copy where the operand is
@@ -631,7 +655,7 @@ __device__ __forceinline__ void copy_async(zdbl* dst, const zdbl* src, bool in, 
 
 template <typename T, bool SIDE_B, int S, int ROWS>
 __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T>& o, size_t plane,
-                                          int block, T* tiles, int* s_max, int* s_min,
+                                          int block, T* tiles, int* s_max, int* s_cnt,
                                           int* s_exp) {
   using O = ops<T>;
   constexpr bool CPLX = O::cplx;
@@ -679,13 +703,10 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
   };
-  // largest (and smallest nonzero) exponents of rows warp + 8 q
-  int best[RQ], low[RQ];
+  // largest exponents of rows warp + 8 q
+  int best[RQ];
 #pragma unroll
-  for (int q = 0; q < RQ; ++q) {
-    best[q] = -2000;
-    low[q] = 2000;
-  }
+  for (int q = 0; q < RQ; ++q) best[q] = -2000;
   for (int t = t_begin; t < t_end; t += g.keep) {
     if (t > t_begin) __syncthreads();
     load_tiles(t);
@@ -695,37 +716,32 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
 #pragma unroll
       for (int q = 0; q < NQ; ++q) {
         const T x = tiles[(i * ROWS + warp + 8 * (q % RQ)) * LD + lane + 32 * (q / RQ)];
-        const int br = expo_bits(O::real(x)), bi = expo_bits(O::imag(x));
-        best[q % RQ] = max(best[q % RQ], max(br, bi));
-        if constexpr (S > 5) {
-          if (br > -2000) low[q % RQ] = min(low[q % RQ], br);
-          if (bi > -2000) low[q % RQ] = min(low[q % RQ], bi);
-        }
+        best[q % RQ] = max(best[q % RQ], max(expo_bits(O::real(x)), expo_bits(O::imag(x))));
       }
   }
 #pragma unroll
   for (int q = 0; q < RQ; ++q) {
     const int b = __reduce_max_sync(0xffffffffu, best[q]);
     if (lane == 0) s_max[warp + 8 * q] = b;
-    if constexpr (S > 5) {
-      const int l = __reduce_min_sync(0xffffffffu, low[q]);
-      if (lane == 0) s_min[warp + 8 * q] = l;
-    }
+    if (S > 5 && lane < 8) s_cnt[(warp + 8 * q) * 8 + lane] = 0;
   }
   __syncthreads();
   if (nranks > 1) cluster.sync();
   if (tid < ROWS) {
-    int b = s_max[tid], lo = S > 5 ? s_min[tid] : 2000;
+    int b = s_max[tid];
     for (int q = 0; q < nranks; ++q)
-      if (q != rank) {
-        b = max(b, cluster.map_shared_rank(s_max, q)[tid]);
-        if constexpr (S > 5) lo = min(lo, cluster.map_shared_rank(s_min, q)[tid]);
+      if (q != rank) b = max(b, cluster.map_shared_rank(s_max, q)[tid]);
+    if (b >= 0x40000000) {  // Inf or NaN in the row
+      if constexpr (S > 5) {
+        if (g.guard)
+          g.guard[(int64_t)blockIdx.z * GUARD_WORDS + GUARD_BAD] = 1;
+        else
+          g.wide[blockIdx.z / g.per] = 1;
+      } else {
+        set_status(g.status, CBC_ERR_NUMERICAL);
       }
-    if constexpr (S > 5) {
-      if (b >= 0x40000000 || (lo < 2000 && b - lo > g.range)) g.wide[blockIdx.z / g.per] = 1;
-    } else if (b >= 0x40000000) {
-      set_status(g.status, CBC_ERR_NUMERICAL);  // Inf or NaN in the row
     }
+    if (S > 5) s_cnt[tid * 8 + 7] = b < -1100 || r0 + tid >= o.rows;  // (without say in the guard)
     b = (b < -1100) ? 0 : b;  // an all-zero (or padding) row
     s_exp[tid] = b;
     if (rank == 0 && r0 + tid < o.rows) o.expo[(int64_t)blockIdx.z * o.ebs + r0 + tid] = b;
@@ -748,8 +764,10 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
       if (r0 + lr >= o.rows) continue;
       const int e = s_exp[lr];
       if constexpr (!CPLX) {
-        const long long w0 = digit_word<S>(tile[lr * LD + 2 * lane], e);
-        const long long w1 = digit_word<S>(tile[lr * LD + 2 * lane + 1], e);
+        const T x0 = tile[lr * LD + 2 * lane], x1 = tile[lr * LD + 2 * lane + 1];
+        const long long w0 = digit_word<S>(x0, e);
+        const long long w1 = digit_word<S>(x1, e);
+        if (S > 5 && g.guard) count_levels(x0, x1, e, s_cnt + lr * 8);
         uint32_t* d = out + (size_t)(r0 + lr) * ld + t * 32 + lane;
 #pragma unroll
         for (int sl = 0; sl < S; ++sl)
@@ -761,6 +779,7 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
         // -x has digits of its own (a digit of -128 carries), and products that leave out the
         // last levels depend on them
         const long long wn = negated_word<S>(wi);
+        if (S > 5 && g.guard) count_levels(O::real(x), O::imag(x), e, s_cnt + lr * 8);
         uint32_t* d = out + (size_t)(SIDE_B ? 2 : 1) * (r0 + lr) * ld + t * 32 + lane;
 #pragma unroll
         for (int sl = 0; sl < S; ++sl) {
@@ -775,19 +794,37 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
       }
     }
   }
-  if (nranks > 1) cluster.sync();  // no CTA leaves while another still reads its row maxima
+  if (S > 5 && g.guard) {
+    // the most entries of a row below each level, over the row blocks; the zeros behind K
+    // were counted as well
+    __syncthreads();
+    if (nranks > 1) cluster.sync();
+    if (rank == 0 && tid < ROWS * 8) {
+      const int t = tid & 7;
+      int v = 0;
+      if (!s_cnt[tid | 7]) {
+        v = (CPLX ? 2 : 1) * g.K - g.K2p;
+        for (int q = 0; q < nranks; ++q) v += cluster.map_shared_rank(s_cnt, q)[tid];
+      }
+      v = max(v, __shfl_xor_sync(0xffffffffu, v, 8));
+      v = max(v, __shfl_xor_sync(0xffffffffu, v, 16));
+      if (lane < GUARD_LEVELS && v > 0)
+        atomicMax(g.guard + (int64_t)blockIdx.z * GUARD_WORDS + (SIDE_B ? GUARD_B : 0) + t, v);
+    }
+  }
+  if (nranks > 1) cluster.sync();  // no CTA leaves while another still reads its shared memory
 }
 
 template <typename T, int S, int ROWS>
 __global__ void __launch_bounds__(256) pack_kernel(PackArgs<T> g) {
   extern __shared__ __align__(16) unsigned char pack_smem[];
-  __shared__ int s_max[ROWS], s_min[ROWS], s_exp[ROWS];
+  __shared__ int s_max[ROWS], s_exp[ROWS], s_cnt[S > 5 ? ROWS * 8 : 1];
   T* tiles = reinterpret_cast<T*>(pack_smem);
   const int block = blockIdx.x / (int)cooperative_groups::this_cluster().num_blocks();
   if (block < g.blocks_a)
-    pack_rows<T, false, S, ROWS>(g, g.a, g.plane_a, block, tiles, s_max, s_min, s_exp);
+    pack_rows<T, false, S, ROWS>(g, g.a, g.plane_a, block, tiles, s_max, s_cnt, s_exp);
   else
-    pack_rows<T, true, S, ROWS>(g, g.b, g.plane_b, block - g.blocks_a, tiles, s_max, s_min, s_exp);
+    pack_rows<T, true, S, ROWS>(g, g.b, g.plane_b, block - g.blocks_a, tiles, s_max, s_cnt, s_exp);
 }
 
 // strides of the logical (row, k) indices at the origin, to pick the read pattern
@@ -971,11 +1008,8 @@ namespace {
 //            1000 x 1000 x 16 61 / 79, x 1000 2107 / 142
 //   complex  16 x 16 x 16 96 / 55, 1000 x 1000 x 8 158 / 106, 128 x 2048 x 128 556 / 69,
 //            1000^3 8097 / 389 us
-// An operand whose rows span more than this many powers of two, or that holds Inf or NaN, is
-// left to the SIMT kernel.  Within it every entry keeps at least 62 - 36 bits and the largest
-// ones all 53; Gaussian rows span about 2^25.
-constexpr int SPLIT_RANGE = 36;
-constexpr int SPLIT_MIN_K_REAL = 28, SPLIT_MIN_K_CPLX = 8;
+// (Below 28 terms of a real sum split_holds turns down Gaussian operands of many rows.)
+constexpr int SPLIT_MIN_K_REAL = 28, SPLIT_MIN_K_CPLX = 14;
 constexpr size_t SPLIT_MAX_BYTES = size_t(16) << 30;
 }  // namespace
 
@@ -1006,7 +1040,7 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
                     int* status, cudaStream_t s, int nb, const TcWide& opt) {
   using namespace tc;
   if (M <= 0 || N <= 0 || nb <= 0) return cudaSuccess;
-  if ((S < 2 || S > 5) && !(S == 8 && opt.wide)) return cudaErrorInvalidValue;
+  if ((S < 2 || S > 5) && !(S == 8 && (opt.wide || opt.guard))) return cudaErrorInvalidValue;
   // keep the long dimension on the 128-row side: C^T = B^T A^T
   if (M < BM && N > M) {
     return gemm_tc<T>(N, M, K, B, transpose_view(vb), conjB, A, transpose_view(va), conjA, C,
@@ -1042,7 +1076,7 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
   pk.status = status;
   pk.wide = opt.wide;
   pk.per = opt.per;
-  pk.range = opt.range;
+  pk.guard = opt.guard;
   cudaError_t pe = pack_operands<T>(pk, S, nb, s);
   if (pe != cudaSuccess) return pe;
   CUtensorMap ma;
@@ -1074,7 +1108,8 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
     args.C = reinterpret_cast<char*>(C);
     args.vc = vc;
     args.status = status;
-    args.skip = opt.skip ? opt.wide : nullptr;
+    args.guard = opt.guard;
+    args.guard_k = g.K2;
     args.acc = opt.acc;
     args.base = opt.base ? static_cast<const char*>(opt.base) : args.C;
     args.base_shift = opt.base ? (opt.base_bs - vc.bs) * (int64_t)sizeof(T) : 0;
@@ -1136,16 +1171,16 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
 }
 
 // ---- FP64 products on the tensor cores -------------------------------------------------
-// 8 slices hold 62 bits of an entry relative to its row's (column's) maximum and their
-// products are summed exactly, so the only rounding is the one to 53 bits at the end (one
-// more per K split): on rows that span fewer powers of two than SPLIT_RANGE the error is
-// below that of an FP64 sum.  Operands outside that are found while they are cut; then the
-// tensor-core kernel leaves their problem out and the SIMT kernel behind it does it.
-// Relative error against 80-bit sums, Gaussian entries: 4e-17 to 2e-16 where the SIMT kernel
+// 8 slices hold 62 bits of an entry relative to its row's (column's) maximum; the kept products
+// of slices are summed exactly and rounded once to 53 bits (once more per K split).  Whether
+// that is as accurate as an FP64 sum is found while the operands are cut (split_guard.cuh);
+// where it is not, the tensor-core kernel leaves the problem out and the SIMT kernel behind it
+// does it.  Relative error against 80-bit sums, Gaussian entries: 4e-17 to 2e-16 where the SIMT kernel
 // has 1e-16 (K = 16) to 1e-15 (K = 1000).
 size_t gemm_f64_split_bytes(int M, int N, int K, bool cplx, int nb) {
   if (K < (cplx ? SPLIT_MIN_K_CPLX : SPLIT_MIN_K_REAL)) return 0;
-  const size_t b = gemm_tc_workspace_bytes(M, N, K, cplx, 8, nb) + tc::a256(sizeof(int) * nb);
+  const size_t b = gemm_tc_workspace_bytes(M, N, K, cplx, 8, nb) +
+                   tc::a256(sizeof(int) * GUARD_WORDS * nb);
   return b <= SPLIT_MAX_BYTES ? b : 0;
 }
 
@@ -1153,14 +1188,15 @@ template <typename T>
 cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& va, bool conjA,
                            const T* B, const View& vb, bool conjB, T* C, const View& vc, void* ws,
                            int* status, cudaStream_t s) {
-  int* wide = static_cast<int*>(ws);  // one word per problem
-  const size_t wb = tc::a256(sizeof(int) * nb);
-  cudaError_t e = cudaMemsetAsync(wide, 0, wb, s);
+  TcWide opt;
+  opt.guard = static_cast<int*>(ws);
+  const size_t gb = tc::a256(sizeof(int) * GUARD_WORDS * nb);
+  cudaError_t e = cudaMemsetAsync(ws, 0, gb, s);
   if (e != cudaSuccess) return e;
-  e = gemm_tc<T>(M, N, K, A, va, conjA, B, vb, conjB, C, vc, 8, static_cast<char*>(ws) + wb,
-                 status, s, nb, TcWide{wide, 1, SPLIT_RANGE, true});
+  e = gemm_tc<T>(M, N, K, A, va, conjA, B, vb, conjB, C, vc, 8, static_cast<char*>(ws) + gb,
+                 status, s, nb, opt);
   if (e != cudaSuccess) return e;
-  return gemm_f64<T>(M, N, K, nb, A, va, conjA, B, vb, conjB, C, vc, s, wide);
+  return gemm_f64<T>(M, N, K, nb, A, va, conjA, B, vb, conjB, C, vc, s, opt.guard);
 }
 
 template cudaError_t gemm_f64_split<double>(int, int, int, int, const double*, const View&, bool,

@@ -60,11 +60,11 @@ struct View {
 template <typename T>
 cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va, bool conjA,
                      const T* B, const View& vb, bool conjB, T* C, const View& vc,
-                     cudaStream_t s, const int* cond = nullptr);
-// (cond: a device word per problem; not NULL: only the problems whose word is set.)
+                     cudaStream_t s, const int* guard = nullptr);
+// (guard: not NULL: only the problems that split_holds, split_guard.cuh, turns down.)
 
-// The FP64 product as 8 bf16 slices per operand on the tensor cores, with an error no larger
-// than gemm_f64's (gemm_tc.cu).  gemm_f64_split_bytes gives the bytes it needs at `ws`, or 0
+// The FP64 product as 8 bf16 slices per operand on the tensor cores, where their error is no
+// larger than an FP64 sum's; the other problems through gemm_f64 (gemm_tc.cu, split_guard.cuh).  gemm_f64_split_bytes gives the bytes it needs at `ws`, or 0
 // where gemm_f64 is to be used: small products, and slices beyond 16 GB.
 size_t gemm_f64_split_bytes(int M, int N, int K, bool cplx, int nb);
 template <typename T>
@@ -76,14 +76,14 @@ cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& 
 // `ws` must hold gemm_tc_workspace_bytes(M, N, K, cplx, S, nb) bytes.  nb problems of
 // one shape, their operands va.bs / vb.bs / vc.bs elements apart, in one launch.
 // S = 8 (62 bits of every entry, relative to its row's maximum) needs TcWide::wide, device
-// words of which number p / per is set when an operand of problem p holds Inf or NaN or one of
-// its rows spans more than 2^range; `skip` (per = 1): then the problem's C is left alone.  acc = 1 or -1: base + A B or base - A B into C, with
+// words of which number p / per is set when an operand of problem p holds Inf or NaN, or
+// TcWide::guard, GUARD_WORDS zeroed words per problem: C of a problem that split_holds turns
+// down is left alone.  acc = 1 or -1: base + A B or base - A B into C, with
 // base (NULL: C itself) laid out as C but for its problems, base_bs elements apart.
 struct TcWide {
   int* wide = nullptr;
   int per = 0x7fffffff;
-  int range = 1 << 20;
-  bool skip = false;
+  int* guard = nullptr;
   int acc = 0;
   const void* base = nullptr;
   int64_t base_bs = 0;

@@ -30,3 +30,83 @@ def test_a_problem_does_not_send_its_neighbours(nb, cplx):
     for b in range(nb):
         if b != 1:
             assert np.array_equal(Q[b], R[b])
+
+
+def _bound(A, B):
+    """K eps |A||B| (sqrt 2 more per complex product), as for any FP64 sum."""
+    return 4 * (A.shape[1] + 2) * 2.0 ** -53 * (np.abs(A) @ np.abs(B))
+
+
+def _check(A, B):
+    from test_gemm_gpu import _run
+    C, _ = _run(0, 0, A, B)
+    long = np.clongdouble if np.iscomplexobj(A) else np.longdouble
+    err = np.abs(C - A.astype(long) @ B.astype(long))
+    assert np.all(err <= _bound(A, B)), (err / _bound(A, B)).max()
+
+
+def _alternate(K, r, up):
+    w = np.ones(K)
+    w[int(up)::2] = 2.0 ** -r
+    return w
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("shape", [(128, 64, 32), (40, 300, 64), (65, 33, 257), (16, 20, 2049)])
+@pytest.mark.parametrize("r", [0, 4, 8, 12, 20, 30, 36, 45])
+@pytest.mark.parametrize("how", ["slope", "alternate", "half", "one", "rows"])
+def test_opposite_grading(how, r, shape, cplx):
+    """A graded along K and B the other way, so that large entries meet small ones: the plain
+    bound of an FP64 sum, entry by entry."""
+    rng = np.random.default_rng([r, shape[2], cplx])
+    M, N, K = shape
+    A, B = _rand(rng, (M, K), cplx), _rand(rng, (K, N), cplx)
+    if how == "slope":
+        w = 2.0 ** -np.linspace(0, r, K)
+        wb = w[::-1]
+    elif how == "alternate":
+        w, wb = _alternate(K, r, True), _alternate(K, r, False)
+    elif how == "half":
+        w = np.where(np.arange(K) < K // 2, 1.0, 2.0 ** -r)
+        wb = w[::-1]
+    else:  # one large entry, in the same place or, "rows", in one row and column only
+        w = np.where(np.arange(K) == 3, 1.0, 2.0 ** -r)
+        wb = np.where(np.arange(K) == 4, 1.0, 2.0 ** -r)
+    if how == "rows":
+        A[-1], B[:, -1] = A[-1] * w, B[:, -1] * wb
+    else:
+        A, B = A * w, B * wb[:, None]
+    _check(A, B)
+
+
+@pytest.mark.parametrize("r", [3, 6, 9, 20])
+def test_equal_digits(r):
+    """Terms whose dropped digits all add up: equal entries 2^-r below one large one."""
+    rng = np.random.default_rng(r)
+    M, N, K = 40, 40, 512
+    A = np.full((M, K), (1 - 2.0 ** -9 + 2.0 ** -40) * 2.0 ** -r / 1.5)
+    B = np.full((K, N), (1 - 2.0 ** -10 - 2.0 ** -41) * 2.0 ** -r / 1.5)
+    A[:, 0], B[1] = rng.uniform(1, 2, M), rng.uniform(1, 2, N)
+    _check(A, B)
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("kind", ["zero_rows", "sparse", "identity", "subnormal", "ends"])
+def test_forms(kind, cplx):
+    """Rows of zeros, mostly zeros, a permutation, and the ends of the exponent range."""
+    rng = np.random.default_rng(3)
+    M, N, K = 70, 45, 130
+    A, B = _rand(rng, (M, K), cplx), _rand(rng, (K, N), cplx)
+    if kind == "zero_rows":
+        A[::3], B[:, 1::4] = 0, 0
+    elif kind == "sparse":
+        A, B = A * (rng.random(A.shape) < 0.05), B * (rng.random(B.shape) < 0.2)
+    elif kind == "identity":
+        A = np.eye(M, K) * (1 + 1j if cplx else 1)
+        B = B * 2.0 ** -rng.integers(0, 50, B.shape).astype(float)
+    elif kind == "subnormal":
+        A = A * 2.0 ** -1030
+        B = B * 2.0 ** 1000
+    else:
+        A, B = A * 2.0 ** 1000, B * 2.0 ** -1000
+    _check(A, B)
