@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(NT) gemm_f64_kernel(GemmArgs<T> g) {
     const int bn = tile % g.tiles_n * BN, bm = tile / g.tiles_n % g.tiles_m * BM;
     const int z = tile / (g.tiles_n * g.tiles_m);
     const int batch = z / g.splits;
-    if (g.guard && split_holds(g.guard + batch * GUARD_WORDS, O::cplx ? 2 * g.K : g.K)) continue;
+    if (g.guard && split_holds(g.guard + batch * GUARD_WORDS)) continue;
     const int split = z % g.splits;
     const int kbeg = split * g.kchunk;
     const int kend = min(g.K, kbeg + g.kchunk);

@@ -205,7 +205,7 @@ struct TcArgs {
   char* C;               // FP64 output (double or zdbl) through the view
   View vc;               // vc.bs: elements between the outputs of consecutive problems
   int* status;
-  const int* guard;      // not NULL: nothing runs for problems that it turns down (gemm_f64_split)
+  int* guard;            // not NULL: nothing runs for problems that it turns down (gemm_f64_split)
   int guard_k;           // terms of the real sums
   int acc;               // 1 or -1: base + A B or base - A B instead of A B
   const char* base;      // rows and columns as C's (C itself when it is split along K)
@@ -267,8 +267,8 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
   constexpr int A_BYTES = BM * KAS * 2;
   constexpr int B_BYTES = BN * KAS * 2;
   constexpr int STAGE_BYTES = S * (A_BYTES + B_BYTES);
-  constexpr uint32_t TMEM_COLS = 512;
-  static_assert(2 * S * BN <= 512, "TMEM budget");  // hence S BN <= 256, the widest MMA
+  constexpr uint32_t TMEM_COLS = S == 1 ? 2 * BN : 512;
+  static_assert(2 * S * BN <= (int)TMEM_COLS, "TMEM budget");  // hence S BN <= 256, the widest MMA
   static_assert(BN % 16 == 0, "MMA width");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -288,8 +288,10 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
   struct Tile {
     int m0, n0, prob, a_begin, n_atoms, n_chunks;
   };
+  // S = 1: the entries of sum |a||b| against the line of split_guard.cuh, for the problems whose
+  // counts are too few; no output but the guard's word
   int seen = -1;  // the last problem whose guard was looked at
-  bool holds = true;
+  bool runs = true;
   auto tile_of = [&](int t) {
     Tile q;
     const int mt = t % a.tiles_m, r = t / a.tiles_m;
@@ -301,9 +303,10 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
     q.n_atoms = max(0, min(a.atoms_total, q.a_begin + a.atoms_per_split) - q.a_begin);
     if (a.guard && q.prob != seen) {
       seen = q.prob;
-      holds = split_holds(a.guard + (int64_t)q.prob * GUARD_WORDS, a.guard_k);
+      const int* g = a.guard + (int64_t)q.prob * GUARD_WORDS;
+      runs = S == 1 ? !g[GUARD_BAD] && !counts_hold(g, a.guard_k) : split_holds(g);
     }
-    if (!holds) q.n_atoms = 0;  // (no role has anything to do in the tile)
+    if (!runs) q.n_atoms = 0;  // (no role has anything to do in the tile)
     q.n_chunks = (q.n_atoms + a.atoms_per_chunk - 1) / a.atoms_per_chunk;
     return q;
   };
@@ -454,7 +457,21 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
         if (lane == 0) mbar_arrive(tempty + buf);
       }
       if (!run) break;
-      if (q.n_chunks > 0) {
+      if constexpr (S == 1) {
+        if (q.n_chunks > 0) {
+          const int mycol = q.n0 + colg * CW + lane;
+          const bool colok =
+              lane < CW && mycol < a.N2 &&
+              a.expB[(int64_t)q.prob * a.ebsB + (a.cplx ? mycol >> 1 : mycol)] != GUARD_ZERO_ROW;
+          const unsigned cols = __ballot_sync(0xffffffffu, colok);
+          const bool rowok = row < a.M && a.expA[q.prob * a.Mp + row] != GUARD_ZERO_ROW;
+          const long long line = (long long)ceilf(0x1p14f * guard_line(a.guard_k));
+          bool few = false;
+#pragma unroll
+          for (int i = 0; i < CW; ++i) few = few || ((cols >> i & 1u) && acc[0][i] < line);
+          if (few && rowok) a.guard[(int64_t)q.prob * GUARD_WORDS + GUARD_FAIL] = 1;
+        }
+      } else if (q.n_chunks > 0) {
         // the CW columns of this warp are shared by its lanes (the lanes are rows): lane i
         // finds column i's offset and exponent once, the loop takes them by shuffle
         const int* expB = a.expB + (int64_t)q.prob * a.ebsB;
@@ -599,15 +616,24 @@ __device__ __forceinline__ uint32_t bf16_pair(uint32_t flo, uint32_t fhi) {
   return __byte_perm(flo, fhi, 0x7632);
 }
 
-// Adds to cnt[t - 2] how many of the warp's entries x0, x1 are below 2^(e-t), t = 2 .. 8 (at most
-// 64: eight bits each; a subnormal entry counts as below all).
-__device__ __forceinline__ void count_levels(double x0, double x1, int e, int* cnt) {
-  auto below = [&](double x) {
-    const int f = ((unsigned)__double2hiint(x) >> 20) & 0x7ff;
-    const int n = f ? min(max(e + 1021 - f, 0), GUARD_LEVELS) : GUARD_LEVELS;  // levels above |x|
+// The leading 31 bits of an entry's magnitude from its digit word (8 slices: |x| 2^(62-e) as an
+// integer; one's complement, so at most one unit of 2^(e-30) off), for the guard
+__device__ __forceinline__ uint32_t leading_bits(long long w) {
+  const int h = (int)((w - DIGIT_BIAS<8>) >> 32);
+  return (uint32_t)(h ^ (h >> 31));
+}
+// floor(2^7 |x| / 2^e) as the bits of a float
+__device__ __forceinline__ uint32_t leading7(uint32_t h) {
+  return __float_as_uint(__uint_as_float(0x4b000000u + (h >> 23)) - 8388608.0f);
+}
+// Adds to cnt[t - 2] how many of the warp's entries (leading bits h0, h1) are below 2^(e-t),
+// t = 2 .. 8 (at most 64: eight bits each).
+__device__ __forceinline__ void count_levels(uint32_t h0, uint32_t h1, int* cnt) {
+  auto below = [](uint32_t h) {
+    const int n = min(max(__clz((int)h) - 3, 0), GUARD_LEVELS);  // levels above |x|
     return 0x0101010101010101ull & ((1ull << (8 * n)) - 1ull);
   };
-  const unsigned long long w = below(x0) + below(x1);
+  const unsigned long long w = below(h0) + below(h1);
   const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)w);
   const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(w >> 32));
   const int lane = threadIdx.x & 31;
@@ -632,7 +658,8 @@ struct PackArgs {
   int* status;
   int* wide;           // 8 slices: word (problem / per) is set when an operand holds Inf or NaN,
   int per;
-  int* guard;          // or the words of split_guard.cuh are filled in
+  int* guard;          // or the words of split_guard.cuh are filled in, and the magnitudes'
+                       // leading bits go to one plane more
 };
 
 // one element to shared memory, zero if !in; complex ones in one copy where the operand is
@@ -742,9 +769,11 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
       }
     }
     if (S > 5) s_cnt[tid * 8 + 7] = b < -1100 || r0 + tid >= o.rows;  // (without say in the guard)
-    b = (b < -1100) ? 0 : b;  // an all-zero (or padding) row
+    const bool zero = b < -1100;  // an all-zero (or padding) row
+    b = zero ? 0 : b;
     s_exp[tid] = b;
-    if (rank == 0 && r0 + tid < o.rows) o.expo[(int64_t)blockIdx.z * o.ebs + r0 + tid] = b;
+    if (rank == 0 && r0 + tid < o.rows)
+      o.expo[(int64_t)blockIdx.z * o.ebs + r0 + tid] = S > 5 && g.guard && zero ? GUARD_ZERO_ROW : b;
   }
   __syncthreads();
   uint32_t* out = reinterpret_cast<uint32_t*>(o.out + (size_t)blockIdx.z * o.rows_pad * g.K2p);
@@ -764,11 +793,14 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
       if (r0 + lr >= o.rows) continue;
       const int e = s_exp[lr];
       if constexpr (!CPLX) {
-        const T x0 = tile[lr * LD + 2 * lane], x1 = tile[lr * LD + 2 * lane + 1];
-        const long long w0 = digit_word<S>(x0, e);
-        const long long w1 = digit_word<S>(x1, e);
-        if (S > 5 && g.guard) count_levels(x0, x1, e, s_cnt + lr * 8);
+        const long long w0 = digit_word<S>(tile[lr * LD + 2 * lane], e);
+        const long long w1 = digit_word<S>(tile[lr * LD + 2 * lane + 1], e);
         uint32_t* d = out + (size_t)(r0 + lr) * ld + t * 32 + lane;
+        if (S > 5 && g.guard) {
+          const uint32_t h0 = leading_bits(w0), h1 = leading_bits(w1);
+          count_levels(h0, h1, s_cnt + lr * 8);
+          d[S * pl] = bf16_pair(leading7(h0), leading7(h1));
+        }
 #pragma unroll
         for (int sl = 0; sl < S; ++sl)
           d[sl * pl] = bf16_pair(digit_f32<S>(w0, sl), digit_f32<S>(w1, sl));
@@ -779,8 +811,14 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
         // -x has digits of its own (a digit of -128 carries), and products that leave out the
         // last levels depend on them
         const long long wn = negated_word<S>(wi);
-        if (S > 5 && g.guard) count_levels(O::real(x), O::imag(x), e, s_cnt + lr * 8);
         uint32_t* d = out + (size_t)(SIDE_B ? 2 : 1) * (r0 + lr) * ld + t * 32 + lane;
+        if (S > 5 && g.guard) {
+          const uint32_t hr = leading_bits(wr), hi = leading_bits(wi);
+          count_levels(hr, hi, s_cnt + lr * 8);
+          const uint32_t ar = leading7(hr), ai = leading7(hi);
+          d[S * pl] = bf16_pair(ar, ai);
+          if (SIDE_B) d[S * pl + ld] = bf16_pair(ai, ar);
+        }
 #pragma unroll
         for (int sl = 0; sl < S; ++sl) {
           const uint32_t fr = digit_f32<S>(wr, sl), fi = digit_f32<S>(wi, sl);
@@ -913,6 +951,7 @@ bool make_map(CUtensorMap* m, void* base, int K2_pad, int64_t rows_pad, int S, i
   return r == CUDA_SUCCESS;
 }
 
+// (S = 1: 1024 products below 2^14)
 int atoms_per_chunk_for(int S) { return std::max(1, (1024 / S) / ka(S)); }
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -976,6 +1015,7 @@ cudaError_t launch_bn(const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs
 cudaError_t launch(int S, int BN, const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs& args,
                    dim3 grid, cudaStream_t s) {
   switch (S * 1000 + BN) {
+    case 1064: return launch_bn<1, 64>(ma, mb, args, grid, s);
     case 2064: return launch_bn<2, 64>(ma, mb, args, grid, s);
     case 3064: return launch_bn<3, 64>(ma, mb, args, grid, s);
     case 4032: return launch_bn<4, 32>(ma, mb, args, grid, s);
@@ -1008,8 +1048,7 @@ namespace {
 //            1000 x 1000 x 16 61 / 79, x 1000 2107 / 142
 //   complex  16 x 16 x 16 96 / 55, 1000 x 1000 x 8 158 / 106, 128 x 2048 x 128 556 / 69,
 //            1000^3 8097 / 389 us
-// (Below 28 terms of a real sum split_holds turns down Gaussian operands of many rows.)
-constexpr int SPLIT_MIN_K_REAL = 28, SPLIT_MIN_K_CPLX = 14;
+constexpr int SPLIT_MIN_K_REAL = 28, SPLIT_MIN_K_CPLX = 8;
 constexpr size_t SPLIT_MAX_BYTES = size_t(16) << 30;
 }  // namespace
 
@@ -1056,10 +1095,11 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
   char* w = static_cast<char*>(ws);
   w = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(w) + 255) & ~uintptr_t(255));
   const size_t b = (size_t)nb;
+  const size_t planes = b * (S + (opt.guard ? 1 : 0));
   __nv_bfloat16* sa = reinterpret_cast<__nv_bfloat16*>(w);
-  w += a256(b * S * g.Mp * g.K2p * 2);
+  w += a256(planes * g.Mp * g.K2p * 2);
   __nv_bfloat16* sb = reinterpret_cast<__nv_bfloat16*>(w);
-  w += a256(b * S * g.N2p * g.K2p * 2);
+  w += a256(planes * g.N2p * g.K2p * 2);
   int* ea = reinterpret_cast<int*>(w);
   w += a256(b * sizeof(int) * g.Mp);
   int* eb = reinterpret_cast<int*>(w);
@@ -1126,6 +1166,24 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
     args.tiles_n = tiles_n;
     args.total_tiles = args.tiles_m * args.tiles_n * splits * nb;
     dim3 grid(std::min(args.total_tiles, g_sms));
+    if (opt.guard) {
+      // the magnitudes' product first, for the problems that the counts don't decide
+      constexpr int CB = 64;
+      CUtensorMap ca, cb;
+      if (!make_map(&ca, sa + 8 * pk.plane_a, g.K2p, nb * g.Mp, 1, BM) ||
+          !make_map(&cb, sb + 8 * pk.plane_b, g.K2p, nb * g.N2p, 1, CB))
+        return cudaErrorInvalidValue;
+      TcArgs c = args;
+      c.atoms_total = g.K2p / ka(1);
+      c.atoms_per_chunk = atoms_per_chunk_for(1);
+      c.atoms_per_split = (c.atoms_total + c.atoms_per_chunk - 1) / c.atoms_per_chunk * c.atoms_per_chunk;
+      c.splits = 1;
+      c.tiles_n = g.N2p / CB;
+      c.total_tiles = c.tiles_m * c.tiles_n * nb;
+      note_launches(CBC_K_GEMM_F64, 1);
+      cudaError_t e = launch(1, CB, ca, cb, c, dim3(std::min(c.total_tiles, g_sms)), s);
+      if (e != cudaSuccess) return e;
+    }
     note_launches(S == 8 ? CBC_K_GEMM_F64 : CBC_K_GEMM_TC, 1);
     if (S != 8)
       note_flops(CBC_K_TC_ISSUED,
@@ -1179,7 +1237,7 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
 // has 1e-16 (K = 16) to 1e-15 (K = 1000).
 size_t gemm_f64_split_bytes(int M, int N, int K, bool cplx, int nb) {
   if (K < (cplx ? SPLIT_MIN_K_CPLX : SPLIT_MIN_K_REAL)) return 0;
-  const size_t b = gemm_tc_workspace_bytes(M, N, K, cplx, 8, nb) +
+  const size_t b = gemm_tc_workspace_bytes(M, N, K, cplx, 9, nb) +  // (8 slices, the magnitudes)
                    tc::a256(sizeof(int) * GUARD_WORDS * nb);
   return b <= SPLIT_MAX_BYTES ? b : 0;
 }

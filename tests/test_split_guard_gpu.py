@@ -41,8 +41,12 @@ def _check(A, B):
     from test_gemm_gpu import _run
     C, _ = _run(0, 0, A, B)
     long = np.clongdouble if np.iscomplexobj(A) else np.longdouble
-    err = np.abs(C - A.astype(long) @ B.astype(long))
-    assert np.all(err <= _bound(A, B)), (err / _bound(A, B)).max()
+    # of large products the first and last rows and columns of tiles
+    rows = [i for i in range(len(A)) if len(A) < 70 or i % 64 in (0, 63) or i == len(A) - 1]
+    cols = [j for j in range(B.shape[1]) if B.shape[1] < 70 or j % 32 in (0, 31) or j == B.shape[1] - 1]
+    a, b = A[rows], B[:, cols]
+    err = np.abs(C[np.ix_(rows, cols)] - a.astype(long) @ b.astype(long))
+    assert np.all(err <= _bound(a, b)), (err / _bound(a, b)).max()
 
 
 def _alternate(K, r, up):
@@ -109,4 +113,23 @@ def test_forms(kind, cplx):
         B = B * 2.0 ** 1000
     else:
         A, B = A * 2.0 ** 1000, B * 2.0 ** -1000
+    _check(A, B)
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("shape", [(300, 200, 1100), (129, 65, 64), (257, 64, 2049), (20, 20, 28)])
+@pytest.mark.parametrize("r", [2, 4, 6, 9, 14, 22])
+def test_entries_where_counts_are_too_few(r, shape, cplx):
+    """Half of every row below 2^-9: the counts don't decide, the magnitudes' product does.  Then
+    the last row and column are graded against each other, which their one entry shows."""
+    rng = np.random.default_rng([r, shape[0], cplx])
+    M, N, K = shape
+    A, B = _rand(rng, (M, K), cplx), _rand(rng, (K, N), cplx)
+    h = np.where(rng.random(K) < 0.5, 1.0, 2.0 ** -12)
+    A, B = A * h, B * h[:, None]
+    _check(A, B)
+    A[-1] *= np.where(h == 1.0, 2.0 ** -r, 1.0)
+    A[-1, 5] = 2.0
+    B[:, -1] *= np.where(h == 1.0, 2.0 ** -r, 1.0)
+    B[7, -1] = 2.0
     _check(A, B)
