@@ -4,8 +4,8 @@
 //
 // It works on leg views of the node tensors (kernels.cuh: View).  On GB300 the FP64 pipe delivers
 // about 2 DFMA per clock per SM, so this kernel is FP64-throughput bound by design: a
-// 64x64 output tile per CTA, 16-deep K slices staged in shared memory, 4x4 outputs
-// per thread, and a K split (FP64 atomics into a zeroed C) when the output tiles
+// 64x64 (32x32) output tile per CTA, 16-deep K slices staged in shared memory, 4x4 (2x2)
+// outputs per thread, and a K split (FP64 atomics into a zeroed C) when the output tiles
 // alone cannot occupy every SM.
 #include <algorithm>
 
@@ -16,7 +16,7 @@
 namespace cbc {
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
+constexpr int BK = 16, NT = 256;
 
 template <typename T>
 struct GemmArgs {
@@ -31,9 +31,11 @@ struct GemmArgs {
   int tiles_n, tiles_m, total;  // tiles of one (problem, split); of the launch
 };
 
-template <typename T, bool CA, bool CB, bool ATOMIC>
+// R x R outputs per thread, 16 R x 16 R per CTA
+template <typename T, bool CA, bool CB, bool ATOMIC, int R>
 __global__ void __launch_bounds__(NT) gemm_f64_kernel(GemmArgs<T> g) {
   using O = ops<T>;
+  constexpr int BM = 16 * R, BN = 16 * R;
   __shared__ T As[BK][BM + 1];
   __shared__ T Bs[BK][BN + 1];
   __shared__ int64_t a_row[BM];
@@ -58,11 +60,11 @@ __global__ void __launch_bounds__(NT) gemm_f64_kernel(GemmArgs<T> g) {
     for (int i = tid; i < BN; i += NT) b_col[i] = (bn + i < g.N) ? g.vb.coff(bn + i) : -1;
     __syncthreads();
 
-    T acc[4][4];
+    T acc[R][R];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = O::zero();
+      for (int j = 0; j < R; ++j) acc[i][j] = O::zero();
 
     for (int k0 = kbeg; k0 < kend; k0 += BK) {
       // A tile: BM x BK, consecutive threads walk K (the contiguous leg of most views)
@@ -96,26 +98,26 @@ __global__ void __launch_bounds__(NT) gemm_f64_kernel(GemmArgs<T> g) {
       __syncthreads();
 #pragma unroll
       for (int kk = 0; kk < BK; ++kk) {
-        T a[4], b[4];
+        T a[R], b[R];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+        for (int i = 0; i < R; ++i) a[i] = As[kk][ty + 16 * i];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+        for (int j = 0; j < R; ++j) b[j] = Bs[kk][tx + 16 * j];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < R; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = O::fma(a[i], b[j], acc[i][j]);
+          for (int j = 0; j < R; ++j) acc[i][j] = O::fma(a[i], b[j], acc[i][j]);
       }
       __syncthreads();
     }
 
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < R; ++i) {
       int r = bm + ty + 16 * i;
       if (r >= g.M) continue;
       int64_t ro = g.vc.roff(r);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < R; ++j) {
         int c = bn + tx + 16 * j;
         if (c >= g.N) continue;
         T* dst = C + ro + g.vc.coff(c);
@@ -150,49 +152,75 @@ __global__ void zero_view_kernel(T* C, View vc, int M, int N, int batch) {
 
 int g_num_sms = 0;
 
-}  // namespace
-
-template <typename T>
-cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va, bool conjA,
-                     const T* B, const View& vb, bool conjB, T* C, const View& vc,
-                     cudaStream_t s, const int* guard) {
-  if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
+// How a product is dealt to the CTAs.  Behind a split product (guard) tiles of 32 x 32 where
+// those of 64 x 64 leave SMs idle: the same sums in the same order, and what the slicing cost is
+// won back.  A product that the split turns down, cbc_gemm in all, on the SIMT kernel at once /
+// behind the split, us: real 256 x 256 x 64 104 / 79, 64 x 64 x 8192 181 / 181 (without a split
+// of K 9700), complex 64 x 128 x 256 567 / 210, 501 x 777 x 1030 4158 / 3290, 1000 x 1000 x 8
+// 163 / 178.
+struct SimtShape {
+  int edge, tiles, splits, kchunk;
+};
+SimtShape simt_shape(int M, int N, int K, int batch, bool guard) {
   if (g_num_sms == 0) {
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (g_num_sms <= 0) g_num_sms = 148;
   }
-  int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN) * batch;
-  int ksteps = (K + BK - 1) / BK;
-  int splits = 1;
-  int target = 2 * g_num_sms;
-  if (!guard && tiles < target && ksteps >= 16) {
-    splits = (target + tiles - 1) / tiles;
-    splits = min(splits, ksteps / 8);
-    splits = max(splits, 1);
+  const int target = 2 * g_num_sms;
+  auto count = [&](int e) { return ((M + e - 1) / e) * ((N + e - 1) / e) * batch; };
+  SimtShape s;
+  s.edge = guard && count(64) < target ? 32 : 64;
+  s.tiles = count(s.edge);
+  const int ksteps = (K + BK - 1) / BK;
+  s.splits = 1;
+  if (s.tiles < target && ksteps >= 16) {
+    s.splits = (target + s.tiles - 1) / s.tiles;
+    s.splits = min(s.splits, ksteps / 8);
+    s.splits = max(s.splits, 1);
   }
-  int kchunk = ((ksteps + splits - 1) / splits) * BK;
-  splits = max(1, (K + kchunk - 1) / kchunk);
+  s.kchunk = ((ksteps + s.splits - 1) / s.splits) * BK;
+  s.splits = max(1, (K + s.kchunk - 1) / max(s.kchunk, 1));
+  return s;
+}
+
+}  // namespace
+
+bool gemm_f64_adds(int M, int N, int K, int batch) {
+  return simt_shape(M, N, K, batch, true).splits > 1;
+}
+
+template <typename T>
+cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va, bool conjA,
+                     const T* B, const View& vb, bool conjB, T* C, const View& vc,
+                     cudaStream_t s, const int* guard) {
+  if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
+  const SimtShape sh = simt_shape(M, N, K, batch, guard != nullptr);
+  const int edge = sh.edge, tiles = sh.tiles, splits = sh.splits;
   if (K <= 0) {  // empty contraction: C = 0
     note_launches(CBC_K_GEMM_F64, 1);
     zero_view_kernel<T><<<256, 256, 0, s>>>(C, vc, M, N, batch);
     return cudaGetLastError();
   }
-  GemmArgs<T> g{M,  N, K,  splits, kchunk, A, va, B, vb, C, vc, guard,
-                (N + BN - 1) / BN, (M + BM - 1) / BM, tiles * splits};
+  GemmArgs<T> g{M,  N, K,  splits, sh.kchunk, A, va, B, vb, C, vc, guard,
+                (N + edge - 1) / edge, (M + edge - 1) / edge, tiles * splits};
   // a product that usually does not run (guard) is launched as one resident wave
-  const int grid = guard ? std::min(g.total, target) : g.total;
-  note_launches(CBC_K_GEMM_F64, splits > 1 ? 2 : 1);
-  if (splits > 1) {
+  const int grid = guard ? std::min(g.total, 2 * g_num_sms) : g.total;
+  note_launches(CBC_K_GEMM_F64, splits > 1 && !guard ? 2 : 1);
+  if (splits > 1 && !guard) {  // (gemm_f64_adds: the split leaves zeros)
     int zb = (int)std::min<int64_t>(4096, ((int64_t)M * N * batch + 255) / 256);
     zero_view_kernel<T><<<zb, 256, 0, s>>>(C, vc, M, N, batch);
   }
 #define CBC_GEMM_LAUNCH(CA, CB)                                                     \
-  if (splits > 1)                                                                   \
-    gemm_f64_kernel<T, CA, CB, true><<<grid, NT, 0, s>>>(g);                        \
+  if (edge == 32 && splits > 1)                                                     \
+    gemm_f64_kernel<T, CA, CB, true, 2><<<grid, NT, 0, s>>>(g);                     \
+  else if (edge == 32)                                                              \
+    gemm_f64_kernel<T, CA, CB, false, 2><<<grid, NT, 0, s>>>(g);                    \
+  else if (splits > 1)                                                              \
+    gemm_f64_kernel<T, CA, CB, true, 4><<<grid, NT, 0, s>>>(g);                     \
   else                                                                              \
-    gemm_f64_kernel<T, CA, CB, false><<<grid, NT, 0, s>>>(g);
+    gemm_f64_kernel<T, CA, CB, false, 4><<<grid, NT, 0, s>>>(g);
   if (conjA && conjB) {
     CBC_GEMM_LAUNCH(true, true)
   } else if (conjA) {

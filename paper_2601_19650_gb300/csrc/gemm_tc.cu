@@ -198,6 +198,7 @@ struct TcArgs {
   int atoms_total;       // K2_pad / ka(S)
   int atoms_per_split;   // multiple of atoms_per_chunk
   int atoms_per_chunk;
+  int atom_step;         // every how many atoms one is taken (S = 1; else 1)
   const int* expA;       // [M_pad]
   const int* expB;       // [N_pad] (one per complex column when cplx)
   int cplx;
@@ -205,7 +206,8 @@ struct TcArgs {
   char* C;               // FP64 output (double or zdbl) through the view
   View vc;               // vc.bs: elements between the outputs of consecutive problems
   int* status;
-  int* guard;            // not NULL: nothing runs for problems that it turns down (gemm_f64_split)
+  int* guard;            // not NULL: nothing, or C = 0 (zero), for problems that it turns down
+  int zero;              // (gemm_f64_split)
   int guard_k;           // terms of the real sums
   int acc;               // 1 or -1: base + A B or base - A B instead of A B
   const char* base;      // rows and columns as C's (C itself when it is split along K)
@@ -306,7 +308,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
       const int* g = a.guard + (int64_t)q.prob * GUARD_WORDS;
       runs = S == 1 ? !g[GUARD_BAD] && !counts_hold(g, a.guard_k) : split_holds(g);
     }
-    if (!runs) q.n_atoms = 0;  // (no role has anything to do in the tile)
+    if (!runs) q.n_atoms = 0;  // (no role but the epilogue has anything to do in the tile)
     q.n_chunks = (q.n_atoms + a.atoms_per_chunk - 1) / a.atoms_per_chunk;
     return q;
   };
@@ -352,7 +354,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
           uint8_t* sA = smem + stage * STAGE_BYTES;
           uint8_t* sB = sA + S * A_BYTES;
           mbar_expect_tx(full + stage, STAGE_BYTES);
-          const int k = (q.a_begin + j) * KAS;
+          const int k = (q.a_begin + j) * KAS * a.atom_step;
 #pragma unroll
           for (int s = 0; s < S; ++s) {
             tma_load_3d(&tmA, full + stage, sA + s * A_BYTES, k, q.prob * a.Mp + q.m0, s);
@@ -471,7 +473,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
           for (int i = 0; i < CW; ++i) few = few || ((cols >> i & 1u) && acc[0][i] < line);
           if (few && rowok) a.guard[(int64_t)q.prob * GUARD_WORDS + GUARD_FAIL] = 1;
         }
-      } else if (q.n_chunks > 0) {
+      } else if (q.n_chunks > 0 || a.zero) {
         // the CW columns of this warp are shared by its lanes (the lanes are rows): lane i
         // finds column i's offset and exponent once, the loop takes them by shuffle
         const int* expB = a.expB + (int64_t)q.prob * a.ebsB;
@@ -1043,12 +1045,14 @@ std::map<TuneKey, int> g_tuned;
 
 namespace {
 // The SIMT kernel walks K at ~1 us (real) or ~4 us (complex) per 16 terms whatever M and N
-// are, the split costs ~10 us of launches more.  cbc_gemm in all, SIMT / split:
-//   real     256 x 256: K = 16 46 / 57 us, 64 100 / 58; 128 x 128 x 32 63 / 56;
-//            1000 x 1000 x 16 61 / 79, x 1000 2107 / 142
-//   complex  16 x 16 x 16 96 / 55, 1000 x 1000 x 8 158 / 106, 128 x 2048 x 128 556 / 69,
-//            1000^3 8097 / 389 us
-constexpr int SPLIT_MIN_K_REAL = 28, SPLIT_MIN_K_CPLX = 8;
+// are, the split costs ~20 us of launches more.  cbc_gemm in all, SIMT / split / SIMT behind the
+// split, us:
+//   real     256 x 256 x 64 104 / 72 / 79; 1000 x 1000 x 28 101 / 84 / 121, x 1000 2115 / 149 / 1978
+//   complex  16 x 16 x 16 102 / 59 / 69, 1000 x 1000 x 8 163 / 101 / 178, 128 x 2048 x 128
+//            563 / 87 / 328
+// So the line for real K is higher where the SIMT tiles alone fill the GPU.
+constexpr int SPLIT_MIN_K_REAL = 28, SPLIT_MIN_K_REAL_BIG = 33, SPLIT_MIN_K_CPLX = 8;
+constexpr double SPLIT_BIG = 3e5;
 constexpr size_t SPLIT_MAX_BYTES = size_t(16) << 30;
 }  // namespace
 
@@ -1149,6 +1153,8 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
     args.vc = vc;
     args.status = status;
     args.guard = opt.guard;
+    args.zero = opt.zero ? 1 : 0;
+    args.atom_step = 1;
     args.guard_k = g.K2;
     args.acc = opt.acc;
     args.base = opt.base ? static_cast<const char*>(opt.base) : args.C;
@@ -1167,14 +1173,17 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
     args.total_tiles = args.tiles_m * args.tiles_n * splits * nb;
     dim3 grid(std::min(args.total_tiles, g_sms));
     if (opt.guard) {
-      // the magnitudes' product first, for the problems that the counts don't decide
-      constexpr int CB = 64;
+      // the magnitudes' product first, for the problems that the counts don't decide; of a long
+      // K at most 32 atoms evenly apart (a part of the sum is below it too: 64 x 64 x 8192 on
+      // one CTA 58 us with all of its 128 atoms)
+      constexpr int CB = 64, CHECK_ATOMS = 32;
       CUtensorMap ca, cb;
       if (!make_map(&ca, sa + 8 * pk.plane_a, g.K2p, nb * g.Mp, 1, BM) ||
           !make_map(&cb, sb + 8 * pk.plane_b, g.K2p, nb * g.N2p, 1, CB))
         return cudaErrorInvalidValue;
       TcArgs c = args;
-      c.atoms_total = g.K2p / ka(1);
+      c.atom_step = (g.K2p / ka(1) + CHECK_ATOMS - 1) / CHECK_ATOMS;
+      c.atoms_total = (g.K2p / ka(1) + c.atom_step - 1) / c.atom_step;
       c.atoms_per_chunk = atoms_per_chunk_for(1);
       c.atoms_per_split = (c.atoms_total + c.atoms_per_chunk - 1) / c.atoms_per_chunk * c.atoms_per_chunk;
       c.splits = 1;
@@ -1236,7 +1245,8 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
 // does it.  Relative error against 80-bit sums, Gaussian entries: 4e-17 to 2e-16 where the SIMT kernel
 // has 1e-16 (K = 16) to 1e-15 (K = 1000).
 size_t gemm_f64_split_bytes(int M, int N, int K, bool cplx, int nb) {
-  if (K < (cplx ? SPLIT_MIN_K_CPLX : SPLIT_MIN_K_REAL)) return 0;
+  const bool big = (double)M * N * nb > SPLIT_BIG;
+  if (K < (cplx ? SPLIT_MIN_K_CPLX : big ? SPLIT_MIN_K_REAL_BIG : SPLIT_MIN_K_REAL)) return 0;
   const size_t b = gemm_tc_workspace_bytes(M, N, K, cplx, 9, nb) +  // (8 slices, the magnitudes)
                    tc::a256(sizeof(int) * GUARD_WORDS * nb);
   return b <= SPLIT_MAX_BYTES ? b : 0;
@@ -1248,6 +1258,7 @@ cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& 
                            int* status, cudaStream_t s) {
   TcWide opt;
   opt.guard = static_cast<int*>(ws);
+  opt.zero = gemm_f64_adds(M, N, K, nb);
   const size_t gb = tc::a256(sizeof(int) * GUARD_WORDS * nb);
   cudaError_t e = cudaMemsetAsync(ws, 0, gb, s);
   if (e != cudaSuccess) return e;

@@ -133,3 +133,15 @@ def test_entries_where_counts_are_too_few(r, shape, cplx):
     B[:, -1] *= np.where(h == 1.0, 2.0 ** -r, 1.0)
     B[7, -1] = 2.0
     _check(A, B)
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("shape", [(64, 64, 8192), (33, 45, 300), (65, 130, 255), (64, 64, 256),
+                                   (31, 33, 40), (700, 1900, 30), (1300, 1040, 33)])
+def test_products_turned_down(shape, cplx):
+    """Operands graded against each other: few and many tiles of either size, split along K
+    (sums added into the zeros that the tensor-core kernel leaves) and not."""
+    rng = np.random.default_rng([*shape, cplx])
+    M, N, K = shape
+    w = 2.0 ** -np.linspace(0, 45, K)
+    _check(_rand(rng, (M, K), cplx) * w, _rand(rng, (K, N), cplx) * w[::-1][:, None])
