@@ -584,11 +584,12 @@ __device__ __forceinline__ long long digit_word(double x, int e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7ffu);
   const unsigned long long mant = (b & 0xfffffffffffffull) | (ex ? (1ull << 52) : 0ull);
-  // N = mant 2^-sh; the largest exponent of a row, ex = e + 1022, has the smallest sh
+  // N = mant 2^-sh; the largest exponent of a row, ex = e + 1022, has the smallest sh: -9 for 8
+  // slices, 14 and more for up to 5, or less where the whole row is subnormal
   constexpr int MIN_SH = 53 - head(S) - 8 * (S - 1);
   const int sh = MIN_SH + e + 1022 - (ex ? ex : 1);
   unsigned long long n;
-  if (MIN_SH < 1 && sh <= 0)
+  if (sh <= 0)
     n = mant << -sh;
   else
     n = sh < 64 ? (mant + ((1ull << (sh - 1)) - 1ull) + ((mant >> sh) & 1ull)) >> sh : 0ull;
