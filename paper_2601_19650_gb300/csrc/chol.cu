@@ -612,6 +612,7 @@ size_t trsm_products_bytes(int m, int n, bool cplx, int nb, bool df) {
   if ((double)m * m * n * nb * (cplx ? 4 : 1) < line * ((m + TRB - 1) / TRB)) return 0;
   const size_t ts = cplx ? sizeof(zdbl) : sizeof(double);
   const size_t nblk = (m + TRB - 1) / TRB;
+  if (nb * nblk > TC_MAX_PROBLEMS) return 0;  // (the blocks' inverses are one call)
   size_t g = gemm_tc_workspace_bytes(TRH, TRH, TRH, cplx, 8, (int)(nb * nblk));
   g = std::max(g, gemm_tc_workspace_bytes(std::min(TRB, m), n, m, cplx, 8, nb));
   return 256 + al256(2 * nb * nblk * TRB * TRB * ts) + al256(nb * nblk * TRH * TRH * ts) +

@@ -1251,6 +1251,7 @@ size_t eig_bt_bytes(int m, int kmax, bool cplx, int nb) {
   if (!bt_products(m, kmax, nb)) return 0;
   const size_t ts = cplx ? sizeof(zdbl) : sizeof(double);
   const size_t nblk = (m + BT_NB - 1) / BT_NB;
+  if (nb * nblk > TC_MAX_PROBLEMS) return 0;  // (the blocks' T are one call)
   return align256(sizeof(int) * nb) + align256(2 * nb * nblk * BT_NB * BT_NB * ts) +
          align256(nb * nblk * BT_HALF * BT_HALF * ts) + align256((size_t)nb * BT_NB * kmax * ts) +
          bt_gemm_bytes(m, kmax, cplx, nb);

@@ -91,6 +91,7 @@ struct TcWide {
   const void* base = nullptr;
   int64_t base_bs = 0;
 };
+constexpr int TC_MAX_PROBLEMS = 65535;  // of one call
 size_t gemm_tc_workspace_bytes(int M, int N, int K, bool cplx, int S, int nb = 1);
 template <typename T>
 cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA, const T* B,
