@@ -51,7 +51,7 @@ int heev_t(int m, int kmax, int nb, T* A, double* lam, T* U, bool mixed, cudaStr
   // without room for the back transformation by products the call takes the other way
   void* bt = nullptr;
   const size_t btb = eig_bt_bytes(m, kmax, ops<T>::cplx, nb);
-  if (btb > 0 && pool_malloc(&bt, btb, s) != cudaSuccess) {
+  if (btb > 0 && scratch_malloc(&bt, btb, s) != cudaSuccess) {
     cudaGetLastError();
     bt = nullptr;
   }
@@ -83,7 +83,7 @@ int cholqr2_t(int m, int n, int nb, T* S, cudaStream_t s) {
   if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), s);
   void* tw = nullptr;
   const size_t tb = trsm_products_bytes(m, n, ops<T>::cplx, nb, false);
-  if (e == cudaSuccess && tb > 0 && pool_malloc(&tw, tb, s) != cudaSuccess) {
+  if (e == cudaSuccess && tb > 0 && scratch_malloc(&tw, tb, s) != cudaSuccess) {
     cudaGetLastError();  // without room the solve takes the other way
     tw = nullptr;
   }

@@ -39,7 +39,7 @@ struct Arena {
   // room that the caller can do without: NULL, and no error kept, when there is none
   void* try_get(size_t bytes) {
     void* p = nullptr;
-    if (pool_malloc(&p, bytes, s) != cudaSuccess) {
+    if (scratch_malloc(&p, bytes, s) != cudaSuccess) {
       cudaGetLastError();
       return nullptr;
     }

@@ -117,6 +117,8 @@ void note_flops(int cls, double flops);
 // stream-ordered device allocation from the library's own pool on the current device
 // (freed with cudaFreeAsync); the caller's default pool is never touched
 cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t s);
+// the same for workspaces that callers can do without; large ones are not kept
+cudaError_t scratch_malloc(void** p, size_t bytes, cudaStream_t s);
 
 // gemm_f64_split with slices from the library's pool where that is the faster way and the
 // pool has room for them, else gemm_f64
@@ -126,7 +128,7 @@ cudaError_t gemm_f64_pooled(int M, int N, int K, int nb, const T* A, const View&
                             int* status, cudaStream_t s) {
   void* ws = nullptr;
   const size_t wb = gemm_f64_split_bytes(M, N, K, ops<T>::cplx, nb);
-  if (wb > 0 && pool_malloc(&ws, wb, s) == cudaSuccess) {
+  if (wb > 0 && scratch_malloc(&ws, wb, s) == cudaSuccess) {
     cudaError_t e = gemm_f64_split<T>(M, N, K, nb, A, va, conjA, B, vb, conjB, C, vc, ws, status, s);
     const cudaError_t f = cudaFreeAsync(ws, s);
     return e != cudaSuccess ? e : f;
