@@ -138,8 +138,9 @@ int cbc_apply(ttn_t state, ttno_t op, int64_t max_bond, double tol,
 
 /* Apply n operators to n states (independent instances of any sizes and topologies)
  * and compress each; the results equal n calls of cbc_apply.  Tensor-train instances
- * with identical shapes (sites, physical and bond dimensions, real/complex), max_bond
- * and tol form groups of up to opt->max_group (default 32) that run in lockstep: every step of Sec. III A is one
+ * with identical shapes (sites, physical and bond dimensions, real/complex; in the mixed
+ * path also 32-bit or 64-bit data), max_bond and tol form groups of up to opt->max_group
+ * (default 32) that run in lockstep: every step of Sec. III A is one
  * launch for the whole group, on the stream of the group's first state (the group waits
  * for the other members' streams first and has finished when the call returns).  A
  * group whose members choose different ranks at some cut is rerun member by member.

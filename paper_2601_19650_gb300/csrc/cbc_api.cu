@@ -560,11 +560,16 @@ int cbc_apply_batched(int n, const ttn_t* states, const ttno_t* ops, const int64
   for (int j = 0; j < n; ++j) outs[j] = nullptr;
   if (n == 0) return CBC_OK;
   // groups: chains with identical shapes, max_bond and tol (at most kMaxGroup each) run
-  // in lockstep, one launch per step for the whole group; the rest one by one
+  // in lockstep, one launch per step for the whole group; the rest one by one.  64-bit and
+  // 32-bit data in the mixed path take different solvers and so go in different groups.
   int kMaxGroup = 32;
+  bool mixed = false;
   {
     Options o;
-    if (parse_options(opt, &o) == CBC_OK) kMaxGroup = o.max_group;
+    if (parse_options(opt, &o) == CBC_OK) {
+      kMaxGroup = o.max_group;
+      mixed = o.precision == CBC_PREC_MIXED;
+    }
   }
   std::vector<std::vector<int>> tasks;
   {
@@ -580,6 +585,7 @@ int cbc_apply_batched(int n, const ttn_t* states, const ttno_t* ops, const int64
           const ttn_t s2 = states[l];
           const ttno_t o2 = ops[l];
           if (tasks[open_task[q]].size() < (size_t)kMaxGroup && s2->cplx == st->cplx &&
+              (!mixed || (s2->wide || o2->wide) == (st->wide || op->wide)) &&
               s2->n == st->n && s2->parent == st->parent && s2->phys == st->phys &&
               s2->bond == st->bond && o2->bond == op->bond && o2->parent == op->parent &&
               o2->phys == op->phys && (max_bond ? max_bond[l] == max_bond[j] : true) &&
