@@ -105,15 +105,16 @@ cudaError_t cbc::pool_malloc(void** p, size_t bytes, cudaStream_t s) {
   return e == cudaSuccess ? cudaMallocFromPoolAsync(p, bytes, pool, s) : e;
 }
 
-// Workspaces of 1 GB and more from a pool that gives back what exceeds 4 GB at the next
+// Workspaces of 1 GB and more from a pool that gives back what exceeds 8 GB at the next
 // synchronisation, so that one very large product does not keep its slices for good.  Below
 // that nothing is mapped anew: 2.1 ms per GB, complex 4096 x 4096 x 4096 (1.8 GB of slices)
-// 15.4 ms, 19.2 if they went back each time.
+// 15.4 ms, 19.2 if they went back each time.  (The Gram products of 128 benchmark instances in
+// FP64 have 7.2 GB of slices, at every cut.)
 cudaError_t cbc::scratch_malloc(void** p, size_t bytes, cudaStream_t s) {
   if (bytes < (size_t(1) << 30)) return pool_malloc(p, bytes, s);
   static cudaMemPool_t pools[64] = {};
   cudaMemPool_t pool;
-  cudaError_t e = device_pool(pools, uint64_t(4) << 30, &pool);
+  cudaError_t e = device_pool(pools, uint64_t(8) << 30, &pool);
   return e == cudaSuccess ? cudaMallocFromPoolAsync(p, bytes, pool, s) : e;
 }
 

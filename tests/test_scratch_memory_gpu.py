@@ -1,5 +1,5 @@
-"""The slices of a large FP64 product (7.2 GB here) are given back when the call is done, but for
-the 4 GB that the library keeps."""
+"""The slices of a large FP64 product (10.9 GB here) are given back when the call is done, but for
+the 8 GB that the library keeps."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -9,7 +9,7 @@ def test_large_product_gives_its_slices_back():
     import torch
 
     from paper_2601_19650_gb300 import _cbc as c
-    n = 8192
+    n = 10000
     A = torch.randn(n, n, dtype=torch.complex128, device="cuda")
     B = torch.randn(n, n, dtype=torch.complex128, device="cuda")
     C = torch.empty_like(A)
@@ -22,6 +22,6 @@ def test_large_product_gives_its_slices_back():
     free = torch.cuda.mem_get_info()[0]
     for _ in range(2):
         gemm(n)
-        assert free - torch.cuda.mem_get_info()[0] < 9 << 29
+        assert free - torch.cuda.mem_get_info()[0] < 17 << 29
     ref = A[:2] @ B
     assert (C[:2] - ref).abs().max() < 1e-11 * n ** 0.5
