@@ -174,9 +174,11 @@ SimtShape simt_shape(int M, int N, int K, int batch, bool guard) {
   s.edge = guard && count(64) < target ? 32 : 64;
   s.tiles = count(s.edge);
   const int ksteps = (K + BK - 1) / BK;
+  // (by the 64 x 64 tiles in either case: partial sums as long as without a split product before)
+  const int tiles64 = count(64);
   s.splits = 1;
-  if (s.tiles < target && ksteps >= 16) {
-    s.splits = (target + s.tiles - 1) / s.tiles;
+  if (tiles64 < target && ksteps >= 16) {
+    s.splits = (target + tiles64 - 1) / tiles64;
     s.splits = min(s.splits, ksteps / 8);
     s.splits = max(s.splits, 1);
   }

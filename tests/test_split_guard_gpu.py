@@ -145,3 +145,17 @@ def test_products_turned_down(shape, cplx):
     M, N, K = shape
     w = 2.0 ** -np.linspace(0, 45, K)
     _check(_rand(rng, (M, K), cplx) * w, _rand(rng, (K, N), cplx) * w[::-1][:, None])
+
+
+def test_error_of_products_turned_down():
+    """Equal positive terms, whose roundings add up along a partial sum: the split of K keeps
+    them as short as on the SIMT kernel alone (3 parts of 344 terms: 344 / 2 roundings at most
+    of half a unit of the running sum, which is half of the whole on average, and one for each
+    part)."""
+    from test_gemm_gpu import _run
+    M, N, K = 501, 777, 1030
+    A = np.full((M, K), 1 / 3.0) + 0j
+    B = np.full((K, N), 1 / 7.0) + 0j
+    C, _ = _run(0, 0, A, B)
+    ref = float(K * (np.longdouble(1 / 3.0) * np.longdouble(1 / 7.0)))
+    assert np.abs(C - ref).max() <= (344 / 4 + 3) * 2.0 ** -53 * ref
