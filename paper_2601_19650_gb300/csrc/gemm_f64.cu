@@ -138,7 +138,8 @@ __global__ void __launch_bounds__(NT) gemm_f64_kernel(GemmArgs<T> g) {
 }
 
 template <typename T>
-__global__ void zero_view_kernel(T* C, View vc, int M, int N, int batch) {
+__global__ void zero_view_kernel(T* C, View vc, int M, int N, int batch, const int* guard) {
+  if (guard && batch == 1 && split_holds(guard)) return;
   int64_t total = (int64_t)M * N * batch;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
        t += (int64_t)gridDim.x * blockDim.x) {
@@ -146,6 +147,7 @@ __global__ void zero_view_kernel(T* C, View vc, int M, int N, int batch) {
     int64_t rb = t / N;
     int r = (int)(rb % M);
     int b = (int)(rb / M);
+    if (guard && batch > 1 && split_holds(guard + b * GUARD_WORDS)) continue;
     C[(int64_t)b * vc.bs + vc.roff(r) + vc.coff(c)] = ops<T>::zero();
   }
 }
@@ -155,9 +157,8 @@ int g_num_sms = 0;
 // How a product is dealt to the CTAs.  Behind a split product (guard) tiles of 32 x 32 where
 // those of 64 x 64 leave SMs idle: the same sums in the same order, and what the slicing cost is
 // won back.  A product that the split turns down, cbc_gemm in all, on the SIMT kernel at once /
-// behind the split, us: real 256 x 256 x 64 104 / 79, 64 x 64 x 8192 181 / 181 (without a split
-// of K 9700), complex 64 x 128 x 256 567 / 210, 501 x 777 x 1030 4158 / 3290, 1000 x 1000 x 8
-// 163 / 178.
+// behind the split, us: real 256 x 256 x 64 104 / 82, 64 x 64 x 8192 181 / 194 (without a split
+// of K 9700), complex 64 x 128 x 256 565 / 220, 501 x 777 x 1030 4257 / 3155.
 struct SimtShape {
   int edge, tiles, splits, kchunk;
 };
@@ -189,10 +190,6 @@ SimtShape simt_shape(int M, int N, int K, int batch, bool guard) {
 
 }  // namespace
 
-bool gemm_f64_adds(int M, int N, int K, int batch) {
-  return simt_shape(M, N, K, batch, true).splits > 1;
-}
-
 template <typename T>
 cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va, bool conjA,
                      const T* B, const View& vb, bool conjB, T* C, const View& vc,
@@ -202,17 +199,17 @@ cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va,
   const int edge = sh.edge, tiles = sh.tiles, splits = sh.splits;
   if (K <= 0) {  // empty contraction: C = 0
     note_launches(CBC_K_GEMM_F64, 1);
-    zero_view_kernel<T><<<256, 256, 0, s>>>(C, vc, M, N, batch);
+    zero_view_kernel<T><<<256, 256, 0, s>>>(C, vc, M, N, batch, nullptr);
     return cudaGetLastError();
   }
   GemmArgs<T> g{M,  N, K,  splits, sh.kchunk, A, va, B, vb, C, vc, guard,
                 (N + edge - 1) / edge, (M + edge - 1) / edge, tiles * splits};
   // a product that usually does not run (guard) is launched as one resident wave
   const int grid = guard ? std::min(g.total, 2 * g_num_sms) : g.total;
-  note_launches(CBC_K_GEMM_F64, splits > 1 && !guard ? 2 : 1);
-  if (splits > 1 && !guard) {  // (gemm_f64_adds: the split leaves zeros)
-    int zb = (int)std::min<int64_t>(4096, ((int64_t)M * N * batch + 255) / 256);
-    zero_view_kernel<T><<<zb, 256, 0, s>>>(C, vc, M, N, batch);
+  note_launches(CBC_K_GEMM_F64, splits > 1 ? 2 : 1);
+  if (splits > 1) {
+    int zb = (int)std::min<int64_t>(guard ? g_num_sms : 4096, ((int64_t)M * N * batch + 255) / 256);
+    zero_view_kernel<T><<<zb, 256, 0, s>>>(C, vc, M, N, batch, guard);
   }
 #define CBC_GEMM_LAUNCH(CA, CB)                                                     \
   if (edge == 32 && splits > 1)                                                     \

@@ -198,7 +198,6 @@ struct TcArgs {
   int atoms_total;       // K2_pad / ka(S)
   int atoms_per_split;   // multiple of atoms_per_chunk
   int atoms_per_chunk;
-  int atom_step;         // every how many atoms one is taken (S = 1; else 1)
   const int* expA;       // [M_pad]
   const int* expB;       // [N_pad] (one per complex column when cplx)
   int cplx;
@@ -206,9 +205,10 @@ struct TcArgs {
   char* C;               // FP64 output (double or zdbl) through the view
   View vc;               // vc.bs: elements between the outputs of consecutive problems
   int* status;
-  int* guard;            // not NULL: nothing, or C = 0 (zero), for problems that it turns down
-  int zero;              // (gemm_f64_split)
+  int* guard;            // not NULL: the words of split_guard.cuh (gemm_f64_split)
   int guard_k;           // terms of the real sums
+  int check_atoms;       // atoms of the magnitudes' product, check_step apart
+  int check_step;
   int acc;               // 1 or -1: base + A B or base - A B instead of A B
   const char* base;      // rows and columns as C's (C itself when it is split along K)
   int64_t base_shift;    // base's bytes from problem to problem less C's
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
   constexpr int A_BYTES = BM * KAS * 2;
   constexpr int B_BYTES = BN * KAS * 2;
   constexpr int STAGE_BYTES = S * (A_BYTES + B_BYTES);
-  constexpr uint32_t TMEM_COLS = S == 1 ? 2 * BN : 512;
+  constexpr uint32_t TMEM_COLS = 512;
   static_assert(2 * S * BN <= (int)TMEM_COLS, "TMEM budget");  // hence S BN <= 256, the widest MMA
   static_assert(BN % 16 == 0, "MMA width");
   extern __shared__ uint8_t smem_raw[];
@@ -289,11 +289,13 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
   // across tiles, so one tile's epilogue overlaps the next tile's loads and MMAs.
   struct Tile {
     int m0, n0, prob, a_begin, n_atoms, n_chunks;
+    bool check;
   };
-  // S = 1: the entries of sum |a||b| against the line of split_guard.cuh, for the problems whose
-  // counts are too few; no output but the guard's word
+  // FP64 products (a.guard): nothing runs for a problem with Inf or NaN, and the tiles of one with
+  // too few counts begin with a chunk of their own, the product of the magnitudes, whose entries
+  // the epilogue holds against the line of split_guard.cuh
   int seen = -1;  // the last problem whose guard was looked at
-  bool runs = true;
+  bool bad = false, few = false;
   auto tile_of = [&](int t) {
     Tile q;
     const int mt = t % a.tiles_m, r = t / a.tiles_m;
@@ -303,12 +305,14 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
     q.prob = z / a.splits;
     q.a_begin = (z % a.splits) * a.atoms_per_split;
     q.n_atoms = max(0, min(a.atoms_total, q.a_begin + a.atoms_per_split) - q.a_begin);
-    if (a.guard && q.prob != seen) {
+    if (S > 5 && a.guard && q.prob != seen) {
       seen = q.prob;
       const int* g = a.guard + (int64_t)q.prob * GUARD_WORDS;
-      runs = S == 1 ? !g[GUARD_BAD] && !counts_hold(g, a.guard_k) : split_holds(g);
+      bad = g[GUARD_BAD];
+      few = !bad && !counts_hold(g, a.guard_k);
     }
-    if (!runs) q.n_atoms = 0;  // (no role but the epilogue has anything to do in the tile)
+    if (bad) q.n_atoms = 0;  // (no role has anything to do in the tile)
+    q.check = few && q.a_begin == 0;
     q.n_chunks = (q.n_atoms + a.atoms_per_chunk - 1) / a.atoms_per_chunk;
     return q;
   };
@@ -345,6 +349,21 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
       bool run = true;
       for (int t = blockIdx.x; t < a.total_tiles && run; t += gridDim.x) {
         const Tile q = tile_of(t);
+        if (S > 5 && q.check) {
+          for (int j = 0; j < a.check_atoms; ++j, ++jg) {
+            const int stage = jg % NSTAGE, use = jg / NSTAGE;
+            if (!mbar_wait(empty + stage, (use & 1) ^ 1, abort_flag, a.status)) {
+              run = false;
+              break;
+            }
+            uint8_t* sA = smem + stage * STAGE_BYTES;
+            mbar_expect_tx(full + stage, A_BYTES + B_BYTES);
+            const int k = j * a.check_step * KAS;
+            tma_load_3d(&tmA, full + stage, sA, k, q.prob * a.Mp + q.m0, S);
+            tma_load_3d(&tmB, full + stage, sA + S * A_BYTES, k, q.prob * a.N2p + q.n0, S);
+          }
+          if (!run) break;
+        }
         for (int j = 0; j < q.n_atoms; ++j, ++jg) {
           const int stage = jg % NSTAGE, use = jg / NSTAGE;
           if (!mbar_wait(empty + stage, (use & 1) ^ 1, abort_flag, a.status)) {
@@ -354,7 +373,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
           uint8_t* sA = smem + stage * STAGE_BYTES;
           uint8_t* sB = sA + S * A_BYTES;
           mbar_expect_tx(full + stage, STAGE_BYTES);
-          const int k = (q.a_begin + j) * KAS * a.atom_step;
+          const int k = (q.a_begin + j) * KAS;
 #pragma unroll
           for (int s = 0; s < S; ++s) {
             tma_load_3d(&tmA, full + stage, sA + s * A_BYTES, k, q.prob * a.Mp + q.m0, s);
@@ -370,6 +389,29 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
       bool run = true;
       for (int t = blockIdx.x; t < a.total_tiles && run; t += gridDim.x) {
         const Tile q = tile_of(t);
+        if (S > 5 && q.check) {
+          const int buf = cg & 1, use = cg >> 1;
+          if (!mbar_wait(tempty + buf, (use & 1) ^ 1, abort_flag, a.status)) break;
+          tc_fence_after();
+          for (int j = 0; j < a.check_atoms; ++j, ++jg) {
+            const int stage = jg % NSTAGE, su = jg / NSTAGE;
+            if (!mbar_wait(full + stage, su & 1, abort_flag, a.status)) {
+              run = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t sA = smem_u32(smem + stage * STAGE_BYTES);
+#pragma unroll
+            for (int kk = 0; kk < KAS / 16; ++kk)
+              umma_bf16(tmem_base + (uint32_t)(buf * S * BN), sdesc<2 * KAS>(sA + kk * 32),
+                        sdesc<2 * KAS>(sA + S * A_BYTES + kk * 32), idesc_bf16(BM, BN),
+                        (j == 0 && kk == 0) ? 0u : 1u);
+            umma_commit(empty + stage);
+          }
+          if (!run) break;
+          umma_commit(tfull + buf);
+          ++cg;
+        }
         int j = 0;
         for (int c = 0; c < q.n_chunks; ++c, ++cg) {
           const int buf = cg & 1, use = cg >> 1;
@@ -428,6 +470,30 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
     for (int t = blockIdx.x; t < a.total_tiles && run; t += gridDim.x) {
       const Tile q = tile_of(t);
       const int row = q.m0 + quarter * 32 + lane;
+      if (S > 5 && q.check) {
+        const int buf = cg & 1, use = cg >> 1;
+        if (!mbar_wait(tfull + buf, use & 1, abort_flag, a.status)) break;
+        tc_fence_after();
+        uint32_t r[CW];
+        tmem_ld<CW>(tmem_base + ((uint32_t)(quarter * 32) << 16) +
+                        (uint32_t)(buf * S * BN + colg * CW), r);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty + buf);
+        ++cg;
+        const int mycol = q.n0 + colg * CW + lane;
+        const bool colok =
+            lane < CW && mycol < a.N2 &&
+            a.expB[(int64_t)q.prob * a.ebsB + (a.cplx ? mycol >> 1 : mycol)] != GUARD_ZERO_ROW;
+        const unsigned cols = __ballot_sync(0xffffffffu, colok);
+        const bool rowok = row < a.M && a.expA[q.prob * a.Mp + row] != GUARD_ZERO_ROW;
+        const float line = 0x1p14f * guard_line(a.guard_k);
+        bool below = false;
+#pragma unroll
+        for (int i = 0; i < CW; ++i)
+          below = below || ((cols >> i & 1u) && __uint_as_float(r[i]) < line);
+        if (below && rowok) a.guard[(int64_t)q.prob * GUARD_WORDS + GUARD_FAIL] = 1;
+      }
       // 8 slices span 2 x 32 bits more than one int64 holds: levels 0-3 and 4-7 apart
       constexpr int NACC = S > 5 ? 2 : 1;
       constexpr int LV = S / NACC;  // levels per accumulator
@@ -459,21 +525,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
         if (lane == 0) mbar_arrive(tempty + buf);
       }
       if (!run) break;
-      if constexpr (S == 1) {
-        if (q.n_chunks > 0) {
-          const int mycol = q.n0 + colg * CW + lane;
-          const bool colok =
-              lane < CW && mycol < a.N2 &&
-              a.expB[(int64_t)q.prob * a.ebsB + (a.cplx ? mycol >> 1 : mycol)] != GUARD_ZERO_ROW;
-          const unsigned cols = __ballot_sync(0xffffffffu, colok);
-          const bool rowok = row < a.M && a.expA[q.prob * a.Mp + row] != GUARD_ZERO_ROW;
-          const long long line = (long long)ceilf(0x1p14f * guard_line(a.guard_k));
-          bool few = false;
-#pragma unroll
-          for (int i = 0; i < CW; ++i) few = few || ((cols >> i & 1u) && acc[0][i] < line);
-          if (few && rowok) a.guard[(int64_t)q.prob * GUARD_WORDS + GUARD_FAIL] = 1;
-        }
-      } else if (q.n_chunks > 0 || a.zero) {
+      if (q.n_chunks > 0) {
         // the CW columns of this warp are shared by its lanes (the lanes are rows): lane i
         // finds column i's offset and exponent once, the loop takes them by shuffle
         const int* expB = a.expB + (int64_t)q.prob * a.ebsB;
@@ -940,10 +992,11 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-bool make_map(CUtensorMap* m, void* base, int K2_pad, int64_t rows_pad, int S, int box_rows) {
+bool make_map(CUtensorMap* m, void* base, int K2_pad, int64_t rows_pad, int S, int planes,
+              int box_rows) {
   auto fn = encode_fn();
   if (!fn) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)K2_pad, (cuuint64_t)rows_pad, (cuuint64_t)S};
+  cuuint64_t dims[3] = {(cuuint64_t)K2_pad, (cuuint64_t)rows_pad, (cuuint64_t)planes};
   cuuint64_t strides[2] = {(cuuint64_t)K2_pad * 2, (cuuint64_t)rows_pad * K2_pad * 2};
   cuuint32_t box[3] = {(cuuint32_t)ka(S), (cuuint32_t)box_rows, 1};
   cuuint32_t es[3] = {1, 1, 1};
@@ -954,7 +1007,7 @@ bool make_map(CUtensorMap* m, void* base, int K2_pad, int64_t rows_pad, int S, i
   return r == CUDA_SUCCESS;
 }
 
-// (S = 1: 1024 products below 2^14)
+constexpr int CHECK_ATOMS = 64;  // of 32 entries, of the magnitudes' product
 int atoms_per_chunk_for(int S) { return std::max(1, (1024 / S) / ka(S)); }
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -1018,7 +1071,6 @@ cudaError_t launch_bn(const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs
 cudaError_t launch(int S, int BN, const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs& args,
                    dim3 grid, cudaStream_t s) {
   switch (S * 1000 + BN) {
-    case 1064: return launch_bn<1, 64>(ma, mb, args, grid, s);
     case 2064: return launch_bn<2, 64>(ma, mb, args, grid, s);
     case 3064: return launch_bn<3, 64>(ma, mb, args, grid, s);
     case 4032: return launch_bn<4, 32>(ma, mb, args, grid, s);
@@ -1046,14 +1098,15 @@ std::map<TuneKey, int> g_tuned;
 
 namespace {
 // The SIMT kernel walks K at ~1 us (real) or ~4 us (complex) per 16 terms whatever M and N
-// are, the split costs ~20 us of launches more.  cbc_gemm in all, SIMT / split / SIMT behind the
-// split, us:
-//   real     256 x 256 x 64 104 / 72 / 79; 1000 x 1000 x 28 101 / 84 / 121, x 1000 2115 / 149 / 1978
-//   complex  16 x 16 x 16 102 / 59 / 69, 1000 x 1000 x 8 163 / 101 / 178, 128 x 2048 x 128
-//            563 / 87 / 328
-// So the line for real K is higher where the SIMT tiles alone fill the GPU.
-constexpr int SPLIT_MIN_K_REAL = 28, SPLIT_MIN_K_REAL_BIG = 33, SPLIT_MIN_K_CPLX = 8;
-constexpr double SPLIT_BIG = 3e5;
+// are, the split costs ~15 us of launches more.  cbc_gemm in all, SIMT / split / SIMT behind the
+// split (operands graded against each other), us:
+//   real     256 x 256 x 64 104 / 58 / 82; 1000 x 1000 x 28 101 / 78 / 125,
+//            x 1000 2117 / 139 / 2030
+//   complex  16 x 16 x 16 102 / 57 / 78, 1000 x 1000 x 8 164 / 94 / 211, x 24 297 / 91 / 321,
+//            128 x 2048 x 128 565 / 78 / 340
+// So a product that is turned down costs up to a quarter more where K is short and the tiles fill
+// the GPU, up to 8% more elsewhere, and less where the smaller tiles win.
+constexpr int SPLIT_MIN_K_REAL = 28, SPLIT_MIN_K_CPLX = 8;
 constexpr size_t SPLIT_MAX_BYTES = size_t(16) << 30;
 }  // namespace
 
@@ -1100,7 +1153,8 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
   char* w = static_cast<char*>(ws);
   w = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(w) + 255) & ~uintptr_t(255));
   const size_t b = (size_t)nb;
-  const size_t planes = b * (S + (opt.guard ? 1 : 0));
+  const int planes1 = S + (opt.guard ? 1 : 0);  // of one problem: the magnitudes behind the slices
+  const size_t planes = b * planes1;
   __nv_bfloat16* sa = reinterpret_cast<__nv_bfloat16*>(w);
   w += a256(planes * g.Mp * g.K2p * 2);
   __nv_bfloat16* sb = reinterpret_cast<__nv_bfloat16*>(w);
@@ -1125,7 +1179,7 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
   cudaError_t pe = pack_operands<T>(pk, S, nb, s);
   if (pe != cudaSuccess) return pe;
   CUtensorMap ma;
-  if (!make_map(&ma, sa, g.K2p, nb * g.Mp, S, BM)) return cudaErrorInvalidValue;
+  if (!make_map(&ma, sa, g.K2p, nb * g.Mp, S, planes1, BM)) return cudaErrorInvalidValue;
   const int atoms = g.K2p / ka(S);
   const int apc = atoms_per_chunk_for(S);
   const int chunks = (atoms + apc - 1) / apc;
@@ -1133,7 +1187,7 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
   // rows (or the zero fill past the planes) for columns the epilogue never writes
   auto run_bn = [&](int BN) -> cudaError_t {
     CUtensorMap mb;
-    if (!make_map(&mb, sb, g.K2p, nb * g.N2p, S, BN)) return cudaErrorInvalidValue;
+    if (!make_map(&mb, sb, g.K2p, nb * g.N2p, S, planes1, BN)) return cudaErrorInvalidValue;
     const int tiles_n = (g.N2p + BN - 1) / BN;
     const int tiles = (g.Mp / BM) * tiles_n * nb;
     int splits = 1;
@@ -1154,8 +1208,10 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
     args.vc = vc;
     args.status = status;
     args.guard = opt.guard;
-    args.zero = opt.zero ? 1 : 0;
-    args.atom_step = 1;
+    // of a long K at most CHECK_ATOMS atoms of the magnitudes, evenly apart: a part of the sum is
+    // below it too (64 x 64 x 8192 on one CTA 58 us with all of its atoms)
+    args.check_step = (atoms + CHECK_ATOMS - 1) / CHECK_ATOMS;
+    args.check_atoms = (atoms + args.check_step - 1) / args.check_step;
     args.guard_k = g.K2;
     args.acc = opt.acc;
     args.base = opt.base ? static_cast<const char*>(opt.base) : args.C;
@@ -1173,27 +1229,6 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
     args.tiles_n = tiles_n;
     args.total_tiles = args.tiles_m * args.tiles_n * splits * nb;
     dim3 grid(std::min(args.total_tiles, g_sms));
-    if (opt.guard) {
-      // the magnitudes' product first, for the problems that the counts don't decide; of a long
-      // K at most 32 atoms evenly apart (a part of the sum is below it too: 64 x 64 x 8192 on
-      // one CTA 58 us with all of its 128 atoms)
-      constexpr int CB = 64, CHECK_ATOMS = 32;
-      CUtensorMap ca, cb;
-      if (!make_map(&ca, sa + 8 * pk.plane_a, g.K2p, nb * g.Mp, 1, BM) ||
-          !make_map(&cb, sb + 8 * pk.plane_b, g.K2p, nb * g.N2p, 1, CB))
-        return cudaErrorInvalidValue;
-      TcArgs c = args;
-      c.atom_step = (g.K2p / ka(1) + CHECK_ATOMS - 1) / CHECK_ATOMS;
-      c.atoms_total = (g.K2p / ka(1) + c.atom_step - 1) / c.atom_step;
-      c.atoms_per_chunk = atoms_per_chunk_for(1);
-      c.atoms_per_split = (c.atoms_total + c.atoms_per_chunk - 1) / c.atoms_per_chunk * c.atoms_per_chunk;
-      c.splits = 1;
-      c.tiles_n = g.N2p / CB;
-      c.total_tiles = c.tiles_m * c.tiles_n * nb;
-      note_launches(CBC_K_GEMM_F64, 1);
-      cudaError_t e = launch(1, CB, ca, cb, c, dim3(std::min(c.total_tiles, g_sms)), s);
-      if (e != cudaSuccess) return e;
-    }
     note_launches(S == 8 ? CBC_K_GEMM_F64 : CBC_K_GEMM_TC, 1);
     if (S != 8)
       note_flops(CBC_K_TC_ISSUED,
@@ -1242,12 +1277,10 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
 // 8 slices hold 62 bits of an entry relative to its row's (column's) maximum; the kept products
 // of slices are summed exactly and rounded once to 53 bits (once more per K split).  Whether
 // that is as accurate as an FP64 sum is found while the operands are cut (split_guard.cuh);
-// where it is not, the tensor-core kernel leaves the problem out and the SIMT kernel behind it
-// does it.  Relative error against 80-bit sums, Gaussian entries: 4e-17 to 2e-16 where the SIMT kernel
-// has 1e-16 (K = 16) to 1e-15 (K = 1000).
+// where it is not, the SIMT kernel behind does the problem (again).  Relative error against 80-bit sums, Gaussian
+// entries: 4e-17 to 2e-16 where the SIMT kernel has 1e-16 (K = 16) to 1e-15 (K = 1000).
 size_t gemm_f64_split_bytes(int M, int N, int K, bool cplx, int nb) {
-  const bool big = (double)M * N * nb > SPLIT_BIG;
-  if (K < (cplx ? SPLIT_MIN_K_CPLX : big ? SPLIT_MIN_K_REAL_BIG : SPLIT_MIN_K_REAL)) return 0;
+  if (K < (cplx ? SPLIT_MIN_K_CPLX : SPLIT_MIN_K_REAL)) return 0;
   const size_t b = gemm_tc_workspace_bytes(M, N, K, cplx, 9, nb) +  // (8 slices, the magnitudes)
                    tc::a256(sizeof(int) * GUARD_WORDS * nb);
   return b <= SPLIT_MAX_BYTES ? b : 0;
@@ -1259,7 +1292,6 @@ cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& 
                            int* status, cudaStream_t s) {
   TcWide opt;
   opt.guard = static_cast<int*>(ws);
-  opt.zero = gemm_f64_adds(M, N, K, nb);
   const size_t gb = tc::a256(sizeof(int) * GUARD_WORDS * nb);
   cudaError_t e = cudaMemsetAsync(ws, 0, gb, s);
   if (e != cudaSuccess) return e;

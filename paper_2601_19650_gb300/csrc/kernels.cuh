@@ -61,9 +61,7 @@ template <typename T>
 cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va, bool conjA,
                      const T* B, const View& vb, bool conjB, T* C, const View& vc,
                      cudaStream_t s, const int* guard = nullptr);
-// (guard: not NULL: only the problems that split_holds, split_guard.cuh, turns down.  Where
-// gemm_f64_adds says so the sums are then added to C, which must be zero.)
-bool gemm_f64_adds(int M, int N, int K, int batch);
+// (guard: not NULL: only the problems that split_holds, split_guard.cuh, turns down.)
 
 // The FP64 product as 8 bf16 slices per operand on the tensor cores, where their error is no
 // larger than an FP64 sum's; the other problems through gemm_f64 (gemm_tc.cu, split_guard.cuh).  gemm_f64_split_bytes gives the bytes it needs at `ws`, or 0
@@ -80,13 +78,12 @@ cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& 
 // S = 8 (62 bits of every entry, relative to its row's maximum) needs TcWide::wide, device
 // words of which number p / per is set when an operand of problem p holds Inf or NaN, or
 // TcWide::guard, GUARD_WORDS zeroed words per problem: C of a problem that split_holds turns
-// down is left alone or, with `zero`, zeroed.  acc = 1 or -1: base + A B or base - A B into C, with
+// down afterwards is not to be used.  acc = 1 or -1: base + A B or base - A B into C, with
 // base (NULL: C itself) laid out as C but for its problems, base_bs elements apart.
 struct TcWide {
   int* wide = nullptr;
   int per = 0x7fffffff;
   int* guard = nullptr;
-  bool zero = false;
   int acc = 0;
   const void* base = nullptr;
   int64_t base_bs = 0;

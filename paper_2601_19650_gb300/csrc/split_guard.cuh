@@ -13,8 +13,8 @@
 //     2^(ea-t) 2^(eb-v), and summing over the levels
 //       S / 2^(ea+eb) >= sum_{t,v} w_t w_v max(0, K - ma(t) - mb(v)), w_t = 2^-(t+1), w_8 = 2^-8.
 //     Gaussian operands pass from K = 28 on (8000 rows: 2^-10.4 K where 2^-10.6 K is needed);
-//   * where the counts are too few, the product of the magnitudes' leading 7 bits (one slice,
-//     gemm_tc.cu), entry by entry: S / 2^(ea+eb) >= 2^-14 sum_k floor(2^7 |a_k| / 2^ea)
+//   * where the counts are too few, the product of the magnitudes' leading 7 bits, one chunk
+//     more of every tile (gemm_tc.cu), entry by entry: S / 2^(ea+eb) >= 2^-14 sum_k floor(2^7 |a_k| / 2^ea)
 //     floor(2^7 |b_k| / 2^eb).  The contractions and Gram products of a chain pass (by at least a
 //     factor of 4 in the cases looked at), operands graded against each other do not.
 #pragma once
@@ -32,7 +32,8 @@ constexpr int GUARD_ZERO_ROW = -4000;         // exponent of a row of zeros (its
 __device__ __forceinline__ float guard_line(int K) {
   return fmaxf(3.4e-3f * sqrtf((float)K), 0x1p-6f);  // 2^-8.2 sqrt(K)
 }
-__device__ __forceinline__ bool counts_hold(const int* g, int K) {
+// (not inlined: the roles of a kernel must come to one answer)
+static __device__ __noinline__ bool counts_hold(const int* g, int K) {
   float s = 0.f;
 #pragma unroll
   for (int t = 0; t < GUARD_LEVELS; ++t) {
