@@ -36,6 +36,7 @@ template <typename T, bool CA, bool CB, bool ATOMIC, int R>
 __global__ void __launch_bounds__(NT) gemm_f64_kernel(GemmArgs<T> g) {
   using O = ops<T>;
   constexpr int BM = 16 * R, BN = 16 * R;
+  if (g.guard && g.total == g.tiles_m * g.tiles_n * g.splits && split_holds(g.guard)) return;
   __shared__ T As[BK][BM + 1];
   __shared__ T Bs[BK][BN + 1];
   __shared__ int64_t a_row[BM];
@@ -157,8 +158,8 @@ int g_num_sms = 0;
 // How a product is dealt to the CTAs.  Behind a split product (guard) tiles of 32 x 32 where
 // those of 64 x 64 leave SMs idle: the same sums in the same order, and what the slicing cost is
 // won back.  A product that the split turns down, cbc_gemm in all, on the SIMT kernel at once /
-// behind the split, us: real 256 x 256 x 64 104 / 82, 64 x 64 x 8192 181 / 194 (without a split
-// of K 9700), complex 64 x 128 x 256 565 / 220, 501 x 777 x 1030 4257 / 3155.
+// behind the split, us: real 256 x 256 x 64 104 / 77, 64 x 64 x 8192 181 / 166 (without a split
+// of K 9700), complex 64 x 128 x 256 565 / 214, 501 x 777 x 1030 4257 / 3141.
 struct SimtShape {
   int edge, tiles, splits, kchunk;
 };

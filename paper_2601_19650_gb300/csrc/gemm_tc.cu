@@ -291,11 +291,9 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
     int m0, n0, prob, a_begin, n_atoms, n_chunks;
     bool check;
   };
-  // FP64 products (a.guard): nothing runs for a problem with Inf or NaN, and the tiles of one with
-  // too few counts begin with a chunk of their own, the product of the magnitudes, whose entries
-  // the epilogue holds against the line of split_guard.cuh
-  int seen = -1;  // the last problem whose guard was looked at
-  bool bad = false, few = false;
+  // FP64 products (a.guard): nothing runs for a problem with Inf or NaN, and the tiles of the
+  // others begin with a chunk of their own, the product of the magnitudes, whose entries the
+  // epilogue holds against the line of split_guard.cuh
   auto tile_of = [&](int t) {
     Tile q;
     const int mt = t % a.tiles_m, r = t / a.tiles_m;
@@ -305,14 +303,13 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
     q.prob = z / a.splits;
     q.a_begin = (z % a.splits) * a.atoms_per_split;
     q.n_atoms = max(0, min(a.atoms_total, q.a_begin + a.atoms_per_split) - q.a_begin);
-    if (S > 5 && a.guard && q.prob != seen) {
-      seen = q.prob;
-      const int* g = a.guard + (int64_t)q.prob * GUARD_WORDS;
-      bad = g[GUARD_BAD];
-      few = !bad && !counts_hold(g, a.guard_k);
+    q.check = false;
+    if (S > 5 && a.guard) {
+      if (a.guard[(int64_t)q.prob * GUARD_WORDS + GUARD_BAD])
+        q.n_atoms = 0;  // (no role has anything to do in the tile)
+      else
+        q.check = q.a_begin == 0;
     }
-    if (bad) q.n_atoms = 0;  // (no role has anything to do in the tile)
-    q.check = few && q.a_begin == 0;
     q.n_chunks = (q.n_atoms + a.atoms_per_chunk - 1) / a.atoms_per_chunk;
     return q;
   };
@@ -350,17 +347,22 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
       for (int t = blockIdx.x; t < a.total_tiles && run; t += gridDim.x) {
         const Tile q = tile_of(t);
         if (S > 5 && q.check) {
-          for (int j = 0; j < a.check_atoms; ++j, ++jg) {
+          // up to S atoms at once, in the places of the slices
+          for (int j = 0; j < a.check_atoms; j += S, ++jg) {
             const int stage = jg % NSTAGE, use = jg / NSTAGE;
             if (!mbar_wait(empty + stage, (use & 1) ^ 1, abort_flag, a.status)) {
               run = false;
               break;
             }
             uint8_t* sA = smem + stage * STAGE_BYTES;
-            mbar_expect_tx(full + stage, A_BYTES + B_BYTES);
-            const int k = j * a.check_step * KAS;
-            tma_load_3d(&tmA, full + stage, sA, k, q.prob * a.Mp + q.m0, S);
-            tma_load_3d(&tmB, full + stage, sA + S * A_BYTES, k, q.prob * a.N2p + q.n0, S);
+            uint8_t* sB = sA + S * A_BYTES;
+            const int n = min(S, a.check_atoms - j);
+            mbar_expect_tx(full + stage, n * (A_BYTES + B_BYTES));
+            for (int s = 0; s < n; ++s) {
+              const int k = (j + s) * a.check_step * KAS;
+              tma_load_3d(&tmA, full + stage, sA + s * A_BYTES, k, q.prob * a.Mp + q.m0, S);
+              tma_load_3d(&tmB, full + stage, sB + s * B_BYTES, k, q.prob * a.N2p + q.n0, S);
+            }
           }
           if (!run) break;
         }
@@ -393,7 +395,7 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
           const int buf = cg & 1, use = cg >> 1;
           if (!mbar_wait(tempty + buf, (use & 1) ^ 1, abort_flag, a.status)) break;
           tc_fence_after();
-          for (int j = 0; j < a.check_atoms; ++j, ++jg) {
+          for (int j = 0; j < a.check_atoms; j += S, ++jg) {
             const int stage = jg % NSTAGE, su = jg / NSTAGE;
             if (!mbar_wait(full + stage, su & 1, abort_flag, a.status)) {
               run = false;
@@ -401,11 +403,15 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
             }
             tc_fence_after();
             const uint32_t sA = smem_u32(smem + stage * STAGE_BYTES);
+            const uint32_t sB = sA + S * A_BYTES;
+            const int n = min(S, a.check_atoms - j);
+            for (int s = 0; s < n; ++s)
 #pragma unroll
-            for (int kk = 0; kk < KAS / 16; ++kk)
-              umma_bf16(tmem_base + (uint32_t)(buf * S * BN), sdesc<2 * KAS>(sA + kk * 32),
-                        sdesc<2 * KAS>(sA + S * A_BYTES + kk * 32), idesc_bf16(BM, BN),
-                        (j == 0 && kk == 0) ? 0u : 1u);
+              for (int kk = 0; kk < KAS / 16; ++kk)
+                umma_bf16(tmem_base + (uint32_t)(buf * S * BN),
+                          sdesc<2 * KAS>(sA + s * A_BYTES + kk * 32),
+                          sdesc<2 * KAS>(sB + s * B_BYTES + kk * 32), idesc_bf16(BM, BN),
+                          (j + s + kk == 0) ? 0u : 1u);
             umma_commit(empty + stage);
           }
           if (!run) break;
@@ -671,30 +677,13 @@ __device__ __forceinline__ uint32_t bf16_pair(uint32_t flo, uint32_t fhi) {
   return __byte_perm(flo, fhi, 0x7632);
 }
 
-// The leading 31 bits of an entry's magnitude from its digit word (8 slices: |x| 2^(62-e) as an
-// integer; one's complement, so at most one unit of 2^(e-30) off), for the guard
-__device__ __forceinline__ uint32_t leading_bits(long long w) {
+// floor(2^7 |x| / 2^e) as the bits of a float, from the digit word (8 slices: x 2^(62-e) as an
+// integer; the complement of a negative one, so at most one less)
+__device__ __forceinline__ uint32_t leading7(long long w) {
   const int h = (int)((w - DIGIT_BIAS<8>) >> 32);
-  return (uint32_t)(h ^ (h >> 31));
+  return __float_as_uint(__uint_as_float(0x4b000000u + ((uint32_t)(h ^ (h >> 31)) >> 23)) -
+                         8388608.0f);
 }
-// floor(2^7 |x| / 2^e) as the bits of a float
-__device__ __forceinline__ uint32_t leading7(uint32_t h) {
-  return __float_as_uint(__uint_as_float(0x4b000000u + (h >> 23)) - 8388608.0f);
-}
-// Adds to cnt[t - 2] how many of the warp's entries (leading bits h0, h1) are below 2^(e-t),
-// t = 2 .. 8 (at most 64: eight bits each).
-__device__ __forceinline__ void count_levels(uint32_t h0, uint32_t h1, int* cnt) {
-  auto below = [](uint32_t h) {
-    const int n = min(max(__clz((int)h) - 3, 0), GUARD_LEVELS);  // levels above |x|
-    return 0x0101010101010101ull & ((1ull << (8 * n)) - 1ull);
-  };
-  const unsigned long long w = below(h0) + below(h1);
-  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)w);
-  const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(w >> 32));
-  const int lane = threadIdx.x & 31;
-  if (lane < GUARD_LEVELS) cnt[lane] += ((lane < 4 ? lo : hi) >> (8 * (lane & 3))) & 255u;
-}
-
 template <typename T>
 struct PackSide {
   const T* src;
@@ -713,7 +702,7 @@ struct PackArgs {
   int* status;
   int* wide;           // 8 slices: word (problem / per) is set when an operand holds Inf or NaN,
   int per;
-  int* guard;          // or the words of split_guard.cuh are filled in, and the magnitudes'
+  int* guard;          // or the problem's word of split_guard.cuh is, and the magnitudes'
                        // leading bits go to one plane more
 };
 
@@ -737,8 +726,7 @@ __device__ __forceinline__ void copy_async(zdbl* dst, const zdbl* src, bool in, 
 
 template <typename T, bool SIDE_B, int S, int ROWS>
 __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T>& o, size_t plane,
-                                          int block, T* tiles, int* s_max, int* s_cnt,
-                                          int* s_exp) {
+                                          int block, T* tiles, int* s_max, int* s_exp) {
   using O = ops<T>;
   constexpr bool CPLX = O::cplx;
   constexpr int KT = CPLX ? 32 : 64;  // logical K of a tile: one 64-wide packed atom
@@ -805,7 +793,6 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
   for (int q = 0; q < RQ; ++q) {
     const int b = __reduce_max_sync(0xffffffffu, best[q]);
     if (lane == 0) s_max[warp + 8 * q] = b;
-    if (S > 5 && lane < 8) s_cnt[(warp + 8 * q) * 8 + lane] = 0;
   }
   __syncthreads();
   if (nranks > 1) cluster.sync();
@@ -823,7 +810,6 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
         set_status(g.status, CBC_ERR_NUMERICAL);
       }
     }
-    if (S > 5) s_cnt[tid * 8 + 7] = b < -1100 || r0 + tid >= o.rows;  // (without say in the guard)
     const bool zero = b < -1100;  // an all-zero (or padding) row
     b = zero ? 0 : b;
     s_exp[tid] = b;
@@ -851,11 +837,7 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
         const long long w0 = digit_word<S>(tile[lr * LD + 2 * lane], e);
         const long long w1 = digit_word<S>(tile[lr * LD + 2 * lane + 1], e);
         uint32_t* d = out + (size_t)(r0 + lr) * ld + t * 32 + lane;
-        if (S > 5 && g.guard) {
-          const uint32_t h0 = leading_bits(w0), h1 = leading_bits(w1);
-          count_levels(h0, h1, s_cnt + lr * 8);
-          d[S * pl] = bf16_pair(leading7(h0), leading7(h1));
-        }
+        if (S > 5 && g.guard) d[S * pl] = bf16_pair(leading7(w0), leading7(w1));
 #pragma unroll
         for (int sl = 0; sl < S; ++sl)
           d[sl * pl] = bf16_pair(digit_f32<S>(w0, sl), digit_f32<S>(w1, sl));
@@ -868,9 +850,7 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
         const long long wn = negated_word<S>(wi);
         uint32_t* d = out + (size_t)(SIDE_B ? 2 : 1) * (r0 + lr) * ld + t * 32 + lane;
         if (S > 5 && g.guard) {
-          const uint32_t hr = leading_bits(wr), hi = leading_bits(wi);
-          count_levels(hr, hi, s_cnt + lr * 8);
-          const uint32_t ar = leading7(hr), ai = leading7(hi);
+          const uint32_t ar = leading7(wr), ai = leading7(wi);
           d[S * pl] = bf16_pair(ar, ai);
           if (SIDE_B) d[S * pl + ld] = bf16_pair(ai, ar);
         }
@@ -887,37 +867,19 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
       }
     }
   }
-  if (S > 5 && g.guard) {
-    // the most entries of a row below each level, over the row blocks; the zeros behind K
-    // were counted as well
-    __syncthreads();
-    if (nranks > 1) cluster.sync();
-    if (rank == 0 && tid < ROWS * 8) {
-      const int t = tid & 7;
-      int v = 0;
-      if (!s_cnt[tid | 7]) {
-        v = (CPLX ? 2 : 1) * g.K - g.K2p;
-        for (int q = 0; q < nranks; ++q) v += cluster.map_shared_rank(s_cnt, q)[tid];
-      }
-      v = max(v, __shfl_xor_sync(0xffffffffu, v, 8));
-      v = max(v, __shfl_xor_sync(0xffffffffu, v, 16));
-      if (lane < GUARD_LEVELS && v > 0)
-        atomicMax(g.guard + (int64_t)blockIdx.z * GUARD_WORDS + (SIDE_B ? GUARD_B : 0) + t, v);
-    }
-  }
-  if (nranks > 1) cluster.sync();  // no CTA leaves while another still reads its shared memory
+  if (nranks > 1) cluster.sync();  // no CTA leaves while another still reads its row maxima
 }
 
 template <typename T, int S, int ROWS>
 __global__ void __launch_bounds__(256) pack_kernel(PackArgs<T> g) {
   extern __shared__ __align__(16) unsigned char pack_smem[];
-  __shared__ int s_max[ROWS], s_exp[ROWS], s_cnt[S > 5 ? ROWS * 8 : 1];
+  __shared__ int s_max[ROWS], s_exp[ROWS];
   T* tiles = reinterpret_cast<T*>(pack_smem);
   const int block = blockIdx.x / (int)cooperative_groups::this_cluster().num_blocks();
   if (block < g.blocks_a)
-    pack_rows<T, false, S, ROWS>(g, g.a, g.plane_a, block, tiles, s_max, s_cnt, s_exp);
+    pack_rows<T, false, S, ROWS>(g, g.a, g.plane_a, block, tiles, s_max, s_exp);
   else
-    pack_rows<T, true, S, ROWS>(g, g.b, g.plane_b, block - g.blocks_a, tiles, s_max, s_cnt, s_exp);
+    pack_rows<T, true, S, ROWS>(g, g.b, g.plane_b, block - g.blocks_a, tiles, s_max, s_exp);
 }
 
 // strides of the logical (row, k) indices at the origin, to pick the read pattern
@@ -1007,7 +969,7 @@ bool make_map(CUtensorMap* m, void* base, int K2_pad, int64_t rows_pad, int S, i
   return r == CUDA_SUCCESS;
 }
 
-constexpr int CHECK_ATOMS = 64;  // of 32 entries, of the magnitudes' product
+constexpr int CHECK_ATOMS = 16;  // of 32 entries, of the magnitudes' product
 int atoms_per_chunk_for(int S) { return std::max(1, (1024 / S) / ka(S)); }
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -1100,12 +1062,12 @@ namespace {
 // The SIMT kernel walks K at ~1 us (real) or ~4 us (complex) per 16 terms whatever M and N
 // are, the split costs ~15 us of launches more.  cbc_gemm in all, SIMT / split / SIMT behind the
 // split (operands graded against each other), us:
-//   real     256 x 256 x 64 104 / 58 / 82; 1000 x 1000 x 28 101 / 78 / 125,
-//            x 1000 2117 / 139 / 2030
-//   complex  16 x 16 x 16 102 / 57 / 78, 1000 x 1000 x 8 164 / 94 / 211, x 24 297 / 91 / 321,
-//            128 x 2048 x 128 565 / 78 / 340
-// So a product that is turned down costs up to a quarter more where K is short and the tiles fill
-// the GPU, up to 8% more elsewhere, and less where the smaller tiles win.
+//   real     256 x 256 x 64 104 / 63 / 77; 1000 x 1000 x 28 101 / 62 / 137,
+//            x 1000 2117 / 139 / 2006
+//   complex  16 x 16 x 16 102 / 51 / 75, 1000 x 1000 x 8 164 / 90 / 200, x 24 297 / 90 / 321,
+//            128 x 2048 x 128 565 / 79 / 337
+// So a product that is turned down costs up to a third more where K is short and the tiles fill
+// the GPU, up to 8% more at other sizes that fill it, and less elsewhere (the smaller tiles).
 constexpr int SPLIT_MIN_K_REAL = 28, SPLIT_MIN_K_CPLX = 8;
 constexpr size_t SPLIT_MAX_BYTES = size_t(16) << 30;
 }  // namespace
@@ -1209,7 +1171,7 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
     args.status = status;
     args.guard = opt.guard;
     // of a long K at most CHECK_ATOMS atoms of the magnitudes, evenly apart: a part of the sum is
-    // below it too (64 x 64 x 8192 on one CTA 58 us with all of its atoms)
+    // below it too, and the line rises with the square root of K only
     args.check_step = (atoms + CHECK_ATOMS - 1) / CHECK_ATOMS;
     args.check_atoms = (atoms + args.check_step - 1) / args.check_step;
     args.guard_k = g.K2;
@@ -1276,7 +1238,7 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
 // ---- FP64 products on the tensor cores -------------------------------------------------
 // 8 slices hold 62 bits of an entry relative to its row's (column's) maximum; the kept products
 // of slices are summed exactly and rounded once to 53 bits (once more per K split).  Whether
-// that is as accurate as an FP64 sum is found while the operands are cut (split_guard.cuh);
+// that is as accurate as an FP64 sum every tile finds out for its entries (split_guard.cuh);
 // where it is not, the SIMT kernel behind does the problem (again).  Relative error against 80-bit sums, Gaussian
 // entries: 4e-17 to 2e-16 where the SIMT kernel has 1e-16 (K = 16) to 1e-15 (K = 1000).
 size_t gemm_f64_split_bytes(int M, int N, int K, bool cplx, int nb) {
