@@ -634,6 +634,9 @@ __device__ __forceinline__ int expo_bits(double x) {
 // per value would run on the narrow FP64 pipe of this part.
 // Returned is N + sum_{i<S-1} 128 256^i: its byte i is q_{S-1-i} + 128 for i < S-1, and its
 // bits from 8 (S-1) up are q_0.
+// Rows of subnormals below 2^LOW_ROW are scaled by 2^LOW_SHIFT before they are cut (5 slices or
+// fewer; exact)
+constexpr int LOW_ROW = -1021, LOW_SHIFT = 100;
 template <int S>
 constexpr long long DIGIT_BIAS =
     (long long)(0x8080808080808080ull & ((1ull << (8 * (S - 1))) - 1ull));
@@ -643,11 +646,11 @@ __device__ __forceinline__ long long digit_word(double x, int e) {
   const int ex = (int)((b >> 52) & 0x7ffu);
   const unsigned long long mant = (b & 0xfffffffffffffull) | (ex ? (1ull << 52) : 0ull);
   // N = mant 2^-sh; the largest exponent of a row, ex = e + 1022, has the smallest sh: -9 for 8
-  // slices, 14 and more for up to 5, or less where the whole row is subnormal
+  // slices, 14 and more for up to 5 (rows below LOW_ROW come scaled)
   constexpr int MIN_SH = 53 - head(S) - 8 * (S - 1);
   const int sh = MIN_SH + e + 1022 - (ex ? ex : 1);
   unsigned long long n;
-  if (sh <= 0)
+  if (MIN_SH < 1 && sh <= 0)
     n = mant << -sh;
   else
     n = sh < 64 ? (mant + ((1ull << (sh - 1)) - 1ull) + ((mant >> sh) & 1ull)) >> sh : 0ull;
@@ -726,7 +729,7 @@ __device__ __forceinline__ void copy_async(zdbl* dst, const zdbl* src, bool in, 
 
 template <typename T, bool SIDE_B, int S, int ROWS>
 __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T>& o, size_t plane,
-                                          int block, T* tiles, int* s_max, int* s_exp) {
+                                          int block, T* tiles, int* s_max, int* s_exp, int* s_low) {
   using O = ops<T>;
   constexpr bool CPLX = O::cplx;
   constexpr int KT = CPLX ? 32 : 64;  // logical K of a tile: one 64-wide packed atom
@@ -796,6 +799,7 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
   }
   __syncthreads();
   if (nranks > 1) cluster.sync();
+  bool low = false;
   if (tid < ROWS) {
     int b = s_max[tid];
     for (int q = 0; q < nranks; ++q)
@@ -812,11 +816,13 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
     }
     const bool zero = b < -1100;  // an all-zero (or padding) row
     b = zero ? 0 : b;
-    s_exp[tid] = b;
+    low = S <= 5 && b < LOW_ROW;
+    s_low[tid] = low;
+    s_exp[tid] = low ? b + LOW_SHIFT : b;
     if (rank == 0 && r0 + tid < o.rows)
       o.expo[(int64_t)blockIdx.z * o.ebs + r0 + tid] = S > 5 && g.guard && zero ? GUARD_ZERO_ROW : b;
   }
-  __syncthreads();
+  const bool any_low = __syncthreads_or(low);
   uint32_t* out = reinterpret_cast<uint32_t*>(o.out + (size_t)blockIdx.z * o.rows_pad * g.K2p);
   const size_t pl = plane / 2, ld = (size_t)g.K2p / 2;  // in words of two bf16
   const bool held = t_end - t_begin <= g.keep;  // the whole share is still there
@@ -828,6 +834,13 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
       load_tiles(t);
       __syncthreads();
     }
+    if (any_low)
+      for (int q = 0; q < NQ; ++q) {
+        const int lr = warp + 8 * (q % RQ);
+        T* x = tiles + (i * ROWS + lr) * LD + lane + 32 * (q / RQ);
+        if (s_low[lr]) *x = O::scale(0x1p100, *x);
+      }
+    __syncwarp();
 #pragma unroll 1
     for (int q = 0; q < RQ; ++q) {
       const int lr = warp + 8 * q;
@@ -873,13 +886,13 @@ __device__ __forceinline__ void pack_rows(const PackArgs<T>& g, const PackSide<T
 template <typename T, int S, int ROWS>
 __global__ void __launch_bounds__(256) pack_kernel(PackArgs<T> g) {
   extern __shared__ __align__(16) unsigned char pack_smem[];
-  __shared__ int s_max[ROWS], s_exp[ROWS];
+  __shared__ int s_max[ROWS], s_exp[ROWS], s_low[ROWS];
   T* tiles = reinterpret_cast<T*>(pack_smem);
   const int block = blockIdx.x / (int)cooperative_groups::this_cluster().num_blocks();
   if (block < g.blocks_a)
-    pack_rows<T, false, S, ROWS>(g, g.a, g.plane_a, block, tiles, s_max, s_exp);
+    pack_rows<T, false, S, ROWS>(g, g.a, g.plane_a, block, tiles, s_max, s_exp, s_low);
   else
-    pack_rows<T, true, S, ROWS>(g, g.b, g.plane_b, block - g.blocks_a, tiles, s_max, s_exp);
+    pack_rows<T, true, S, ROWS>(g, g.b, g.plane_b, block - g.blocks_a, tiles, s_max, s_exp, s_low);
 }
 
 // strides of the logical (row, k) indices at the origin, to pick the read pattern
