@@ -123,6 +123,7 @@ extern "C" {
 
 int cbc_heev(int dtype, int m, int kmax, int nb, void* A, double* lam_out, void* U_out,
              int mixed, void* stream) {
+  ScratchScope scope;
   if (!A || !lam_out || !U_out || m < 1 || kmax < 1 || kmax > m || nb < 1)
     return fail(CBC_ERR_INVALID_ARG, "cbc_heev: bad arguments");
   if (dtype != CBC_F64 && dtype != CBC_C128)
@@ -136,6 +137,7 @@ int cbc_heev(int dtype, int m, int kmax, int nb, void* A, double* lam_out, void*
 }
 
 int cbc_cholqr2(int dtype, int m, int n, int nb, void* S, void* stream) {
+  ScratchScope scope;
   if (!S || m < 1 || n < m || nb < 1)
     return fail(CBC_ERR_INVALID_ARG, "cbc_cholqr2: bad arguments (need 1 <= m <= n)");
   if (dtype != CBC_F64 && dtype != CBC_C128)

@@ -64,7 +64,8 @@ static size_t dtype_bytes(int dt) {
   }
 }
 
-// the pool of the current device, made on first use, that keeps up to `keep` bytes when idle
+// the pool of the current device, made on first use, that keeps up to `keep` bytes at a
+// synchronisation
 static cudaError_t device_pool(cudaMemPool_t (&pools)[64], uint64_t keep, cudaMemPool_t* pool) {
   static std::mutex mu;
   int dev = 0;
@@ -105,17 +106,32 @@ cudaError_t cbc::pool_malloc(void** p, size_t bytes, cudaStream_t s) {
   return e == cudaSuccess ? cudaMallocFromPoolAsync(p, bytes, pool, s) : e;
 }
 
-// Workspaces of 1 GB and more from a pool that gives back what exceeds 8 GB at the next
-// synchronisation, so that one very large product does not keep its slices for good.  Below
-// that nothing is mapped anew: 2.1 ms per GB, complex 4096 x 4096 x 4096 (1.8 GB of slices)
-// 15.4 ms, 19.2 if they went back each time.  (The Gram products of 128 benchmark instances in
-// FP64 have 7.2 GB of slices, at every cut.)
+// Workspaces of 1 GB and more come from a pool of their own, which keeps them through a call
+// and at its end (ScratchScope) gives back what exceeds 8 GB, so that one very large product does
+// not keep its slices for good.  Mapping memory anew takes 2.1 ms per GB: 128 benchmark instances
+// in FP64, with up to 7.2 GB of slices of many sizes at every cut, take 3478 ms a step and 3659 if
+// the pool is cut back at every synchronisation.
+static cudaMemPool_t g_scratch[64] = {};
+static std::atomic<bool> g_scratch_used[64];
+static std::atomic<int> g_scratch_calls{0};
+
 cudaError_t cbc::scratch_malloc(void** p, size_t bytes, cudaStream_t s) {
   if (bytes < (size_t(1) << 30)) return pool_malloc(p, bytes, s);
-  static cudaMemPool_t pools[64] = {};
   cudaMemPool_t pool;
-  cudaError_t e = device_pool(pools, uint64_t(8) << 30, &pool);
-  return e == cudaSuccess ? cudaMallocFromPoolAsync(p, bytes, pool, s) : e;
+  cudaError_t e = device_pool(g_scratch, UINT64_MAX, &pool);
+  if (e != cudaSuccess) return e;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  g_scratch_used[dev] = true;
+  return cudaMallocFromPoolAsync(p, bytes, pool, s);
+}
+
+cbc::ScratchScope::ScratchScope() { ++g_scratch_calls; }
+cbc::ScratchScope::~ScratchScope() {
+  // by the last of the calls under way
+  if (--g_scratch_calls != 0) return;
+  for (int dev = 0; dev < 64; ++dev)
+    if (g_scratch_used[dev].exchange(false)) cudaMemPoolTrimTo(g_scratch[dev], size_t(8) << 30);
 }
 
 static int build_network(Net* net, int kind, int n_nodes, const int32_t* parent,
@@ -392,6 +408,7 @@ static int apply_one(ttn_t state, ttno_t op, int64_t max_bond, double tol,
 
 int cbc_apply(ttn_t state, ttno_t op, int64_t max_bond, double tol, const cbc_options* opt,
               ttn_t* out) {
+  ScratchScope scope;
   return apply_one(state, op, max_bond, tol, opt, false, out);
 }
 
@@ -444,6 +461,7 @@ static int run_method(ttn_t state, ttno_t op, int64_t max_bond, double tol, Opti
 
 int zipup_apply(ttn_t state, ttno_t op, int64_t max_bond, double tol, const cbc_options* opt,
                 ttn_t* out) {
+  ScratchScope scope;
   if (!out) return fail(CBC_ERR_INVALID_ARG, "zipup_apply: out is NULL");
   *out = nullptr;
   int rc = check_chain_pair(state, op, "zipup_apply");
@@ -458,6 +476,7 @@ int zipup_apply(ttn_t state, ttno_t op, int64_t max_bond, double tol, const cbc_
 
 int direct_apply(ttn_t state, ttno_t op, int64_t max_bond, double tol, const cbc_options* opt,
                  ttn_t* out) {
+  ScratchScope scope;
   if (!out) return fail(CBC_ERR_INVALID_ARG, "direct_apply: out is NULL");
   *out = nullptr;
   int rc = check_chain_pair(state, op, "direct_apply");
@@ -472,6 +491,7 @@ int direct_apply(ttn_t state, ttno_t op, int64_t max_bond, double tol, const cbc
 
 int src_apply(ttn_t state, ttno_t op, int64_t sketch_size, const void* const* omega,
               int omega_dtype, int omega_on_device, const cbc_options* opt, ttn_t* out) {
+  ScratchScope scope;
   if (!out) return fail(CBC_ERR_INVALID_ARG, "src_apply: out is NULL");
   *out = nullptr;
   int rc = check_chain_pair(state, op, "src_apply");
@@ -556,6 +576,7 @@ int cbc_rank_rule(int n, const double* w, double beyond, int64_t max_bond, doubl
 
 int cbc_apply_batched(int n, const ttn_t* states, const ttno_t* ops, const int64_t* max_bond,
                       const double* tol, const cbc_options* opt, int workers, ttn_t* outs) {
+  ScratchScope scope;
   if (n < 0 || (n > 0 && (!states || !ops || !outs)))
     return fail(CBC_ERR_INVALID_ARG, "cbc_apply_batched: bad arguments");
   for (int j = 0; j < n; ++j) outs[j] = nullptr;
@@ -676,6 +697,7 @@ int cbc_apply_batched(int n, const ttn_t* states, const ttno_t* ops, const int64
 int cbc_gemm(int precision, int slices, int dtype, int M, int N, int K, const void* A,
              int64_t lda, int transA, int conjA, const void* B, int64_t ldb, int transB,
              int conjB, void* C, int64_t ldc, void* stream) {
+  ScratchScope scope;
   if (!A || !B || !C || M < 1 || N < 1 || K < 1 || ldc < N)
     return fail(CBC_ERR_INVALID_ARG, "cbc_gemm: bad arguments");
   if (dtype != CBC_F64 && dtype != CBC_C128)

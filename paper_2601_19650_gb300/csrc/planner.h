@@ -117,8 +117,13 @@ void note_flops(int cls, double flops);
 // stream-ordered device allocation from the library's own pool on the current device
 // (freed with cudaFreeAsync); the caller's default pool is never touched
 cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t s);
-// the same for workspaces that callers can do without; large ones are not kept
+// the same for workspaces that callers can do without; of large ones a bounded amount is kept
+// behind a call (one ScratchScope)
 cudaError_t scratch_malloc(void** p, size_t bytes, cudaStream_t s);
+struct ScratchScope {
+  ScratchScope();
+  ~ScratchScope();
+};
 
 // gemm_f64_split with slices from the library's pool where that is the faster way and the
 // pool has room for them, else gemm_f64
