@@ -70,9 +70,11 @@ enum cbc_dtype { CBC_F32 = 0, CBC_F64 = 1, CBC_C64 = 2, CBC_C128 = 3 };
 
 /* Arithmetic of cbc_apply.
  * CBC_PREC_FP64 : every contraction, Gram matrix, eigensolve, Cholesky and triangular
- *                 solve in FP64.  Products whose operands' rows span less than 2^36 run on
- *                 the tensor cores with 8 bf16 slices per operand, summed exactly and
- *                 rounded to FP64 at the end; the others on the FP64 pipes.
+ *                 solve in FP64.  A product runs on the tensor cores with 8 bf16 slices
+ *                 per operand where every entry of |A| |B| is large enough beside its row's
+ *                 and column's largest entries that the error is within that of an FP64
+ *                 sum, K 2^-53 (|A| |B|); else (operands graded against each other along K,
+ *                 Inf, NaN, short K) on the FP64 pipes.
  * CBC_PREC_MIXED: the dense contractions and Gram products run on the tensor cores
  *                 (tcgen05) with bf16 operand slices and FP32 partial sums that are
  *                 combined in FP64; the eigensolve, Cholesky and triangular solves stay
@@ -253,8 +255,9 @@ int ttno_destroy(ttno_t t); /* NULL is a no-op */
 /* Dense product used by every contraction of the sweeps, exposed as a building block
  * (and for kernel-level tests): C = op(A) op(B) with row-major DEVICE matrices of
  * dtype CBC_F64 or CBC_C128.  op(X) = X, X^T (trans), conj(X) (conj) or X^H (both).
- *   precision  CBC_PREC_FP64: FP64 accuracy (see cbc_apply); CBC_PREC_MIXED: tensor cores with `slices`
- *              bf16 slices per operand (2..5; 0 = 4), exact FP32 partial sums, FP64
+ *   precision  CBC_PREC_FP64: entry by entry within the error of an FP64 sum (see
+ *              enum cbc_prec); CBC_PREC_MIXED: tensor cores with `slices` bf16 slices per
+ *              operand (2..5; 0 = 4), exact FP32 partial sums, FP64
  *              result (see cbc_apply)
  *   M, N, K    op(A) is M x K, op(B) is K x N, C is M x N (ldc >= N), K >= 1
  *   lda, ldb   leading dimensions of A and B as stored

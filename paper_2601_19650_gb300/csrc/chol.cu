@@ -536,8 +536,8 @@ cudaError_t cholesky_lower(T* G, int m, int* status, void* bar, int num_sms, cud
                            int nb, bool steady) {
   // the rows in the shared memory of one cluster per matrix: as many CTAs (and FP64 units) as
   // the batch leaves idle, 4 rows each at least; where that is one, a kernel without a cluster.
-  // (`steady`: the column blocks below, one CTA per matrix from 8 matrices on.  A change of the
-  // order of these sums by 1e-16 has moved mixed results on 64-bit data by 2e-9.)
+  // (`steady`: the earlier choice, the column blocks below, one CTA per matrix from 8 matrices on.
+  // A change of the order of these sums by 1e-16 has moved mixed results on 64-bit data by 2e-9.)
   const size_t tri_bytes = (size_t)m * (m + 1) / 2 * sizeof(T);
   if (!steady) {
     const void* kc = (const void*)chol_cluster_kernel<T>;
@@ -631,7 +631,9 @@ cudaError_t trsm_products(const T* C, T* S, int m, int n, int* status, void* ws,
     return p;
   };
   TcWide set;
-  set.wide = reinterpret_cast<int*>(take(4));  // (Inf and NaN are met by the next Gram)
+  // Not read: S has finite rows of unit norm and C is the factor of its Gram, which a row with Inf
+  // or NaN would have failed (the call then returns that status whatever the solve makes of it).
+  set.wide = reinterpret_cast<int*>(take(4));
   T* D = reinterpret_cast<T*>(take(2 * nb * bs * sizeof(T)));
   T* Inv = D + nb * bs;
   T* tmp = reinterpret_cast<T*>(take(sizeof(T) * nb * nblk * hf));

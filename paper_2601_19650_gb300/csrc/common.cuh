@@ -169,8 +169,9 @@ __device__ __forceinline__ double rsqrt64(double x) {
 }
 
 // The same in the way of rcp64: r (1 + e/2 + 3 e^2/8) with e = 1 - x r^2, five dependent
-// operations.  (The pivots of Cholesky keep rsqrt64: whether a rank-deficient block breaks
-// down hangs on its last bit.)
+// operations.  (chol1_kernel and chol_kernel keep rsqrt64 for their pivots: whether a
+// rank-deficient block breaks down hangs on its last bit.  chol_cluster_kernel updates with
+// 1 / pivot and takes its roots from here.)
 __device__ __forceinline__ double rsqrt64_short(double x) {
   const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
   if (ex - 1u >= 2046u) return rsqrt64(x);

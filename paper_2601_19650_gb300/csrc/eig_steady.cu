@@ -2,9 +2,12 @@
 //
 // A slice of the mixed path's products has a last digit of 2^-31 of a row's maximum, so a
 // change of rounding of 1e-13 in an eigenvector turns some digits over and moves a whole
-// chain's result by 1e-9 to 6e-9: less than its error, but more than 64-bit results may move
-// from one version of this library to the next.  The order of the sums in these kernels is
-// therefore fixed.  Data of 32 bits carries 6e-8 of its own and takes eig.cu, as FP64 calls do
+// chain's result by 1e-9 to 6e-9: less than its error (1e-8 to 1e-7), but more than 64-bit
+// results should move from one version of this library to the next.  These are therefore the
+// earlier solvers, with their operations in their order.  That order is not fixed altogether:
+// large lone matrices add v^H p over the CTAs by atomics in order of arrival, the products around
+// add K splits by atomics and pick their tile width by timing, and now and then (8 of 112 cases)
+// the same call moves as much from process to process.  Data of 32 bits carries 6e-8 of its own and takes eig.cu, as FP64 calls do
 // (their results move by 1e-13).  64 of 256 x 256 complex: 13.6 ms here, 10.1 ms there; one of
 // 256 x 256 complex in FP64: 2.9 and 1.4 ms for the reduction.
 //

@@ -28,12 +28,11 @@
 // Kernel: persistent, one CTA per SM (cta_group::1) looping over 128 x BN output tiles of
 // all the problems of a call (a lockstep group of CBC instances is one call).  Warp 0
 // issues TMA loads of 64-wide K atoms (32-wide for 8 slices; S slices of A and of B per
-// atom, 128B or 64B swizzle, two smem stages), warp 1 issues tcgen05.mma (one elected thread; one MMA per slice of A,
-// against all the slices of B it meets side by side) into S TMEM accumulators per K chunk,
-// double buffered across chunks and tiles so the epilogue of
-// one chunk overlaps the MMAs of the next, and 4 epilogue warps per 16
-// columns drain TMEM (tcgen05.ld) into int64 registers and write FP64, assembled with integer
-// operations.  Every wait is bounded (clock64); a timeout raises CBC_ERR_TIMEOUT in the
+// atom, 128B or 64B swizzle, two smem stages), warp 1 issues tcgen05.mma (one elected thread;
+// one MMA per slice of A, against all the slices of B it meets side by side) into S TMEM
+// accumulators per K chunk, double buffered across chunks and tiles so the epilogue of one chunk
+// overlaps the MMAs of the next, and 4 epilogue warps per 16 columns drain TMEM (tcgen05.ld) into
+// int64 registers and write FP64, assembled with integer operations.  Every wait is bounded (clock64); a timeout raises CBC_ERR_TIMEOUT in the
 // status word, all roles leave their loops, and TMEM is freed before the CTA exits.
 #include <cooperative_groups.h>
 #include <cuda.h>
@@ -442,8 +441,9 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
             // B: level s + t) back to back in TMEM, so they are one operand of (S-s) BN
             // columns.  Issued one pair of slices at a time the MMAs were bound by reading
             // A's 4 KB from shared memory again for every BN columns (8192 x 4096 x 1024
-            // complex, S = 5: 5.1 ms; stacked 3.3 ms, then bound by L2 reads of the slices).  s = 0 covers every
-            // level, so its first MMA of a chunk clears them all.
+            // complex, S = 5: 5.1 ms; stacked 3.3 ms: 39 GB of slices from L2 by the tiles' shapes,
+            // tensor pipe busy 59% of the time).  s = 0 covers every level, so its first MMA of a
+            // chunk clears them all.
 #pragma unroll
             for (int kk = 0; kk < KAS / 16; ++kk) {
 #pragma unroll
@@ -545,7 +545,8 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
         const int ea = rowok ? a.expA[q.prob * a.Mp + row] : 0;
         const int bias = -2 * head(S) - 8 * (S - 1);
         const int64_t ro = rowok ? a.vc.roff(row) : 0;
-        const bool pair = a.cplx && !a.atomic && !a.acc && (reinterpret_cast<uintptr_t>(a.C) & 15) == 0;
+        const bool pair =
+            a.cplx && !a.atomic && !a.acc && (reinterpret_cast<uintptr_t>(a.C) & 15) == 0;
         auto value = [&](int i, int e) {
           if constexpr (NACC == 2)
             return i96_ldexp(acc[0][i], acc[1][i], e);
@@ -604,14 +605,15 @@ __global__ void __launch_bounds__(nthreads(BN), 1)
 // those rows' K range.  The elements are copied to shared memory once, along whichever index
 // is contiguous in memory and all at once (up to `keep` tiles; a longer share is copied a
 // second time, from L2), the rows' exponents are combined through the cluster's shared
-// memory, and the slices leave coalesced along K to the [S][rows][K2_pad] planes.  Bound by HBM: 16 B read
-// and 4 S (A) or 8 S (B) B written per complex element.  Rows of padding are not written:
+// memory, and the slices leave coalesced along K to the [S][rows][K2_pad] planes.  16 B are read
+// and 4 S (A) or 8 S (B) B written per complex element; 4096 x 4096 x 1024 with 5 slices keeps
+// issue slots 54% and DRAM 38% busy: between the arithmetic on digits and the wait for the one
+// copy in, three CTAs of an SM at a time.  Rows of padding are not written:
 // they reach only rows and columns of the accumulators that the epilogue skips.
 constexpr int PACK_ROWS = 32;
 // tiles held in shared memory: more cover a longer share in one copy, fewer leave room for
 // other CTAs on the SM
-constexpr int PACK_KEEP = 4, PACK_KEEP_FEW = 8;
-constexpr int PACK_FEW_CTAS = 304;
+constexpr int PACK_KEEP = 4;
 constexpr int PACK_CLUSTER = 8;  // most CTAs that share the K range of one row block
 
 // exponent of |x| (biased-exponent field) without FP64 arithmetic: max|x| < 2^e with
@@ -1252,8 +1254,10 @@ cudaError_t gemm_tc(int M, int N, int K, const T* A, const View& va, bool conjA,
 // 8 slices hold 62 bits of an entry relative to its row's (column's) maximum; the kept products
 // of slices are summed exactly and rounded once to 53 bits (once more per K split).  Whether
 // that is as accurate as an FP64 sum every tile finds out for its entries (split_guard.cuh);
-// where it is not, the SIMT kernel behind does the problem (again).  Relative error against 80-bit sums, Gaussian
-// entries: 4e-17 to 2e-16 where the SIMT kernel has 1e-16 (K = 16) to 1e-15 (K = 1000).
+// where it is not, the SIMT kernel behind does the problem (again).  Largest error
+// in units of 2^-53 |A| |B|, SIMT kernel / split: Gaussian 64 x 64 x 28 2.4 / 0.5, complex
+// 501 x 777 x 1030 1.3 / 0.07; positive entries 300 x 300 x 100 8.2 / 1.0; half of the entries
+// zero 1.9 / 0.4; rows and columns scaled by 2^-30 to 2^30 2.4 / 0.2.
 size_t gemm_f64_split_bytes(int M, int N, int K, bool cplx, int nb) {
   if (K < (cplx ? SPLIT_MIN_K_CPLX : SPLIT_MIN_K_REAL)) return 0;
   const size_t b = gemm_tc_workspace_bytes(M, N, K, cplx, 9, nb) +  // (8 slices, the magnitudes)

@@ -64,8 +64,9 @@ cudaError_t gemm_f64(int M, int N, int K, int batch, const T* A, const View& va,
 // (guard: not NULL: only the problems that split_holds, split_guard.cuh, turns down.)
 
 // The FP64 product as 8 bf16 slices per operand on the tensor cores, where their error is no
-// larger than an FP64 sum's; the other problems through gemm_f64 (gemm_tc.cu, split_guard.cuh).  gemm_f64_split_bytes gives the bytes it needs at `ws`, or 0
-// where gemm_f64 is to be used: small products, and slices beyond 16 GB.
+// larger than an FP64 sum's; the other problems through gemm_f64 (gemm_tc.cu, split_guard.cuh).
+// gemm_f64_split_bytes gives the bytes it needs at `ws`, or 0 where gemm_f64 is to be used: short
+// sums, and slices beyond 16 GB.
 size_t gemm_f64_split_bytes(int M, int N, int K, bool cplx, int nb);
 template <typename T>
 cudaError_t gemm_f64_split(int M, int N, int K, int nb, const T* A, const View& va, bool conjA,
@@ -123,8 +124,8 @@ cudaError_t tridiag_cluster(const T* A, int m, double* d, double* e, T* tau, T* 
                             size_t wb, int nb, const TriClusterShape& sh, bool df,
                             cudaStream_t s);
 
-// The same outputs with a fixed order of all sums, for mixed calls on 64-bit data (eig_steady.cu
-// says why); workspace: nb * eig_workspace_bytes_steady(m, kmax).
+// The same outputs from the earlier solvers, for mixed calls on 64-bit data (eig_steady.cu says
+// why); workspace: nb * eig_workspace_bytes_steady(m, kmax).
 size_t eig_workspace_bytes_steady(int m, int kmax, bool cplx);
 template <typename T>
 cudaError_t heev_top_steady(T* A, int m, int kmax, double* lam, T* U, void* work, int* status,
@@ -138,8 +139,8 @@ cudaError_t tridiag_cluster_steady(const T* A, int m, double* d, double* e, T* t
 
 // ---- Cholesky QR (FP64) ------------------------------------------------------------
 // Q = C^{-1} S with G = S S^H = C C^H, S: m x n (m <= n), row-major, in place on S.
-// nb problems: G, C m*m and S m*n elements apart; `bar` holds nb GridBarriers.  `steady`: a fixed
-// order of the sums, for mixed calls on 64-bit data.
+// nb problems: G, C m*m and S m*n elements apart; `bar` holds nb GridBarriers.  `steady`: the
+// earlier kernels, for mixed calls on 64-bit data.
 template <typename T>
 cudaError_t cholesky_lower(T* G, int m, int* status, void* bar, int num_sms, cudaStream_t s,
                            int nb = 1, bool steady = false);
@@ -149,9 +150,8 @@ template <typename T>
 cudaError_t trsm_lower_left(const T* C, T* S, int m, int n, int* status, void* bar,
                             int num_sms, cudaStream_t s, int nb = 1, void* dfbuf = nullptr);
 // The same solve by products on the tensor cores, to FP64 accuracy (`df`: the other way would
-// be double-float): `ws` holds
-// trsm_products_bytes (0 where trsm_lower_left is the better way) bytes; S has
-// rows of unit norm.
+// be double-float): `ws` holds trsm_products_bytes (0 where trsm_lower_left is the better way)
+// bytes; S has rows of unit norm.
 size_t trsm_products_bytes(int m, int n, bool cplx, int nb, bool df);
 template <typename T>
 cudaError_t trsm_products(const T* C, T* S, int m, int n, int* status, void* ws, cudaStream_t s,

@@ -121,7 +121,7 @@ T host_one() {
 struct Prec {
   bool mixed = false;
   bool cholqr_f64 = false;  // CholeskyQR2's Gram in FP64 even on the mixed path
-  bool steady = false;      // mixed on 64-bit data: a fixed order of all sums (eig_steady.cu)
+  bool steady = false;      // mixed on 64-bit data: the earlier solvers (eig_steady.cu)
   int s_fwd = 5, s_bwd = 4;
   Arena* ar = nullptr;
   int* status = nullptr;

@@ -8,7 +8,8 @@
 // S / 2^(ea+eb) is at least 2^-8.2 sqrt(K) and 2^-6 for every entry of the product: its error is
 // then at most 4.6 sqrt(K) u S and K u S, and on digits that are not all alike about u S / 2.
 // S is bounded from below by the product of the magnitudes' leading 7 bits (gemm_tc.cu, one chunk
-// more of every tile): S / 2^(ea+eb) >= 2^-14 sum_k floor(2^7 |a_k| / 2^ea) floor(2^7 |b_k| / 2^eb).
+// more of every tile):
+//   S / 2^(ea+eb) >= 2^-14 sum_k floor(2^7 |a_k| / 2^ea) floor(2^7 |b_k| / 2^eb).
 // Gaussian operands are a factor of 2^3.5 to 2^6 above the line, the contractions and Gram
 // products of an FP64 application by at least 4 (but for a few whose operands are graded); operands
 // graded against each other along K are below it.

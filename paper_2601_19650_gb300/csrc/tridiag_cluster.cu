@@ -22,7 +22,7 @@
 // cover its dependent operations.  Two barriers,
 // one row at a time and the update behind the scalars / this, double-float: 64 of m = 256 complex
 // 7.9 / 7.2 ms, 8 of 512 real 6.9 / 6.0, 64 of 64 complex 0.60 / 0.38; FP64: 2 of 512 real 10.1
-// / 7.0.  (Issue slots 41% busy, FP32 pipe 27%, at m = 256.)
+// / 7.0.  (16 of m = 256 complex: issue slots of the busy SMs 37%, FP32 pipe 29%.)
 // DF (the mixed path): the rows and every per-element quantity as double-float pairs, so all
 // O(m) and O(m^2) work per column runs in FP32 arithmetic with error-free transformations;
 // FP64 only for the handful of Householder scalars.  Otherwise FP64 throughout.
@@ -49,7 +49,7 @@ struct TriClArgs {
   int m;
   double* d;       // per-matrix outputs, workspaces wb bytes apart:
   double* e;       //   diagonal, off-diagonal (beta_j), tau_j, and the reflectors
-  T* tau;          //   V (row j: [j] = tau_j, [j+1] = 1, [c] = v_c)
+  T* tau;          //   V (row j: [j+1] = 1, [c] = v_c for c > j + 1)
   T* V;
   int64_t a_bs;    // elements between consecutive matrices A
   size_t wb;       // bytes between consecutive workspaces
@@ -476,9 +476,9 @@ TriClusterShape tridiag_cluster_shape(int m, int nb, bool df) {
   static_assert(sizeof(typename dfof<T>::type) == sizeof(T), "double-float element size");
   // Double-float: the fewest CTAs (at least 4) that hold the matrix, since every CTA repeats
   // the O(m) work of a column; 8 warps where m gives them rows (4 warps cost 8 of m = 512
-  // real 23% more, 8 warps cost 64 of 64 complex 21% more).  FP64: as many SMs' FP64 units as the batch
-  // leaves idle (2 of m = 512 real on 8 / 16 CTAs 8220 / 6960 us; 4 of 256 complex on 4 / 8 / 16
-  // 7010 / 5210 / 5290).
+  // real 23% more, 8 warps cost 64 of 64 complex 21% more).  FP64: as many SMs' FP64 units as the
+  // batch leaves idle (2 of m = 512 real on 8 / 16 CTAs 8220 / 6960 us; 4 of 256 complex on 4 /
+  // 8 / 16 7010 / 5210 / 5290).
   const int lead = m > 256 || !df ? 256 : 128;
   int low = 4;
   if (!df)

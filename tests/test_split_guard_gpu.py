@@ -119,9 +119,9 @@ def test_forms(kind, cplx):
 @pytest.mark.parametrize("cplx", [False, True])
 @pytest.mark.parametrize("shape", [(300, 200, 1100), (129, 65, 64), (257, 64, 2049), (20, 20, 28)])
 @pytest.mark.parametrize("r", [2, 4, 6, 9, 14, 22])
-def test_entries_where_counts_are_too_few(r, shape, cplx):
-    """Half of every row below 2^-9: the counts don't decide, the magnitudes' product does.  Then
-    the last row and column are graded against each other, which their one entry shows."""
+def test_one_entry_below_the_line(r, shape, cplx):
+    """Half of every row small, in the same places in A and B, and then the last row and column
+    graded against each other besides, which one entry of the last tile shows."""
     rng = np.random.default_rng([r, shape[0], cplx])
     M, N, K = shape
     A, B = _rand(rng, (M, K), cplx), _rand(rng, (K, N), cplx)
